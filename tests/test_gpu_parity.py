@@ -229,6 +229,32 @@ def test_select_ragged_batch_and_ties():
     _select_case([32, 128, 64], 196, 100, 4, ties=True)
 
 
+@pytest.mark.parametrize("F,T", [(1, 1), (1, 31), (1, 33), (8, 256), (1, 2049), (1024, 8), (683, 12), (3, 8191), (24577, 1),
+                                 (7, 3511), (1024, 28), (14336, 2), (1, 57298), (28, 2045)])
+def test_select_at_the_edges_of_its_launch_shapes(F, T):
+    """Token counts around the cluster sizes and keys per thread of the selection kernel, one frame of
+    every token and 1024 frames; scores with ties, all equal, and spread over the whole exponent range.
+    Indices and counts are exact."""
+    if F > 1024:
+        F, T = 1, F * T
+    nv = F * T
+    rng = np.random.default_rng(nv)
+    wide = np.exp2(rng.uniform(-140, 0, nv)).astype(np.float32)
+    for i, s in enumerate((rng.random(nv).astype(np.float32), (rng.integers(0, 3, nv) * 0.25).astype(np.float32),
+                           np.full(nv, 0.5, np.float32), wide)):
+        kt, k1 = (nv // 3, nv // 7) if i != 1 else (nv - nv // 5, nv // 2)
+        dev = torch.from_numpy(s).cuda()
+        got = specvlm.select(dev, [0, nv], [F], T, [k1], [kt], [0, kt]).cpu().numpy()[:kt]
+        assert np.array_equal(got, oracle.select(s, F, T, k1, kt))
+        kept, n1 = specvlm.select_top_p(dev, [0, nv], [F], T, [400], [kt], [0, kt])
+        ref, ref_k1 = oracle.select_top_p(s, F, T, 400, kt)
+        assert int(n1[0]) == ref_k1 and np.array_equal(kept.cpu().numpy()[:kt], ref)
+
+
+def test_select_batch_of_long_sequences():
+    _select_case([128, 32, 128, 1] * 4, 196, 100, 6)
+
+
 def test_select_stage_split_extremes():
     # k1 = 0 (Stage II only), k1 = k_total (Stage I only)
     rng = np.random.default_rng(5)
