@@ -19,7 +19,7 @@
 namespace specvlm {
 
 constexpr int kSchedMaxBatch = 127;     // sequences per call (their tile counts live in shared memory)
-constexpr int kSchedMinTilesPerCta = 4;   // below this a slice is not worth a CTA of its own
+constexpr int kSchedMinTilesPerCta = 2;   // below this a slice is not worth a CTA of its own (a tile per softmax group)
 
 // Number of CTAs that get a non-empty slice.
 SPECVLM_HD int sched_active_ctas(int64_t total_tiles, int grid) {

@@ -5,7 +5,7 @@
 //
 // One persistent CTA per SM streams a contiguous slice of the flat (layer, sequence, KV head, tile)
 // list (attn_sched.h), so the cache is read exactly once, every SM moves the same number of bytes
-// and only two partial results per CTA ever touch scratch memory.  A tile is 128 tokens: two
+// and only two partial results per CTA ever touch scratch memory (attn_merge_kernel folds them).  A tile is 128 tokens: two
 // 64-token sub-tiles (one cache page each) as the TMA moves them.
 //
 // Roles inside a CTA (12 warps = 3 warpgroups; the first gives registers to the other two):
@@ -39,7 +39,7 @@ struct AttnTcParams {
   float* lse;                 // [L][B][n_win][Hq] or null
   float* ws_o;                // partial results: [2 * grid][rows][D], normalised
   float* ws_lse;              // [2 * grid][rows], log2 units
-  int32_t* ws_cnt;            // [items] arrival counters, zero at launch
+  int4* ws_cut;               // [grid]: the cut item whose first part a CTA holds, see attn_merge_kernel
   const int32_t* block_table; // [B][max_blocks] or null
   const int32_t* seq_lens;    // [B]
   int32_t* d_status;
@@ -190,7 +190,7 @@ struct TcCfg {
   static constexpr int OFF_Q = OFF_V + NVP * 2 * SUB_BYTES;
   static constexpr int OFF_P = OFF_Q + NQ * Q_BYTES;
   static constexpr int BIG = OFF_P + 2 * P_BYTES;
-  static constexpr int N_BARS = 2 * NKP + 2 * NVP + 17;
+  static constexpr int N_BARS = 2 * NKP + 2 * NVP + 15;
   static constexpr int SM_BAR = 0;
   static constexpr int SM_MISC = SM_BAR + 8 * N_BARS;
   static constexpr int SM_PREFIX = SM_MISC + 32;
@@ -204,6 +204,22 @@ struct TcCfg {
   static constexpr uint32_t TMEM_COLS = 512;
   static_assert(SMALL + BIG <= kMaxSmem, "shared-memory plan does not fit");
 };
+
+// Which item, if any, this CTA's slice holds the first part of while a slice boundary cuts it: (layer *
+// batch + sequence, KV head, scratch slot of the first part, number of parts), no parts if there is none.
+// Written before any wait, so that the merge never reads a stale entry.
+__device__ __forceinline__ void publish_cut_item(const AttnTcParams& p, bool active, int cta, int gcta, int n_active,
+                                                 int64_t total, int64_t T0, int64_t T1, const int* prefix) {
+  int4 cut = make_int4(0, 0, 0, 0);
+  if (active && T1 < total) {
+    const Segment s = segment_at(T1 - 1, T1, prefix, p.batch, p.n_kv_heads);   // the item of the slice's last tile
+    const int64_t item_end = s.item_begin + s.item_tiles;
+    if (item_end > T1 && s.item_begin >= T0)
+      cut = make_int4(s.layer * p.batch + s.b, s.g, partial_slot(gcta, T0, s.item_begin),
+                      slice_owner(item_end - 1, n_active, total) - cta + 1);
+  }
+  p.ws_cut[gcta] = cut;
+}
 
 // TREE: the window's visibility comes from per-token ancestor masks instead of the chain rule.
 // A template parameter, not a run-time branch: the chain kernel's code is untouched by the tree
@@ -236,11 +252,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const uint32_t bar_o_full = bar_p_empty + 16;
   const uint32_t bar_o_empty = bar_o_full + 8;
   const uint32_t bar_ep_stats = bar_o_empty + 8;       // both groups' row statistics are in shared memory
-  const uint32_t bar_ep_done = bar_ep_stats + 8;       // a partial result has been written
-  const uint32_t bar_ep_flag = bar_ep_done + 8;        // ... and the arrival counter has been read
   volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem_raw + C::SM_MISC);
   volatile uint32_t* const tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_raw + C::SM_MISC + 8);
-  volatile int* const last_flag = reinterpret_cast<volatile int*>(smem_raw + C::SM_MISC + 16);
   volatile int* const any_empty = reinterpret_cast<volatile int*>(smem_raw + C::SM_MISC + 20);
   int* const prefix = reinterpret_cast<int*>(smem_raw + C::SM_PREFIX);
   float2* const stats = reinterpret_cast<float2*>(smem_raw + C::SM_STATS);
@@ -249,11 +262,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 
   // the plan needs the tiles inside the allocation (true whenever the base is 1024-byte aligned)
   if (big + C::BIG > raw_addr + C::TOTAL) {
-    if (tid == 0 && p.d_status) *p.d_status = SPECVLM_ERR_CUDA;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tid == 0) {
+      p.ws_cut[blockIdx.x] = make_int4(0, 0, 0, 0);
+      if (p.d_status) *p.d_status = SPECVLM_ERR_CUDA;
+    }
     return;
   }
 
   // ------------------------------------------------------------------ set-up
+  // Everything up to griddepcontrol.wait touches no global memory and runs while the kernel before
+  // this one drains; one barrier separates the set-up from the roles.
   if (tid == 0) {
     for (int s = 0; s < NKP; ++s) {
       mbar_init(bar_k_full + 8 * s, 1);
@@ -274,32 +293,39 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     mbar_init(bar_o_full, 1);
     mbar_init(bar_o_empty, 8);
     mbar_init(bar_ep_stats, 8);
-    mbar_init(bar_ep_done, 8);
-    mbar_init(bar_ep_flag, 1);
     *abort_flag = 0;
-    *any_empty = 0;
-    prefix[0] = 0;
     mbar_fence_init();
   }
-  __syncthreads();
   if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS);
-  // tiles per sequence, then their running sum
-  for (int b = tid; b < p.batch; b += blockDim.x) {
-    const int n = clamp_len(p.seq_lens[b], p.max_seq_len);
-    prefix[b + 1] = (n + kBigTokens - 1) / kBigTokens;
-    if (n == 0) *any_empty = 1;
+  if (warp == 3 && lane == 0) {
+    tma_prefetch_desc(&tm_k);
+    tma_prefetch_desc(&tm_v);
+    tma_prefetch_desc(&tm_q);
   }
-  // query rows that no item uses stay zero (the TMA only ever writes the first `rows` rows)
-  for (int idx = tid; idx < NQ * Q_BYTES / 16; idx += blockDim.x)
-    *reinterpret_cast<uint4*>(big_ptr + C::OFF_Q + idx * 16) = make_uint4(0, 0, 0, 0);
-  fence_proxy_async();
-  tc_fence_before_sync();
-  __syncthreads();
+  if (warp >= 4) {
+    // query rows that no item uses stay zero (the TMA only ever writes the first p.rows rows of a
+    // 64-channel block)
+    const int n16 = (M - p.rows) * 8;
+    for (int idx = tid - 128; idx < NQ * (D / 64) * n16; idx += kTcThreads - 128) {
+      const int blk = idx / n16;
+      *reinterpret_cast<uint4*>(big_ptr + C::OFF_Q + blk * (M * 128) + p.rows * 128 + (idx - blk * n16) * 16) =
+          make_uint4(0, 0, 0, 0);
+    }
+    fence_proxy_async();
+  }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 0) {
+    // running sum of the tiles per sequence
     int carry = 0;
+    bool empty = false;
     for (int b0 = 0; b0 < p.batch; b0 += 32) {
       const int b = b0 + lane;
-      int v = b < p.batch ? prefix[b + 1] : 0;
+      int v = 0;
+      if (b < p.batch) {
+        v = (clamp_len(p.seq_lens[b], p.max_seq_len) + kBigTokens - 1) / kBigTokens;
+        empty |= v == 0;
+      }
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
         const int o = __shfl_up_sync(0xffffffffu, v, off);
@@ -308,7 +334,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       if (b < p.batch) prefix[b + 1] = v + carry;
       carry += __shfl_sync(0xffffffffu, v, 31);
     }
+    empty = __any_sync(0xffffffffu, empty);
+    if (lane == 0) {
+      prefix[0] = 0;
+      *any_empty = empty ? 1 : 0;
+    }
   }
+  tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
@@ -340,8 +372,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     if (lane == 0 && active) {
       const bool is_k = warp == 0;
       const CUtensorMap* const tm = is_k ? &tm_k : &tm_v;
-      tma_prefetch_desc(tm);
-      if (is_k) tma_prefetch_desc(&tm_q);
       const uint64_t policy = l2_policy_evict_first();
       const uint64_t policy_q = l2_policy_evict_last();
       const int subs_per_block = p.block_table ? p.block_tokens / kTileTokens : 1;
@@ -412,6 +442,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   } else if (warp == 1) {
     // ================================================================ S = Q K^T issuer
     setmaxnreg_dec<kRegsLight>();
+    if (lane == 0) publish_cut_item(p, active, cta, gcta, n_active, total, T0, T1, prefix);
     if (lane == 0 && active) {
       SliceCursor c;
       c.start(T0, T1, prefix, p.batch, hkv);
@@ -538,7 +569,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     c.start(T0, T1, prefix, p.batch, hkv);
     bool ok = true;
     int i0 = 0;           // index (inside the slice) of the current segment's first tile
-    int n_partial = 0;    // partial epilogues so far
 #define SM_WAIT(bar, parity)                                                        \
   do {                                                                              \
     ok = __all_sync(0xffffffffu, mbar_wait((bar), (parity), abort_flag));           \
@@ -938,104 +968,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_o_empty);
 
-      if (!complete) {
-        // the CTA that brings an item's last partial result merges all of them, in slice order
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_ep_done);
-        const int64_t item_end = sg.item_begin + sg.item_tiles;
-        const int c_first = slice_owner(sg.item_begin, n_active, total);
-        const int c_last = slice_owner(item_end - 1, n_active, total);
-        if (st == 0) {
-          if (mbar_wait(bar_ep_done, n_partial & 1, abort_flag)) {
-            const int old = atomicAdd(p.ws_cnt + (size_t)part * n_items + sg.item, 1);
-            __threadfence();
-            *last_flag = (old == c_last - c_first) ? 1 : 0;
-          } else {
-            *last_flag = 0;
-          }
-          mbar_arrive(bar_ep_flag);
-        }
-        SM_WAIT(bar_ep_flag, n_partial & 1);
-        ++n_partial;
-        if (*last_flag) {
-          __threadfence();
-          // Two output positions per thread and pass, the parts in chunks of kMergeChunk: every
-          // load of a chunk is issued before the first is used, so a pass costs one trip to the L2
-          // instead of one per part and value.  Parts are folded in slice order (fixed).
-          constexpr int kMergeChunk = 4;
-          const int n_parts = c_last - c_first + 1;
-          const int n_idx = rows * (D / 4);
-          for (int idx0 = st; idx0 < n_idx; idx0 += 512) {
-            int r[2], c4[2];
-            bool on[2];
-            float mm[2] = {-INFINITY, -INFINITY}, den[2] = {0.f, 0.f};
-            float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              const int idx = idx0 + 256 * u;
-              on[u] = idx < n_idx;
-              r[u] = on[u] ? idx / (D / 4) : 0;
-              c4[u] = on[u] ? idx - r[u] * (D / 4) : 0;
-            }
-            for (int pc = 0; pc < n_parts; pc += kMergeChunk) {
-              float ls[2][kMergeChunk];
-              float4 x[2][kMergeChunk];
-#pragma unroll
-              for (int q = 0; q < kMergeChunk; ++q) {
-                const bool have = pc + q < n_parts;
-                const int cpart = c_first + pc + q;
-                const int sl = have ? partial_slot(part * ctas_per_part + cpart, slice_begin(cpart, n_active, total), sg.item_begin) : 0;
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                  if (have && on[u]) {
-                    ls[u][q] = ldg_cg_f32(p.ws_lse + (size_t)sl * p.rows + r[u]);
-                    x[u][q] = ldg_cg_f32x4(p.ws_o + ((size_t)sl * p.rows + r[u]) * D + c4[u] * 4);
-                  } else {
-                    ls[u][q] = -INFINITY;
-                    x[u][q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                  }
-                }
-              }
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                float m2 = mm[u];
-#pragma unroll
-                for (int q = 0; q < kMergeChunk; ++q) m2 = fmaxf(m2, ls[u][q]);
-                if (m2 == -INFINITY) continue;
-                const float sc = mm[u] == -INFINITY ? 0.f : fast_exp2(mm[u] - m2);
-                acc[u].x *= sc;
-                acc[u].y *= sc;
-                acc[u].z *= sc;
-                acc[u].w *= sc;
-                den[u] *= sc;
-#pragma unroll
-                for (int q = 0; q < kMergeChunk; ++q) {
-                  const float w = ls[u][q] == -INFINITY ? 0.f : fast_exp2(ls[u][q] - m2);
-                  acc[u].x += w * x[u][q].x;
-                  acc[u].y += w * x[u][q].y;
-                  acc[u].z += w * x[u][q].z;
-                  acc[u].w += w * x[u][q].w;
-                  den[u] += w;
-                }
-                mm[u] = m2;
-              }
-            }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              if (!on[u]) continue;
-              const float invd = den[u] > 0.f ? 1.f / den[u] : 0.f;
-              const int t = r[u] / p.group, hq = sg.g * p.group + (r[u] - t * p.group);
-              const size_t orow = ((size_t)lb * p.n_win + q0 + t) * p.n_q_heads + hq;
-              uint2 packed;
-              packed.x = pack_bf16x2(acc[u].x * invd, acc[u].y * invd);
-              packed.y = pack_bf16x2(acc[u].z * invd, acc[u].w * invd);
-              *reinterpret_cast<uint2*>(p.out + orow * D + c4[u] * 4) = packed;
-              if (p.lse && c4[u] == 0) p.lse[orow] = den[u] > 0.f ? (mm[u] + log2f(den[u])) * kLn2 : -INFINITY;
-            }
-          }
-        }
-      }
       i0 += sg.n_tiles;
       c.next_segment(prefix, p.batch, hkv);
     }
@@ -1051,6 +983,116 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     tc_fence_after_sync();
     tmem_dealloc(tmem_base, C::TMEM_COLS);
   }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Merge of the items that slice boundaries cut, a kernel of its own behind the attention kernel
+// (launched with programmatic stream serialization).  blockIdx.x = the CTA that holds an item's
+// first part (most hold none and leave), blockIdx.y = a block of output positions (four channels of
+// a row each).  The parts of an item sit in the scratch slots first_slot and 2 (c + 1), 2 (c + 2), ..
+//   out = sum_s w_s o_s / sum_s w_s,  w_s = 2^(lse_s - max),  parts folded in slice order (fixed).
+// LANES warps share an item's parts, for launches that cut few items into many parts.
+// One CTA per item used to do this at the end of the attention kernel, after an atomic counter said that
+// it was the last: with one layer of 6400 tokens (8 items in 13 parts each) that was 21 of the
+// call's 37.8 us, plus a memset of the counters and 2.5 us of fences per partial result.
+// ---------------------------------------------------------------------------------------------
+constexpr int kMergeThreads = 256;
+constexpr int kMergeChunk = 8;         // parts whose loads are in flight together
+
+template <int D, int LANES>
+__global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnTcParams p) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int gcta = blockIdx.x;
+  const int4 cut = __ldcg(p.ws_cut + gcta);
+  if (cut.w == 0) return;
+  const int ctas_per_part = (int)gridDim.x / p.n_parts;
+  const int part = gcta / ctas_per_part, q0 = part * p.q_per;
+  const int rows = (p.n_win - q0 < p.q_per ? p.n_win - q0 : p.q_per) * p.group;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kPos = kMergeThreads / LANES;              // output positions of a block
+  const int wl = warp % LANES;                              // this warp's share of the parts: wl, wl + LANES, ..
+  const int pos = (warp / LANES) * 32 + lane;
+  const int idx = blockIdx.y * kPos + pos;
+  const bool on = idx < rows * (D / 4);
+  const int r = on ? idx / (D / 4) : 0, c4 = on ? idx - r * (D / 4) : 0;
+  float mm = -INFINITY, den = 0.f;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k0 = wl; k0 < cut.w; k0 += LANES * kMergeChunk) {
+    float ls[kMergeChunk];
+    float4 x[kMergeChunk];
+#pragma unroll
+    for (int q = 0; q < kMergeChunk; ++q) {
+      const int k = k0 + q * LANES;
+      ls[q] = -INFINITY;
+      x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (on && k < cut.w) {
+        const size_t row = (size_t)(k == 0 ? cut.z : 2 * (gcta + k)) * p.rows + r;
+        ls[q] = ldg_cg_f32(p.ws_lse + row);
+        x[q] = ldg_cg_f32x4(p.ws_o + row * D + c4 * 4);
+      }
+    }
+    float m2 = mm;
+#pragma unroll
+    for (int q = 0; q < kMergeChunk; ++q) m2 = fmaxf(m2, ls[q]);
+    if (m2 == -INFINITY) continue;
+    const float sc = mm == -INFINITY ? 0.f : fast_exp2(mm - m2);
+    acc.x *= sc;
+    acc.y *= sc;
+    acc.z *= sc;
+    acc.w *= sc;
+    den *= sc;
+#pragma unroll
+    for (int q = 0; q < kMergeChunk; ++q) {
+      const float w = ls[q] == -INFINITY ? 0.f : fast_exp2(ls[q] - m2);
+      acc.x += w * x[q].x;
+      acc.y += w * x[q].y;
+      acc.z += w * x[q].z;
+      acc.w += w * x[q].w;
+      den += w;
+    }
+    mm = m2;
+  }
+  if constexpr (LANES > 1) {
+    __shared__ float4 acc_sm[LANES - 1][kPos];
+    __shared__ float2 md_sm[LANES - 1][kPos];
+    if (wl > 0) {
+      acc_sm[wl - 1][pos] = acc;
+      md_sm[wl - 1][pos] = make_float2(mm, den);
+    }
+    __syncthreads();
+    if (wl > 0) return;
+    float m2 = mm;
+#pragma unroll
+    for (int w = 0; w < LANES - 1; ++w) m2 = fmaxf(m2, md_sm[w][pos].x);
+    const float sc = mm == -INFINITY ? 0.f : fast_exp2(mm - m2);
+    acc.x *= sc;
+    acc.y *= sc;
+    acc.z *= sc;
+    acc.w *= sc;
+    den *= sc;
+#pragma unroll
+    for (int w = 0; w < LANES - 1; ++w) {
+      const float2 md = md_sm[w][pos];
+      const float4 x = acc_sm[w][pos];
+      const float f = md.x == -INFINITY ? 0.f : fast_exp2(md.x - m2);
+      acc.x += f * x.x;
+      acc.y += f * x.y;
+      acc.z += f * x.z;
+      acc.w += f * x.w;
+      den += f * md.y;
+    }
+    mm = m2;
+  }
+  if (!on) return;
+  const float inv = den > 0.f ? 1.f / den : 0.f;
+  const int t = r / p.group, h = cut.y * p.group + (r - t * p.group);
+  const size_t orow = ((size_t)cut.x * p.n_win + q0 + t) * p.n_q_heads + h;
+  uint2 packed;
+  packed.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+  packed.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+  *reinterpret_cast<uint2*>(p.out + orow * D + c4 * 4) = packed;
+  if (p.lse && c4 == 0) p.lse[orow] = den > 0.f ? (mm + log2f(den)) * kLn2 : -INFINITY;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1073,18 +1115,16 @@ static int tc_grid(const specvlm_kv_t* kv, int32_t batch, int n_parts) {
   return n_parts * sched_active_ctas(tiles_max, per_part);
 }
 
-// scratch: two partial results per CTA (rows of a full part each), their LSEs, one arrival counter
-// per (part, item)
+// scratch: two partial results per CTA (rows of a full part each), their LSEs, and the cut item of each CTA
 static void tc_ws_layout(const specvlm_kv_t* kv, int32_t batch, int rows, int group, size_t& o_bytes, size_t& lse_bytes,
-                         size_t& cnt_bytes) {
+                         size_t& cut_bytes) {
   int n_parts, q_per;
   tc_parts(rows, group, n_parts, q_per);
   const int grid = tc_grid(kv, batch, n_parts);
-  const size_t items = (size_t)kv->n_layers * batch * kv->n_kv_heads;
   const size_t rows_part = (size_t)q_per * group;
   o_bytes = round_up((size_t)2 * grid * rows_part * kv->head_dim * sizeof(float), 256);
   lse_bytes = round_up((size_t)2 * grid * rows_part * sizeof(float), 256);
-  cnt_bytes = round_up(items * n_parts * sizeof(int32_t), 256);
+  cut_bytes = round_up((size_t)grid * sizeof(int4), 256);
 }
 
 size_t attn_tc_ws_bytes(const specvlm_kv_t* kv, int32_t batch, int rows, int group) {
@@ -1127,8 +1167,23 @@ static int32_t launch_tc_t(const CUtensorMap& tk, const CUtensorMap& tv, const C
     if (fa.numRegs * kTcThreads < kRegsNeeded) return SPECVLM_ERR_CUDA;   // setmaxnreg could never be satisfied
     if (!smem_attr_once(attr_done, reinterpret_cast<const void*>(kern), C::TOTAL)) return SPECVLM_ERR_CUDA;
   }
-  kern<<<grid, kTcThreads, C::TOTAL, st>>>(tk, tv, tq, p);
-  return launch_status();
+  return launch_after(kern, dim3((unsigned)grid), dim3(kTcThreads), C::TOTAL, st, tk, tv, tq, p);
+}
+
+template <int D>
+static int32_t launch_merge(const AttnTcParams& p, int grid, cudaStream_t st) {
+  const int ctas = grid / p.n_parts;
+  if (ctas <= 1) return SPECVLM_OK;                       // no slice boundary: nothing is ever cut
+  // Two parts per cut item where the items outnumber the CTAs; many where a few items fill the chip.
+  const int64_t items = (int64_t)p.n_layers * p.batch * p.n_kv_heads;
+  const int positions = p.rows * (D / 4);
+  if (ctas > 4 * items) {
+    constexpr int kPos = kMergeThreads / 4;
+    return launch_after(attn_merge_kernel<D, 4>, dim3((unsigned)grid, (unsigned)((positions + kPos - 1) / kPos)),
+                        dim3(kMergeThreads), 0, st, p);
+  }
+  return launch_after(attn_merge_kernel<D, 1>, dim3((unsigned)grid, (unsigned)((positions + kMergeThreads - 1) / kMergeThreads)),
+                      dim3(kMergeThreads), 0, st, p);
 }
 
 // Ancestor masks of a draft tree: bit w of anc[b][t] says that node t attends window position w
@@ -1174,9 +1229,9 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   const int64_t items = (int64_t)kv->n_layers * batch * kv->n_kv_heads;
   if (items > 0x3fffffff) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SPECVLM_ERR_INVALID_ARG;
-  size_t o_bytes, lse_bytes, cnt_bytes;
-  tc_ws_layout(kv, batch, rows, group, o_bytes, lse_bytes, cnt_bytes);
-  const size_t base_bytes = o_bytes + lse_bytes + cnt_bytes;
+  size_t o_bytes, lse_bytes, cut_bytes;
+  tc_ws_layout(kv, batch, rows, group, o_bytes, lse_bytes, cut_bytes);
+  const size_t base_bytes = o_bytes + lse_bytes + cut_bytes;
   if (ws_bytes < base_bytes + (tree_parents ? attn_tc_tree_extra_bytes(batch, n_q) : 0))
     return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
   if (tree_parents && n_q > kMaxTreeNodes) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
@@ -1199,7 +1254,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   uint8_t* w = static_cast<uint8_t*>(ws);
   p.ws_o = reinterpret_cast<float*>(w);
   p.ws_lse = reinterpret_cast<float*>(w + o_bytes);
-  p.ws_cnt = reinterpret_cast<int32_t*>(w + o_bytes + lse_bytes);
+  p.ws_cut = reinterpret_cast<int4*>(w + o_bytes + lse_bytes);
   p.n_parts = n_parts;
   p.q_per = q_per;
   p.rows = q_per * group;
@@ -1229,13 +1284,12 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   CUtensorMap tq;
   rc = encode_q_map(&tq, q, kv->head_dim, group, n_q, q_per, kv->n_kv_heads, (int64_t)kv->n_layers * batch);
   if (rc != SPECVLM_OK) return rc;
-  if (cudaMemsetAsync(p.ws_cnt, 0, (size_t)items * n_parts * sizeof(int32_t), st) != cudaSuccess) return SPECVLM_ERR_CUDA;
   if (kv->head_dim == 128)
     rc = p.rows <= 64 ? launch_tc<128, 64>(tk, tv, tq, p, grid, st) : launch_tc<128, 128>(tk, tv, tq, p, grid, st);
   else
     rc = p.rows <= 64 ? launch_tc<64, 64>(tk, tv, tq, p, grid, st) : launch_tc<64, 128>(tk, tv, tq, p, grid, st);
   if (rc != SPECVLM_OK) return rc;
-  return SPECVLM_OK;
+  return kv->head_dim == 128 ? launch_merge<128>(p, grid, st) : launch_merge<64>(p, grid, st);
 }
 
 }  // namespace specvlm

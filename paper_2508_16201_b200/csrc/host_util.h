@@ -91,6 +91,26 @@ inline int32_t launch_status() {
   return cudaGetLastError() == cudaSuccess ? SPECVLM_OK : SPECVLM_ERR_CUDA;
 }
 
+// Launches `kern` so that it may be scheduled while the kernel before it in the stream still runs
+// (programmatic stream serialization).  The kernel itself has to wait (griddepcontrol.wait) for that
+// kernel's completion, in every CTA and before its first access to global memory.
+template <typename... KArgs, typename... Args>
+inline int32_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                            const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...) != cudaSuccess) return SPECVLM_ERR_CUDA;
+  return launch_status();
+}
+
 inline int sm_count() {
   // one process drives one GPU; the count of the first device seen is kept
   static std::atomic<int> cached{0};
