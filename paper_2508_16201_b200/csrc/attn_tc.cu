@@ -1,7 +1,6 @@
 // Streaming softmax attention over a bf16 K/V cache on the 5th-generation tensor cores of sm_100a:
-// (gamma+1)-query verification attention and tree verification, i.e. windows of 17 to 128 rows per
-// KV head and set of CTAs (a wider window is cut into parts that share one launch; up to 16 rows run on the kernel of
-// attn.cu).
+// (gamma+1)-query verification attention and tree verification, windows of up to 128 rows per KV head
+// (chains of up to 16 rows run on the kernel of attn.cu, wider windows on that of attn_pair.cu).
 //
 // One persistent CTA per SM streams a contiguous slice of the flat (layer, sequence, KV head, tile)
 // list (attn_sched.h), so the cache is read exactly once, every SM moves the same number of bytes
@@ -28,151 +27,9 @@
 // The running maximum of a row is only raised when a tile's maximum exceeds it by more than 2^8; O
 // is then rescaled in place in TMEM.  Probabilities stay below 2^8, well inside bf16 / fp32 range,
 // and the common tile needs no pass over O at all.
-#include "attn.cuh"
-#include "attn_sched.h"
-#include "host_util.h"
+#include "attn_tc.cuh"
 
 namespace specvlm {
-
-struct AttnTcParams {
-  __nv_bfloat16* out;         // [L][B][n_win][Hq][D]
-  float* lse;                 // [L][B][n_win][Hq] or null
-  float* ws_o;                // partial results: [2 * grid][rows][D], normalised
-  float* ws_lse;              // [2 * grid][rows], log2 units
-  int4* ws_cut;               // [grid]: the cut item whose first part a CTA holds, see attn_merge_kernel
-  const int32_t* block_table; // [B][max_blocks] or null
-  const int32_t* seq_lens;    // [B]
-  int32_t* d_status;
-  const uint64_t* anc;        // [B][n_win] ancestor masks of a draft tree (<= 64 nodes), or null: the window is a chain
-  int32_t batch, n_layers, n_q_heads, n_kv_heads, group;
-  int32_t n_win;              // tokens of the whole window
-  int32_t n_parts, q_per;     // the window is cut into n_parts parts of q_per tokens (the last may be shorter)
-  int32_t rows;               // rows of a full part = q_per * group (<= 128): the row pitch of the scratch slots
-  int32_t max_blocks, block_tokens, max_seq_len;
-  float scale_log2;           // sm_scale * log2(e)
-};
-
-constexpr float kRescaleThreshold = 8.f;   // log2 units
-constexpr int kMaxTreeNodes = 64;          // a window mask is one 64-bit word per node
-constexpr int kBigTokens = 2 * kTileTokens;          // tokens per MMA tile
-constexpr int kTcThreads = 384;
-// setmaxnreg moves registers between the warps of a CTA inside the pool the CTA got at launch
-// (threads x registers per thread as compiled: 384 x 168), and an increase blocks until the pool
-// has them -- for ever, if the requests add up to more than the pool.  The launch code checks the
-// sum against the compiled kernel's pool and refuses to launch otherwise.
-constexpr int kRegsLight = 96, kRegsSoftmax = 200;
-constexpr int kRegsNeeded = 128 * kRegsLight + 256 * kRegsSoftmax;
-
-template <int N> __device__ __forceinline__ void setmaxnreg_dec() {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
-}
-template <int N> __device__ __forceinline__ void setmaxnreg_inc() {
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
-}
-
-// 16 TMEM lanes x 64 fp32 columns -> 32 registers per thread: registers 4j, 4j+1 hold lane
-// (base + tid/4), columns 8j + 2(tid%4) + {0,1}; registers 4j+2, 4j+3 the same columns of lane
-// (base + 8 + tid/4).
-__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st_16x256b_x8(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ float ldg_cg_f32(const float* p) {
-  float v;
-  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ float4 ldg_cg_f32x4(const float* p) {
-  float4 v;
-  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
-  return v;
-}
-
-__device__ __forceinline__ int clamp_len(int n, int max_len) { return n < 0 ? 0 : (n > max_len ? max_len : n); }
-
-// Cold paths of the softmax loop, kept out of line: the loop's code has to stay small enough for
-// the instruction cache (with the mask logic inline the 128-row variant ran 25 % slower, although
-// only one or two tiles of an item ever need a mask).
-//
-// Tiles that overlap the window of new tokens: the invisible logits of this thread's two rows
-// (a 16-lane half of S: rows lr and lr + 8, columns 8j + lc + {0, 1} of each 64-column block) are
-// overwritten with -inf in tensor memory, so the loop itself knows no masks.  Visibility of key
-// `tok` for the row of query token t: every key before the window, and inside the window the
-// positions whose bit is set in the row's mask -- the token's ancestors and itself for a tree
-// (a0, a1 = the rows' masks), positions up to t for a chain (a0, a1 = the rows' limits `lim`:
-// key tok is visible when tok < lim).
-template <bool TREE>
-__device__ __noinline__ void mask_s_half(uint32_t saddr, int tile_tok0, int win0, int lc, uint64_t a0, uint64_t a1) {
-  const uint64_t a[2] = {a0, a1};
-#pragma unroll 1
-  for (int c = 0; c < 2; ++c) {
-    uint64_t mk[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      if constexpr (TREE) {
-        // 128 visibility bits of the tile: the keys before the window, then the row's window mask
-        // at the window's offset in the tile
-        const int sh = win0 - tile_tok0;                       // tile column of window position 0
-        unsigned __int128 full = 0;
-        if (a[e]) {
-          if (sh > 0) full = sh >= 128 ? ~(unsigned __int128)0 : (((unsigned __int128)1 << sh) - 1);
-          const unsigned __int128 w = a[e];
-          full |= sh >= 0 ? (sh < 128 ? w << sh : (unsigned __int128)0)
-                          : (sh > -64 ? w >> (-sh) : (unsigned __int128)0);
-        }
-        mk[e] = (uint64_t)(full >> (64 * c)) >> lc;
-      } else {
-        const int n_vis = (int)a[e] - tile_tok0 - 64 * c;       // visible columns of the block
-        mk[e] = (n_vis <= 0 ? 0ull : (n_vis >= 64 ? ~0ull : ((1ull << n_vis) - 1ull))) >> lc;
-      }
-    }
-    uint32_t v[32];
-    tmem_ld_16x256b_x8(saddr + 64 * c, v);
-    tmem_ld_wait();
-#pragma unroll
-    for (int k = 0; k < 32; ++k)
-      if (!((mk[(k >> 1) & 1] >> ((k >> 2) * 8 + (k & 1))) & 1ull)) v[k] = 0xff800000u;   // -inf
-    tmem_st_16x256b_x8(saddr + 64 * c, v);
-  }
-  tmem_st_wait();
-}
-
-// A row maximum grew past the lazy-rescale threshold: the rows' O accumulators (16-lane half,
-// d columns from oaddr on) are multiplied by f0 (row lr) and f1 (row lr + 8) in tensor memory.
-template <int D>
-__device__ __noinline__ void rescale_o_half(uint32_t oaddr, float f0, float f1) {
-#pragma unroll 1
-  for (int cc = 0; cc < D / 64; ++cc) {
-    uint32_t o[32];
-    tmem_ld_16x256b_x8(oaddr + cc * 64, o);
-    tmem_ld_wait();
-#pragma unroll
-    for (int k = 0; k < 32; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * (((k >> 1) & 1) ? f1 : f0));
-    tmem_st_16x256b_x8(oaddr + cc * 64, o);
-  }
-  tmem_st_wait();
-}
 
 // Shared-memory plan.  A small region (barriers, flags, per-sequence tile counts, the softmax
 // groups' row statistics) sits at the start of the dynamic shared memory; the tile rings and the
@@ -204,22 +61,6 @@ struct TcCfg {
   static constexpr uint32_t TMEM_COLS = 512;
   static_assert(SMALL + BIG <= kMaxSmem, "shared-memory plan does not fit");
 };
-
-// Which item, if any, this CTA's slice holds the first part of while a slice boundary cuts it: (layer *
-// batch + sequence, KV head, scratch slot of the first part, number of parts), no parts if there is none.
-// Written before any wait, so that the merge never reads a stale entry.
-__device__ __forceinline__ void publish_cut_item(const AttnTcParams& p, bool active, int cta, int gcta, int n_active,
-                                                 int64_t total, int64_t T0, int64_t T1, const int* prefix) {
-  int4 cut = make_int4(0, 0, 0, 0);
-  if (active && T1 < total) {
-    const Segment s = segment_at(T1 - 1, T1, prefix, p.batch, p.n_kv_heads);   // the item of the slice's last tile
-    const int64_t item_end = s.item_begin + s.item_tiles;
-    if (item_end > T1 && s.item_begin >= T0)
-      cut = make_int4(s.layer * p.batch + s.b, s.g, partial_slot(gcta, T0, s.item_begin),
-                      slice_owner(item_end - 1, n_active, total) - cta + 1);
-  }
-  p.ws_cut[gcta] = cut;
-}
 
 // TREE: the window's visibility comes from per-token ancestor masks instead of the chain rule.
 // A template parameter, not a run-time branch: the chain kernel's code is untouched by the tree
@@ -316,29 +157,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 0) {
-    // running sum of the tiles per sequence
-    int carry = 0;
-    bool empty = false;
-    for (int b0 = 0; b0 < p.batch; b0 += 32) {
-      const int b = b0 + lane;
-      int v = 0;
-      if (b < p.batch) {
-        v = (clamp_len(p.seq_lens[b], p.max_seq_len) + kBigTokens - 1) / kBigTokens;
-        empty |= v == 0;
-      }
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, v, off);
-        if (lane >= off) v += o;
-      }
-      if (b < p.batch) prefix[b + 1] = v + carry;
-      carry += __shfl_sync(0xffffffffu, v, 31);
-    }
-    empty = __any_sync(0xffffffffu, empty);
-    if (lane == 0) {
-      prefix[0] = 0;
-      *any_empty = empty ? 1 : 0;
-    }
+    const bool empty = tile_prefix(p, prefix, lane);
+    if (lane == 0) *any_empty = empty ? 1 : 0;
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -346,20 +166,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const uint32_t tmem_base = *tmem_slot;
   const int hkv = p.n_kv_heads;
   const int64_t total = (int64_t)p.n_layers * hkv * prefix[p.batch];
-  // A window of more than 128 rows is cut into parts of q_per query tokens, the accumulators of one
-  // part filling the tensor memory.  The parts run side by side in this one launch: the grid is
-  // n_parts sets of CTAs, every set slices the same flat tile list in the same way, so CTA c of each
-  // set streams the same K/V tiles at about the same time and all but the first to ask find them in
-  // the L2 cache -- HBM delivers every tile once, not once per part.
-  const int ctas_per_part = (int)gridDim.x / p.n_parts;
-  const int part = blockIdx.x / ctas_per_part;          // >= n_parts: a spare CTA without work
-  const int cta = blockIdx.x - part * ctas_per_part;    // index inside the part's set
-  const int gcta = blockIdx.x;                          // index of this CTA's scratch slots
-  const int q0 = part * p.q_per;                        // first window token of the part
-  const int n_q_part = part < p.n_parts ? (p.n_win - q0 < p.q_per ? p.n_win - q0 : p.q_per) : 0;
-  const int rows = n_q_part > 0 ? n_q_part * p.group : 0;   // rows in use (of the M rows of a tile)
-  const int n_active = sched_active_ctas(total, ctas_per_part);
-  const bool active = total > 0 && rows > 0 && cta < n_active;
+  const int cta = blockIdx.x;
+  const int rows = p.rows;                              // rows in use (of the M rows of a tile)
+  const int n_active = sched_active_ctas(total, (int)gridDim.x);
+  const bool active = total > 0 && cta < n_active;
   const int64_t T0 = active ? slice_begin(cta, n_active, total) : 0;
   const int64_t T1 = active ? slice_begin(cta + 1, n_active, total) : 0;
   const int n_items = p.n_layers * p.batch * hkv;
@@ -396,7 +206,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           mbar_arrive_expect_tx(bar_q_full + 8 * qb, (uint32_t)p.rows * 128u * (D / 64));
 #pragma unroll
           for (int h = 0; h < D / 64; ++h)
-            tma_load_5d(q_sm + qb * Q_BYTES + h * (M * 128), &tm_q, bar_q_full + 8 * qb, h * 64, 0, q0, sg.g,
+            tma_load_5d(q_sm + qb * Q_BYTES + h * (M * 128), &tm_q, bar_q_full + 8 * qb, h * 64, 0, 0, sg.g,
                         sg.layer * p.batch + sg.b, policy_q);
         }
         const int n_sub_seq = (clamp_len(p.seq_lens[sg.b], p.max_seq_len) + kTileTokens - 1) / kTileTokens;
@@ -442,7 +252,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   } else if (warp == 1) {
     // ================================================================ S = Q K^T issuer
     setmaxnreg_dec<kRegsLight>();
-    if (lane == 0) publish_cut_item(p, active, cta, gcta, n_active, total, T0, T1, prefix);
+    if (lane == 0) publish_cut_item(p, active, cta, cta, n_active, total, T0, T1, prefix);
     if (lane == 0 && active) {
       SliceCursor c;
       c.start(T0, T1, prefix, p.batch, hkv);
@@ -551,14 +361,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const int nh = (rows > row0(0) ? 1 : 0) + (NH > 1 && rows > row0(1) ? 1 : 0);
 
     // sequences without any token: their outputs are zero, their LSE -inf
-    if (*any_empty && rows > 0) {
-      for (int item = cta; item < n_items; item += ctas_per_part) {
+    if (*any_empty) {
+      for (int item = cta; item < n_items; item += (int)gridDim.x) {
         const int lb = item / hkv, g = item - lb * hkv, b = lb % p.batch;
         if (prefix[b + 1] != prefix[b]) continue;
         for (int idx = st; idx < rows * (D / 8); idx += 256) {
           const int r = idx / (D / 8), c8 = idx - r * (D / 8);
           const int t = r / p.group, h = g * p.group + (r - t * p.group);
-          const size_t orow = ((size_t)lb * p.n_win + q0 + t) * p.n_q_heads + h;
+          const size_t orow = ((size_t)lb * p.n_win + t) * p.n_q_heads + h;
           *reinterpret_cast<uint4*>(p.out + orow * D + c8 * 8) = make_uint4(0, 0, 0, 0);
           if (p.lse && c8 == 0) p.lse[orow] = -INFINITY;
         }
@@ -596,9 +406,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const bool warp_on = rows > 32 * quarter;         // warp-uniform: some row of this quadrant is in use
         uint64_t my_a;                                       // the row's window mask (tree) or key limit (chain)
         if constexpr (TREE) {
-          my_a = my_row < rows ? __ldg(p.anc + (size_t)sg.b * p.n_win + q0 + my_row / p.group) : 0ull;
+          my_a = my_row < rows ? __ldg(p.anc + (size_t)sg.b * p.n_win + my_row / p.group) : 0ull;
         } else {
-          my_a = my_row < rows ? (uint64_t)(win0 + q0 + my_row / p.group + 1) : 0ull;
+          my_a = my_row < rows ? (uint64_t)(win0 + my_row / p.group + 1) : 0ull;
         }
         float m_row = -INFINITY, l_row = 0.f;
         const uint32_t prow = p_sm + grp * P_BYTES + my_row * 128;
@@ -744,9 +554,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           const int r = row0(h) + lr + 8 * e;
           const int t = r / p.group;
           if constexpr (TREE) {
-            vis[h][e] = r < rows ? __ldg(p.anc + (size_t)sg.b * p.n_win + q0 + t) : 0ull;
+            vis[h][e] = r < rows ? __ldg(p.anc + (size_t)sg.b * p.n_win + t) : 0ull;
           } else {
-            lim[h][e] = r < rows ? win0 + q0 + t + 1 : 0;
+            lim[h][e] = r < rows ? win0 + t + 1 : 0;
           }
           m_used[h][e] = -INFINITY;
           l_sum[h][e] = 0.f;
@@ -896,7 +706,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       //   O = (w0 O0 + w1 O1) / (w0 l0 + w1 l1),  w_g = 2^(m_g - max(m0, m1))
       const bool complete = sg.tile0 == 0 && sg.n_tiles == sg.item_tiles;
       const int lb = sg.layer * p.batch + sg.b;
-      const int slot = partial_slot(gcta, T0, sg.item_begin);
+      const int slot = partial_slot(cta, T0, sg.item_begin);
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_ep_stats);
       SM_WAIT(bar_ep_stats, seg_idx & 1);
@@ -948,7 +758,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
               }
             if (complete) {
               const int t = r / p.group, hq = sg.g * p.group + (r - t * p.group);
-              const size_t orow = ((size_t)lb * p.n_win + q0 + t) * p.n_q_heads + hq;
+              const size_t orow = ((size_t)lb * p.n_win + t) * p.n_q_heads + hq;
               __nv_bfloat16* dst = p.out + orow * D + cc * 64 + lc;
 #pragma unroll
               for (int jj = 0; jj < 8; ++jj)
@@ -1106,21 +916,24 @@ static void tc_parts(int rows, int group, int& n_parts, int& q_per) {
   q_per = (n_q + n_parts - 1) / n_parts;               // the parts are made as equal as the tokens allow
 }
 
-// One set of CTAs per part, every set as large as the SMs allow (and the tile count is worth).
-static int tc_grid(const specvlm_kv_t* kv, int32_t batch, int n_parts) {
+// CTAs of a launch's set (as many as the SMs allow and the tile count is worth).  A window of one
+// part is one set; a wider one has a set per two parts (attn_pair.cu), the sets side by side in one launch
+// over the same slices, so that all but the first reader of a tile find it in the L2 cache.
+static int tc_set_ctas(const specvlm_kv_t* kv, int32_t batch, int n_parts) {
   const int64_t tiles_max = (int64_t)kv->n_layers * batch * kv->n_kv_heads *
                             ((kv->max_seq_len + kBigTokens - 1) / kBigTokens);
-  int per_part = sm_count() / n_parts;
-  if (per_part < 1) per_part = 1;
-  return n_parts * sched_active_ctas(tiles_max, per_part);
+  int per_set = sm_count() / ((n_parts + 1) / 2);
+  if (per_set < 1) per_set = 1;
+  return sched_active_ctas(tiles_max, per_set);
 }
 
-// scratch: two partial results per CTA (rows of a full part each), their LSEs, and the cut item of each CTA
+// scratch, per part and CTA of its set: two partial results (rows of a full part each), their LSEs, and the
+// item that the CTA's slice cuts
 static void tc_ws_layout(const specvlm_kv_t* kv, int32_t batch, int rows, int group, size_t& o_bytes, size_t& lse_bytes,
                          size_t& cut_bytes) {
   int n_parts, q_per;
   tc_parts(rows, group, n_parts, q_per);
-  const int grid = tc_grid(kv, batch, n_parts);
+  const int grid = n_parts * tc_set_ctas(kv, batch, n_parts);
   const size_t rows_part = (size_t)q_per * group;
   o_bytes = round_up((size_t)2 * grid * rows_part * kv->head_dim * sizeof(float), 256);
   lse_bytes = round_up((size_t)2 * grid * rows_part * sizeof(float), 256);
@@ -1151,29 +964,10 @@ static int32_t encode_q_map(CUtensorMap* map, const void* q, int D, int group, i
   return r == CUDA_SUCCESS ? SPECVLM_OK : SPECVLM_ERR_CUDA;
 }
 
-template <int D, int M, bool TREE>
-static int32_t launch_tc_t(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const AttnTcParams& p,
-                         int grid, cudaStream_t st) {
-  using C = TcCfg<D, M>;
-  auto kern = attn_tc_kernel<D, M, TREE>;
-  // once per device and kernel variant: the opt-in shared-memory size, and the check that the
-  // compiled kernel's register pool can satisfy the setmaxnreg requests (it never changes)
-  static std::atomic<uint64_t> attr_done{0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return SPECVLM_ERR_CUDA;
-  if (!(attr_done.load(std::memory_order_acquire) & (1ull << (dev & 63)))) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return SPECVLM_ERR_CUDA;
-    if (fa.numRegs * kTcThreads < kRegsNeeded) return SPECVLM_ERR_CUDA;   // setmaxnreg could never be satisfied
-    if (!smem_attr_once(attr_done, reinterpret_cast<const void*>(kern), C::TOTAL)) return SPECVLM_ERR_CUDA;
-  }
-  return launch_after(kern, dim3((unsigned)grid), dim3(kTcThreads), C::TOTAL, st, tk, tv, tq, p);
-}
-
 template <int D>
-static int32_t launch_merge(const AttnTcParams& p, int grid, cudaStream_t st) {
-  const int ctas = grid / p.n_parts;
+static int32_t launch_merge(const AttnTcParams& p, int ctas, cudaStream_t st) {
   if (ctas <= 1) return SPECVLM_OK;                       // no slice boundary: nothing is ever cut
+  const int grid = p.n_parts * ctas;
   // Two parts per cut item where the items outnumber the CTAs; many where a few items fill the chip.
   const int64_t items = (int64_t)p.n_layers * p.batch * p.n_kv_heads;
   const int positions = p.rows * (D / 4);
@@ -1217,8 +1011,14 @@ size_t attn_tc_tree_extra_bytes(int32_t batch, int32_t n_nodes) {
 template <int D, int M>
 static int32_t launch_tc(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const AttnTcParams& p,
                          int grid, cudaStream_t st) {
-  return p.anc ? launch_tc_t<D, M, true>(tk, tv, tq, p, grid, st) : launch_tc_t<D, M, false>(tk, tv, tq, p, grid, st);
+  constexpr int kSmem = TcCfg<D, M>::TOTAL;
+  return p.anc ? launch_tc_kernel<attn_tc_kernel<D, M, true>>(kSmem, tk, tv, tq, p, grid, st)
+               : launch_tc_kernel<attn_tc_kernel<D, M, false>>(kSmem, tk, tv, tq, p, grid, st);
 }
+
+// attn_pair.cu
+int32_t attn_pair_launch(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const AttnTcParams& p,
+                         int head_dim, int grid, cudaStream_t st);
 
 int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int32_t n_q_heads, int32_t n_q,
                        float sm_scale, void* out, float* lse, void* ws, size_t ws_bytes, int32_t* d_status,
@@ -1235,12 +1035,11 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   if (ws_bytes < base_bytes + (tree_parents ? attn_tc_tree_extra_bytes(batch, n_q) : 0))
     return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
   if (tree_parents && n_q > kMaxTreeNodes) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
-  // A window of more than 128 rows is cut into parts of equal numbers of query tokens (the
-  // accumulators of one part fill the tensor memory); the parts share one launch (see the kernel).
+  // A window of more than 128 rows is cut into parts of equal numbers of query tokens that share one launch.
   int n_parts, q_per;
   tc_parts(rows, group, n_parts, q_per);
   if (q_per * group > 128) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
-  const int grid = tc_grid(kv, batch, n_parts);
+  const int ctas = tc_set_ctas(kv, batch, n_parts);
 
   CUtensorMap tk, tv;
   int32_t rc = encode_kv_map(&tk, kv, kv->k, kTileTokens);
@@ -1284,12 +1083,14 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   CUtensorMap tq;
   rc = encode_q_map(&tq, q, kv->head_dim, group, n_q, q_per, kv->n_kv_heads, (int64_t)kv->n_layers * batch);
   if (rc != SPECVLM_OK) return rc;
-  if (kv->head_dim == 128)
-    rc = p.rows <= 64 ? launch_tc<128, 64>(tk, tv, tq, p, grid, st) : launch_tc<128, 128>(tk, tv, tq, p, grid, st);
+  if (n_parts > 1)
+    rc = attn_pair_launch(tk, tv, tq, p, kv->head_dim, (n_parts + 1) / 2 * ctas, st);
+  else if (kv->head_dim == 128)
+    rc = p.rows <= 64 ? launch_tc<128, 64>(tk, tv, tq, p, ctas, st) : launch_tc<128, 128>(tk, tv, tq, p, ctas, st);
   else
-    rc = p.rows <= 64 ? launch_tc<64, 64>(tk, tv, tq, p, grid, st) : launch_tc<64, 128>(tk, tv, tq, p, grid, st);
+    rc = p.rows <= 64 ? launch_tc<64, 64>(tk, tv, tq, p, ctas, st) : launch_tc<64, 128>(tk, tv, tq, p, ctas, st);
   if (rc != SPECVLM_OK) return rc;
-  return kv->head_dim == 128 ? launch_merge<128>(p, grid, st) : launch_merge<64>(p, grid, st);
+  return kv->head_dim == 128 ? launch_merge<128>(p, ctas, st) : launch_merge<64>(p, ctas, st);
 }
 
 }  // namespace specvlm

@@ -142,6 +142,14 @@ def test_verify_window_wider_than_one_launch(paged):
     _run_attn(1, 16, 1, 64, [200], 8, paged=paged, seed=12)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("n", [9, 16, 65, 79, 80, 127, 128, 129, 193, 385, 897])
+def test_wide_window_at_sequence_ends(D, n):
+    """A window of two parts (144 rows at 16 heads per KV head) over sequences that end at every kind of
+    place inside a tile, with NaN past the end; the second sequence makes slices cut items."""
+    _run_attn(1, 16, 1, D, [n, 1500], 8, paged=n % 2 == 1, seed=90 + n, poison=True)
+
+
 def test_verify_window_crossing_tile_boundary():
     # the gamma+1 new tokens straddle a 64-token tile edge, and sit alone in the last tile
     for n in [64 + 3, 128, 128 + 6, 6]:
