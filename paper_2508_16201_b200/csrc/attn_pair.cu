@@ -203,7 +203,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         const Segment sg = c.sg;
         if (is_k) {
           // both parts' query rows: a box of (64 channels) x (group heads) x (q_per tokens) per 64-channel block
-          if (c.seg_idx >= 1) ok = mbar_wait(bar_q_empty, (c.seg_idx - 1) & 1, abort_flag);
+          if (c.seg_idx >= 1) ok = mbar_wait_soon(bar_q_empty, (c.seg_idx - 1) & 1, abort_flag);
           if (!ok) break;
           mbar_arrive_expect_tx(bar_q_full, (uint32_t)(n_here * p.rows) * 128u * (D / 64));
           for (int g = 0; g < n_here; ++g)
@@ -231,7 +231,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             blk_next[1] = s0 + 3 < n_sub_seq ? __ldg(table + (s0 + 3) / subs_per_block) : 0;
           }
           const int slot = i % n_ring;
-          if (i >= n_ring) ok = mbar_wait(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
+          if (i >= n_ring) ok = mbar_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
           if (!ok) break;
           mbar_arrive_expect_tx(bar_full + 8 * slot, n_sub * SUB_BYTES);
           for (int u = 0; u < n_sub; ++u) {
@@ -279,7 +279,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                        umma_desc_advance(db, (s >> 2) * (kBigTokens * 128) + (s & 3) * 32), kIdescQK, s > 0 ? 1u : 0u);
         umma_commit(bar_s_full + 8 * g);
       };
-      ok = mbar_wait(bar_q_full, 0, abort_flag) && mbar_wait(bar_k_full, 0, abort_flag);
+      ok = mbar_wait_soon(bar_q_full, 0, abort_flag) && mbar_wait_soon(bar_k_full, 0, abort_flag);
       if (ok) {
         issue_qk(0);
         umma_commit(bar_k_empty);
@@ -299,7 +299,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         c.next_tile(prefix, p.batch, hkv);               // the cursor stands on tile i + 1 from here on
         const bool more = i + 1 < n_my;
         // waits that are over by the time P arrives come before the wait for P
-        ok = mbar_wait(bar_v_full + 8 * vp, (i / NVP) & 1, abort_flag);
+        ok = mbar_wait_soon(bar_v_full + 8 * vp, (i / NVP) & 1, abort_flag);
         if (ok && tail && (last_rows & 15) != 0) {
           // Steps of 16 tokens past the sequence's end are left out; inside the last step the V rows past
           // the end hold whatever the page held and are cleared (a zero probability times a stale
@@ -311,13 +311,13 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                   make_uint4(0, 0, 0, 0);
           fence_proxy_async();
         }
-        if (ok && more) ok = mbar_wait(bar_k_full + 8 * ((i + 1) % NKP), ((i + 1) / NKP) & 1, abort_flag);
+        if (ok && more) ok = mbar_wait_soon(bar_k_full + 8 * ((i + 1) % NKP), ((i + 1) / NKP) & 1, abort_flag);
         // the first product of an item overwrites O: the previous item's must have been read
-        if (ok && j == 0 && seg_idx >= 1) ok = mbar_wait(bar_o_empty + 8 * g, (seg_idx - 1) & 1, abort_flag);
+        if (ok && j == 0 && seg_idx >= 1) ok = mbar_wait_soon(bar_o_empty + 8 * g, (seg_idx - 1) & 1, abort_flag);
         const uint64_t db = umma_desc_advance(dv0, vp * 2 * SUB_BYTES);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          if (ok) ok = mbar_wait((u ? bar_p_full : bar_p_half) + 8 * g, i & 1, abort_flag);
+          if (ok) ok = mbar_wait_soon((u ? bar_p_full : bar_p_half) + 8 * g, i & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
           const int n_kt = u >= n_sub ? 0 : (tail && u == n_sub - 1 ? (last_rows + 15) >> 4 : kTileTokens / 16);
@@ -335,7 +335,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         umma_commit(bar_v_empty + 8 * vp);
         if (more) {
           if (last) {
-            ok = mbar_wait(bar_q_full, (seg_idx + 1) & 1, abort_flag);
+            ok = mbar_wait_soon(bar_q_full, (seg_idx + 1) & 1, abort_flag);
             if (!ok) break;
             issue_qk(i + 1);
           }
@@ -386,7 +386,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     int i = 0;
 #define SM_WAIT(bar, parity)                                                        \
   do {                                                                              \
-    ok = __all_sync(0xffffffffu, mbar_wait((bar), (parity), abort_flag));           \
+    ok = __all_sync(0xffffffffu, mbar_wait_soon((bar), (parity), abort_flag));           \
     if (!ok) goto softmax_done;                                                     \
   } while (0)
     // The two parts' warps of a lane quadrant sit on the same scheduler and take turns with its
@@ -395,7 +395,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     const uint32_t my_turn = bar_turn + 8 * (4 * g + quarter), other_turn = bar_turn + 8 * (4 * (1 - g) + quarter);
     const bool turns = n_here == 2;
     auto take_turn = [&](int n) {               // part 0 goes first: its n-th turn follows part 1's (n - 1)-th
-      if (turns && (g == 1 || n > 0)) ok = __all_sync(0xffffffffu, mbar_wait(my_turn, (g == 1 ? n : n - 1) & 1, abort_flag));
+      if (turns && (g == 1 || n > 0)) ok = __all_sync(0xffffffffu, mbar_wait_soon(my_turn, (g == 1 ? n : n - 1) & 1, abort_flag));
     };
     auto pass_turn = [&]() {
       __syncwarp();

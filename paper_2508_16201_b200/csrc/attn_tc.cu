@@ -201,7 +201,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if (is_k) {
           // the item's query rows: a box of (64 channels) x (group heads) x (n_q tokens) per 64-channel block
           const int qb = c.seg_idx % NQ;
-          if (c.seg_idx >= NQ) ok = mbar_wait(bar_q_empty + 8 * qb, ((c.seg_idx / NQ) - 1) & 1, abort_flag);
+          if (c.seg_idx >= NQ) ok = mbar_wait_soon(bar_q_empty + 8 * qb, ((c.seg_idx / NQ) - 1) & 1, abort_flag);
           if (!ok) break;
           mbar_arrive_expect_tx(bar_q_full + 8 * qb, (uint32_t)p.rows * 128u * (D / 64));
 #pragma unroll
@@ -227,7 +227,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             blk_next[1] = s0 + 3 < n_sub_seq ? __ldg(table + (s0 + 3) / subs_per_block) : 0;
           }
           const int slot = i % n_ring;
-          if (i >= n_ring) ok = mbar_wait(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
+          if (i >= n_ring) ok = mbar_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
           if (!ok) break;
           mbar_arrive_expect_tx(bar_full + 8 * slot, n_sub * SUB_BYTES);
           for (int u = 0; u < n_sub; ++u) {
@@ -260,9 +260,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       bool ok = true;
       for (int i = 0; i < n_my; ++i) {
         const int g = i & 1, kp = i % NKP, qb = c.seg_idx % NQ;
-        ok = mbar_wait(bar_k_full + 8 * kp, (i / NKP) & 1, abort_flag);
-        if (ok && c.j == 0) ok = mbar_wait(bar_q_full + 8 * qb, (c.seg_idx / NQ) & 1, abort_flag);
-        if (ok && i >= 2) ok = mbar_wait(bar_s_empty + 8 * g, ((i >> 1) - 1) & 1, abort_flag);
+        ok = mbar_wait_soon(bar_k_full + 8 * kp, (i / NKP) & 1, abort_flag);
+        if (ok && c.j == 0) ok = mbar_wait_soon(bar_q_full + 8 * qb, (c.seg_idx / NQ) & 1, abort_flag);
+        if (ok && i >= 2) ok = mbar_wait_soon(bar_s_empty + 8 * g, ((i >> 1) - 1) & 1, abort_flag);
         if (!ok) break;
         tc_fence_after_sync();
         const uint64_t da = umma_desc_advance(dq0, qb * Q_BYTES), db = umma_desc_advance(dk0, kp * 2 * SUB_BYTES);
@@ -296,7 +296,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       int n_sub_seq = 0, kv_len = 0;
 #define PV_WAIT(bar, parity)                                                        \
   do {                                                                              \
-    ok = __all_sync(0xffffffffu, mbar_wait((bar), (parity), abort_flag));           \
+    ok = __all_sync(0xffffffffu, mbar_wait_soon((bar), (parity), abort_flag));           \
   } while (0)
       for (int i = 0; i < n_my; ++i) {
         const int g = i & 1, vp = i % NVP;
@@ -381,7 +381,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     int i0 = 0;           // index (inside the slice) of the current segment's first tile
 #define SM_WAIT(bar, parity)                                                        \
   do {                                                                              \
-    ok = __all_sync(0xffffffffu, mbar_wait((bar), (parity), abort_flag));           \
+    ok = __all_sync(0xffffffffu, mbar_wait_soon((bar), (parity), abort_flag));           \
     if (!ok) goto softmax_done;                                                     \
   } while (0)
 
