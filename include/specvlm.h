@@ -18,6 +18,9 @@
  *     library allocates nothing and keeps no state between calls.
  *   - Work is enqueued on the CUDA stream passed as `stream` (a cudaStream_t cast to void*;
  *     NULL = the legacy default stream).  No call synchronises the host with the device.
+ *     The kernels are launched with programmatic stream serialization: one may begin while the kernel
+ *     before it on the stream is still running, and touches no global memory until that kernel's
+ *     writes are complete and visible.
  *   - `d_status` (device int32_t*, optional): a kernel that gives up a bounded wait stores
  *     SPECVLM_ERR_TIMEOUT there and returns.  A kernel that finds device-side data it would have
  *     to turn into an address out of range (a kept index, a block-table entry, a tree-path node,
@@ -246,9 +249,6 @@ int32_t specvlm_gather_kv(const specvlm_kv_t* src, const int32_t* kept_idx, cons
  *   lse_or_null device fp32 [n_layers][batch][n_q][n_q_heads]: natural-log sum-exp of the logits
  *   ws          device scratch, specvlm_attn_workspace_bytes(kv, batch, n_q_heads, gamma)
  * fp32 softmax and accumulation; probabilities are rounded to bf16 before the PV product.
- * Stream order: the decode kernel (windows of at most 16 rows) is launched with programmatic stream
- * serialization; it may begin while the kernel before it on the stream is still running, and
- * touches no global memory until that kernel's writes are complete and visible.
  * Supported: head_dim 64/128; group = n_q_heads/n_kv_heads in 1..16; 0 <= gamma <= 8;
  * batch <= 127 when group * (gamma+1) > 16.  A window of more than 128 rows (group * (gamma+1))
  * is cut into parts of at most 128 rows that run side by side in one launch, so that the cache

@@ -1,9 +1,8 @@
 // Step 4c: greedy acceptance.  Kernel 1 streams the fp32 logits once (16-byte loads, all of a
 // thread's loads in flight together) and leaves one (max, lowest index) candidate per (row, vocab
 // chunk); kernel 2 finishes the argmax of the gamma+1 rows of a sequence and counts the leading
-// draft tokens that equal it.  Kernel 2 is launched with programmatic stream serialization: its
-// CTAs are scheduled while kernel 1 still runs and wait (griddepcontrol.wait) for kernel 1's
-// results, so the second launch costs no gap on the stream.
+// draft tokens that equal it; its CTAs are scheduled while kernel 1 still runs (programmatic dependent
+// launch), so the second launch costs no gap on the stream.
 #include <mutex>
 
 #include "common.cuh"
@@ -29,9 +28,9 @@ __device__ __forceinline__ void take_better(float& av, int& ai, float bv, int bi
 }
 
 __global__ void __launch_bounds__(kAcceptThreads)
-accept_partial_kernel(const float* __restrict__ logits, int vocab, int n_chunks, Cand* __restrict__ part) {
-  // the dependent kernel may be scheduled from now on; it waits for this grid's completion itself
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+accept_partial_kernel(const float* logits, int vocab, int n_chunks, Cand* __restrict__ part) {
+  pdl_launch_next();
+  pdl_wait();
   const int row = blockIdx.y, chunk = blockIdx.x;
   const float* base = logits + (size_t)row * vocab;
   const int lo = chunk * kAcceptChunk;
@@ -81,13 +80,14 @@ accept_partial_kernel(const float* __restrict__ logits, int vocab, int n_chunks,
 
 // one warp per (sequence, t); one CTA of (gamma+1) warps per sequence
 __global__ void accept_finish_kernel(const Cand* part, int n_chunks,
-                                     const int32_t* __restrict__ draft, int gamma,
+                                     const int32_t* draft, int gamma,
                                      int32_t* __restrict__ accept_len, int32_t* __restrict__ next_token,
                                      int32_t* __restrict__ g_out) {
   __shared__ int g_sm[16];
   const int b = blockIdx.x, t = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Cand* row = part + ((size_t)b * (gamma + 1) + t) * n_chunks;
-  asm volatile("griddepcontrol.wait;" ::: "memory");         // kernel 1 has completed, its candidates are visible
+  pdl_launch_next();
+  pdl_wait();                            // kernel 1 has completed, its candidates are visible
   float bv = -INFINITY;
   int bi = 0x7fffffff;
   for (int c = lane; c < n_chunks; c += 32) {
@@ -116,13 +116,14 @@ __global__ void accept_finish_kernel(const Cand* part, int n_chunks,
 // Tree drafting: one warp per node finishes its arg-max, then one thread walks from the root to
 // the child whose token is the target's choice at the current node, as long as there is one.
 __global__ void accept_tree_finish_kernel(const Cand* part, int n_chunks,
-                                          const int32_t* __restrict__ node_tokens,
-                                          const int32_t* __restrict__ parents, int n_nodes,
+                                          const int32_t* node_tokens,
+                                          const int32_t* parents, int n_nodes,
                                           int32_t* __restrict__ accept_len, int32_t* __restrict__ next_token,
                                           int32_t* __restrict__ path, int32_t* __restrict__ g_out) {
   __shared__ int g_sm[64];
   const int b = blockIdx.x, lane = threadIdx.x & 31;
-  asm volatile("griddepcontrol.wait;" ::: "memory");         // kernel 1 has completed, its candidates are visible
+  pdl_launch_next();
+  pdl_wait();                            // kernel 1 has completed, its candidates are visible
   // a warp per node; with more than 32 nodes the warps take a second one each
   for (int t = threadIdx.x >> 5; t < n_nodes; t += blockDim.x >> 5) {
     const Cand* row = part + ((size_t)b * n_nodes + t) * n_chunks;
@@ -166,24 +167,6 @@ __global__ void accept_tree_finish_kernel(const Cand* part, int n_chunks,
   }
 }
 
-// Launches `kern` so that it may be scheduled while the kernel before it in the stream still runs
-// (programmatic stream serialization); the kernel itself waits for that kernel's results.
-template <typename... KArgs, typename... Args>
-static int32_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...) != cudaSuccess) return SPECVLM_ERR_CUDA;
-  return launch_status();
-}
-
 // Built-in scratch of specvlm_accept_noalloc: room for kStaticCands (row, vocab chunk) candidates.
 // Every GPU that loads the library holds these 128 KB until the process exits.
 constexpr int kStaticCands = 16384;
@@ -215,11 +198,10 @@ extern "C" int32_t specvlm_accept(const float* target_logits, const int32_t* dra
   const int n_chunks = (vocab + kAcceptChunk - 1) / kAcceptChunk;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Cand* part = static_cast<Cand*>(ws);
-  accept_partial_kernel<<<dim3((unsigned)n_chunks, (unsigned)(batch * (gamma + 1))), kAcceptThreads, 0, st>>>(
-      target_logits, vocab, n_chunks, part);
-  int32_t rc = launch_status();
+  int32_t rc = launch_after(accept_partial_kernel, dim3((unsigned)n_chunks, (unsigned)(batch * (gamma + 1))), dim3(kAcceptThreads), 0, st,
+                            target_logits, vocab, n_chunks, part);
   if (rc != SPECVLM_OK) return rc;
-  return launch_dependent(accept_finish_kernel, dim3((unsigned)batch), dim3(32u * (gamma + 1)), st,
+  return launch_after(accept_finish_kernel, dim3((unsigned)batch), dim3(32u * (gamma + 1)), 0, st,
                           static_cast<const Cand*>(part), n_chunks, draft_tokens, gamma, accept_len, next_token,
                           target_argmax_or_null);
 }
@@ -257,11 +239,10 @@ extern "C" int32_t specvlm_accept_noalloc(const float* target_logits, const int3
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // every candidate slot that kernel 2 reads is written by kernel 1 of the same call first, so
   // nothing left over from an earlier call has to be cleared
-  accept_partial_kernel<<<dim3((unsigned)n_chunks, (unsigned)(batch * (gamma + 1))), kAcceptThreads, 0, st>>>(
-      target_logits, vocab, n_chunks, part);
-  int32_t rc = launch_status();
+  int32_t rc = launch_after(accept_partial_kernel, dim3((unsigned)n_chunks, (unsigned)(batch * (gamma + 1))), dim3(kAcceptThreads), 0, st,
+                            target_logits, vocab, n_chunks, part);
   if (rc != SPECVLM_OK) return rc;
-  return launch_dependent(accept_finish_kernel, dim3((unsigned)batch), dim3(32u * (gamma + 1)), st,
+  return launch_after(accept_finish_kernel, dim3((unsigned)batch), dim3(32u * (gamma + 1)), 0, st,
                           static_cast<const Cand*>(part), n_chunks, draft_tokens, gamma, accept_len, next_token,
                           target_argmax_or_null);
 }
@@ -281,11 +262,10 @@ extern "C" int32_t specvlm_accept_tree(const float* target_logits, const int32_t
   const int n_chunks = (vocab + kAcceptChunk - 1) / kAcceptChunk;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Cand* part = static_cast<Cand*>(ws);
-  accept_partial_kernel<<<dim3((unsigned)n_chunks, (unsigned)(batch * n_nodes)), kAcceptThreads, 0, st>>>(
-      target_logits, vocab, n_chunks, part);
-  int32_t rc = launch_status();
+  int32_t rc = launch_after(accept_partial_kernel, dim3((unsigned)n_chunks, (unsigned)(batch * n_nodes)), dim3(kAcceptThreads), 0, st,
+                            target_logits, vocab, n_chunks, part);
   if (rc != SPECVLM_OK) return rc;
-  return launch_dependent(accept_tree_finish_kernel, dim3((unsigned)batch), dim3(32u * (n_nodes < 32 ? n_nodes : 32)), st,
+  return launch_after(accept_tree_finish_kernel, dim3((unsigned)batch), dim3(32u * (n_nodes < 32 ? n_nodes : 32)), 0, st,
                           static_cast<const Cand*>(part), n_chunks, node_tokens, parents, n_nodes, accept_len,
                           next_token, path, target_argmax_or_null);
 }

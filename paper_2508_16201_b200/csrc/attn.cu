@@ -65,8 +65,8 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     tma_prefetch_desc(&tm_v);
   }
   __syncthreads();                       // the barriers are initialised
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch_next();
+  pdl_wait();
 
   // The first tile of an unsplit, contiguous cache sits at a known place whatever the sequence's
   // length (rows past the cache's end are zero-filled by the copy): the producer asks for it
@@ -470,19 +470,7 @@ static int32_t launch_rows16_s(const CUtensorMap& tk, const CUtensorMap& tv, con
   auto kern = attn_rows16_kernel<D, STAGES, NG>;
   static std::atomic<uint64_t> attr_done{0};
   if (!smem_attr_once(attr_done, reinterpret_cast<const void*>(kern), SMEM)) return SPECVLM_ERR_CUDA;
-  // launched with programmatic stream serialization: see the kernel's griddepcontrol.wait
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(32 * (4 * NG + 1), 1, 1);
-  cfg.dynamicSmemBytes = SMEM;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, kern, tk, tv, p) != cudaSuccess) return SPECVLM_ERR_CUDA;
-  return launch_status();
+  return launch_after(kern, grid, dim3(32 * (4 * NG + 1)), (size_t)SMEM, st, tk, tv, p);
 }
 
 // Ring depth: 3 stages let two CTAs share an SM; a launch with no more CTAs than SMs would leave

@@ -113,7 +113,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 
   // the plan needs the tiles inside the allocation (true whenever the base is 1024-byte aligned)
   if (big + C::BIG > raw_addr + C::TOTAL) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
     if (tid < n_here) {
       p.ws_cut[(2 * set + tid) * ctas + cta] = make_int4(0, 0, 0, 0);
       if (p.d_status) *p.d_status = SPECVLM_ERR_CUDA;
@@ -161,8 +161,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     }
     fence_proxy_async();
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch_next();
+  pdl_wait();
   if (warp == 0) {
     const bool empty = tile_prefix(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;
@@ -218,8 +218,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         int blk[2], blk_next[2] = {sg.b, sg.b};
         if (table) {
           const int s0 = 2 * sg.tile0;
-          blk_next[0] = __ldg(table + s0 / subs_per_block);
-          blk_next[1] = s0 + 1 < n_sub_seq ? __ldg(table + (s0 + 1) / subs_per_block) : 0;
+          blk_next[0] = __ldcg(table + s0 / subs_per_block);
+          blk_next[1] = s0 + 1 < n_sub_seq ? __ldcg(table + (s0 + 1) / subs_per_block) : 0;
         }
         for (int j = 0; j < sg.n_tiles; ++j, ++i) {
           const int s0 = 2 * (sg.tile0 + j);                    // first sub-tile of this tile
@@ -227,8 +227,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
           blk[0] = blk_next[0];
           blk[1] = blk_next[1];
           if (table && j + 1 < sg.n_tiles) {                    // table entries of the next tile, one tile ahead
-            blk_next[0] = __ldg(table + (s0 + 2) / subs_per_block);
-            blk_next[1] = s0 + 3 < n_sub_seq ? __ldg(table + (s0 + 3) / subs_per_block) : 0;
+            blk_next[0] = __ldcg(table + (s0 + 2) / subs_per_block);
+            blk_next[1] = s0 + 3 < n_sub_seq ? __ldcg(table + (s0 + 3) / subs_per_block) : 0;
           }
           const int slot = i % n_ring;
           if (i >= n_ring) ok = mbar_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
@@ -409,7 +409,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       const int win0 = kv_len - p.n_win;
       uint64_t my_a;
       if constexpr (TREE) {
-        my_a = row_on ? __ldg(p.anc + (size_t)sg.b * p.n_win + q0 + my_t) : 0ull;
+        my_a = row_on ? __ldcg(p.anc + (size_t)sg.b * p.n_win + q0 + my_t) : 0ull;
       } else {
         my_a = row_on ? (uint64_t)(win0 + q0 + my_t + 1) : 0ull;
       }

@@ -103,7 +103,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 
   // the plan needs the tiles inside the allocation (true whenever the base is 1024-byte aligned)
   if (big + C::BIG > raw_addr + C::TOTAL) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
     if (tid == 0) {
       p.ws_cut[blockIdx.x] = make_int4(0, 0, 0, 0);
       if (p.d_status) *p.d_status = SPECVLM_ERR_CUDA;
@@ -154,8 +154,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
     fence_proxy_async();
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch_next();
+  pdl_wait();
   if (warp == 0) {
     const bool empty = tile_prefix(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;
@@ -214,8 +214,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         int blk[2], blk_next[2] = {sg.b, sg.b};
         if (table) {
           const int s0 = 2 * sg.tile0;
-          blk_next[0] = __ldg(table + s0 / subs_per_block);
-          blk_next[1] = s0 + 1 < n_sub_seq ? __ldg(table + (s0 + 1) / subs_per_block) : 0;
+          blk_next[0] = __ldcg(table + s0 / subs_per_block);
+          blk_next[1] = s0 + 1 < n_sub_seq ? __ldcg(table + (s0 + 1) / subs_per_block) : 0;
         }
         for (int j = 0; j < sg.n_tiles; ++j, ++i) {
           const int s0 = 2 * (sg.tile0 + j);                    // first sub-tile of this tile
@@ -223,8 +223,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           blk[0] = blk_next[0];
           blk[1] = blk_next[1];
           if (table && j + 1 < sg.n_tiles) {                    // table entries of the next tile, one tile ahead
-            blk_next[0] = __ldg(table + (s0 + 2) / subs_per_block);
-            blk_next[1] = s0 + 3 < n_sub_seq ? __ldg(table + (s0 + 3) / subs_per_block) : 0;
+            blk_next[0] = __ldcg(table + (s0 + 2) / subs_per_block);
+            blk_next[1] = s0 + 3 < n_sub_seq ? __ldcg(table + (s0 + 3) / subs_per_block) : 0;
           }
           const int slot = i % n_ring;
           if (i >= n_ring) ok = mbar_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
@@ -406,7 +406,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const bool warp_on = rows > 32 * quarter;         // warp-uniform: some row of this quadrant is in use
         uint64_t my_a;                                       // the row's window mask (tree) or key limit (chain)
         if constexpr (TREE) {
-          my_a = my_row < rows ? __ldg(p.anc + (size_t)sg.b * p.n_win + my_row / p.group) : 0ull;
+          my_a = my_row < rows ? __ldcg(p.anc + (size_t)sg.b * p.n_win + my_row / p.group) : 0ull;
         } else {
           my_a = my_row < rows ? (uint64_t)(win0 + my_row / p.group + 1) : 0ull;
         }
@@ -554,7 +554,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           const int r = row0(h) + lr + 8 * e;
           const int t = r / p.group;
           if constexpr (TREE) {
-            vis[h][e] = r < rows ? __ldg(p.anc + (size_t)sg.b * p.n_win + t) : 0ull;
+            vis[h][e] = r < rows ? __ldcg(p.anc + (size_t)sg.b * p.n_win + t) : 0ull;
           } else {
             lim[h][e] = r < rows ? win0 + t + 1 : 0;
           }
@@ -811,8 +811,8 @@ constexpr int kMergeChunk = 8;         // parts whose loads are in flight togeth
 
 template <int D, int LANES>
 __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnTcParams p) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch_next();
+  pdl_wait();
   const int gcta = blockIdx.x;
   const int4 cut = __ldcg(p.ws_cut + gcta);
   if (cut.w == 0) return;
@@ -982,8 +982,10 @@ static int32_t launch_merge(const AttnTcParams& p, int ctas, cudaStream_t st) {
 
 // Ancestor masks of a draft tree: bit w of anc[b][t] says that node t attends window position w
 // (itself and the nodes on its path to a root).  parents[b][t] < t, -1 for a root.
-__global__ void tree_ancestors_kernel(const int32_t* __restrict__ parents, int n, int n_nodes,
+__global__ void tree_ancestors_kernel(const int32_t* parents, int n, int n_nodes,
                                       uint64_t* __restrict__ anc, int32_t* d_status) {
+  pdl_launch_next();
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int t = i % n_nodes;
@@ -1074,8 +1076,8 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   if (tree_parents) {
     uint64_t* anc = reinterpret_cast<uint64_t*>(static_cast<uint8_t*>(ws) + base_bytes);
     const int n = batch * n_q;
-    tree_ancestors_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(tree_parents, n, n_q, anc, d_status);
-    rc = launch_status();
+    rc = launch_after(tree_ancestors_kernel, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, st, tree_parents, n, n_q, anc,
+                      d_status);
     if (rc != SPECVLM_OK) return rc;
     p.anc = anc;
   }

@@ -25,6 +25,8 @@ struct AppendParams {
 
 // one thread per 16-byte chunk of a new token row
 __global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ AppendParams p) {
+  pdl_launch_next();
+  pdl_wait();
   const int64_t total = (int64_t)p.n_layers * p.batch * p.n_new * p.n_kv_heads * p.chunks_per_row;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     int64_t r = i;
@@ -42,7 +44,7 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ 
     }
     int blk = b, off = pos;
     if (p.table) {
-      blk = __ldg(p.table + (size_t)b * p.max_blocks + pos / p.block_tokens);
+      blk = *(p.table + (size_t)b * p.max_blocks + pos / p.block_tokens);
       off = pos % p.block_tokens;
       if (blk < 0 || blk >= p.n_blocks) {
         if (p.d_status) *p.d_status = SPECVLM_ERR_INVALID_ARG;
@@ -58,6 +60,8 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ 
 // seq_lens[b] += delta, or, with accept_len, seq_lens[b] -= gamma - accept_len[b]
 __global__ void seq_len_update_kernel(int32_t* seq_lens, const int32_t* accept_len, int batch, int delta, int gamma,
                                       int max_seq_len, int32_t* d_status) {
+  pdl_launch_next();
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= batch) return;
   int n = seq_lens[b];
@@ -90,6 +94,8 @@ struct CompactParams {
 // One CTA per (layer, KV head, sequence): the accepted nodes' rows move up behind the root.  A
 // destination row can be a later move's source, so every row is read before any is written.
 __global__ void __launch_bounds__(256) compact_tree_kernel(const __grid_constant__ CompactParams p) {
+  pdl_launch_next();
+  pdl_wait();
   const int b = blockIdx.y;
   const int layer = blockIdx.x / p.n_kv_heads, head = blockIdx.x - layer * p.n_kv_heads;
   const int n = min(max(p.accept_len[b], 0), p.n_nodes - 1);
@@ -100,7 +106,7 @@ __global__ void __launch_bounds__(256) compact_tree_kernel(const __grid_constant
   auto addr = [&](int pos, int chunk) -> int64_t {
     int blk = b, off = pos;
     if (p.table) {
-      blk = __ldg(p.table + (size_t)b * p.max_blocks + pos / p.block_tokens);
+      blk = *(p.table + (size_t)b * p.max_blocks + pos / p.block_tokens);
       off = pos % p.block_tokens;
       if (blk < 0 || blk >= p.n_blocks) return -1;
     }
@@ -147,6 +153,8 @@ __global__ void __launch_bounds__(256) compact_tree_kernel(const __grid_constant
 // seq_lens[b] = seq_lens[b] - n_nodes + 1 + accept_len[b]
 __global__ void tree_len_kernel(int32_t* seq_lens, const int32_t* accept_len, int batch, int n_nodes,
                                 int32_t* d_status) {
+  pdl_launch_next();
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= batch) return;
   const int a = accept_len[b], n = seq_lens[b];
@@ -189,22 +197,19 @@ extern "C" int32_t specvlm_append_kv(const specvlm_kv_t* kv, const void* new_k, 
   const int64_t cap = (int64_t)sm_count() * 8;
   if (blocks > cap) blocks = cap;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  append_kv_kernel<<<(unsigned)blocks, 256, 0, st>>>(p);
-  rc = launch_status();
+  rc = launch_after(append_kv_kernel, dim3((unsigned)blocks), dim3(256), 0, st, p);
   if (rc != SPECVLM_OK) return rc;
   // the lengths change only after every row has been placed by the kernel above
-  seq_len_update_kernel<<<(unsigned)((batch + 127) / 128), 128, 0, st>>>(seq_lens_inout, nullptr, batch, n_new, 0,
-                                                                         c.max_seq_len, d_status);
-  return launch_status();
+  return launch_after(seq_len_update_kernel, dim3((unsigned)((batch + 127) / 128)), dim3(128), 0, st, seq_lens_inout, nullptr,
+                      batch, n_new, 0, c.max_seq_len, d_status);
 }
 
 extern "C" int32_t specvlm_rollback_kv(int32_t* seq_lens_inout, const int32_t* accept_len, int32_t batch,
                                        int32_t gamma, int32_t* d_status, void* stream) {
   NvtxRange nvtx_range(__func__);
   if (!seq_lens_inout || !accept_len || batch < 1 || gamma < 0) return SPECVLM_ERR_INVALID_ARG;
-  seq_len_update_kernel<<<(unsigned)((batch + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream)>>>(
-      seq_lens_inout, accept_len, batch, 0, gamma, 0, d_status);
-  return launch_status();
+  return launch_after(seq_len_update_kernel, dim3((unsigned)((batch + 127) / 128)), dim3(128), 0,
+                      static_cast<cudaStream_t>(stream), seq_lens_inout, accept_len, batch, 0, gamma, 0, d_status);
 }
 
 extern "C" int32_t specvlm_compact_tree_kv(const specvlm_kv_t* kv, const int32_t* path, const int32_t* accept_len,
@@ -231,10 +236,8 @@ extern "C" int32_t specvlm_compact_tree_kv(const specvlm_kv_t* kv, const int32_t
   p.n_blocks = c.n_blocks; p.max_seq_len = c.max_seq_len; p.d_status = d_status;
   p.n_kv_heads = c.n_kv_heads; p.chunks_per_row = c.head_dim / 8;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  compact_tree_kernel<<<dim3((unsigned)(c.n_layers * c.n_kv_heads), (unsigned)batch), 256, 0, st>>>(p);
-  rc = launch_status();
+  rc = launch_after(compact_tree_kernel, dim3((unsigned)(c.n_layers * c.n_kv_heads), (unsigned)batch), dim3(256), 0, st, p);
   if (rc != SPECVLM_OK) return rc;
-  tree_len_kernel<<<(unsigned)((batch + 127) / 128), 128, 0, st>>>(seq_lens_inout, accept_len, batch, n_nodes,
-                                                                   d_status);
-  return launch_status();
+  return launch_after(tree_len_kernel, dim3((unsigned)((batch + 127) / 128)), dim3(128), 0, st, seq_lens_inout, accept_len,
+                      batch, n_nodes, d_status);
 }

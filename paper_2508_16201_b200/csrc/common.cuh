@@ -19,6 +19,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Programmatic dependent launch.  Every kernel of the library is launched so that it may start while the
+// kernel before it in the stream still runs (launch_after), lets its own successor start as soon as all
+// its CTAs run, and waits for the predecessor's completion, in every CTA, before its first access to global
+// memory: what precedes the wait (barriers, tensor memory, descriptors, the launch itself) costs no time on the
+// stream.  Data that an earlier kernel may have written is therefore never read through the non-coherent path
+// (__ldg, const __restrict__): a line cached before the wait would not be dropped by it.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

@@ -35,6 +35,8 @@ struct GatherParams {
 };
 
 __global__ void __launch_bounds__(256) gather_kv_kernel(const __grid_constant__ GatherParams p) {
+  pdl_launch_next();
+  pdl_wait();
   const int bl = blockIdx.z;                 // sequence within this launch
   const GatherSeq sq = p.seq[bl];
   const int b = p.batch0 + bl;
@@ -49,7 +51,7 @@ __global__ void __launch_bounds__(256) gather_kv_kernel(const __grid_constant__ 
     if (j < sq.video_start) {
       sp = j;
     } else if (j < sq.video_start + sq.kept_n) {
-      const int kj = __ldg(p.kept_idx + sq.kept_off + (j - sq.video_start));
+      const int kj = *(p.kept_idx + sq.kept_off + (j - sq.video_start));
       ok = kj >= 0 && kj < sq.video_len;
       sp = sq.video_start + kj;
     } else {
@@ -57,13 +59,13 @@ __global__ void __launch_bounds__(256) gather_kv_kernel(const __grid_constant__ 
     }
     int sblk = b, soff = sp;
     if (ok && p.src_table) {
-      sblk = __ldg(p.src_table + (size_t)b * p.src_max_blocks + sp / p.src_block_tokens);
+      sblk = *(p.src_table + (size_t)b * p.src_max_blocks + sp / p.src_block_tokens);
       soff = sp % p.src_block_tokens;
       ok = sblk >= 0 && sblk < p.src_n_blocks;
     }
     int dblk = b, doff = j;
     if (ok && p.dst_table) {
-      dblk = __ldg(p.dst_table + (size_t)b * p.dst_max_blocks + j / p.dst_block_tokens);
+      dblk = *(p.dst_table + (size_t)b * p.dst_max_blocks + j / p.dst_block_tokens);
       doff = j % p.dst_block_tokens;
       ok = dblk >= 0 && dblk < p.dst_n_blocks;
     }
@@ -153,8 +155,7 @@ extern "C" int32_t specvlm_gather_kv(const specvlm_kv_t* src, const int32_t* kep
     if (gx > 64) gx = 64;                    // each CTA strides over the rest of its slab
     if (gx < 1) gx = 1;
     dim3 grid((unsigned)gx, (unsigned)(s.n_layers * s.n_kv_heads), (unsigned)nb);
-    gather_kv_kernel<<<grid, 256, 0, st>>>(p);
-    rc = launch_status();
+    rc = launch_after(gather_kv_kernel, grid, dim3(256), 0, st, p);
     if (rc != SPECVLM_OK) return rc;
   }
   return SPECVLM_OK;

@@ -168,6 +168,8 @@ scores_colsum_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   }
   if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
   tc_fence_before_sync();
+  pdl_launch_next();
+  pdl_wait();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
@@ -260,7 +262,7 @@ scores_colsum_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
       float v = 0.f;
       if (fu < n_units) {
         const int rows_valid = min(p.qt, sq.n_text - ft * p.qt) * p.group;
-        v = et < rows_valid ? -__ldg(lse_row + (size_t)(ft * p.qt) * p.n_q_heads + fu * p.group) * kLog2e : -INFINITY;
+        v = et < rows_valid ? -__ldcg(lse_row + (size_t)(ft * p.qt) * p.n_q_heads + fu * p.group) * kLog2e : -INFINITY;
       }
       ft += NG;                                 // this group's next tile
       while (ft >= n_qt) {
@@ -410,6 +412,8 @@ scores_lse_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   }
   if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
   tc_fence_before_sync();
+  pdl_launch_next();
+  pdl_wait();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
@@ -563,6 +567,8 @@ scores_lse_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
 // scores[j] = (sum over layers, in order, of partial[l][j]) / (L * Hq * n_text of j's sequence)
 __global__ void scores_finish_kernel(const __grid_constant__ ScoreParams p, float* __restrict__ scores) {
+  pdl_launch_next();
+  pdl_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= p.sum_video) return;
   int b = 0;
@@ -697,8 +703,7 @@ static int32_t launch_lse(ScoreSetup& su, cudaStream_t st) {
   auto k = scores_lse_tc_kernel<D, STAGES>;
   static std::atomic<uint64_t> attr_done{0};
   if (!smem_attr_once(attr_done, reinterpret_cast<const void*>(k), SMEM)) return SPECVLM_ERR_CUDA;
-  k<<<grid, 320, SMEM, st>>>(su.tk, su.tq, su.p1);
-  return launch_status();
+  return launch_after(k, grid, dim3(320), (size_t)SMEM, st, su.tk, su.tq, su.p1);
 }
 
 template <int D>
@@ -709,8 +714,8 @@ static int32_t launch_colsum(ScoreSetup& su, cudaStream_t st) {
   auto k = scores_colsum_tc_kernel<D, STAGES>;
   static std::atomic<uint64_t> attr_done{0};
   if (!smem_attr_once(attr_done, reinterpret_cast<const void*>(k), SMEM)) return SPECVLM_ERR_CUDA;
-  k<<<dim3((unsigned)su.n_key_blocks, (unsigned)su.layer_count), kColsumThreads, SMEM, st>>>(su.tk, su.tq, su.p2);
-  return launch_status();
+  return launch_after(k, dim3((unsigned)su.n_key_blocks, (unsigned)su.layer_count), dim3(kColsumThreads), (size_t)SMEM, st,
+                      su.tk, su.tq, su.p2);
 }
 
 }  // namespace specvlm
@@ -788,8 +793,7 @@ static int32_t stage1_scores_range(const specvlm_kv_t* target_kv, const void* q_
   ScoreParams pf = su.p2;                  // all layers' partial sums, in layer order
   pf.partial = partial_all;
   pf.n_layers = su.kv.n_layers;
-  scores_finish_kernel<<<(unsigned)((pf.sum_video + 255) / 256), 256, 0, st>>>(pf, scores);
-  return launch_status();
+  return launch_after(scores_finish_kernel, dim3((unsigned)((pf.sum_video + 255) / 256)), dim3(256), 0, st, pf, scores);
 }
 
 extern "C" int32_t specvlm_stage1_scores(const specvlm_kv_t* target_kv, const void* q_text,

@@ -218,6 +218,10 @@ __global__ void __launch_bounds__(kSelThreads, KEYS <= 6 ? 2 : 1) select_kernel(
   const int n_keys = (n_v + n_cta * kSelThreads - 1) / (n_cta * kSelThreads);
   const int j0 = (rank * kSelWarps + warp) * 32 * n_keys + lane;   // this thread's tokens: j0 + 32 i
 
+  pdl_launch_next();
+  for (int i = tid; i < 3 * 256 * kSelCopies / 4; i += kSelThreads)
+    reinterpret_cast<uint4*>(&sm.hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+  pdl_wait();
   // order-preserving map float -> uint32 (larger float <=> larger key)
   uint32_t key[KEYS];
   uint32_t valid = 0u;
@@ -232,13 +236,11 @@ __global__ void __launch_bounds__(kSelThreads, KEYS <= 6 ? 2 : 1) select_kernel(
         const float r = (float)(philox4x32_10_word0((uint32_t)j, (uint32_t)sq.seq_index, p.seed_lo, p.seed_hi) >> 8);
         key[i] = __float_as_uint(r) | 0x80000000u;
       } else {
-        const uint32_t u = __float_as_uint(__ldg(p.scores + sq.score_off + j));
+        const uint32_t u = __float_as_uint(__ldcg(p.scores + sq.score_off + j));
         key[i] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
       }
     }
   }
-  for (int i = tid; i < 3 * 256 * kSelCopies / 4; i += kSelThreads)
-    reinterpret_cast<uint4*>(&sm.hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
 
   uint32_t thr = 0u;                   // selected: keys above thr, and the first k_rem keys equal to it
   int k_rem = 0;
@@ -495,6 +497,8 @@ struct RangeParams {
 };
 
 __global__ void baseline_ranges_kernel(const __grid_constant__ RangeParams p) {
+  pdl_launch_next();
+  pdl_wait();
   const int i = blockIdx.x;
   const int F = p.n_frames[i], T = p.tokens_per_frame, K = p.k_total[i], n_v = F * T;
   int32_t* out = p.kept_idx + p.kept_off[i];
@@ -523,13 +527,15 @@ static int32_t launch_select(const SelParams& p, int n_seq, int n_cta, cudaStrea
   cfg.blockDim = dim3(kSelThreads);
   cfg.dynamicSmemBytes = sizeof(SelSmem);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)n_cta;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   if (cudaLaunchKernelEx(&cfg, select_kernel<KEYS>, p) != cudaSuccess) return SPECVLM_ERR_CUDA;
   return launch_status();
 }
@@ -661,8 +667,7 @@ extern "C" int32_t specvlm_select_baseline(int32_t mode, uint64_t seed, const in
       p.k_total[i] = k_total[b];
       p.kept_off[i] = kept_cu[b];
     }
-    baseline_ranges_kernel<<<(unsigned)nb, 256, 0, st>>>(p);
-    const int32_t rc = launch_status();
+    const int32_t rc = launch_after(baseline_ranges_kernel, dim3((unsigned)nb), dim3(256), 0, st, p);
     if (rc != SPECVLM_OK) return rc;
   }
   return SPECVLM_OK;
