@@ -402,9 +402,11 @@ int32_t specvlm_debug_wait_timeout(int32_t limit_ms, int32_t* d_status, int32_t*
                                    void* stream);
 
 /*
- * Test hook; the paper has no counterpart.  n_splits > 0 makes every later attention call of up
- * to 16 rows per KV head cut each sequence into that many CTAs (capped by its tile count), so
- * that tests reach the split-merge path at any size; 0 restores the built-in choice.  Process-wide.
+ * Test hook; the paper has no counterpart.  For every later attention call of up to 16 rows per KV
+ * head, n_splits = 1 forces a CTA per (layer, sequence, KV head) and n_splits > 1 slices of the list
+ * of all tiles that cut a sequence about that many times (capped by its tile count), so that tests
+ * reach both kernels and the merge of cut sequences at any size; 0 restores the built-in choice.
+ * Process-wide.
  */
 void specvlm_debug_set_attn_splits(int32_t n_splits);
 

@@ -164,7 +164,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   pdl_launch_next();
   pdl_wait();
   if (warp == 0) {
-    const bool empty = tile_prefix(p, prefix, lane);
+    const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;
   }
   tc_fence_before_sync();

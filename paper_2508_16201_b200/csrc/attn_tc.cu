@@ -157,7 +157,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   pdl_launch_next();
   pdl_wait();
   if (warp == 0) {
-    const bool empty = tile_prefix(p, prefix, lane);
+    const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;
   }
   tc_fence_before_sync();
@@ -1010,6 +1010,10 @@ size_t attn_tc_tree_extra_bytes(int32_t batch, int32_t n_nodes) {
   return round_up((size_t)batch * n_nodes * sizeof(uint64_t), 256);
 }
 
+int32_t attn_merge_launch(const AttnTcParams& p, int head_dim, int ctas, cudaStream_t st) {
+  return head_dim == 128 ? launch_merge<128>(p, ctas, st) : launch_merge<64>(p, ctas, st);
+}
+
 template <int D, int M>
 static int32_t launch_tc(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const AttnTcParams& p,
                          int grid, cudaStream_t st) {
@@ -1050,6 +1054,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   if (rc != SPECVLM_OK) return rc;
 
   AttnTcParams p;
+  p.q = static_cast<const __nv_bfloat16*>(q);
   p.out = static_cast<__nv_bfloat16*>(out);
   p.lse = lse;
   uint8_t* w = static_cast<uint8_t*>(ws);
@@ -1092,7 +1097,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   else
     rc = p.rows <= 64 ? launch_tc<64, 64>(tk, tv, tq, p, ctas, st) : launch_tc<64, 128>(tk, tv, tq, p, ctas, st);
   if (rc != SPECVLM_OK) return rc;
-  return kv->head_dim == 128 ? launch_merge<128>(p, ctas, st) : launch_merge<64>(p, ctas, st);
+  return attn_merge_launch(p, kv->head_dim, ctas, st);
 }
 
 }  // namespace specvlm

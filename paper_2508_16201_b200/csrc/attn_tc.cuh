@@ -1,6 +1,6 @@
-// Shared by the two tcgen05 attention kernels (attn_tc.cu: windows of up to 128 rows; attn_pair.cu: wider
-// ones): launch parameters, tensor-memory access, the cold paths of the softmax loops and the
-// hand-over of cut items to the merge kernel.
+// Shared by the attention kernels that work on slices of the flat tile list (attn_tc.cu: windows of up to 128
+// rows; attn_pair.cu: wider ones; attn.cu: up to 16 rows): launch parameters, tensor-memory access, the cold paths of
+// the softmax loops and the hand-over of cut items to the merge kernel.
 #pragma once
 #include "attn.cuh"
 #include "attn_sched.h"
@@ -9,6 +9,7 @@
 namespace specvlm {
 
 struct AttnTcParams {
+  const __nv_bfloat16* q;     // [L][B][n_win][Hq][D] (the kernels of attn_tc.cu and attn_pair.cu read it through a tensor map)
   __nv_bfloat16* out;         // [L][B][n_win][Hq][D]
   float* lse;                 // [L][B][n_win][Hq] or null
   float* ws_o;                // partial results: [2 * grid][rows][D], normalised
@@ -148,8 +149,9 @@ __device__ __noinline__ void rescale_o_half(uint32_t oaddr, float f0, float f1) 
   tmem_st_wait();
 }
 
-// Running sum of the tiles per sequence, by one warp: prefix[b] = tiles of the sequences before b.
+// Running sum of the tiles (of TILE tokens) per sequence, by one warp: prefix[b] = tiles of the sequences before b.
 // Returns whether some sequence has no token.
+template <int TILE>
 __device__ __forceinline__ bool tile_prefix(const AttnTcParams& p, int* prefix, int lane) {
   int carry = 0;
   bool empty = false;
@@ -157,7 +159,7 @@ __device__ __forceinline__ bool tile_prefix(const AttnTcParams& p, int* prefix, 
     const int b = b0 + lane;
     int v = 0;
     if (b < p.batch) {
-      v = (clamp_len(p.seq_lens[b], p.max_seq_len) + kBigTokens - 1) / kBigTokens;
+      v = (clamp_len(p.seq_lens[b], p.max_seq_len) + TILE - 1) / TILE;
       empty |= v == 0;
     }
 #pragma unroll
@@ -187,6 +189,9 @@ __device__ __forceinline__ void publish_cut_item(const AttnTcParams& p, bool act
   }
   p.ws_cut[gcta] = cut;
 }
+
+// attn_tc.cu: the merge of the items that slice boundaries cut, for a launch of n_parts sets of `ctas` CTAs
+int32_t attn_merge_launch(const AttnTcParams& p, int head_dim, int ctas, cudaStream_t st);
 
 // (a template of the kernel itself: kernels of one signature must not share the flag below)
 template <auto kern>

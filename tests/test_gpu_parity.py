@@ -97,6 +97,33 @@ def test_decode_ragged_batch_paged_poisoned():
               splits=4, extra_capacity=5)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("lens", [[1], [64, 0, 65], [0, 0], [3, 1000, 63, 130], [2111], [257] * 40])
+def test_decode_on_slices(lens, D):
+    """The slice kernel at every kind of slice: one tile, empty sequences between others, all empty, items cut
+    by several boundaries, several items per CTA with the ring running over their boundaries (NaN past every end)."""
+    from gpu_util import make_cache
+    if max(lens) > 0 and min(lens) > 0:
+        for splits in (2, 7, 64):
+            _run_attn(2, 28, 4, D, lens, 0, paged=len(lens) % 2 == 0, seed=60 + len(lens), decode_api=True, splits=splits,
+                      poison=True)
+        return
+    cache, k, v = make_cache(1, 4, D, [max(n, 1) for n in lens], paged=False, seed=61, extra_capacity=3)
+    cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    q = synth.randn_bf16((1, len(lens), 28, D), "cuda", 61, "Q")
+    specvlm.debug_set_attn_splits(5)
+    try:
+        out = f64(specvlm.draft_decode_attn(cache, q, 0.1))
+    finally:
+        specvlm.debug_set_attn_splits(0)
+    for b, n in enumerate(lens):
+        if n == 0:
+            assert (out[0, b] == 0).all()
+        else:
+            ref, _ = oracle.attention(bits(q)[0, b][None], k[b][0], v[b][0], n, 0.1)
+            assert row_rel_err(out[0, b], ref[0]) <= ATTN_TOL
+
+
 def test_decode_group_sizes():
     for Hq, Hkv in [(4, 4), (16, 1), (10, 2), (32, 4)]:
         _run_attn(1, Hq, Hkv, 128, [200], 0, paged=False, seed=4, decode_api=True)
