@@ -268,9 +268,9 @@ class Path:
                                   device=device)
         self.status = torch.zeros(1, dtype=torch.int32, device=device)
         # launches of our kernels per step: row LSE 1, rating 2 (column sums + finish), select 1,
-        # gather 1, one per draft decode step, verify 1, accept 2 (split merges run inside the
-        # attention kernels; the counter resets before them are memsets, not counted)
-        self.launches_per_step = 1 + 2 + 1 + 1 + w.gamma + 1 + 2
+        # gather 1, one per draft decode step (a CTA per item at this size, no merge), verify 2 (the attention
+        # kernel and the merge of the items that its slices cut), accept 2
+        self.launches_per_step = 1 + 2 + 1 + 1 + w.gamma + 2 + 2
 
     # the calls, in path order ------------------------------------------------------------------
     def row_lse_call(self):
