@@ -807,12 +807,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 // call's 37.8 us, plus a memset of the counters and 2.5 us of fences per partial result.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMergeThreads = 256;
-constexpr int kMergeChunk = 8;         // parts whose loads are in flight together
 
 template <int D, int LANES>
 __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnTcParams p) {
   pdl_launch_next();
   pdl_wait();
+  // parts whose loads are in flight together: most cut items have two parts, and the registers of more would
+  // keep blocks off the SMs (26-node tree under sustained load 677 -> 668 us, and 80-layer chain 359.5 -> 358.1); the
+  // many parts of a few items are what LANES is for
+  constexpr int kMergeChunk = LANES == 1 ? 2 : 8;
   const int gcta = blockIdx.x;
   const int4 cut = __ldcg(p.ws_cut + gcta);
   if (cut.w == 0) return;
