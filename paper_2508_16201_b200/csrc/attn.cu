@@ -323,6 +323,18 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   }
 
   // -------------------------------------------------------------------- consumers
+  if (n_my == 0) {
+    // An empty sequence: its outputs are zero, its LSE -inf.  The ring stays untouched: the tile that the producer
+    // asked for before it knew the length may still be landing there, with whatever the cache rows hold.
+    for (int idx = tid; idx < p.rows * (D / 8); idx += 128 * NG) {
+      const int r = idx / (D / 8), c8 = idx - r * (D / 8);
+      const int t = r / p.group, h = g * p.group + (r - t * p.group);
+      const size_t orow = ((size_t)lb * p.n_q + t) * p.n_q_heads + h;
+      *reinterpret_cast<uint4*>(p.out + orow * D + c8 * 8) = make_uint4(0, 0, 0, 0);
+      if (p.lse && c8 == 0) p.lse[orow] = -INFINITY;
+    }
+    return;
+  }
   const int cw = warp & 3, grp = warp >> 2;                           // token slice, consumer group
   Rows16<D> st;
   st.start(p, p.n_q, p.rows, lb, g, kv_len, lane);

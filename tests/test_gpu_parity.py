@@ -108,17 +108,48 @@ def test_decode_on_slices(lens, D):
             _run_attn(2, 28, 4, D, lens, 0, paged=len(lens) % 2 == 0, seed=60 + len(lens), decode_api=True, splits=splits,
                       poison=True)
         return
+    # empty sequences, whose rows are NaN throughout: on the slices, with a CTA per item (1) and as the rule has it
     cache, k, v = make_cache(1, 4, D, [max(n, 1) for n in lens], paged=False, seed=61, extra_capacity=3)
     cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    for b, n in enumerate(lens):
+        cache.k[:, b, :, n:] = float("nan")
+        cache.v[:, b, :, n:] = float("nan")
     q = synth.randn_bf16((1, len(lens), 28, D), "cuda", 61, "Q")
-    specvlm.debug_set_attn_splits(5)
+    lse = torch.zeros((1, len(lens), 28), dtype=torch.float32, device="cuda")
+    for splits in (5, 1, 0):
+        specvlm.debug_set_attn_splits(splits)
+        try:
+            out = f64(specvlm.draft_decode_attn(cache, q, 0.1, lse=lse))
+        finally:
+            specvlm.debug_set_attn_splits(0)
+        for b, n in enumerate(lens):
+            if n == 0:
+                assert (out[0, b] == 0).all() and torch.isneginf(lse[0, b]).all(), splits
+            else:
+                ref, _ = oracle.attention(bits(q)[0, b][None], k[b][0], v[b][0], n, 0.1)
+                assert row_rel_err(out[0, b], ref[0]) <= ATTN_TOL, splits
+
+
+def test_decode_empty_sequences_among_many_items():
+    """More items than SMs (the launch shape of two CTAs per SM) with every other sequence empty, all of whose
+    cache rows are NaN: zeros and an LSE of -inf there, the others as the oracle has them."""
+    from gpu_util import make_cache
+    lens = [70 if b % 2 else 0 for b in range(48)]
+    cache, k, v = make_cache(1, 4, 128, [max(n, 1) for n in lens], paged=False, seed=62)
+    cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    for b, n in enumerate(lens):
+        cache.k[:, b, :, n:] = float("nan")
+        cache.v[:, b, :, n:] = float("nan")
+    q = synth.randn_bf16((1, len(lens), 28, 128), "cuda", 62, "Q")
+    lse = torch.zeros((1, len(lens), 28), dtype=torch.float32, device="cuda")
+    specvlm.debug_set_attn_splits(1)
     try:
-        out = f64(specvlm.draft_decode_attn(cache, q, 0.1))
+        out = f64(specvlm.draft_decode_attn(cache, q, 0.1, lse=lse))
     finally:
         specvlm.debug_set_attn_splits(0)
     for b, n in enumerate(lens):
         if n == 0:
-            assert (out[0, b] == 0).all()
+            assert (out[0, b] == 0).all() and torch.isneginf(lse[0, b]).all()
         else:
             ref, _ = oracle.attention(bits(q)[0, b][None], k[b][0], v[b][0], n, 0.1)
             assert row_rel_err(out[0, b], ref[0]) <= ATTN_TOL
