@@ -249,6 +249,8 @@ int32_t specvlm_gather_kv(const specvlm_kv_t* src, const int32_t* kept_idx, cons
  *   lse_or_null device fp32 [n_layers][batch][n_q][n_q_heads]: natural-log sum-exp of the logits
  *   ws          device scratch, specvlm_attn_workspace_bytes(kv, batch, n_q_heads, gamma)
  * fp32 softmax and accumulation; probabilities are rounded to bf16 before the PV product.
+ * After SPECVLM_ERR_TIMEOUT out and lse hold nothing that was computed from unfinished partial results: the heads
+ * whose work was given up keep, in whole or in part, what was there before the call.
  * Supported: head_dim 64/128; group = n_q_heads/n_kv_heads in 1..16; 0 <= gamma <= 8;
  * batch <= 127 when group * (gamma+1) > 16.  A window of more than 128 rows (group * (gamma+1))
  * is cut into parts of at most 128 rows that run side by side in one launch, so that the cache
@@ -409,6 +411,18 @@ int32_t specvlm_debug_wait_timeout(int32_t limit_ms, int32_t* d_status, int32_t*
  * Process-wide.
  */
 void specvlm_debug_set_attn_splits(int32_t n_splits);
+
+/*
+ * Test hook; the paper has no counterpart.  Runs the second kernel of an attention call again, the one that folds the
+ * partial results of the (layer, sequence, KV head) items that more than one CTA has worked on, over the
+ * scratch that the call left in ws: kv, batch, n_q_heads and ws as in specvlm_draft_decode_attn (n_q = 1) or
+ * specvlm_verify_attn (n_q = gamma + 1).  lost_cta >= 0 first marks that CTA's partial results as not to be used, as the
+ * CTA itself does when a bounded wait expires: items with such a part stay as they are in out and lse.  n_ctas (host int32 out): the CTAs of the
+ * call, 0 (with SPECVLM_ERR_UNSUPPORTED_SHAPE) if it has no second kernel.  The mark stays in ws.
+ */
+int32_t specvlm_debug_attn_merge(const specvlm_kv_t* kv, int32_t batch, int32_t n_q_heads, int32_t n_q, void* out,
+                                 float* lse_or_null, void* ws, size_t ws_bytes, int32_t lost_cta, int32_t* n_ctas,
+                                 void* stream);
 
 /*
  * Test hook, host only; the paper has no counterpart.  Reports how a verification window of n_q

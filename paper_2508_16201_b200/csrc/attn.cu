@@ -372,6 +372,18 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   }
 }
 
+// bar.sync 1 over n threads (whole warps) that also answers whether the predicate holds for all of them
+__device__ __forceinline__ bool bar_and(bool pred, int n) {
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(all) : "r"((uint32_t)pred), "r"(n) : "memory");
+  return all != 0;
+}
+
 // ---------------------------------------------------------------------------------------------
 // The same on slices: a persistent CTA per SM streams a contiguous slice of the flat (layer, sequence, KV
 // head, 64-token tile) list (attn_sched.h), whatever the items' number and lengths, so that every SM moves the
@@ -430,6 +442,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
     const bool empty = tile_prefix<kTileTokens>(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;
   }
+  if (warp > 0 && warp < NW) unwritten_parts(p, blockIdx.x, D, tid - 32, 32 * (NW - 1));
   __syncthreads();
   const int hkv = p.n_kv_heads, cta = blockIdx.x;
   const int64_t total = (int64_t)p.n_layers * hkv * prefix[p.batch];
@@ -528,10 +541,11 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
     // merge the consumer warps' partials; the first barrier also says that the previous item's have been read
     const bool complete = sg.tile0 == 0 && sg.n_tiles == sg.item_tiles;
     const int slot = partial_slot(cta, T0, sg.item_begin);
-    asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
+    // and whether every consumer has seen all its tiles: one answer for all threads, so that a row is stored whole or not at all
+    const bool whole = bar_and(alive, 128 * NG);
     st.publish(o_sm, m_sm, l_sm, p.rows, warp, lane);
     asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
-    if (alive && !*abort_flag) {
+    if (whole) {
       for (int idx = tid; idx < p.rows * (D / 4); idx += 128 * NG) {
         const int r = idx / (D / 4), ch = (idx - r * (D / 4)) * 4;
         float4 acc;
@@ -544,7 +558,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
         } else {
           const size_t prow = (size_t)slot * p.rows + r;
           *reinterpret_cast<float4*>(p.ws_o + prow * D + ch) = acc;
-          if (ch == 0) p.ws_lse[prow] = lse2;
+          if (ch % 64 == 0) p.ws_lse[(size_t)(ch / 64) * p.lse_block + prow] = lse2;
         }
       }
     }
@@ -598,20 +612,9 @@ static int rows16_slices(const specvlm_kv_t* kv, int32_t batch) {
   return sched_active_ctas(items * tiles, (int)sms);
 }
 
-// scratch of a launch on slices: two partial results [rows][D] fp32 per CTA, their LSEs, and the item that
-// the CTA's slice cuts
-static void rows16_ws_layout(int ctas, int rows, int head_dim, size_t& o_bytes, size_t& lse_bytes, size_t& cut_bytes) {
-  o_bytes = round_up((size_t)2 * ctas * rows * head_dim * sizeof(float), 256);
-  lse_bytes = round_up((size_t)2 * ctas * rows * sizeof(float), 256);
-  cut_bytes = round_up((size_t)ctas * sizeof(int4), 256);
-}
-
 static size_t rows16_ws_bytes(const specvlm_kv_t* kv, int32_t batch, int rows) {
   const int ctas = rows16_slices(kv, batch);
-  if (ctas == 0) return 256;
-  size_t a, b, c;
-  rows16_ws_layout(ctas, rows, kv->head_dim, a, b, c);
-  return a + b + c;
+  return ctas == 0 ? 256 : SliceScratch(ctas, rows, kv->head_dim).bytes();
 }
 
 // tcgen05 path (attn_tc.cu)
@@ -652,6 +655,12 @@ static int32_t launch_slices(const CUtensorMap& tk, const CUtensorMap& tv, const
   return launch_after(kern, dim3((unsigned)ctas), dim3(32 * (4 * C::NG + 1)), (size_t)C::SMEM, st, tk, tv, p);
 }
 
+// Test hook (specvlm_debug_attn_merge): one CTA's partial results as if it had given up, without a wait that expires.
+__global__ void give_up_kernel(const __grid_constant__ AttnTcParams p, int gcta, int head_dim) {
+  pdl_wait();
+  unwritten_parts(p, gcta, head_dim, threadIdx.x, blockDim.x);
+}
+
 static int32_t attn_common(const specvlm_kv_t* kv, const void* q, int32_t batch, int32_t n_q_heads,
                            int32_t n_q, float sm_scale, void* out, float* lse, void* ws,
                            size_t ws_bytes, int32_t* d_status, void* stream) {
@@ -677,33 +686,10 @@ static int32_t attn_common(const specvlm_kv_t* kv, const void* q, int32_t batch,
 
   const int ctas = rows16_slices(kv, batch);
   if (ctas > 0) {
-    size_t o_bytes, lse_bytes, cut_bytes;
-    rows16_ws_layout(ctas, rows, kv->head_dim, o_bytes, lse_bytes, cut_bytes);
+    const SliceScratch sc(ctas, rows, kv->head_dim);
     if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SPECVLM_ERR_INVALID_ARG;
-    if (ws_bytes < o_bytes + lse_bytes + cut_bytes) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
-    AttnTcParams p = {};
-    p.q = static_cast<const __nv_bfloat16*>(q);
-    p.out = static_cast<__nv_bfloat16*>(out);
-    p.lse = lse;
-    uint8_t* const w = static_cast<uint8_t*>(ws);
-    p.ws_o = reinterpret_cast<float*>(w);
-    p.ws_lse = reinterpret_cast<float*>(w + o_bytes);
-    p.ws_cut = reinterpret_cast<int4*>(w + o_bytes + lse_bytes);
-    p.block_table = kv->block_table;
-    p.seq_lens = kv->seq_lens;
-    p.d_status = d_status;
-    p.batch = batch;
-    p.n_layers = kv->n_layers;
-    p.n_q_heads = n_q_heads;
-    p.n_kv_heads = kv->n_kv_heads;
-    p.group = group;
-    p.n_win = p.q_per = n_q;
-    p.n_parts = 1;
-    p.rows = rows;
-    p.max_blocks = kv->max_blocks;
-    p.block_tokens = kv->block_tokens;
-    p.max_seq_len = kv->max_seq_len;
-    p.scale_log2 = sm_scale * kLog2e;
+    if (ws_bytes < sc.bytes()) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
+    const AttnTcParams p = slice_params(kv, q, batch, n_q_heads, n_q, sm_scale, out, lse, d_status, 1, n_q, ws, sc);
     rc = kv->head_dim == 128 ? launch_slices<128>(tk, tv, p, ctas, st) : launch_slices<64>(tk, tv, p, ctas, st);
     return rc != SPECVLM_OK ? rc : attn_merge_launch(p, kv->head_dim, ctas, st);
   }
@@ -736,6 +722,30 @@ using namespace specvlm;
 
 extern "C" void specvlm_debug_set_attn_splits(int32_t n_splits) {
   g_forced_splits.store(n_splits > 0 ? n_splits : 0, std::memory_order_relaxed);
+}
+
+extern "C" int32_t specvlm_debug_attn_merge(const specvlm_kv_t* kv, int32_t batch, int32_t n_q_heads, int32_t n_q,
+                                            void* out, float* lse_or_null, void* ws, size_t ws_bytes, int32_t lost_cta,
+                                            int32_t* n_ctas, void* stream) {
+  const int32_t rc = validate_kv(kv, batch, true);
+  if (rc != SPECVLM_OK) return rc;
+  if (!out || !ws || !n_ctas || n_q_heads < 1 || n_q < 1 || n_q_heads % kv->n_kv_heads != 0) return SPECVLM_ERR_INVALID_ARG;
+  const int group = n_q_heads / kv->n_kv_heads;
+  if (group > 16 || n_q > 9 || batch > kSchedMaxBatch) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
+  const SlicePlan pl = group * n_q > kRows16Max ? attn_tc_plan(kv, batch, group, n_q) : SlicePlan{rows16_slices(kv, batch), 1, n_q};
+  const int grid = pl.n_parts * pl.ctas;
+  *n_ctas = grid;
+  if (grid == 0) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
+  const SliceScratch sc(grid, pl.q_per * group, kv->head_dim);
+  if (ws_bytes < sc.bytes()) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
+  if (lost_cta >= grid) return SPECVLM_ERR_INVALID_ARG;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const AttnTcParams p = slice_params(kv, nullptr, batch, n_q_heads, n_q, 1.f, out, lse_or_null, nullptr, pl.n_parts, pl.q_per, ws, sc);
+  if (lost_cta >= 0) {
+    const int32_t marked = launch_after(give_up_kernel, dim3(1), dim3(128), 0, st, p, lost_cta, kv->head_dim);
+    if (marked != SPECVLM_OK) return marked;
+  }
+  return attn_merge_launch(p, kv->head_dim, pl.ctas, st);
 }
 
 extern "C" size_t specvlm_attn_workspace_bytes(const specvlm_kv_t* kv, int32_t batch,

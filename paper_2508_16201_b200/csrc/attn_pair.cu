@@ -163,6 +163,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   }
   pdl_launch_next();
   pdl_wait();
+  if (warp >= 4 && (warp - 4) >> 2 < n_here) unwritten_parts(p, (2 * set + ((warp - 4) >> 2)) * ctas + cta, D, tid & 127, 128);
   if (warp == 0) {
     const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;
@@ -544,7 +545,10 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
           }
         }
         if (row_on) {
-          if (!complete) p.ws_lse[prow] = lse2;
+          if (!complete) {
+#pragma unroll
+            for (int b = 0; b < D / 64; ++b) p.ws_lse[(size_t)b * p.lse_block + prow] = lse2;
+          }
           else if (p.lse) p.lse[orow] = lse2 * kLn2;
         }
       }

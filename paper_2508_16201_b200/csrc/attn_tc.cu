@@ -156,6 +156,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   }
   pdl_launch_next();
   pdl_wait();
+  if (warp >= 4) unwritten_parts(p, blockIdx.x, D, tid - 128, kTcThreads - 128);
   if (warp == 0) {
     const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;
@@ -769,7 +770,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 #pragma unroll
               for (int jj = 0; jj < 8; ++jj)
                 *reinterpret_cast<float2*>(dst + jj * 8) = make_float2(res[2 * jj], res[2 * jj + 1]);
-              if (cc == 0 && (lane & 3) == 0) p.ws_lse[(size_t)slot * p.rows + r] = lse2[e];
+              if ((lane & 3) == 0) p.ws_lse[(size_t)cc * p.lse_block + (size_t)slot * p.rows + r] = lse2[e];
             }
           }
         }
@@ -801,6 +802,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 // first part (most hold none and leave), blockIdx.y = a block of output positions (four channels of
 // a row each).  The parts of an item sit in the scratch slots first_slot and 2 (c + 1), 2 (c + 2), ..
 //   out = sum_s w_s o_s / sum_s w_s,  w_s = 2^(lse_s - max),  parts folded in slice order (fixed).
+// A row with a part that was never written (its CTA gave up) is left alone.
 // LANES warps share an item's parts, for launches that cut few items into many parts.
 // One CTA per item used to do this at the end of the attention kernel, after an atomic counter said that
 // it was the last: with one layer of 6400 tokens (8 items in 13 parts each) that was 21 of the
@@ -831,6 +833,7 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_
   const int r = on ? idx / (D / 4) : 0, c4 = on ? idx - r * (D / 4) : 0;
   float mm = -INFINITY, den = 0.f;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool lost = false;
   for (int k0 = wl; k0 < cut.w; k0 += LANES * kMergeChunk) {
     float ls[kMergeChunk];
     float4 x[kMergeChunk];
@@ -841,7 +844,8 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_
       x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (on && k < cut.w) {
         const size_t row = (size_t)(k == 0 ? cut.z : 2 * (gcta + k)) * p.rows + r;
-        ls[q] = ldg_cg_f32(p.ws_lse + row);
+        ls[q] = ldg_cg_f32(p.ws_lse + (size_t)(c4 >> 4) * p.lse_block + row);
+        lost |= unwritten(ls[q]);
         x[q] = ldg_cg_f32x4(p.ws_o + row * D + c4 * 4);
       }
     }
@@ -871,13 +875,16 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_
     __shared__ float2 md_sm[LANES - 1][kPos];
     if (wl > 0) {
       acc_sm[wl - 1][pos] = acc;
-      md_sm[wl - 1][pos] = make_float2(mm, den);
+      md_sm[wl - 1][pos] = make_float2(lost ? __uint_as_float(kUnwritten) : mm, den);
     }
     __syncthreads();
     if (wl > 0) return;
     float m2 = mm;
 #pragma unroll
-    for (int w = 0; w < LANES - 1; ++w) m2 = fmaxf(m2, md_sm[w][pos].x);
+    for (int w = 0; w < LANES - 1; ++w) {
+      lost |= unwritten(md_sm[w][pos].x);
+      m2 = fmaxf(m2, md_sm[w][pos].x);
+    }
     const float sc = mm == -INFINITY ? 0.f : fast_exp2(mm - m2);
     acc.x *= sc;
     acc.y *= sc;
@@ -897,7 +904,7 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_
     }
     mm = m2;
   }
-  if (!on) return;
+  if (!on || lost) return;
   const float inv = den > 0.f ? 1.f / den : 0.f;
   const int t = r / p.group, h = cut.y * p.group + (r - t * p.group);
   const size_t orow = ((size_t)cut.x * p.n_win + q0 + t) * p.n_q_heads + h;
@@ -930,23 +937,19 @@ static int tc_set_ctas(const specvlm_kv_t* kv, int32_t batch, int n_parts) {
   return sched_active_ctas(tiles_max, per_set);
 }
 
-// scratch, per part and CTA of its set: two partial results (rows of a full part each), their LSEs, and the
-// item that the CTA's slice cuts
-static void tc_ws_layout(const specvlm_kv_t* kv, int32_t batch, int rows, int group, size_t& o_bytes, size_t& lse_bytes,
-                         size_t& cut_bytes) {
-  int n_parts, q_per;
-  tc_parts(rows, group, n_parts, q_per);
-  const int grid = n_parts * tc_set_ctas(kv, batch, n_parts);
-  const size_t rows_part = (size_t)q_per * group;
-  o_bytes = round_up((size_t)2 * grid * rows_part * kv->head_dim * sizeof(float), 256);
-  lse_bytes = round_up((size_t)2 * grid * rows_part * sizeof(float), 256);
-  cut_bytes = round_up((size_t)grid * sizeof(int4), 256);
+SlicePlan attn_tc_plan(const specvlm_kv_t* kv, int32_t batch, int32_t group, int32_t n_q) {
+  SlicePlan pl;
+  tc_parts(group * n_q, group, pl.n_parts, pl.q_per);
+  pl.ctas = tc_set_ctas(kv, batch, pl.n_parts);
+  return pl;
+}
+
+static SliceScratch tc_scratch(const specvlm_kv_t* kv, const SlicePlan& pl, int group) {
+  return SliceScratch(pl.n_parts * pl.ctas, pl.q_per * group, kv->head_dim);
 }
 
 size_t attn_tc_ws_bytes(const specvlm_kv_t* kv, int32_t batch, int rows, int group) {
-  size_t a, b, c;
-  tc_ws_layout(kv, batch, rows, group, a, b, c);
-  return a + b + c;
+  return tc_scratch(kv, attn_tc_plan(kv, batch, group, rows / group), group).bytes();
 }
 
 // Queries as a 5-D tensor (channel, head in group, query token, KV head, layer * batch + sequence):
@@ -1038,17 +1041,14 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   const int64_t items = (int64_t)kv->n_layers * batch * kv->n_kv_heads;
   if (items > 0x3fffffff) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SPECVLM_ERR_INVALID_ARG;
-  size_t o_bytes, lse_bytes, cut_bytes;
-  tc_ws_layout(kv, batch, rows, group, o_bytes, lse_bytes, cut_bytes);
-  const size_t base_bytes = o_bytes + lse_bytes + cut_bytes;
-  if (ws_bytes < base_bytes + (tree_parents ? attn_tc_tree_extra_bytes(batch, n_q) : 0))
+  // A window of more than 128 rows is cut into parts of equal numbers of query tokens that share one launch.
+  const SlicePlan pl = attn_tc_plan(kv, batch, group, n_q);
+  const SliceScratch sc = tc_scratch(kv, pl, group);
+  if (ws_bytes < sc.bytes() + (tree_parents ? attn_tc_tree_extra_bytes(batch, n_q) : 0))
     return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
   if (tree_parents && n_q > kMaxTreeNodes) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
-  // A window of more than 128 rows is cut into parts of equal numbers of query tokens that share one launch.
-  int n_parts, q_per;
-  tc_parts(rows, group, n_parts, q_per);
-  if (q_per * group > 128) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
-  const int ctas = tc_set_ctas(kv, batch, n_parts);
+  if (pl.q_per * group > 128) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
+  const int ctas = pl.ctas, n_parts = pl.n_parts;
 
   CUtensorMap tk, tv;
   int32_t rc = encode_kv_map(&tk, kv, kv->k, kTileTokens);
@@ -1056,33 +1056,9 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   rc = encode_kv_map(&tv, kv, kv->v, kTileTokens);
   if (rc != SPECVLM_OK) return rc;
 
-  AttnTcParams p;
-  p.q = static_cast<const __nv_bfloat16*>(q);
-  p.out = static_cast<__nv_bfloat16*>(out);
-  p.lse = lse;
-  uint8_t* w = static_cast<uint8_t*>(ws);
-  p.ws_o = reinterpret_cast<float*>(w);
-  p.ws_lse = reinterpret_cast<float*>(w + o_bytes);
-  p.ws_cut = reinterpret_cast<int4*>(w + o_bytes + lse_bytes);
-  p.n_parts = n_parts;
-  p.q_per = q_per;
-  p.rows = q_per * group;
-  p.block_table = kv->block_table;
-  p.seq_lens = kv->seq_lens;
-  p.d_status = d_status;
-  p.batch = batch;
-  p.n_layers = kv->n_layers;
-  p.n_win = n_q;
-  p.n_q_heads = n_q_heads;
-  p.n_kv_heads = kv->n_kv_heads;
-  p.group = group;
-  p.max_blocks = kv->max_blocks;
-  p.block_tokens = kv->block_tokens;
-  p.max_seq_len = kv->max_seq_len;
-  p.scale_log2 = sm_scale * kLog2e;
-  p.anc = nullptr;
+  AttnTcParams p = slice_params(kv, q, batch, n_q_heads, n_q, sm_scale, out, lse, d_status, n_parts, pl.q_per, ws, sc);
   if (tree_parents) {
-    uint64_t* anc = reinterpret_cast<uint64_t*>(static_cast<uint8_t*>(ws) + base_bytes);
+    uint64_t* anc = reinterpret_cast<uint64_t*>(static_cast<uint8_t*>(ws) + sc.bytes());
     const int n = batch * n_q;
     rc = launch_after(tree_ancestors_kernel, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, st, tree_parents, n, n_q, anc,
                       d_status);
@@ -1091,7 +1067,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   }
 
   CUtensorMap tq;
-  rc = encode_q_map(&tq, q, kv->head_dim, group, n_q, q_per, kv->n_kv_heads, (int64_t)kv->n_layers * batch);
+  rc = encode_q_map(&tq, q, kv->head_dim, group, n_q, pl.q_per, kv->n_kv_heads, (int64_t)kv->n_layers * batch);
   if (rc != SPECVLM_OK) return rc;
   if (n_parts > 1)
     rc = attn_pair_launch(tk, tv, tq, p, kv->head_dim, (n_parts + 1) / 2 * ctas, st);

@@ -13,7 +13,7 @@ struct AttnTcParams {
   __nv_bfloat16* out;         // [L][B][n_win][Hq][D]
   float* lse;                 // [L][B][n_win][Hq] or null
   float* ws_o;                // partial results: [2 * grid][rows][D], normalised
-  float* ws_lse;              // [2 * grid][rows], log2 units
+  float* ws_lse;              // [D / 64][2 * grid][rows], log2 units: per 64-channel block, see unwritten_parts
   int4* ws_cut;               // [grid]: the cut item whose first part a CTA holds, see attn_merge_kernel
   const int32_t* block_table; // [B][max_blocks] or null
   const int32_t* seq_lens;    // [B]
@@ -24,6 +24,7 @@ struct AttnTcParams {
   int32_t n_parts, q_per;     // the window is cut into n_parts parts of q_per tokens (the last may be shorter)
   int32_t rows;               // rows of a full part = q_per * group (<= 128): the row pitch of the scratch slots
   int32_t max_blocks, block_tokens, max_seq_len;
+  int32_t lse_block;          // floats from one 64-channel block's LSEs to the next one's
   float scale_log2;           // sm_scale * log2(e)
 };
 
@@ -190,8 +191,73 @@ __device__ __forceinline__ void publish_cut_item(const AttnTcParams& p, bool act
   p.ws_cut[gcta] = cut;
 }
 
+// A CTA that gives up (a wait expired) leaves partial results unwritten, and the merge must make nothing of what their
+// slots hold.  So every CTA first fills the LSEs of its two slots with a bit pattern that no LSE has (a CTA stores -inf, a
+// finite value or +inf), before the barrier behind its set-up, and the merge leaves a row alone that has such a part.  Where two
+// groups of warps store a row's channels (attn_tc.cu at d = 128) one of them may give up where the other does not: each
+// stores an LSE of its own with its 64-channel block.
+constexpr uint32_t kUnwritten = 0xffffffffu;
+__device__ __forceinline__ bool unwritten(float lse) { return __float_as_uint(lse) == kUnwritten; }
+// by n_threads threads t = 0 ..
+__device__ __forceinline__ void unwritten_parts(const AttnTcParams& p, int gcta, int head_dim, int t, int n_threads) {
+  for (int i = t; i < 2 * p.rows * (head_dim / 64); i += n_threads) {
+    const int block = i / (2 * p.rows);
+    p.ws_lse[(size_t)block * p.lse_block + (size_t)2 * gcta * p.rows + (i - block * 2 * p.rows)] = __uint_as_float(kUnwritten);
+  }
+}
+
 // attn_tc.cu: the merge of the items that slice boundaries cut, for a launch of n_parts sets of `ctas` CTAs
 int32_t attn_merge_launch(const AttnTcParams& p, int head_dim, int ctas, cudaStream_t st);
+
+// Scratch of a launch: partial results [2 * grid][rows][D], their LSEs, and the item that each CTA's slice cuts.
+struct SliceScratch {
+  int grid;
+  size_t o_bytes, lse_bytes, cut_bytes;
+  SliceScratch(int grid, int rows, int head_dim)
+      : grid(grid),
+        o_bytes(round_up((size_t)2 * grid * rows * head_dim * sizeof(float), 256)),
+        lse_bytes(round_up((size_t)2 * grid * rows * (head_dim / 64) * sizeof(float), 256)),
+        cut_bytes(round_up((size_t)grid * sizeof(int4), 256)) {}
+  size_t bytes() const { return o_bytes + lse_bytes + cut_bytes; }
+};
+
+inline AttnTcParams slice_params(const specvlm_kv_t* kv, const void* q, int32_t batch, int32_t n_q_heads, int32_t n_q,
+                                 float sm_scale, void* out, float* lse, int32_t* d_status, int n_parts, int q_per, void* ws,
+                                 const SliceScratch& sc) {
+  AttnTcParams p;
+  p.q = static_cast<const __nv_bfloat16*>(q);
+  p.out = static_cast<__nv_bfloat16*>(out);
+  p.lse = lse;
+  uint8_t* const w = static_cast<uint8_t*>(ws);
+  p.ws_o = reinterpret_cast<float*>(w);
+  p.ws_lse = reinterpret_cast<float*>(w + sc.o_bytes);
+  p.ws_cut = reinterpret_cast<int4*>(w + sc.o_bytes + sc.lse_bytes);
+  p.block_table = kv->block_table;
+  p.seq_lens = kv->seq_lens;
+  p.d_status = d_status;
+  p.anc = nullptr;
+  p.batch = batch;
+  p.n_layers = kv->n_layers;
+  p.n_q_heads = n_q_heads;
+  p.n_kv_heads = kv->n_kv_heads;
+  p.group = n_q_heads / kv->n_kv_heads;
+  p.n_win = n_q;
+  p.n_parts = n_parts;
+  p.q_per = q_per;
+  p.rows = q_per * p.group;
+  p.max_blocks = kv->max_blocks;
+  p.block_tokens = kv->block_tokens;
+  p.max_seq_len = kv->max_seq_len;
+  p.lse_block = 2 * sc.grid * p.rows;
+  p.scale_log2 = sm_scale * kLog2e;
+  return p;
+}
+
+// How a launch on slices of a given window is laid out: `ctas` CTAs in each of n_parts sets (0: a CTA per item).
+struct SlicePlan {
+  int ctas, n_parts, q_per;
+};
+SlicePlan attn_tc_plan(const specvlm_kv_t* kv, int32_t batch, int32_t group, int32_t n_q);      // attn_tc.cu
 
 // (a template of the kernel itself: kernels of one signature must not share the flag below)
 template <auto kern>

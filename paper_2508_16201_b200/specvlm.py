@@ -55,7 +55,7 @@ EXPORTS = [
     "specvlm_append_kv", "specvlm_rollback_kv",
     "specvlm_verify_tree_workspace_bytes", "specvlm_verify_tree_attn", "specvlm_accept_tree",
     "specvlm_compact_tree_kv", "specvlm_debug_poison_shared_memory", "specvlm_debug_wait_timeout",
-    "specvlm_debug_set_attn_splits", "specvlm_debug_window_parts",
+    "specvlm_debug_set_attn_splits", "specvlm_debug_window_parts", "specvlm_debug_attn_merge",
 ]
 
 
@@ -102,6 +102,9 @@ def lib():
         L.specvlm_debug_wait_timeout.argtypes = [c_int32, c_void_p, c_void_p, c_void_p]
         L.specvlm_debug_window_parts.restype = c_int32
         L.specvlm_debug_window_parts.argtypes = [c_int32, c_int32, i32p, i32p]
+        L.specvlm_debug_attn_merge.restype = c_int32
+        L.specvlm_debug_attn_merge.argtypes = [kvp, c_int32, c_int32, c_int32, c_void_p, c_void_p, c_void_p, c_size_t,
+                                               c_int32, i32p, c_void_p]
         L.specvlm_debug_set_attn_splits.restype = None
         L.specvlm_debug_set_attn_splits.argtypes = [c_int32]
         L.specvlm_verify_tree_workspace_bytes.restype = c_size_t
@@ -465,6 +468,18 @@ def debug_wait_timeout(limit_ms: int, d_status: torch.Tensor, d_abort_flag: torc
 def debug_set_attn_splits(n_splits: int) -> None:
     """Forces the split count of the 16-row attention kernel (0 = built-in choice; test hook)."""
     lib().specvlm_debug_set_attn_splits(int(n_splits))
+
+
+def debug_attn_merge(kv: KvCache, out: torch.Tensor, ws: torch.Tensor, lse: torch.Tensor | None = None,
+                     lost_cta: int = -1) -> int:
+    """Runs the merge of an attention call (out: [n_layers][batch][n_q][n_q_heads][head_dim]) again over the scratch that
+    it left, with one CTA marked as having given up; returns the number of CTAs (test hook)."""
+    L, B, NQ, Hq, D = out.shape
+    n = c_int32()
+    rc = lib().specvlm_debug_attn_merge(byref(kv.struct), B, Hq, NQ, _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), int(lost_cta),
+                                        byref(n), _stream())
+    _check(rc, "specvlm_debug_attn_merge")
+    return n.value
 
 
 def compact_tree_kv(kv: KvCache, path: torch.Tensor, accept_len: torch.Tensor,

@@ -7,6 +7,8 @@ could leave the allocation even if a guard were missing.  Expected: the offendin
 (its destination keeps the sentinel it held), every other row equals the oracle, and
 SPECVLM_ERR_INVALID_ARG arrives in d_status.  The last test makes a bounded barrier wait run out
 on a barrier nothing arrives at and reads SPECVLM_ERR_TIMEOUT back; the kernel returns normally."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -164,3 +166,54 @@ def test_bounded_wait_runs_out_and_reports_timeout():
     n, nxt, _ = specvlm.accept(logits, drafts)
     a, nx, _ = oracle.accept(logits[0].cpu().numpy(), drafts[0].cpu().numpy())
     assert (int(n[0]), int(nxt[0])) == (a, nx)
+
+
+@pytest.mark.parametrize("Hq,Hkv,gamma,D,lens", [
+    (28, 4, 0, 128, [6000]),                     # 16-row slices, few items in many parts (four warps share the parts)
+    (28, 4, 0, 64, [700, 0, 3000, 129] * 3),     # the same with items that no boundary cuts and empty sequences
+    (64, 8, 5, 128, [1500, 300]),                # 48 rows
+    (16, 2, 8, 64, [3000, 300]),                 # 72 rows, d = 64
+    (64, 4, 8, 128, [1100, 0, 2000]),            # 144 rows: two parts of the window per CTA
+    (32, 2, 8, 64, [260, 2500])])                # the same at d = 64
+def test_items_with_a_part_that_was_given_up_are_left_alone(Hq, Hkv, gamma, D, lens):
+    """An item that slice boundaries cut is folded from several CTAs' partial results.  Where one of the CTAs gave
+    up, nothing may be made of what its slots hold.  The second kernel of a finished call runs again over the call's
+    scratch: as it is, it stores the cut items once more, bit for bit; with a CTA marked as having given up, all of them
+    but the ones that this CTA has a part of, which keep a sentinel.  (No wait is made to expire.)"""
+    L, B, nq = 2, len(lens), gamma + 1
+    group, n_parts, q_per = Hq // Hkv, ctypes.c_int32(), ctypes.c_int32()
+    assert specvlm.lib().specvlm_debug_window_parts(nq, group, ctypes.byref(n_parts), ctypes.byref(q_per)) == 0
+    q_per = q_per.value                              # query tokens of a part of a window wider than 128 rows
+    cache, _, _ = make_cache(L, Hkv, D, [max(n, 1) for n in lens], paged=False, seed=80)
+    cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    q = synth.randn_bf16((L, B, nq, Hq, D), "cuda", 81, "Q")
+    lse = torch.empty((L, B, nq, Hq), dtype=torch.float32, device="cuda")
+    specvlm.debug_set_attn_splits(6 if gamma == 0 else 0)
+    try:
+        ws = torch.full((specvlm.attn_workspace_bytes(cache, B, Hq, gamma),), 255, dtype=torch.uint8, device="cuda")
+        whole = specvlm.verify_attn(cache, q, gamma, 0.1, lse=lse, ws=ws)
+        saved = ws.clone()
+
+        def merge(cta=-1):
+            """Items [part of the window][L][B][Hkv] that the merge has stored: whole, and as in the call."""
+            out, lse2 = torch.full_like(whole, 7.0), torch.full_like(lse, 7.0)
+            ws.copy_(saved)
+            n = specvlm.debug_attn_merge(cache, out, ws, lse2, cta)
+            stored = (out != 7.0).any(-1)
+            assert torch.equal(stored, lse2 != 7.0)
+            assert torch.equal(out[stored], whole[stored]) and torch.equal(lse2[stored], lse[stored])
+            items = [h.unflatten(3, (Hkv, group)).transpose(2, 3).flatten(3) for h in stored.split(q_per, dim=2)]
+            assert all(torch.equal(i.any(-1), i.all(-1)) for i in items)
+            return n, torch.stack([i.all(-1) for i in items])
+
+        n, cut = merge()
+        assert cut.any()
+        left, parts = torch.zeros_like(cut), 0
+        for cta in range(n):
+            stored = merge(cta)[1]
+            assert not (stored & ~cut).any()
+            left |= cut & ~stored
+            parts += int((cut & ~stored).sum())
+        assert torch.equal(left, cut) and parts >= 2 * int(cut.sum())   # a cut item has parts in two CTAs at least
+    finally:
+        specvlm.debug_set_attn_splits(0)
