@@ -144,7 +144,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     *abort_flag = 0;
     mbar_fence_init();
   }
-  if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS);
+  if (warp == 1) tmem_alloc_launch_next(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS);
   if (warp == 3 && lane == 0) {
     tma_prefetch_desc(&tm_k);
     tma_prefetch_desc(&tm_v);
@@ -161,7 +161,6 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     }
     fence_proxy_async();
   }
-  pdl_launch_next();
   pdl_wait();
   if (warp >= 4 && (warp - 4) >> 2 < n_here) unwritten_parts(p, (2 * set + ((warp - 4) >> 2)) * ctas + cta, D, tid & 127, 128);
   if (warp == 0) {

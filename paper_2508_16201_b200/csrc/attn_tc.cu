@@ -137,7 +137,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     *abort_flag = 0;
     mbar_fence_init();
   }
-  if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS);
+  if (warp == 1) tmem_alloc_launch_next(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS);
   if (warp == 3 && lane == 0) {
     tma_prefetch_desc(&tm_k);
     tma_prefetch_desc(&tm_v);
@@ -154,7 +154,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
     fence_proxy_async();
   }
-  pdl_launch_next();
   pdl_wait();
   if (warp >= 4) unwritten_parts(p, blockIdx.x, D, tid - 128, kTcThreads - 128);
   if (warp == 0) {

@@ -19,11 +19,12 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Programmatic dependent launch.  Every kernel of the library is launched so that it may start while the
-// kernel before it in the stream still runs (launch_after), lets its own successor start as soon as all
-// its CTAs run, and waits for the predecessor's completion, in every CTA, before its first access to global
-// memory: what precedes the wait (barriers, tensor memory, descriptors, the launch itself) costs no time on the
-// stream.  Data that an earlier kernel may have written is therefore never read through the non-coherent path
+// Programmatic dependent launch.  Every kernel of the path is launched so that it may start while the
+// kernel before it in the stream still runs (launch_after) and waits for the predecessor's completion, in every CTA,
+// before its first access to global memory: what precedes the wait (barriers, tensor memory, descriptors, the launch
+// itself) costs no time on the stream.  It lets its own successor start once all its CTAs run, and have their tensor
+// memory where they use it (tmem_alloc_launch_next), so that a successor's CTA that waits holds nothing that the kernel
+// it waits for still needs.  The finishing kernels of acceptance do not release early (accept.cu).  Data that an earlier kernel may have written is therefore never read through the non-coherent path
 // (__ldg, const __restrict__): a line cached before the wait would not be dropped by it.
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -262,6 +263,13 @@ __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols)
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+// The allocation of a kernel that takes part in programmatic dependent launch, by the one warp that releases the
+// successor, once the CTA has its columns.  A release by another warp could come while this one still waits for columns:
+// a successor's CTA that took them and then waited for this kernel would leave both waiting for ever.
+__device__ __forceinline__ void tmem_alloc_launch_next(uint32_t smem_dst, uint32_t ncols) {
+  tmem_alloc(smem_dst, ncols);
+  pdl_launch_next();
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");

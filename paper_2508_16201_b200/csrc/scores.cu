@@ -166,9 +166,8 @@ scores_colsum_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     }
     fence_proxy_async();                                           // the MMAs read it through the async proxy
   }
-  if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+  if (warp == 1) tmem_alloc_launch_next(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
   tc_fence_before_sync();
-  pdl_launch_next();
   pdl_wait();
   __syncthreads();
   tc_fence_after_sync();
@@ -410,9 +409,8 @@ scores_lse_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     *abort_flag = 0;
     mbar_fence_init();
   }
-  if (warp == 1) tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+  if (warp == 1) tmem_alloc_launch_next(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
   tc_fence_before_sync();
-  pdl_launch_next();
   pdl_wait();
   __syncthreads();
   tc_fence_after_sync();

@@ -118,3 +118,24 @@ def test_rating_kernels_compile_without_heavy_spills():
         seen += 1
         assert int(m.group(3)) <= 64 and int(m.group(4)) <= 64, m.group(0)
     assert seen >= 4
+
+
+def test_kernels_with_tensor_memory_release_their_successor_after_the_allocation():
+    """A kernel may let its successor start only once each of its CTAs has its tensor memory: a successor's CTA that
+    took the columns first and then waited for that kernel would leave both waiting.  In the sources: every allocation
+    is the helper that releases after it, and no kernel that calls it releases anywhere else."""
+    csrc = os.path.join(ROOT, "paper_2508_16201_b200", "csrc")
+    seen = 0
+    for f in sorted(os.listdir(csrc)):
+        src = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, f)).read())
+        if f == "common.cuh":
+            body = src[src.index("void tmem_alloc_launch_next("):]
+            assert body.index("tmem_alloc(smem_dst") < body.index("pdl_launch_next();") < body.index("}")
+            continue
+        assert not re.search(r"\btmem_alloc\(|tcgen05\.alloc|griddepcontrol\.launch_dependents", src), f
+        for kernel in src.split("__global__")[1:]:
+            if "tmem_alloc_launch_next(" in kernel:
+                seen += 1
+                # up to the kernel's end: the first line that is a closing brace alone
+                assert "pdl_launch_next()" not in kernel[:kernel.index("\n}\n")], (f, kernel[:80])
+    assert seen == 4
