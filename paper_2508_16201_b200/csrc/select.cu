@@ -36,6 +36,7 @@ constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelMaxCluster = 8;      // the portable cluster size
 constexpr int kSelMaxKeys = 14;        // keys per thread: 8 x 512 x 14 = 57 344 tokens
+constexpr int kSelMaxFrames = 1024;
 constexpr int kSelCopies = 8;          // interleaved copies of a histogram bin: lanes with equal digits spread over them
 constexpr int kSelMaxBatch = 64;
 constexpr int kTopPFracBits = 36;
@@ -92,8 +93,8 @@ struct SelSmem {
   int wcount[kSelWarps];
   int digit, count, same;                                  // result of a pass's scan
   int less[kSelMaxCluster], equal[kSelMaxCluster];         // every CTA's keys below and equal to the threshold
-  int cf[1024 + 1];                                        // unselected tokens before each frame
-  uint32_t quota[1024 + 1];                                // Stage-II picks before each frame
+  int cf[kSelMaxFrames + 1];                                        // unselected tokens before each frame
+  uint32_t quota[kSelMaxFrames + 1];                                // Stage-II picks before each frame
 };
 
 // One pass of the descent over the live keys [base, base + (n_digits << shift)), n_digits <= 256: into the CTA's histogram, the
@@ -562,7 +563,8 @@ static int32_t select_common(const float* scores, const int32_t* video_cu, const
   int64_t max_tokens = 0;
   for (int b = 0; b < batch; ++b) {
     const int64_t n_v = (int64_t)n_frames[b] * tokens_per_frame;
-    if (n_frames[b] < 1 || n_frames[b] > 1024 || n_v > 57344) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
+    if (n_frames[b] < 1 || n_frames[b] > kSelMaxFrames || n_v > kSelMaxCluster * kSelThreads * kSelMaxKeys)
+      return SPECVLM_ERR_UNSUPPORTED_SHAPE;
     if (k_total[b] < 0 || k_total[b] > n_v) return SPECVLM_ERR_INVALID_ARG;
     if (lambda_permille) {
       if (lambda_permille[b] < 0 || lambda_permille[b] > 1000) return SPECVLM_ERR_INVALID_ARG;
@@ -571,9 +573,6 @@ static int32_t select_common(const float* scores, const int32_t* video_cu, const
     }
     if ((!random_keys && video_cu[b + 1] - video_cu[b] < n_v) || kept_cu[b + 1] - kept_cu[b] < k_total[b])
       return SPECVLM_ERR_INVALID_ARG;
-    // a further limit on tokens + frames (a key per token and a count per frame in one 227 KB budget)
-    const size_t words = (size_t)n_v + n_frames[b] + 1 + 256 + 32 + 8;
-    if ((words + (words & 1)) * 4 + (256 + 2) * 8 > 232448) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
     if (n_v > max_tokens) max_tokens = n_v;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);

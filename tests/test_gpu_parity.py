@@ -296,7 +296,8 @@ def test_select_ragged_batch_and_ties():
 
 
 @pytest.mark.parametrize("F,T", [(1, 1), (1, 31), (1, 33), (8, 256), (1, 2049), (1024, 8), (683, 12), (3, 8191), (24577, 1),
-                                 (7, 3511), (1024, 28), (14336, 2), (1, 57298), (28, 2045)])
+                                 (7, 3511), (1024, 28), (14336, 2), (1, 57298), (28, 2045),
+                                 (1, 57344), (1024, 56), (2, 28672), (896, 64)])     # the documented limits
 def test_select_at_the_edges_of_its_launch_shapes(F, T):
     """Token counts around the cluster sizes and keys per thread of the selection kernel, one frame of
     every token and 1024 frames; scores with ties, all equal, and spread over the whole exponent range.
