@@ -162,7 +162,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     fence_proxy_async();
   }
   pdl_wait();
-  if (warp >= 4 && (warp - 4) >> 2 < n_here) unwritten_parts(p, (2 * set + ((warp - 4) >> 2)) * ctas + cta, D, tid & 127, 128);
+  if (warp >= 2 && warp - 2 < n_here) unwritten_parts(p, (2 * set + warp - 2) * ctas + cta, D, lane, 32);
   if (warp == 0) {
     const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;

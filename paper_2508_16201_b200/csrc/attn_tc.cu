@@ -155,7 +155,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     fence_proxy_async();
   }
   pdl_wait();
-  if (warp >= 4) unwritten_parts(p, blockIdx.x, D, tid - 128, kTcThreads - 128);
+  if (warp == 3) unwritten_parts(p, blockIdx.x, D, lane, 32);
   if (warp == 0) {
     const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
     if (lane == 0) *any_empty = empty ? 1 : 0;

@@ -200,9 +200,11 @@ constexpr uint32_t kUnwritten = 0xffffffffu;
 __device__ __forceinline__ bool unwritten(float lse) { return __float_as_uint(lse) == kUnwritten; }
 // by n_threads threads t = 0 ..
 __device__ __forceinline__ void unwritten_parts(const AttnTcParams& p, int gcta, int head_dim, int t, int n_threads) {
-  for (int i = t; i < 2 * p.rows * (head_dim / 64); i += n_threads) {
-    const int block = i / (2 * p.rows);
-    p.ws_lse[(size_t)block * p.lse_block + (size_t)2 * gcta * p.rows + (i - block * 2 * p.rows)] = __uint_as_float(kUnwritten);
+  float* const slots = p.ws_lse + (size_t)2 * gcta * p.rows;
+#pragma unroll 1
+  for (int i = t; i < 2 * p.rows; i += n_threads) {
+    slots[i] = __uint_as_float(kUnwritten);
+    if (head_dim == 128) slots[p.lse_block + i] = __uint_as_float(kUnwritten);
   }
 }
 
