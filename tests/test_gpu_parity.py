@@ -566,7 +566,9 @@ def test_scores_row_lse_entry():
 @pytest.mark.parametrize("Hq,Hkv,gamma,D", [(64, 8, 8, 128),    # 72 rows: the 128-row tiles
                                             (64, 8, 5, 128),    # 48 rows: the 64-row tiles
                                             (28, 4, 0, 128),    # 7 rows: the decode kernel
-                                            (16, 2, 8, 64)])    # 72 rows, d = 64
+                                            (16, 2, 8, 64),     # 72 rows, d = 64
+                                            (32, 2, 8, 128),    # 144 rows: two parts of the window per CTA
+                                            (16, 1, 8, 64)])    # the same, d = 64
 def test_attention_with_maxima_rising_along_the_sequence(Hq, Hkv, gamma, D):
     """Random N(0,1) logits never move a row's running maximum by much after the first tile, so the
     kernels' rescaling of the running sums and of the O accumulator would go untested.  Here the

@@ -138,10 +138,14 @@ def test_tree_step_chain_verify_accept_compact(paged, n_nodes):
         assert np.array_equal(gk[b], rk[:, :, :nl]) and np.array_equal(gv[b], rv[:, :, :nl])
 
 
-def test_tree_attention_with_maxima_rising_along_the_sequence():
-    """The 128-row tree variant on logits that rise by about 12 log2 units per 128 tokens for some
+@pytest.mark.parametrize("Hq,Hkv,D,n_nodes", [(64, 8, 128, 16),      # 128 rows
+                                              (64, 8, 128, 26),      # 208 rows: two parts of the window per CTA
+                                              (16, 2, 64, 26),       # the same, d = 64
+                                              (32, 2, 128, 20)])     # 320 rows: three parts, the last alone in its CTA
+def test_tree_attention_with_maxima_rising_along_the_sequence(Hq, Hkv, D, n_nodes):
+    """The wide tree variants on logits that rise by about 12 log2 units per 128 tokens for some
     rows and fall for others: the reference maximum of a row has to be raised tile after tile."""
-    L, Hq, Hkv, D, n_nodes = 2, 64, 8, 128, 16
+    L = 2
     lens = [1400 + n_nodes, 300]
     rng = np.random.default_rng(95)
     cache, _, _ = make_cache(L, Hkv, D, lens, paged=False, seed=95)
