@@ -572,12 +572,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           __syncwarp();
           if (lane == 0) mbar_arrive(bar_s_empty + 8 * grp);
         }
-        // One copy of the code serves both 16-row halves of a warp (the 128-row variant): the loop is
-        // rolled, the current half's state sits at index 0 of its arrays, and the two halves' states
-        // change places after each half -- twice per tile, so every tile finds them as it left them.
+        // (none where the window has no rows for this warp)
 #pragma unroll 1
         for (int h = 0; h < nh; ++h) {
-          // The half's 16 rows x 128 columns are read from TMEM twice, 64 columns at a time, by the
+          // The warp's 16 rows x 128 columns are read from TMEM twice, 64 columns at a time, by the
           // same (rolled) code: once for the row maxima, once for the probabilities.  That halves
           // the live registers and the code of the loop; a TMEM load costs far less than the spills.
           const uint32_t saddr = tmem_base + ((uint32_t)(32 * quarter + 16 * h) << 16) + C::COL_S + grp * kBigTokens;
@@ -658,25 +656,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           }
           l_sum[0][0] += ps[0] + ps[1];
           l_sum[0][1] += ps[2] + ps[3];
-          if (NH == 2 && nh == 2) {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float tm = m_used[0][e], tl = l_sum[0][e];
-              m_used[0][e] = m_used[NH - 1][e];
-              m_used[NH - 1][e] = tm;
-              l_sum[0][e] = l_sum[NH - 1][e];
-              l_sum[NH - 1][e] = tl;
-              if constexpr (TREE) {
-                const uint64_t tv = vis[0][e];
-                vis[0][e] = vis[NH - 1][e];
-                vis[NH - 1][e] = tv;
-              } else {
-                const int tv = lim[0][e];
-                lim[0][e] = lim[NH - 1][e];
-                lim[NH - 1][e] = tv;
-              }
-            }
-          }
         }
         if (nh == 0 && i >= 2) SM_WAIT(bar_p_empty + 8 * grp, ((i >> 1) - 1) & 1);
         fence_proxy_async();
