@@ -423,7 +423,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
           take_turn(i);
           if (!ok) goto softmax_done;
           pass_turn();
-          // rows of zero queries: their logits are zero bits, which P may stay
+          // no row of the window here: whatever S holds (zeros, or NaN from K rows past a sequence's end) may stand as P,
+          // since rows of a product do not mix and nobody reads these
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) {

@@ -466,7 +466,8 @@ def debug_wait_timeout(limit_ms: int, d_status: torch.Tensor, d_abort_flag: torc
 
 
 def debug_set_attn_splits(n_splits: int) -> None:
-    """Forces the split count of the 16-row attention kernel (0 = built-in choice; test hook)."""
+    """Attention of up to 16 rows per KV head: 1 forces a CTA per (layer, sequence, KV head), more than 1 slices that cut a
+    sequence about that many times, 0 is the built-in choice (test hook, process-wide)."""
     lib().specvlm_debug_set_attn_splits(int(n_splits))
 
 

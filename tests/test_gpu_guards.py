@@ -5,8 +5,9 @@ nodes, sequence lengths) into addresses.  Each guard is fed one value that is ou
 the call's arguments declare but still inside the tensor the test allocated, so that no access
 could leave the allocation even if a guard were missing.  Expected: the offending row is skipped
 (its destination keeps the sentinel it held), every other row equals the oracle, and
-SPECVLM_ERR_INVALID_ARG arrives in d_status.  The last test makes a bounded barrier wait run out
-on a barrier nothing arrives at and reads SPECVLM_ERR_TIMEOUT back; the kernel returns normally."""
+SPECVLM_ERR_INVALID_ARG arrives in d_status.  One test makes a bounded barrier wait run out
+on a barrier nothing arrives at and reads SPECVLM_ERR_TIMEOUT back; the kernel returns normally.
+The last one checks what attention makes of the partial results of a CTA that gave up."""
 import ctypes
 
 import numpy as np
