@@ -182,7 +182,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   if (warp == 0 || warp == 3) {
     // ================================================================ TMA producers
     setmaxnreg_dec<kRegsLight>();
-    if (lane == 0 && active) {
+    if (active) {
+      const bool leader = elect_one();
       const bool is_k = warp == 0;
       const CUtensorMap* const tm = is_k ? &tm_k : &tm_v;
       const uint64_t policy = l2_policy_evict_first();
@@ -203,14 +204,16 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         const Segment sg = c.sg;
         if (is_k) {
           // both parts' query rows: a box of (64 channels) x (group heads) x (q_per tokens) per 64-channel block
-          if (c.seg_idx >= 1) ok = mbar_wait_soon(bar_q_empty, (c.seg_idx - 1) & 1, abort_flag);
+          if (c.seg_idx >= 1) ok = warp_wait_soon(bar_q_empty, (c.seg_idx - 1) & 1, abort_flag);
           if (!ok) break;
-          mbar_arrive_expect_tx(bar_q_full, (uint32_t)(n_here * p.rows) * 128u * (D / 64));
-          for (int g = 0; g < n_here; ++g)
+          if (leader) {
+            mbar_arrive_expect_tx(bar_q_full, (uint32_t)(n_here * p.rows) * 128u * (D / 64));
+            for (int g = 0; g < n_here; ++g)
 #pragma unroll
-            for (int h = 0; h < D / 64; ++h)
-              tma_load_5d(q_sm + g * Q_BYTES + h * (M * 128), &tm_q, bar_q_full, h * 64, 0, (2 * set + g) * p.q_per, sg.g,
-                          sg.layer * p.batch + sg.b, policy_q);
+              for (int h = 0; h < D / 64; ++h)
+                tma_load_5d(q_sm + g * Q_BYTES + h * (M * 128), &tm_q, bar_q_full, h * 64, 0, (2 * set + g) * p.q_per, sg.g,
+                            sg.layer * p.batch + sg.b, policy_q);
+          }
           n_q = c.seg_idx + 1;
         }
         const int n_sub_seq = (clamp_len(p.seq_lens[sg.b], p.max_seq_len) + kTileTokens - 1) / kTileTokens;
@@ -231,22 +234,24 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             blk_next[1] = s0 + 3 < n_sub_seq ? __ldcg(table + (s0 + 3) / subs_per_block) : 0;
           }
           const int slot = i % n_ring;
-          if (i >= n_ring) ok = mbar_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
+          if (i >= n_ring) ok = warp_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
           if (!ok) break;
-          mbar_arrive_expect_tx(bar_full + 8 * slot, n_sub * SUB_BYTES);
-          for (int u = 0; u < n_sub; ++u) {
-            const int tok = table ? ((s0 + u) % subs_per_block) * kTileTokens : (s0 + u) * kTileTokens;
+          if (leader) {
+            mbar_arrive_expect_tx(bar_full + 8 * slot, n_sub * SUB_BYTES);
+            for (int u = 0; u < n_sub; ++u) {
+              const int tok = table ? ((s0 + u) % subs_per_block) * kTileTokens : (s0 + u) * kTileTokens;
 #pragma unroll
-            for (int h = 0; h < D / 64; ++h)
-              tma_load_5d(ring_sm + slot * 2 * SUB_BYTES + h * blk_stride + u * sub_stride, tm, bar_full + 8 * slot,
-                          h * 64, tok, sg.g, blk[u], sg.layer, policy);
+              for (int h = 0; h < D / 64; ++h)
+                tma_load_5d(ring_sm + slot * 2 * SUB_BYTES + h * blk_stride + u * sub_stride, tm, bar_full + 8 * slot,
+                            h * 64, tok, sg.g, blk[u], sg.layer, policy);
+            }
           }
         }
         if (ok) c.next_segment(prefix, p.batch, hkv);
       }
       if (!ok) {
-        // a wait expired: report, then stay until this thread's copies in flight have landed (bounded)
-        if (p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
+        // a wait expired: report, then stay until this warp's copies in flight have landed (bounded)
+        if (p.d_status && leader) *p.d_status = SPECVLM_ERR_TIMEOUT;
         const uint64_t t0 = global_timer_ns();
         for (int k = i > n_ring ? i - n_ring : 0; k < i; ++k)
           while (!mbar_test_wait(bar_full + 8 * (k % n_ring), (k / n_ring) & 1) && global_timer_ns() - t0 < kWaitLimitNs) {
@@ -256,12 +261,13 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       }
     }
   } else if (warp < 3) {
-    // ================================================================ product issuers, one thread per part
+    // ================================================================ product issuers, a warp per part, one lane of which issues
     setmaxnreg_dec<kRegsLight>();
     const int g = warp - 1;
     if (g < n_here && lane == 0)
       publish_cut_item(p, active, cta, (2 * set + g) * ctas + cta, n_active, total, T0, T1, prefix);
-    if (g < n_here && lane == 0 && active) {
+    if (g < n_here && active) {
+      const bool leader = elect_one();
       SliceCursor c;
       c.start(T0, T1, prefix, p.batch, hkv);
       const uint64_t dq = umma_desc_sw128(q_sm + g * Q_BYTES, 16, 1024), dk0 = umma_desc_sw128(k_sm, 16, 1024);
@@ -271,6 +277,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       int n_sub_seq = 0, last_rows = 0;
       auto issue_qk = [&](int i) {                       // S of tile i
         const uint64_t db = umma_desc_advance(dk0, (i % NKP) * 2 * SUB_BYTES);
+        if (!leader) return;
 #pragma unroll
         for (int s = 0; s < D / 16; ++s)
           // 16 channels per step = 32 bytes along the swizzled 128-byte row; channels 64.. are the
@@ -279,11 +286,13 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                        umma_desc_advance(db, (s >> 2) * (kBigTokens * 128) + (s & 3) * 32), kIdescQK, s > 0 ? 1u : 0u);
         umma_commit(bar_s_full + 8 * g);
       };
-      ok = mbar_wait_soon(bar_q_full, 0, abort_flag) && mbar_wait_soon(bar_k_full, 0, abort_flag);
+      ok = warp_all(mbar_wait_soon(bar_q_full, 0, abort_flag) && mbar_wait_soon(bar_k_full, 0, abort_flag));
       if (ok) {
         issue_qk(0);
-        umma_commit(bar_k_empty);
-        if (c.last_of_segment()) umma_commit(bar_q_empty);
+        if (leader) {
+          umma_commit(bar_k_empty);
+          if (c.last_of_segment()) umma_commit(bar_q_empty);
+        }
       }
       for (int i = 0; i < n_my && ok; ++i) {
         const int vp = i % NVP, seg_idx = c.seg_idx, j = c.j;
@@ -299,51 +308,58 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         c.next_tile(prefix, p.batch, hkv);               // the cursor stands on tile i + 1 from here on
         const bool more = i + 1 < n_my;
         // waits that are over by the time P arrives come before the wait for P
-        ok = mbar_wait_soon(bar_v_full + 8 * vp, (i / NVP) & 1, abort_flag);
+        ok = warp_wait_soon(bar_v_full + 8 * vp, (i / NVP) & 1, abort_flag);
         if (ok && tail && (last_rows & 15) != 0) {
           // Steps of 16 tokens past the sequence's end are left out; inside the last step the V rows past
           // the end hold whatever the page held and are cleared (a zero probability times a stale
           // non-finite value must not reach O).  Both issuers do it: either may come first.
           uint8_t* const vt = big_ptr + C::OFF_V + vp * 2 * SUB_BYTES + (n_sub - 1) * SUB_BYTES;
-          for (int t = last_rows; t < ((last_rows + 15) & ~15); ++t)
-            for (int c16 = 0; c16 < D / 8; ++c16)
-              *reinterpret_cast<uint4*>(vt + (c16 >> 3) * (kTileTokens * 128) + t * 128 + (c16 & 7) * 16) =
-                  make_uint4(0, 0, 0, 0);
+          const int n_clear = (((last_rows + 15) & ~15) - last_rows) * (D / 8);
+          for (int idx = lane; idx < n_clear; idx += 32) {
+            const int t = last_rows + idx / (D / 8), c16 = idx % (D / 8);
+            *reinterpret_cast<uint4*>(vt + (c16 >> 3) * (kTileTokens * 128) + t * 128 + (c16 & 7) * 16) =
+                make_uint4(0, 0, 0, 0);
+          }
           fence_proxy_async();
+          __syncwarp();
         }
-        if (ok && more) ok = mbar_wait_soon(bar_k_full + 8 * ((i + 1) % NKP), ((i + 1) / NKP) & 1, abort_flag);
+        if (ok && more) ok = warp_wait_soon(bar_k_full + 8 * ((i + 1) % NKP), ((i + 1) / NKP) & 1, abort_flag);
         // the first product of an item overwrites O: the previous item's must have been read
-        if (ok && j == 0 && seg_idx >= 1) ok = mbar_wait_soon(bar_o_empty + 8 * g, (seg_idx - 1) & 1, abort_flag);
+        if (ok && j == 0 && seg_idx >= 1) ok = warp_wait_soon(bar_o_empty + 8 * g, (seg_idx - 1) & 1, abort_flag);
         const uint64_t db = umma_desc_advance(dv0, vp * 2 * SUB_BYTES);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          if (ok) ok = mbar_wait_soon((u ? bar_p_full : bar_p_half) + 8 * g, i & 1, abort_flag);
+          if (ok) ok = warp_wait_soon((u ? bar_p_full : bar_p_half) + 8 * g, i & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
           const int n_kt = u >= n_sub ? 0 : (tail && u == n_sub - 1 ? (last_rows + 15) >> 4 : kTileTokens / 16);
 #pragma unroll
           for (int kt = 0; kt < kTileTokens / 16; ++kt)
             // 16 tokens per step: 8 columns of bf16 pairs of P, 16 rows of 128 bytes down the V sub-tile
-            if (kt < n_kt)
+            if (leader && kt < n_kt)
               umma_bf16_ts(o_tmem, s_tmem + u * 32 + kt * 8, umma_desc_advance(db, u * SUB_BYTES + kt * 2048), kIdescPV,
                            u > 0 || kt > 0 || j > 0 ? 1u : 0u);
         }
         if (!ok) break;
         // S of the next tile first: the softmax is waiting for it
         if (more && !last) issue_qk(i + 1);
-        if (last) umma_commit(bar_o_full + 8 * g);
-        umma_commit(bar_v_empty + 8 * vp);
+        if (leader) {
+          if (last) umma_commit(bar_o_full + 8 * g);
+          umma_commit(bar_v_empty + 8 * vp);
+        }
         if (more) {
           if (last) {
-            ok = mbar_wait_soon(bar_q_full, (seg_idx + 1) & 1, abort_flag);
+            ok = warp_wait_soon(bar_q_full, (seg_idx + 1) & 1, abort_flag);
             if (!ok) break;
             issue_qk(i + 1);
           }
-          umma_commit(bar_k_empty + 8 * ((i + 1) % NKP));
-          if (c.last_of_segment()) umma_commit(bar_q_empty);
+          if (leader) {
+            umma_commit(bar_k_empty + 8 * ((i + 1) % NKP));
+            if (c.last_of_segment()) umma_commit(bar_q_empty);
+          }
         }
       }
-      if (!ok && p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
+      if (!ok && p.d_status && leader) *p.d_status = SPECVLM_ERR_TIMEOUT;
     }
   } else {
     // ================================================================ softmax / epilogue (warps 4..11)
@@ -386,7 +402,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     int i = 0;
 #define SM_WAIT(bar, parity)                                                        \
   do {                                                                              \
-    ok = __all_sync(0xffffffffu, mbar_wait_soon((bar), (parity), abort_flag));           \
+    ok = warp_wait_soon((bar), (parity), abort_flag);                                \
     if (!ok) goto softmax_done;                                                     \
   } while (0)
     // The two parts' warps of a lane quadrant sit on the same scheduler and take turns with its
@@ -395,7 +411,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     const uint32_t my_turn = bar_turn + 8 * (4 * g + quarter), other_turn = bar_turn + 8 * (4 * (1 - g) + quarter);
     const bool turns = n_here == 2;
     auto take_turn = [&](int n) {               // part 0 goes first: its n-th turn follows part 1's (n - 1)-th
-      if (turns && (g == 1 || n > 0)) ok = __all_sync(0xffffffffu, mbar_wait_soon(my_turn, (g == 1 ? n : n - 1) & 1, abort_flag));
+      if (turns && (g == 1 || n > 0)) ok = warp_wait_soon(my_turn, (g == 1 ? n : n - 1) & 1, abort_flag);
     };
     auto pass_turn = [&]() {
       __syncwarp();

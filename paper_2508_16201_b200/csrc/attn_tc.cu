@@ -179,7 +179,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // ================================================================ TMA producers
     // warp 0: query rows + K tiles; warp 3: V tiles.  Both walk the same slice.
     setmaxnreg_dec<kRegsLight>();
-    if (lane == 0 && active) {
+    if (active) {
+      const bool leader = elect_one();
       const bool is_k = warp == 0;
       const CUtensorMap* const tm = is_k ? &tm_k : &tm_v;
       const uint64_t policy = l2_policy_evict_first();
@@ -201,13 +202,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if (is_k) {
           // the item's query rows: a box of (64 channels) x (group heads) x (n_q tokens) per 64-channel block
           const int qb = c.seg_idx % NQ;
-          if (c.seg_idx >= NQ) ok = mbar_wait_soon(bar_q_empty + 8 * qb, ((c.seg_idx / NQ) - 1) & 1, abort_flag);
+          if (c.seg_idx >= NQ) ok = warp_wait_soon(bar_q_empty + 8 * qb, ((c.seg_idx / NQ) - 1) & 1, abort_flag);
           if (!ok) break;
-          mbar_arrive_expect_tx(bar_q_full + 8 * qb, (uint32_t)p.rows * 128u * (D / 64));
+          if (leader) {
+            mbar_arrive_expect_tx(bar_q_full + 8 * qb, (uint32_t)p.rows * 128u * (D / 64));
 #pragma unroll
-          for (int h = 0; h < D / 64; ++h)
-            tma_load_5d(q_sm + qb * Q_BYTES + h * (M * 128), &tm_q, bar_q_full + 8 * qb, h * 64, 0, 0, sg.g,
-                        sg.layer * p.batch + sg.b, policy_q);
+            for (int h = 0; h < D / 64; ++h)
+              tma_load_5d(q_sm + qb * Q_BYTES + h * (M * 128), &tm_q, bar_q_full + 8 * qb, h * 64, 0, 0, sg.g,
+                          sg.layer * p.batch + sg.b, policy_q);
+          }
         }
         const int n_sub_seq = (clamp_len(p.seq_lens[sg.b], p.max_seq_len) + kTileTokens - 1) / kTileTokens;
         const int32_t* table = p.block_table ? p.block_table + (size_t)sg.b * p.max_blocks : nullptr;
@@ -227,22 +230,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             blk_next[1] = s0 + 3 < n_sub_seq ? __ldcg(table + (s0 + 3) / subs_per_block) : 0;
           }
           const int slot = i % n_ring;
-          if (i >= n_ring) ok = mbar_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
+          if (i >= n_ring) ok = warp_wait_soon(bar_empty + 8 * slot, ((i / n_ring) - 1) & 1, abort_flag);
           if (!ok) break;
-          mbar_arrive_expect_tx(bar_full + 8 * slot, n_sub * SUB_BYTES);
-          for (int u = 0; u < n_sub; ++u) {
-            const int tok = table ? ((s0 + u) % subs_per_block) * kTileTokens : (s0 + u) * kTileTokens;
+          if (leader) {
+            mbar_arrive_expect_tx(bar_full + 8 * slot, n_sub * SUB_BYTES);
+            for (int u = 0; u < n_sub; ++u) {
+              const int tok = table ? ((s0 + u) % subs_per_block) * kTileTokens : (s0 + u) * kTileTokens;
 #pragma unroll
-            for (int h = 0; h < D / 64; ++h)
-              tma_load_5d(ring_sm + slot * 2 * SUB_BYTES + h * blk_stride + u * sub_stride, tm, bar_full + 8 * slot,
-                          h * 64, tok, sg.g, blk[u], sg.layer, policy);
+              for (int h = 0; h < D / 64; ++h)
+                tma_load_5d(ring_sm + slot * 2 * SUB_BYTES + h * blk_stride + u * sub_stride, tm, bar_full + 8 * slot,
+                            h * 64, tok, sg.g, blk[u], sg.layer, policy);
+            }
           }
         }
         if (ok) c.next_segment(prefix, p.batch, hkv);
       }
       if (!ok) {
-        // a wait expired: report, then stay until this thread's copies in flight have landed (bounded)
-        if (p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
+        // a wait expired: report, then stay until this warp's copies in flight have landed (bounded)
+        if (p.d_status && leader) *p.d_status = SPECVLM_ERR_TIMEOUT;
         const uint64_t t0 = global_timer_ns();
         for (int k = i > n_ring ? i - n_ring : 0; k < i; ++k)
           while (!mbar_test_wait(bar_full + 8 * (k % n_ring), (k / n_ring) & 1) && global_timer_ns() - t0 < kWaitLimitNs) {
@@ -253,7 +258,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // ================================================================ S = Q K^T issuer
     setmaxnreg_dec<kRegsLight>();
     if (lane == 0) publish_cut_item(p, active, cta, cta, n_active, total, T0, T1, prefix);
-    if (lane == 0 && active) {
+    if (active) {
+      const bool leader = elect_one();
       SliceCursor c;
       c.start(T0, T1, prefix, p.batch, hkv);
       const uint64_t dq0 = umma_desc_sw128(q_sm, 16, 1024), dk0 = umma_desc_sw128(k_sm, 16, 1024);
@@ -263,41 +269,40 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         ok = mbar_wait_soon(bar_k_full + 8 * kp, (i / NKP) & 1, abort_flag);
         if (ok && c.j == 0) ok = mbar_wait_soon(bar_q_full + 8 * qb, (c.seg_idx / NQ) & 1, abort_flag);
         if (ok && i >= 2) ok = mbar_wait_soon(bar_s_empty + 8 * g, ((i >> 1) - 1) & 1, abort_flag);
+        ok = warp_all(ok);
         if (!ok) break;
         tc_fence_after_sync();
         const uint64_t da = umma_desc_advance(dq0, qb * Q_BYTES), db = umma_desc_advance(dk0, kp * 2 * SUB_BYTES);
         const uint32_t d_tmem = tmem_base + C::COL_S + g * kBigTokens;
+        if (leader) {
 #pragma unroll
-        for (int s = 0; s < D / 16; ++s)
-          // 16 channels per step = 32 bytes along the swizzled 128-byte row; channels 64.. are the
-          // second 64-channel block of each operand
-          umma_bf16_ss(d_tmem, umma_desc_advance(da, (s >> 2) * (M * 128) + (s & 3) * 32),
-                       umma_desc_advance(db, (s >> 2) * (kBigTokens * 128) + (s & 3) * 32), kIdescQK, s > 0 ? 1u : 0u);
-        umma_commit(bar_s_full + 8 * g);
-        umma_commit(bar_k_empty + 8 * kp);
-        if (c.last_of_segment()) umma_commit(bar_q_empty + 8 * qb);
+          for (int s = 0; s < D / 16; ++s)
+            // 16 channels per step = 32 bytes along the swizzled 128-byte row; channels 64.. are the
+            // second 64-channel block of each operand
+            umma_bf16_ss(d_tmem, umma_desc_advance(da, (s >> 2) * (M * 128) + (s & 3) * 32),
+                         umma_desc_advance(db, (s >> 2) * (kBigTokens * 128) + (s & 3) * 32), kIdescQK, s > 0 ? 1u : 0u);
+          umma_commit(bar_s_full + 8 * g);
+          umma_commit(bar_k_empty + 8 * kp);
+          if (c.last_of_segment()) umma_commit(bar_q_empty + 8 * qb);
+        }
         c.next_tile(prefix, p.batch, hkv);
       }
-      if (!ok && p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
+      if (!ok && p.d_status && leader) *p.d_status = SPECVLM_ERR_TIMEOUT;
     }
   } else if (warp == 2) {
     // ================================================================ O += P V issuer
-    // The whole warp walks the slice; lane 0 issues.  The other lanes are there for the one job
-    // that needs hands: where a sequence ends inside a sub-tile, the V rows past its end hold
+    // The whole warp walks the slice; one lane issues.  The others lend a hand where a sequence ends inside a sub-tile, the V rows past its end hold
     // whatever the page held, and are cleared so that a zero probability times a stale non-finite
     // value cannot reach O.
     setmaxnreg_dec<kRegsLight>();
     if (active) {
+      const bool leader = elect_one();
       SliceCursor c;
       c.start(T0, T1, prefix, p.batch, hkv);
       const uint64_t dp0 = umma_desc_sw128(p_sm, 16, 1024);
       const uint64_t dv0 = umma_desc_sw128(v_sm, kTileTokens * 128, 1024);   // 64-channel blocks 8 KB apart
       bool ok = true;
       int n_sub_seq = 0, kv_len = 0;
-#define PV_WAIT(bar, parity)                                                        \
-  do {                                                                              \
-    ok = __all_sync(0xffffffffu, mbar_wait_soon((bar), (parity), abort_flag));           \
-  } while (0)
       for (int i = 0; i < n_my; ++i) {
         const int g = i & 1, vp = i % NVP;
         if (c.j == 0) {
@@ -306,7 +311,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         }
         const int s0 = 2 * (c.sg.tile0 + c.j);
         const int n_sub = n_sub_seq - s0 < 2 ? n_sub_seq - s0 : 2;
-        PV_WAIT(bar_v_full + 8 * vp, (i / NVP) & 1);
+        ok = warp_wait_soon(bar_v_full + 8 * vp, (i / NVP) & 1, abort_flag);
         if (!ok) break;
         if (s0 + n_sub == n_sub_seq && (kv_len & (kTileTokens - 1)) != 0) {
           uint8_t* vt = big_ptr + C::OFF_V + vp * 2 * SUB_BYTES + (n_sub - 1) * SUB_BYTES;
@@ -320,11 +325,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           __syncwarp();
         }
         // the first product of each group overwrites that group's O: the previous item must be out
-        if (c.j < 2 && c.seg_idx >= 1) PV_WAIT(bar_o_empty, (c.seg_idx - 1) & 1);
-        if (ok) PV_WAIT(bar_p_full + 8 * g, (i >> 1) & 1);
+        if (c.j < 2 && c.seg_idx >= 1) ok = warp_wait_soon(bar_o_empty, (c.seg_idx - 1) & 1, abort_flag);
+        if (ok) ok = warp_wait_soon(bar_p_full + 8 * g, (i >> 1) & 1, abort_flag);
         if (!ok) break;
-        if (lane == 0) {
-          tc_fence_after_sync();
+        tc_fence_after_sync();
+        if (leader) {
           const uint64_t da = umma_desc_advance(dp0, g * P_BYTES), db = umma_desc_advance(dv0, vp * 2 * SUB_BYTES);
           const uint32_t d_tmem = tmem_base + C::COL_O + g * D;
           const uint32_t acc0 = c.j >= 2 ? 1u : 0u;
@@ -342,11 +347,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           umma_commit(bar_v_empty + 8 * vp);
           if (c.last_of_segment()) umma_commit(bar_o_full);
         }
-        __syncwarp();
         c.next_tile(prefix, p.batch, hkv);
       }
-#undef PV_WAIT
-      if (!ok && p.d_status && lane == 0) *p.d_status = SPECVLM_ERR_TIMEOUT;
+      if (!ok && p.d_status && leader) *p.d_status = SPECVLM_ERR_TIMEOUT;
     }
   } else {
     // ================================================================ softmax / epilogue (warps 4..11)
@@ -381,7 +384,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     int i0 = 0;           // index (inside the slice) of the current segment's first tile
 #define SM_WAIT(bar, parity)                                                        \
   do {                                                                              \
-    ok = __all_sync(0xffffffffu, mbar_wait_soon((bar), (parity), abort_flag));           \
+    ok = warp_wait_soon((bar), (parity), abort_flag);                                \
     if (!ok) goto softmax_done;                                                     \
   } while (0)
 

@@ -121,8 +121,35 @@ __device__ __forceinline__ bool mbar_wait_soon(uint32_t bar, uint32_t parity, vo
   return mbar_test_wait(bar, parity) || mbar_wait(bar, parity, abort_flag);
 }
 
+// Waits of a whole warp: the vote makes the outcome the same in every lane, whichever lanes saw the abort flag.
+__device__ __forceinline__ bool warp_all(bool ok) { return __all_sync(0xffffffffu, ok) != 0; }
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return warp_all(mbar_wait(bar, parity, abort_flag));
+}
+__device__ __forceinline__ bool warp_wait_soon(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return warp_all(mbar_wait_soon(bar, parity, abort_flag));
+}
+
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// True in one lane of the (whole, converged) warp, the same one every time.  What a warp issues for itself -- tensor
+// instructions, their commits, TMA copies -- goes behind this in code that all of its lanes run: in a branch of
+// `lane == 0` the compiler takes the operands for different in each lane and moves them to the uniform registers that
+// these instructions read one instruction at a time.  Eight tcgen05.mma of fixed operands: 402 cycles to
+// issue behind `lane == 0`, 133 behind this; with operands that change from tile to tile 760 in the first form.
+// Verification, sustained, at 80 layers of 6400 tokens: a tree of 208 rows 669 -> 648 us (4310 -> 3700 cycles a
+// tile), 48 rows 360 -> 353.5; 40 layers x 4 sequences, 72 rows 1974 -> 1954.  Not in the rating passes, whose
+// issuer is never late: 32 polling lanes there cost 0.6 to 1 % at the power cap; nor for the decode kernel's copies (even).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(e));
+  return e != 0;
 }
 
 // ------------------------------------------------------------------------------ TMA
