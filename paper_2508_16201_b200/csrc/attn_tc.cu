@@ -779,121 +779,160 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 
 // ---------------------------------------------------------------------------------------------
 // Merge of the items that slice boundaries cut, a kernel of its own behind the attention kernel
-// (launched with programmatic stream serialization).  blockIdx.x = the CTA that holds an item's
-// first part (most hold none and leave), blockIdx.y = a block of output positions (four channels of
-// a row each).  The parts of an item sit in the scratch slots first_slot and 2 (c + 1), 2 (c + 2), ..
+// (launched with programmatic stream serialization).  A unit of work is a cut item and a block of its output
+// positions (four channels of a row each).  The parts of an item sit in the scratch slots first_slot and
+// 2 (c + 1), 2 (c + 2), ..
 //   out = sum_s w_s o_s / sum_s w_s,  w_s = 2^(lse_s - max),  parts folded in slice order (fixed).
 // A row with a part that was never written (its CTA gave up) is left alone.
-// LANES warps share an item's parts, for launches that cut few items into many parts.
-// One CTA per item used to do this at the end of the attention kernel, after an atomic counter said that
-// it was the last: with one layer of 6400 tokens (8 items in 13 parts each) that was 21 of the
-// call's 37.8 us, plus a memset of the counters and 2.5 us of fences per partial result.
+// LANES warps share an item's parts: 1 where most items are cut in two, 4 where few items are cut into many parts.
+// blockIdx.x = the CTA that holds an item's first part, blockIdx.y the block of positions; most CTAs of few items hold
+// no first part, and their blocks leave.  Where that would take several rounds of blocks (TABLE) every block reads the
+// whole table of cut items (2.4 KB), finds the valid entries by ballots and takes units in turn: one layer of 6400
+// tokens launched 3552 blocks for 192 units, in eight rounds, and the merge took 6.4 of the call's 19.2 us; now 17.3
+// (208 rows: 43.9 -> 31.2).  Elsewhere the table costs more than it saves (4 layers x 4 heads of 6400 tokens, one
+// query row: 13.3 -> 14.5; 1 layer of 12 800: 13.6 -> 14.1).
 // ---------------------------------------------------------------------------------------------
 constexpr int kMergeThreads = 256;
+constexpr int kMergeMaxCtas = 640;                       // entries of the table: CTAs of all sets (4 per SM at most)
 
-template <int D, int LANES>
-__global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnTcParams p) {
-  pdl_launch_next();
-  pdl_wait();
+template <int D, int LANES, bool TABLE>
+__global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __grid_constant__ AttnTcParams p, int n_ctas) {
   // parts whose loads are in flight together: most cut items have two parts, and the registers of more would
   // keep blocks off the SMs (26-node tree under sustained load 677 -> 668 us, and 80-layer chain 359.5 -> 358.1); the
   // many parts of a few items are what LANES is for
   constexpr int kMergeChunk = LANES == 1 ? 2 : 8;
-  const int gcta = blockIdx.x;
-  const int4 cut = __ldcg(p.ws_cut + gcta);
-  if (cut.w == 0) return;
-  const int ctas_per_part = (int)gridDim.x / p.n_parts;
-  const int part = gcta / ctas_per_part, q0 = part * p.q_per;
-  const int rows = (p.n_win - q0 < p.q_per ? p.n_win - q0 : p.q_per) * p.group;
+  constexpr int kPos = kMergeThreads / LANES;              // output positions of a unit
+  constexpr int kRounds = (kMergeMaxCtas + kMergeThreads - 1) / kMergeThreads;
+  __shared__ int4 cuts[TABLE ? kMergeMaxCtas : 1];
+  __shared__ uint32_t valid[TABLE ? kRounds * (kMergeThreads / 32) : 1];
+  __shared__ float4 acc_sm[LANES > 1 ? LANES - 1 : 1][kPos];
+  __shared__ float2 md_sm[LANES > 1 ? LANES - 1 : 1][kPos];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kPos = kMergeThreads / LANES;              // output positions of a block
   const int wl = warp % LANES;                              // this warp's share of the parts: wl, wl + LANES, ..
   const int pos = (warp / LANES) * 32 + lane;
-  const int idx = blockIdx.y * kPos + pos;
-  const bool on = idx < rows * (D / 4);
-  const int r = on ? idx / (D / 4) : 0, c4 = on ? idx - r * (D / 4) : 0;
-  float mm = -INFINITY, den = 0.f;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool lost = false;
-  for (int k0 = wl; k0 < cut.w; k0 += LANES * kMergeChunk) {
-    float ls[kMergeChunk];
-    float4 x[kMergeChunk];
-#pragma unroll
-    for (int q = 0; q < kMergeChunk; ++q) {
-      const int k = k0 + q * LANES;
-      ls[q] = -INFINITY;
-      x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (on && k < cut.w) {
-        const size_t row = (size_t)(k == 0 ? cut.z : 2 * (gcta + k)) * p.rows + r;
-        ls[q] = ldg_cg_f32(p.ws_lse + (size_t)(c4 >> 4) * p.lse_block + row);
-        lost |= unwritten(ls[q]);
-        x[q] = ldg_cg_f32x4(p.ws_o + row * D + c4 * 4);
-      }
-    }
-    float m2 = mm;
-#pragma unroll
-    for (int q = 0; q < kMergeChunk; ++q) m2 = fmaxf(m2, ls[q]);
-    if (m2 == -INFINITY) continue;
-    const float sc = mm == -INFINITY ? 0.f : fast_exp2(mm - m2);
-    acc.x *= sc;
-    acc.y *= sc;
-    acc.z *= sc;
-    acc.w *= sc;
-    den *= sc;
-#pragma unroll
-    for (int q = 0; q < kMergeChunk; ++q) {
-      const float w = ls[q] == -INFINITY ? 0.f : fast_exp2(ls[q] - m2);
-      acc.x += w * x[q].x;
-      acc.y += w * x[q].y;
-      acc.z += w * x[q].z;
-      acc.w += w * x[q].w;
-      den += w;
-    }
-    mm = m2;
-  }
-  if constexpr (LANES > 1) {
-    __shared__ float4 acc_sm[LANES - 1][kPos];
-    __shared__ float2 md_sm[LANES - 1][kPos];
-    if (wl > 0) {
-      acc_sm[wl - 1][pos] = acc;
-      md_sm[wl - 1][pos] = make_float2(lost ? __uint_as_float(kUnwritten) : mm, den);
+  pdl_launch_next();
+  pdl_wait();
+  int n_units = 0, chunks = 1;
+  if constexpr (TABLE) {
+    for (int r = 0, i = threadIdx.x; r * kMergeThreads < n_ctas; ++r, i += kMergeThreads) {
+      const int4 c = i < n_ctas ? __ldcg(p.ws_cut + i) : make_int4(0, 0, 0, 0);
+      if (i < n_ctas) cuts[i] = c;
+      const uint32_t v = __ballot_sync(0xffffffffu, c.w != 0);
+      if (lane == 0) valid[r * (kMergeThreads / 32) + warp] = v;
     }
     __syncthreads();
-    if (wl > 0) return;
-    float m2 = mm;
-#pragma unroll
-    for (int w = 0; w < LANES - 1; ++w) {
-      lost |= unwritten(md_sm[w][pos].x);
-      m2 = fmaxf(m2, md_sm[w][pos].x);
-    }
-    const float sc = mm == -INFINITY ? 0.f : fast_exp2(mm - m2);
-    acc.x *= sc;
-    acc.y *= sc;
-    acc.z *= sc;
-    acc.w *= sc;
-    den *= sc;
-#pragma unroll
-    for (int w = 0; w < LANES - 1; ++w) {
-      const float2 md = md_sm[w][pos];
-      const float4 x = acc_sm[w][pos];
-      const float f = md.x == -INFINITY ? 0.f : fast_exp2(md.x - m2);
-      acc.x += f * x.x;
-      acc.y += f * x.y;
-      acc.z += f * x.z;
-      acc.w += f * x.w;
-      den += f * md.y;
-    }
-    mm = m2;
+    for (int w = 0; w < (n_ctas + 31) / 32; ++w) n_units += __popc(valid[w]);
+    chunks = (p.rows * (D / 4) + kPos - 1) / kPos;
+    n_units *= chunks;
   }
-  if (!on || lost) return;
-  const float inv = den > 0.f ? 1.f / den : 0.f;
-  const int t = r / p.group, h = cut.y * p.group + (r - t * p.group);
-  const size_t orow = ((size_t)cut.x * p.n_win + q0 + t) * p.n_q_heads + h;
-  uint2 packed;
-  packed.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-  packed.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-  *reinterpret_cast<uint2*>(p.out + orow * D + c4 * 4) = packed;
-  if (p.lse && c4 == 0) p.lse[orow] = den > 0.f ? (mm + log2f(den)) * kLn2 : -INFINITY;
+  const int ctas_per_part = n_ctas / p.n_parts;
+  for (int unit = blockIdx.x; !TABLE || unit < n_units; unit += gridDim.x) {
+    int gcta, idx;
+    int4 cut;
+    if constexpr (!TABLE) {
+      gcta = unit;
+      cut = __ldcg(p.ws_cut + gcta);
+      if (cut.w == 0) return;
+      idx = blockIdx.y * kPos + pos;
+    } else {
+      int k_th = unit / chunks;
+      idx = (unit - k_th * chunks) * kPos + pos;
+      int word = 0;
+      for (int n = __popc(valid[0]); k_th >= n; n = __popc(valid[++word])) k_th -= n;
+      uint32_t bits = valid[word];
+      for (; k_th > 0; --k_th) bits &= bits - 1;
+      gcta = word * 32 + __ffs((int)bits) - 1;
+      cut = cuts[gcta];
+    }
+    const int part = gcta / ctas_per_part, q0 = part * p.q_per;
+    const int rows = (p.n_win - q0 < p.q_per ? p.n_win - q0 : p.q_per) * p.group;
+    const bool on = idx < rows * (D / 4);
+    const int r = on ? idx / (D / 4) : 0, c4 = on ? idx - r * (D / 4) : 0;
+    float mm = -INFINITY, den = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool lost = false;
+    for (int k0 = wl; k0 < cut.w; k0 += LANES * kMergeChunk) {
+      float ls[kMergeChunk];
+      float4 x[kMergeChunk];
+#pragma unroll
+      for (int q = 0; q < kMergeChunk; ++q) {
+        const int k = k0 + q * LANES;
+        ls[q] = -INFINITY;
+        x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (on && k < cut.w) {
+          const size_t row = (size_t)(k == 0 ? cut.z : 2 * (gcta + k)) * p.rows + r;
+          ls[q] = ldg_cg_f32(p.ws_lse + (size_t)(c4 >> 4) * p.lse_block + row);
+          lost |= unwritten(ls[q]);
+          x[q] = ldg_cg_f32x4(p.ws_o + row * D + c4 * 4);
+        }
+      }
+      float m2 = mm;
+#pragma unroll
+      for (int q = 0; q < kMergeChunk; ++q) m2 = fmaxf(m2, ls[q]);
+      if (m2 == -INFINITY) continue;
+      const float sc = mm == -INFINITY ? 0.f : fast_exp2(mm - m2);
+      acc.x *= sc;
+      acc.y *= sc;
+      acc.z *= sc;
+      acc.w *= sc;
+      den *= sc;
+#pragma unroll
+      for (int q = 0; q < kMergeChunk; ++q) {
+        const float w = ls[q] == -INFINITY ? 0.f : fast_exp2(ls[q] - m2);
+        acc.x += w * x[q].x;
+        acc.y += w * x[q].y;
+        acc.z += w * x[q].z;
+        acc.w += w * x[q].w;
+        den += w;
+      }
+      mm = m2;
+    }
+    if constexpr (LANES > 1) {
+      if (wl > 0) {
+        acc_sm[wl - 1][pos] = acc;
+        md_sm[wl - 1][pos] = make_float2(lost ? __uint_as_float(kUnwritten) : mm, den);
+      }
+      __syncthreads();
+      if (wl == 0) {
+        float m2 = mm;
+#pragma unroll
+        for (int w = 0; w < LANES - 1; ++w) {
+          lost |= unwritten(md_sm[w][pos].x);
+          m2 = fmaxf(m2, md_sm[w][pos].x);
+        }
+        const float sc = mm == -INFINITY ? 0.f : fast_exp2(mm - m2);
+        acc.x *= sc;
+        acc.y *= sc;
+        acc.z *= sc;
+        acc.w *= sc;
+        den *= sc;
+#pragma unroll
+        for (int w = 0; w < LANES - 1; ++w) {
+          const float2 md = md_sm[w][pos];
+          const float4 x = acc_sm[w][pos];
+          const float f = md.x == -INFINITY ? 0.f : fast_exp2(md.x - m2);
+          acc.x += f * x.x;
+          acc.y += f * x.y;
+          acc.z += f * x.z;
+          acc.w += f * x.w;
+          den += f * md.y;
+        }
+        mm = m2;
+      }
+      if (TABLE) __syncthreads();                           // the next unit's sums overwrite these
+    }
+    if (!TABLE && (wl > 0 || !on || lost)) return;
+    if (wl > 0 || !on || lost) continue;
+    const float inv = den > 0.f ? 1.f / den : 0.f;
+    const int t = r / p.group, h = cut.y * p.group + (r - t * p.group);
+    const size_t orow = ((size_t)cut.x * p.n_win + q0 + t) * p.n_q_heads + h;
+    uint2 packed;
+    packed.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+    packed.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+    *reinterpret_cast<uint2*>(p.out + orow * D + c4 * 4) = packed;
+    if (p.lse && c4 == 0) p.lse[orow] = den > 0.f ? (mm + log2f(den)) * kLn2 : -INFINITY;
+    if (!TABLE) return;
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -958,13 +997,15 @@ static int32_t launch_merge(const AttnTcParams& p, int ctas, cudaStream_t st) {
   // Two parts per cut item where the items outnumber the CTAs; many where a few items fill the chip.
   const int64_t items = (int64_t)p.n_layers * p.batch * p.n_kv_heads;
   const int positions = p.rows * (D / 4);
-  if (ctas > 4 * items) {
-    constexpr int kPos = kMergeThreads / 4;
-    return launch_after(attn_merge_kernel<D, 4>, dim3((unsigned)grid, (unsigned)((positions + kPos - 1) / kPos)),
-                        dim3(kMergeThreads), 0, st, p);
-  }
-  return launch_after(attn_merge_kernel<D, 1>, dim3((unsigned)grid, (unsigned)((positions + kMergeThreads - 1) / kMergeThreads)),
-                      dim3(kMergeThreads), 0, st, p);
+  const int chunks1 = (positions + kMergeThreads - 1) / kMergeThreads, chunks4 = (4 * positions + kMergeThreads - 1) / kMergeThreads;
+  if (ctas <= 4 * items)
+    return launch_after(attn_merge_kernel<D, 1, false>, dim3((unsigned)grid, (unsigned)chunks1), dim3(kMergeThreads), 0, st, p, grid);
+  const int64_t resident = 3 * sm_count();                // blocks that the chip holds at once
+  if ((int64_t)grid * chunks4 <= 2 * resident || grid > kMergeMaxCtas)
+    return launch_after(attn_merge_kernel<D, 4, false>, dim3((unsigned)grid, (unsigned)chunks4), dim3(kMergeThreads), 0, st, p, grid);
+  const int64_t units = p.n_parts * items * chunks4;
+  return launch_after(attn_merge_kernel<D, 4, true>, dim3((unsigned)(units < resident ? units : resident)), dim3(kMergeThreads), 0,
+                      st, p, grid);
 }
 
 // Ancestor masks of a draft tree: bit w of anc[b][t] says that node t attends window position w
