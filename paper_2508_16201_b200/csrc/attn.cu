@@ -402,7 +402,8 @@ struct SliceCfg {
   static constexpr int OFF_ML = OFF_O + 4 * NG * 16 * Rows16<D>::OPITCH * 4;
   static constexpr int OFF_BAR = OFF_ML + 2 * 4 * NG * 16 * 4;
   static constexpr int OFF_MISC = OFF_BAR + 16 * STAGES;
-  static constexpr int OFF_PREFIX = OFF_MISC + 16;
+  static constexpr int OFF_PLAN = OFF_MISC + 16;
+  static constexpr int OFF_PREFIX = OFF_PLAN + (kPlanBytes + 7) / 8 * 8;
   static constexpr int SMEM = OFF_PREFIX + (kSchedMaxBatch + 1) * 4 + 1024;
   static_assert(STAGES % NG == 0, "ring depth must be a multiple of the number of consumer groups");
   static_assert(SMEM <= 232448, "shared-memory plan does not fit");
@@ -420,7 +421,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
   uint8_t* const smem = smem_raw + (base - raw_addr);
   const uint32_t bar_full = base + C::OFF_BAR, bar_empty = bar_full + 8 * STAGES;
   volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC);
-  volatile int* const any_empty = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
+  CtaSlice* const slice = reinterpret_cast<CtaSlice*>(smem + C::OFF_PLAN);
   int* const prefix = reinterpret_cast<int*>(smem + C::OFF_PREFIX);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -438,18 +439,11 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
   }
   pdl_launch_next();
   pdl_wait();
-  if (warp == 0) {
-    const bool empty = tile_prefix<kTileTokens>(p, prefix, lane);
-    if (lane == 0) *any_empty = empty ? 1 : 0;
-  }
+  if (warp == 0) plan_slice<kTileTokens>(p, prefix, slice, blockIdx.x, gridDim.x, lane);
   if (warp > 0 && warp < NW) unwritten_parts(p, blockIdx.x, D, tid - 32, 32 * (NW - 1));
   __syncthreads();
   const int hkv = p.n_kv_heads, cta = blockIdx.x;
-  const int64_t total = (int64_t)p.n_layers * hkv * prefix[p.batch];
-  const int n_active = sched_active_ctas(total, (int)gridDim.x);
-  const bool active = total > 0 && cta < n_active;
-  const int64_t T0 = active ? slice_begin(cta, n_active, total) : 0;
-  const int64_t T1 = active ? slice_begin(cta + 1, n_active, total) : 0;
+  const int64_t T0 = slice->begin, T1 = slice->end;
 
   if (warp == NW) {
     // ------------------------------------------------------------------ producer
@@ -478,12 +472,12 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
           tma_load_5d(dst + TILE_BYTES + h * (kTileTokens * 128), &tm_v, full, h * 64, tok, c.sg.g, blk, c.sg.layer, policy);
         }
         if (!told && i == STAGES - 1) {                     // the ring is full: time for the hand-over of a cut item
-          publish_cut_item(p, active, cta, cta, n_active, total, T0, T1, prefix);
+          publish_cut_item(p, *slice, cta, cta, prefix);
           told = true;
         }
         c.next_tile(prefix, p.batch, hkv);
       }
-      if (!told) publish_cut_item(p, active, cta, cta, n_active, total, T0, T1, prefix);
+      if (!told) publish_cut_item(p, *slice, cta, cta, prefix);
       if (!ok) {
         // a wait expired: report, then stay until this CTA's copies in flight have landed
         if (p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
@@ -502,7 +496,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
   float* const m_sm = reinterpret_cast<float*>(smem + C::OFF_ML);     // [NW][16]
   float* const l_sm = m_sm + NW * 16;                                  // [NW][16]
   // sequences without any token: their outputs are zero, their LSE -inf
-  if (*any_empty) {
+  if (slice->any_empty) {
     const int n_items = p.n_layers * p.batch * hkv;
     for (int item = cta; item < n_items; item += (int)gridDim.x) {
       const int lb = item / hkv, g = item - lb * hkv, b = lb % p.batch;
@@ -609,7 +603,10 @@ static int rows16_slices(const specvlm_kv_t* kv, int32_t batch) {
   }
   const double slices = 4.5 + ragged * hbm + 2.0 * (1.0 + (double)items / sms);
   if (slices + 1.5 >= per_item) return 0;
-  return sched_active_ctas(items * tiles, (int)sms);
+  const int even = sched_active_ctas(items * tiles, (int)sms);
+  // slices that keep to item boundaries may use more CTAs: every item rounds its own up
+  const int64_t aligned = items * sched_active_ctas(tiles, (int)sms);
+  return aligned > even && items <= sms ? (int)(aligned < sms ? aligned : sms) : even;
 }
 
 static size_t rows16_ws_bytes(const specvlm_kv_t* kv, int32_t batch, int rows) {

@@ -41,7 +41,8 @@ struct PairCfg {
   static constexpr int BIG = OFF_Q + 2 * Q_BYTES;
   static constexpr int N_BARS = 2 * NKP + 2 * NVP + 20;
   static constexpr int SM_MISC = 8 * N_BARS;
-  static constexpr int SM_PREFIX = SM_MISC + 32;
+  static constexpr int SM_PLAN = SM_MISC + 16;
+  static constexpr int SM_PREFIX = SM_PLAN + (kPlanBytes + 7) / 8 * 8;
   static constexpr int SMALL_USED = SM_PREFIX + (kSchedMaxBatch + 1) * 4;
   static constexpr int SMALL = (SMALL_USED + 1023) / 1024 * 1024;
   static constexpr int kMaxSmem = 232448;                       // 227 KB
@@ -102,7 +103,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   const uint32_t bar_turn = bar_o_empty + 16;          // [2][4]: the turn of part g's warp of a TMEM lane quadrant
   volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem_raw + C::SM_MISC);
   volatile uint32_t* const tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_raw + C::SM_MISC + 8);
-  volatile int* const any_empty = reinterpret_cast<volatile int*>(smem_raw + C::SM_MISC + 16);
+  CtaSlice* const slice = reinterpret_cast<CtaSlice*>(smem_raw + C::SM_PLAN);
   int* const prefix = reinterpret_cast<int*>(smem_raw + C::SM_PREFIX);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -163,20 +164,14 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   }
   pdl_wait();
   if (warp >= 2 && warp - 2 < n_here) unwritten_parts(p, (2 * set + warp - 2) * ctas + cta, D, lane, 32);
-  if (warp == 0) {
-    const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
-    if (lane == 0) *any_empty = empty ? 1 : 0;
-  }
+  if (warp == 0) plan_slice<kBigTokens>(p, prefix, slice, cta, ctas, lane);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   const int hkv = p.n_kv_heads;
-  const int64_t total = (int64_t)p.n_layers * hkv * prefix[p.batch];
-  const int n_active = sched_active_ctas(total, ctas);
-  const bool active = total > 0 && cta < n_active;
-  const int64_t T0 = active ? slice_begin(cta, n_active, total) : 0;
-  const int64_t T1 = active ? slice_begin(cta + 1, n_active, total) : 0;
+  const int64_t T0 = slice->begin, T1 = slice->end;
+  const bool active = T0 < T1;
   const int n_my = (int)(T1 - T0);
 
   if (warp == 0 || warp == 3) {
@@ -265,7 +260,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     setmaxnreg_dec<kRegsLight>();
     const int g = warp - 1;
     if (g < n_here && lane == 0)
-      publish_cut_item(p, active, cta, (2 * set + g) * ctas + cta, n_active, total, T0, T1, prefix);
+      publish_cut_item(p, *slice, cta, (2 * set + g) * ctas + cta, prefix);
     if (g < n_here && active) {
       const bool leader = elect_one();
       SliceCursor c;
@@ -380,7 +375,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     const uint32_t saddr = lane_base + C::COL_S + g * kBigTokens, oaddr = lane_base + C::COL_O + g * D;
 
     // sequences without any token: their outputs are zero, their LSE -inf
-    if (*any_empty && rows > 0) {
+    if (slice->any_empty && rows > 0) {
       const int n_items = p.n_layers * p.batch * hkv;
       for (int item = cta; item < n_items; item += ctas) {
         const int lb = item / hkv, kvh = item - lb * hkv, b = lb % p.batch;

@@ -38,6 +38,38 @@ SPECVLM_HD int slice_owner(int64_t f, int n_active, int64_t total_tiles) {
   return (int)(((f + 1) * n_active - 1) / total_tiles);
 }
 
+// Where the items are fewer than the CTAs, slices that keep to item boundaries: an item of t tiles gets ceil(t / q)
+// CTAs of its own, as equal as its tiles allow.  No CTA then works on two items, one after the other (with a few tiles a
+// CTA the second one's hand-over is as long as its tiles).  part_prefix[b] = CTAs of one KV head of the sequences < b.
+constexpr int kSchedAlignedBatch = 32;
+
+// Tiles a CTA from which to look for such a split, and up to which it is worth it.
+SPECVLM_HD int aligned_q_first(int64_t total_tiles, int grid) {
+  const int64_t q = (total_tiles + grid - 1) / grid;
+  return q > kSchedMinTilesPerCta ? (int)q : kSchedMinTilesPerCta;
+}
+SPECVLM_HD int aligned_q_last(int q_first) { return q_first + 1; }
+
+// The slice of CTA c, its item's CTAs in `parts`; false if c has no work.
+SPECVLM_HD bool aligned_slice(int c, const int* prefix, const int* part_prefix, int batch, int n_layers, int n_kv_heads,
+                              int64_t* begin, int64_t* end, int* parts) {
+  const int per_layer = n_kv_heads * part_prefix[batch];
+  if (per_layer == 0 || c >= n_layers * per_layer) return false;
+  const int layer = c / per_layer, rem = c - layer * per_layer;
+  int lo = 0, hi = batch - 1;             // last b with n_kv_heads * part_prefix[b] <= rem
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (n_kv_heads * part_prefix[mid] <= rem) lo = mid; else hi = mid - 1;
+  }
+  const int n = part_prefix[lo + 1] - part_prefix[lo], t = prefix[lo + 1] - prefix[lo];
+  const int rem2 = rem - n_kv_heads * part_prefix[lo], g = rem2 / n, part = rem2 - g * n;
+  const int64_t item = (int64_t)n_kv_heads * ((int64_t)layer * prefix[batch] + prefix[lo]) + (int64_t)g * t;
+  *begin = item + (int64_t)part * t / n;
+  *end = item + (int64_t)(part + 1) * t / n;
+  *parts = n;
+  return true;
+}
+
 struct Segment {
   int layer, b, g;        // the item
   int item;               // (layer * batch + b) * n_kv_heads + g

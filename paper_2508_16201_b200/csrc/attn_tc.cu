@@ -50,7 +50,8 @@ struct TcCfg {
   static constexpr int N_BARS = 2 * NKP + 2 * NVP + 15;
   static constexpr int SM_BAR = 0;
   static constexpr int SM_MISC = SM_BAR + 8 * N_BARS;
-  static constexpr int SM_PREFIX = SM_MISC + 32;
+  static constexpr int SM_PLAN = SM_MISC + 16;
+  static constexpr int SM_PREFIX = SM_PLAN + (kPlanBytes + 7) / 8 * 8;
   static constexpr int SM_STATS = SM_PREFIX + (kSchedMaxBatch + 1) * 4;     // [2 groups][M rows] float2
   static constexpr int SMALL_USED = SM_STATS + 2 * M * 8;
   static constexpr int SMALL = (SMALL_USED + 1023) / 1024 * 1024;
@@ -95,7 +96,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const uint32_t bar_ep_stats = bar_o_empty + 8;       // both groups' row statistics are in shared memory
   volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem_raw + C::SM_MISC);
   volatile uint32_t* const tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_raw + C::SM_MISC + 8);
-  volatile int* const any_empty = reinterpret_cast<volatile int*>(smem_raw + C::SM_MISC + 20);
+  CtaSlice* const slice = reinterpret_cast<CtaSlice*>(smem_raw + C::SM_PLAN);
   int* const prefix = reinterpret_cast<int*>(smem_raw + C::SM_PREFIX);
   float2* const stats = reinterpret_cast<float2*>(smem_raw + C::SM_STATS);
 
@@ -156,22 +157,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   }
   pdl_wait();
   if (warp == 3) unwritten_parts(p, blockIdx.x, D, lane, 32);
-  if (warp == 0) {
-    const bool empty = tile_prefix<kBigTokens>(p, prefix, lane);
-    if (lane == 0) *any_empty = empty ? 1 : 0;
-  }
+  if (warp == 0) plan_slice<kBigTokens>(p, prefix, slice, blockIdx.x, gridDim.x, lane);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   const int hkv = p.n_kv_heads;
-  const int64_t total = (int64_t)p.n_layers * hkv * prefix[p.batch];
   const int cta = blockIdx.x;
   const int rows = p.rows;                              // rows in use (of the M rows of a tile)
-  const int n_active = sched_active_ctas(total, (int)gridDim.x);
-  const bool active = total > 0 && cta < n_active;
-  const int64_t T0 = active ? slice_begin(cta, n_active, total) : 0;
-  const int64_t T1 = active ? slice_begin(cta + 1, n_active, total) : 0;
+  const int64_t T0 = slice->begin, T1 = slice->end;
+  const bool active = T0 < T1;
   const int n_items = p.n_layers * p.batch * hkv;
   const int n_my = (int)(T1 - T0);
 
@@ -257,7 +252,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   } else if (warp == 1) {
     // ================================================================ S = Q K^T issuer
     setmaxnreg_dec<kRegsLight>();
-    if (lane == 0) publish_cut_item(p, active, cta, cta, n_active, total, T0, T1, prefix);
+    if (lane == 0) publish_cut_item(p, *slice, cta, cta, prefix);
     if (active) {
       const bool leader = elect_one();
       SliceCursor c;
@@ -364,7 +359,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const int nh = (rows > row0(0) ? 1 : 0) + (NH > 1 && rows > row0(1) ? 1 : 0);
 
     // sequences without any token: their outputs are zero, their LSE -inf
-    if (*any_empty) {
+    if (slice->any_empty) {
       for (int item = cta; item < n_items; item += (int)gridDim.x) {
         const int lb = item / hkv, g = item - lb * hkv, b = lb % p.batch;
         if (prefix[b + 1] != prefix[b]) continue;
@@ -954,7 +949,11 @@ static int tc_set_ctas(const specvlm_kv_t* kv, int32_t batch, int n_parts) {
                             ((kv->max_seq_len + kBigTokens - 1) / kBigTokens);
   int per_set = sm_count() / ((n_parts + 1) / 2);
   if (per_set < 1) per_set = 1;
-  return sched_active_ctas(tiles_max, per_set);
+  const int even = sched_active_ctas(tiles_max, per_set);
+  // slices that keep to item boundaries may use more CTAs: every item rounds its own up
+  const int64_t items = (int64_t)kv->n_layers * batch * kv->n_kv_heads;
+  const int64_t aligned = items * sched_active_ctas((kv->max_seq_len + kBigTokens - 1) / kBigTokens, per_set);
+  return aligned > even && items <= per_set ? (int)(aligned < per_set ? aligned : per_set) : even;
 }
 
 SlicePlan attn_tc_plan(const specvlm_kv_t* kv, int32_t batch, int32_t group, int32_t n_q) {

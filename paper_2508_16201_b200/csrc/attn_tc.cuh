@@ -24,6 +24,7 @@ struct AttnTcParams {
   int32_t n_parts, q_per;     // the window is cut into n_parts parts of q_per tokens (the last may be shorter)
   int32_t rows;               // rows of a full part = q_per * group (<= 128): the row pitch of the scratch slots
   int32_t max_blocks, block_tokens, max_seq_len;
+  int32_t align;              // slices may keep to item boundaries (attn_sched.h): no more items than CTAs
   int32_t lse_block;          // floats from one 64-channel block's LSEs to the next one's
   float scale_log2;           // sm_scale * log2(e)
 };
@@ -175,18 +176,71 @@ __device__ __forceinline__ bool tile_prefix(const AttnTcParams& p, int* prefix, 
   return __any_sync(0xffffffffu, empty);
 }
 
+// A CTA's slice of the flat tile list.
+struct CtaSlice {
+  int64_t total, begin, end;   // tiles of the list; the slice (empty: the CTA has no work)
+  int n_active;                // CTAs with work, of slices of equal length
+  int parts;                   // slices that keep to item boundaries: the CTAs of this one's item; 0 otherwise
+  int any_empty;               // some sequence has no token
+};
+constexpr int kPlanBytes = (int)sizeof(CtaSlice) + (kSchedAlignedBatch + 1) * 4;   // with the CTAs per sequence behind it
+
+// The plan of CTA `cta` of `ctas`, by one warp: the running sums of the tiles and the CTA's slice, to shared memory.
+template <int TILE>
+__device__ __forceinline__ void plan_slice(const AttnTcParams& p, int* prefix, CtaSlice* out, int cta, int ctas, int lane) {
+  const bool empty = tile_prefix<TILE>(p, prefix, lane);
+  __syncwarp();
+  const int per_head = prefix[p.batch], lh = p.n_layers * p.n_kv_heads;
+  const int64_t total = (int64_t)lh * per_head;
+  int q = 0;
+  if (p.align && total > 0) {
+    int* const part_prefix = reinterpret_cast<int*>(out + 1);
+    const int t = lane < p.batch ? prefix[lane + 1] - prefix[lane] : 0;
+    const int q_first = aligned_q_first(total, ctas);
+    for (int c = q_first; c <= aligned_q_last(q_first) && q == 0; ++c) {
+      int n = (t + c - 1) / c;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, n, off);
+        if (lane >= off) n += o;
+      }
+      if ((int64_t)lh * __shfl_sync(0xffffffffu, n, 31) <= ctas) {
+        q = c;
+        part_prefix[lane + 1] = n;
+        if (lane == 0) part_prefix[0] = 0;
+      }
+    }
+    __syncwarp();
+  }
+  if (lane == 0) {
+    CtaSlice s;
+    s.total = total;
+    s.begin = s.end = 0;
+    s.n_active = sched_active_ctas(total, ctas);
+    s.parts = 0;
+    s.any_empty = empty ? 1 : 0;
+    if (q > 0) {
+      aligned_slice(cta, prefix, reinterpret_cast<const int*>(out + 1), p.batch, p.n_layers, p.n_kv_heads, &s.begin, &s.end,
+                    &s.parts);
+    } else if (total > 0 && cta < s.n_active) {
+      s.begin = slice_begin(cta, s.n_active, total);
+      s.end = slice_begin(cta + 1, s.n_active, total);
+    }
+    *out = s;
+  }
+}
+
 // Which item, if any, this CTA's slice holds the first part of while a slice boundary cuts it: (layer *
 // batch + sequence, KV head, scratch slot of the first part, number of parts), no parts if there is none.
 // Written before any wait, so that the merge never reads a stale entry.
-__device__ __forceinline__ void publish_cut_item(const AttnTcParams& p, bool active, int cta, int gcta, int n_active,
-                                                 int64_t total, int64_t T0, int64_t T1, const int* prefix) {
+__device__ __forceinline__ void publish_cut_item(const AttnTcParams& p, const CtaSlice& sl, int cta, int gcta, const int* prefix) {
   int4 cut = make_int4(0, 0, 0, 0);
-  if (active && T1 < total) {
-    const Segment s = segment_at(T1 - 1, T1, prefix, p.batch, p.n_kv_heads);   // the item of the slice's last tile
+  if (sl.begin < sl.end && sl.end < sl.total) {
+    const Segment s = segment_at(sl.end - 1, sl.end, prefix, p.batch, p.n_kv_heads);   // the item of the slice's last tile
     const int64_t item_end = s.item_begin + s.item_tiles;
-    if (item_end > T1 && s.item_begin >= T0)
-      cut = make_int4(s.layer * p.batch + s.b, s.g, partial_slot(gcta, T0, s.item_begin),
-                      slice_owner(item_end - 1, n_active, total) - cta + 1);
+    if (item_end > sl.end && s.item_begin >= sl.begin)
+      cut = make_int4(s.layer * p.batch + s.b, s.g, partial_slot(gcta, sl.begin, s.item_begin),
+                      sl.parts > 0 ? sl.parts : slice_owner(item_end - 1, sl.n_active, sl.total) - cta + 1);
   }
   p.ws_cut[gcta] = cut;
 }
@@ -250,6 +304,7 @@ inline AttnTcParams slice_params(const specvlm_kv_t* kv, const void* q, int32_t 
   p.max_blocks = kv->max_blocks;
   p.block_tokens = kv->block_tokens;
   p.max_seq_len = kv->max_seq_len;
+  p.align = (int64_t)p.n_layers * batch * p.n_kv_heads <= sc.grid / n_parts && batch <= kSchedAlignedBatch;
   p.lse_block = 2 * sc.grid * p.rows;
   p.scale_log2 = sm_scale * kLog2e;
   return p;

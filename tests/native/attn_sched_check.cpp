@@ -101,22 +101,61 @@ static int check(const std::vector<int>& tiles, int n_layers, int hkv, int grid)
   return 0;
 }
 
+// Slices that keep to item boundaries: every CTA stays inside one item, an item's CTAs are consecutive and share its
+// tiles out in order, none longer than the q they were cut by.
+static int check_aligned(const std::vector<int>& tiles, int n_layers, int hkv, int grid) {
+  const int batch = (int)tiles.size();
+  std::vector<int> prefix(batch + 1, 0);
+  for (int b = 0; b < batch; ++b) prefix[b + 1] = prefix[b] + tiles[b];
+  const int64_t total = (int64_t)n_layers * hkv * prefix[batch];
+  if (total == 0) return 0;
+  const int q_first = aligned_q_first(total, grid);
+  for (int q = q_first; q <= aligned_q_last(q_first); ++q) {
+    std::vector<int> parts(batch + 1, 0);
+    for (int b = 0; b < batch; ++b) parts[b + 1] = parts[b] + (tiles[b] + q - 1) / q;
+    if ((int64_t)n_layers * hkv * parts[batch] > grid) continue;
+    int64_t f = 0;
+    int left = 0;                                            // CTAs of the current item still to come
+    for (int c = 0; c < grid; ++c) {
+      int64_t t0 = -1, t1 = -1;
+      int n = 0;
+      const bool active = aligned_slice(c, prefix.data(), parts.data(), batch, n_layers, hkv, &t0, &t1, &n);
+      if (active != (c < n_layers * hkv * parts[batch])) return 30;
+      if (!active) continue;
+      if (t0 != f || t1 <= t0 || t1 - t0 > q) return 31;     // in order, none empty, none longer than q
+      const Segment s = segment_at(t0, t1, prefix.data(), batch, hkv);
+      if (s.n_tiles != t1 - t0) return 32;                   // inside one item
+      if (n != (tiles[s.b] + q - 1) / q) return 33;
+      if ((left == 0) != (s.tile0 == 0)) return 34;
+      if (left == 0) left = n;
+      if ((--left == 0) != (s.tile0 + s.n_tiles == s.item_tiles)) return 35;
+      if (partial_slot(c, t0, s.item_begin) != 2 * c) return 36;
+      f = t1;
+    }
+    if (f != total || left != 0) return 37;
+    break;
+  }
+  return 0;
+}
+
 int main() {
   unsigned rng = 12345u;
   auto rnd = [&](int m) { rng = rng * 1664525u + 1013904223u; return (int)((rng >> 8) % (unsigned)m); };
   struct Fixed { std::vector<int> tiles; int L, H, grid; };
   const std::vector<Fixed> fixed = {
       {{101}, 80, 8, 148}, {{12}, 28, 4, 148}, {{100}, 28, 4, 148}, {{3}, 1, 1, 148}, {{1}, 1, 1, 148},
-      {{0, 5, 0, 9, 0}, 3, 2, 7}, {{785, 1}, 2, 8, 148}, {{99, 197, 295, 393}, 80, 8, 148}};
+      {{0, 5, 0, 9, 0}, 3, 2, 7}, {{51}, 1, 8, 148}, {{51, 0, 26}, 1, 8, 148}, {{101}, 4, 8, 148}, {{785, 1}, 2, 8, 148}, {{99, 197, 295, 393}, 80, 8, 148}};
   for (const Fixed& f : fixed) {
-    const int rc = check(f.tiles, f.L, f.H, f.grid);
+    int rc = check(f.tiles, f.L, f.H, f.grid);
+    if (!rc) rc = check_aligned(f.tiles, f.L, f.H, f.grid);
     if (rc) { std::printf("fixed case failed: property %d\n", rc); return 1; }
   }
   for (int iter = 0; iter < 4000; ++iter) {
     const int batch = 1 + rnd(6), L = 1 + rnd(5), H = 1 + rnd(4), grid = 1 + rnd(40);
     std::vector<int> tiles(batch);
     for (int& t : tiles) t = rnd(4) == 0 ? 0 : 1 + rnd(30);
-    const int rc = check(tiles, L, H, grid);
+    int rc = check(tiles, L, H, grid);
+    if (!rc) rc = check_aligned(tiles, L, H, iter & 1 ? grid : 8 * grid);
     if (rc) { std::printf("random case %d failed: property %d\n", iter, rc); return 1; }
   }
   std::printf("ok\n");
