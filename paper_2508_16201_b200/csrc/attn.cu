@@ -449,7 +449,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
     // ------------------------------------------------------------------ producer
     if (lane == 0) {
       SliceCursor c;
-      c.start(T0, T1, prefix, p.batch, hkv);
+      c.start(T0, T1, slice->first);
       const uint64_t policy = l2_policy_evict_first();
       const int tiles_per_block = p.block_table ? p.block_tokens / kTileTokens : 1;
       bool ok = true, told = false;
@@ -511,7 +511,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
     }
   }
   SliceCursor c;
-  c.start(T0, T1, prefix, p.batch, hkv);
+  c.start(T0, T1, slice->first);
   bool alive = true;
   int i0 = 0;                                                          // slice index of the item's first tile
   while (!c.done()) {

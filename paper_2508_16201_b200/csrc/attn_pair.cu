@@ -192,7 +192,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       const uint32_t blk_stride = is_k ? kBigTokens * 128 : kTileTokens * 128;
       const uint32_t sub_stride = is_k ? kTileTokens * 128 : SUB_BYTES;
       SliceCursor c;
-      c.start(T0, T1, prefix, p.batch, hkv);
+      c.start(T0, T1, slice->first);
       bool ok = true;
       int i = 0, n_q = 0;
       while (!c.done() && ok) {
@@ -264,7 +264,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     if (g < n_here && active) {
       const bool leader = elect_one();
       SliceCursor c;
-      c.start(T0, T1, prefix, p.batch, hkv);
+      c.start(T0, T1, slice->first);
       const uint64_t dq = umma_desc_sw128(q_sm + g * Q_BYTES, 16, 1024), dk0 = umma_desc_sw128(k_sm, 16, 1024);
       const uint64_t dv0 = umma_desc_sw128(v_sm, kTileTokens * 128, 1024);   // 64-channel blocks 8 KB apart
       const uint32_t s_tmem = tmem_base + C::COL_S + g * kBigTokens, o_tmem = tmem_base + C::COL_O + g * D;
@@ -391,8 +391,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     }
 
     SliceCursor c;
-    if (rows > 0) c.start(T0, T1, prefix, p.batch, hkv);
-    else c.start(0, 0, prefix, p.batch, hkv);     // no second part here: the group has nothing to do
+    if (rows > 0) c.start(T0, T1, slice->first);
+    else c.start(0, 0, slice->first);     // no second part here: the group has nothing to do
     bool ok = true;
     int i = 0;
 #define SM_WAIT(bar, parity)                                                        \

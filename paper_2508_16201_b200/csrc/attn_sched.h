@@ -38,38 +38,6 @@ SPECVLM_HD int slice_owner(int64_t f, int n_active, int64_t total_tiles) {
   return (int)(((f + 1) * n_active - 1) / total_tiles);
 }
 
-// Where the items are fewer than the CTAs, slices that keep to item boundaries: an item of t tiles gets ceil(t / q)
-// CTAs of its own, as equal as its tiles allow.  No CTA then works on two items, one after the other (with a few tiles a
-// CTA the second one's hand-over is as long as its tiles).  part_prefix[b] = CTAs of one KV head of the sequences < b.
-constexpr int kSchedAlignedBatch = 32;
-
-// Tiles a CTA from which to look for such a split, and up to which it is worth it.
-SPECVLM_HD int aligned_q_first(int64_t total_tiles, int grid) {
-  const int64_t q = (total_tiles + grid - 1) / grid;
-  return q > kSchedMinTilesPerCta ? (int)q : kSchedMinTilesPerCta;
-}
-SPECVLM_HD int aligned_q_last(int q_first) { return q_first + 1; }
-
-// The slice of CTA c, its item's CTAs in `parts`; false if c has no work.
-SPECVLM_HD bool aligned_slice(int c, const int* prefix, const int* part_prefix, int batch, int n_layers, int n_kv_heads,
-                              int64_t* begin, int64_t* end, int* parts) {
-  const int per_layer = n_kv_heads * part_prefix[batch];
-  if (per_layer == 0 || c >= n_layers * per_layer) return false;
-  const int layer = c / per_layer, rem = c - layer * per_layer;
-  int lo = 0, hi = batch - 1;             // last b with n_kv_heads * part_prefix[b] <= rem
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (n_kv_heads * part_prefix[mid] <= rem) lo = mid; else hi = mid - 1;
-  }
-  const int n = part_prefix[lo + 1] - part_prefix[lo], t = prefix[lo + 1] - prefix[lo];
-  const int rem2 = rem - n_kv_heads * part_prefix[lo], g = rem2 / n, part = rem2 - g * n;
-  const int64_t item = (int64_t)n_kv_heads * ((int64_t)layer * prefix[batch] + prefix[lo]) + (int64_t)g * t;
-  *begin = item + (int64_t)part * t / n;
-  *end = item + (int64_t)(part + 1) * t / n;
-  *parts = n;
-  return true;
-}
-
 struct Segment {
   int layer, b, g;        // the item
   int item;               // (layer * batch + b) * n_kv_heads + g
@@ -104,6 +72,46 @@ SPECVLM_HD Segment segment_at(int64_t f, int64_t slice_end, const int* prefix, i
   return s;
 }
 
+// Where the items are fewer than the CTAs, slices that keep to item boundaries: an item of t tiles gets ceil(t / q)
+// CTAs of its own, as equal as its tiles allow.  No CTA then works on two items, one after the other (with a few tiles a
+// CTA the second one's hand-over is as long as its tiles).  part_prefix[b] = CTAs of one KV head of the sequences < b.
+// The arithmetic is in 32 bits (it is on the way to the first tile): total < 2^31.
+constexpr int kSchedAlignedBatch = 32;
+
+// Tiles a CTA from which to look for such a split, and up to which it is worth it.
+SPECVLM_HD int aligned_q_first(int total_tiles, int grid) {
+  const int q = (int)(((uint32_t)total_tiles + (uint32_t)grid - 1u) / (uint32_t)grid);
+  return q > kSchedMinTilesPerCta ? q : kSchedMinTilesPerCta;
+}
+SPECVLM_HD int aligned_q_last(int q_first) { return q_first + 1; }
+
+// The slice of CTA c, one segment, and its item's CTAs in `parts`; false if c has no work.
+SPECVLM_HD bool aligned_slice(int c, const int* prefix, const int* part_prefix, int batch, int n_layers, int n_kv_heads,
+                              Segment* s, int* parts) {
+  const int per_layer = n_kv_heads * part_prefix[batch];
+  if (per_layer == 0 || c >= n_layers * per_layer) return false;
+  const int layer = n_layers == 1 ? 0 : (int)((uint32_t)c / (uint32_t)per_layer), rem = c - layer * per_layer;
+  int lo = 0, hi = batch - 1;             // last b with n_kv_heads * part_prefix[b] <= rem
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (n_kv_heads * part_prefix[mid] <= rem) lo = mid; else hi = mid - 1;
+  }
+  const int n = part_prefix[lo + 1] - part_prefix[lo], t = prefix[lo + 1] - prefix[lo];
+  const int rem2 = rem - n_kv_heads * part_prefix[lo], g = (int)((uint32_t)rem2 / (uint32_t)n), part = rem2 - g * n;
+  s->layer = layer;
+  s->b = lo;
+  s->g = g;
+  s->item = (layer * batch + lo) * n_kv_heads + g;
+  s->item_tiles = t;
+  s->item_begin = (int64_t)n_kv_heads * ((int64_t)layer * prefix[batch] + prefix[lo]) + (int64_t)g * t;
+  // part * t / n and (part + 1) * t / n: the first t % n parts' worth of remainders falls evenly
+  const int base = (int)((uint32_t)t / (uint32_t)n), rest = t - base * n;
+  s->tile0 = part * base + (int)((uint32_t)(part * rest) / (uint32_t)n);
+  s->n_tiles = (part + 1) * base + (int)((uint32_t)((part + 1) * rest) / (uint32_t)n) - s->tile0;
+  *parts = n;
+  return true;
+}
+
 // Scratch slot of the partial result that CTA c holds for the item starting at flat tile item_begin:
 // slot 2c when the item is the first segment of c's slice, 2c + 1 otherwise (then it is the last).
 SPECVLM_HD int partial_slot(int c, int64_t cta_slice_begin, int64_t item_begin) {
@@ -124,6 +132,14 @@ struct SliceCursor {
     j = 0;
     seg_idx = 0;
     if (f < end) sg = segment_at(f, end, prefix, batch, hkv);
+  }
+  // the same with the slice's first segment at hand
+  SPECVLM_HD void start(int64_t begin, int64_t end_, const Segment& first) {
+    f = begin;
+    end = end_;
+    j = 0;
+    seg_idx = 0;
+    sg = first;
   }
   SPECVLM_HD bool done() const { return f >= end; }
   SPECVLM_HD bool last_of_segment() const { return j == sg.n_tiles - 1; }

@@ -189,7 +189,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       const uint32_t blk_stride = is_k ? kBigTokens * 128 : kTileTokens * 128;
       const uint32_t sub_stride = is_k ? kTileTokens * 128 : SUB_BYTES;
       SliceCursor c;
-      c.start(T0, T1, prefix, p.batch, hkv);
+      c.start(T0, T1, slice->first);
       bool ok = true;
       int i = 0;
       while (!c.done() && ok) {
@@ -256,7 +256,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     if (active) {
       const bool leader = elect_one();
       SliceCursor c;
-      c.start(T0, T1, prefix, p.batch, hkv);
+      c.start(T0, T1, slice->first);
       const uint64_t dq0 = umma_desc_sw128(q_sm, 16, 1024), dk0 = umma_desc_sw128(k_sm, 16, 1024);
       bool ok = true;
       for (int i = 0; i < n_my; ++i) {
@@ -293,7 +293,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     if (active) {
       const bool leader = elect_one();
       SliceCursor c;
-      c.start(T0, T1, prefix, p.batch, hkv);
+      c.start(T0, T1, slice->first);
       const uint64_t dp0 = umma_desc_sw128(p_sm, 16, 1024);
       const uint64_t dv0 = umma_desc_sw128(v_sm, kTileTokens * 128, 1024);   // 64-channel blocks 8 KB apart
       bool ok = true;
@@ -374,7 +374,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
 
     SliceCursor c;
-    c.start(T0, T1, prefix, p.batch, hkv);
+    c.start(T0, T1, slice->first);
     bool ok = true;
     int i0 = 0;           // index (inside the slice) of the current segment's first tile
 #define SM_WAIT(bar, parity)                                                        \

@@ -179,6 +179,7 @@ __device__ __forceinline__ bool tile_prefix(const AttnTcParams& p, int* prefix, 
 // A CTA's slice of the flat tile list.
 struct CtaSlice {
   int64_t total, begin, end;   // tiles of the list; the slice (empty: the CTA has no work)
+  Segment first;               // the slice's first segment
   int n_active;                // CTAs with work, of slices of equal length
   int parts;                   // slices that keep to item boundaries: the CTAs of this one's item; 0 otherwise
   int any_empty;               // some sequence has no token
@@ -193,18 +194,20 @@ __device__ __forceinline__ void plan_slice(const AttnTcParams& p, int* prefix, C
   const int per_head = prefix[p.batch], lh = p.n_layers * p.n_kv_heads;
   const int64_t total = (int64_t)lh * per_head;
   int q = 0;
-  if (p.align && total > 0) {
-    int* const part_prefix = reinterpret_cast<int*>(out + 1);
+  int* const part_prefix = reinterpret_cast<int*>(out + 1);
+  if (p.align && total > 0 && total < 0x7fffffff) {
     const int t = lane < p.batch ? prefix[lane + 1] - prefix[lane] : 0;
-    const int q_first = aligned_q_first(total, ctas);
+    const int q_first = aligned_q_first((int)total, ctas);
     for (int c = q_first; c <= aligned_q_last(q_first) && q == 0; ++c) {
-      int n = (t + c - 1) / c;
+      int n = (int)((uint32_t)(t + c - 1) / (uint32_t)c);
+      if (p.batch > 1) {
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, n, off);
-        if (lane >= off) n += o;
+        for (int off = 1; off < 32; off <<= 1) {
+          const int o = __shfl_up_sync(0xffffffffu, n, off);
+          if (lane >= off) n += o;
+        }
       }
-      if ((int64_t)lh * __shfl_sync(0xffffffffu, n, 31) <= ctas) {
+      if ((int64_t)lh * __shfl_sync(0xffffffffu, n, p.batch - 1) <= ctas) {
         q = c;
         part_prefix[lane + 1] = n;
         if (lane == 0) part_prefix[0] = 0;
@@ -213,20 +216,29 @@ __device__ __forceinline__ void plan_slice(const AttnTcParams& p, int* prefix, C
     __syncwarp();
   }
   if (lane == 0) {
-    CtaSlice s;
-    s.total = total;
-    s.begin = s.end = 0;
-    s.n_active = sched_active_ctas(total, ctas);
-    s.parts = 0;
-    s.any_empty = empty ? 1 : 0;
+    out->total = total;
+    out->any_empty = empty ? 1 : 0;
+    int64_t begin = 0, end = 0;
+    int n_active = 1, parts = 0;
+    Segment s = {};
     if (q > 0) {
-      aligned_slice(cta, prefix, reinterpret_cast<const int*>(out + 1), p.batch, p.n_layers, p.n_kv_heads, &s.begin, &s.end,
-                    &s.parts);
-    } else if (total > 0 && cta < s.n_active) {
-      s.begin = slice_begin(cta, s.n_active, total);
-      s.end = slice_begin(cta + 1, s.n_active, total);
+      if (aligned_slice(cta, prefix, part_prefix, p.batch, p.n_layers, p.n_kv_heads, &s, &parts)) {
+        begin = s.item_begin + s.tile0;
+        end = begin + s.n_tiles;
+      }
+    } else if (total > 0) {
+      n_active = sched_active_ctas(total, ctas);
+      if (cta < n_active) {
+        begin = slice_begin(cta, n_active, total);
+        end = slice_begin(cta + 1, n_active, total);
+        s = segment_at(begin, end, prefix, p.batch, p.n_kv_heads);
+      }
     }
-    *out = s;
+    out->begin = begin;
+    out->end = end;
+    out->first = s;
+    out->n_active = n_active;
+    out->parts = parts;
   }
 }
 

@@ -109,7 +109,7 @@ static int check_aligned(const std::vector<int>& tiles, int n_layers, int hkv, i
   for (int b = 0; b < batch; ++b) prefix[b + 1] = prefix[b] + tiles[b];
   const int64_t total = (int64_t)n_layers * hkv * prefix[batch];
   if (total == 0) return 0;
-  const int q_first = aligned_q_first(total, grid);
+  const int q_first = aligned_q_first((int)total, grid);
   for (int q = q_first; q <= aligned_q_last(q_first); ++q) {
     std::vector<int> parts(batch + 1, 0);
     for (int b = 0; b < batch; ++b) parts[b + 1] = parts[b] + (tiles[b] + q - 1) / q;
@@ -117,14 +117,16 @@ static int check_aligned(const std::vector<int>& tiles, int n_layers, int hkv, i
     int64_t f = 0;
     int left = 0;                                            // CTAs of the current item still to come
     for (int c = 0; c < grid; ++c) {
-      int64_t t0 = -1, t1 = -1;
+      Segment s = {};
       int n = 0;
-      const bool active = aligned_slice(c, prefix.data(), parts.data(), batch, n_layers, hkv, &t0, &t1, &n);
+      const bool active = aligned_slice(c, prefix.data(), parts.data(), batch, n_layers, hkv, &s, &n);
       if (active != (c < n_layers * hkv * parts[batch])) return 30;
       if (!active) continue;
+      const int64_t t0 = s.item_begin + s.tile0, t1 = t0 + s.n_tiles;
       if (t0 != f || t1 <= t0 || t1 - t0 > q) return 31;     // in order, none empty, none longer than q
-      const Segment s = segment_at(t0, t1, prefix.data(), batch, hkv);
-      if (s.n_tiles != t1 - t0) return 32;                   // inside one item
+      const Segment w = segment_at(t0, t1, prefix.data(), batch, hkv);
+      if (w.layer != s.layer || w.b != s.b || w.g != s.g || w.item != s.item || w.tile0 != s.tile0 || w.n_tiles != s.n_tiles ||
+          w.item_tiles != s.item_tiles || w.item_begin != s.item_begin) return 32;   // one segment, the one that is there
       if (n != (tiles[s.b] + q - 1) / q) return 33;
       if ((left == 0) != (s.tile0 == 0)) return 34;
       if (left == 0) left = n;

@@ -72,7 +72,7 @@ def _run_attn(L, Hq, Hkv, D, seq_lens, gamma, *, paged, seed, decode_api=False, 
     return err
 
 
-@pytest.mark.parametrize("lens", [[800], [3200], [1601, 7, 900], [12000]])
+@pytest.mark.parametrize("lens", [[800], [3200], [1601, 9, 900], [12000]])
 @pytest.mark.parametrize("L,gamma", [(1, 5), (2, 8)])
 def test_verify_few_items_many_parts(L, gamma, lens):
     """Items fewer than the CTAs: slices that keep to item boundaries, and the merge that reads the whole table."""
