@@ -77,13 +77,13 @@ SPECVLM_HD Segment segment_at(int64_t f, int64_t slice_end, const int* prefix, i
 // CTA the second one's hand-over is as long as its tiles).  part_prefix[b] = CTAs of one KV head of the sequences < b.
 // The arithmetic is in 32 bits (it is on the way to the first tile): total < 2^31.
 constexpr int kSchedAlignedBatch = 32;
+constexpr int kSchedAlignedTries = 2;     // q from the smallest that could fit; more tiles a CTA are not worth it
 
-// Tiles a CTA from which to look for such a split, and up to which it is worth it.
+// Tiles a CTA from which to look for such a split.
 SPECVLM_HD int aligned_q_first(int total_tiles, int grid) {
   const int q = (int)(((uint32_t)total_tiles + (uint32_t)grid - 1u) / (uint32_t)grid);
   return q > kSchedMinTilesPerCta ? q : kSchedMinTilesPerCta;
 }
-SPECVLM_HD int aligned_q_last(int q_first) { return q_first + 1; }
 
 // The slice of CTA c, one segment, and its item's CTAs in `parts`; false if c has no work.
 SPECVLM_HD bool aligned_slice(int c, const int* prefix, const int* part_prefix, int batch, int n_layers, int n_kv_heads,

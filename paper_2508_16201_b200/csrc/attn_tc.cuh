@@ -198,8 +198,16 @@ __device__ __forceinline__ void plan_slice(const AttnTcParams& p, int* prefix, C
   if (p.align && total > 0 && total < 0x7fffffff) {
     const int t = lane < p.batch ? prefix[lane + 1] - prefix[lane] : 0;
     const int q_first = aligned_q_first((int)total, ctas);
-    for (int c = q_first; c <= aligned_q_last(q_first) && q == 0; ++c) {
-      int n = (int)((uint32_t)(t + c - 1) / (uint32_t)c);
+    int n = 0;
+#pragma unroll
+    for (int c = kSchedAlignedTries - 1; c >= 0; --c) {    // the first that fits is kept; sums of both, then one scan
+      const int m = (int)((uint32_t)(t + q_first + c - 1) / (uint32_t)(q_first + c));
+      if ((int64_t)lh * __reduce_add_sync(0xffffffffu, m) <= ctas) {
+        q = q_first + c;
+        n = m;
+      }
+    }
+    if (q > 0) {
       if (p.batch > 1) {
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -207,11 +215,8 @@ __device__ __forceinline__ void plan_slice(const AttnTcParams& p, int* prefix, C
           if (lane >= off) n += o;
         }
       }
-      if ((int64_t)lh * __shfl_sync(0xffffffffu, n, p.batch - 1) <= ctas) {
-        q = c;
-        part_prefix[lane + 1] = n;
-        if (lane == 0) part_prefix[0] = 0;
-      }
+      part_prefix[lane + 1] = n;
+      if (lane == 0) part_prefix[0] = 0;
     }
     __syncwarp();
   }

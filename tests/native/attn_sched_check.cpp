@@ -110,7 +110,7 @@ static int check_aligned(const std::vector<int>& tiles, int n_layers, int hkv, i
   const int64_t total = (int64_t)n_layers * hkv * prefix[batch];
   if (total == 0) return 0;
   const int q_first = aligned_q_first((int)total, grid);
-  for (int q = q_first; q <= aligned_q_last(q_first); ++q) {
+  for (int q = q_first; q < q_first + kSchedAlignedTries; ++q) {
     std::vector<int> parts(batch + 1, 0);
     for (int b = 0; b < batch; ++b) parts[b + 1] = parts[b] + (tiles[b] + q - 1) / q;
     if ((int64_t)n_layers * hkv * parts[batch] > grid) continue;
