@@ -447,7 +447,8 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
 
   if (warp == NW) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       SliceCursor c;
       c.start(T0, T1, slice->first);
       const uint64_t policy = l2_policy_evict_first();
@@ -456,7 +457,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
       int i = 0;
       for (; !c.done() && ok; ++i) {
         const int s = i % STAGES;
-        if (i >= STAGES) ok = mbar_wait(bar_empty + 8 * s, ((i / STAGES) - 1) & 1, abort_flag);
+        if (i >= STAGES) ok = warp_wait(bar_empty + 8 * s, ((i / STAGES) - 1) & 1, abort_flag);
         if (!ok) break;
         const int t = c.sg.tile0 + c.j;
         int blk = c.sg.b, tok = t * kTileTokens;
@@ -465,22 +466,24 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
           tok = (t % tiles_per_block) * kTileTokens;
         }
         const uint32_t full = bar_full + 8 * s, dst = base + s * STAGE_BYTES;
-        mbar_arrive_expect_tx(full, STAGE_BYTES);
+        if (leader) {
+          mbar_arrive_expect_tx(full, STAGE_BYTES);
 #pragma unroll
-        for (int h = 0; h < D / 64; ++h) {
-          tma_load_5d(dst + h * (kTileTokens * 128), &tm_k, full, h * 64, tok, c.sg.g, blk, c.sg.layer, policy);
-          tma_load_5d(dst + TILE_BYTES + h * (kTileTokens * 128), &tm_v, full, h * 64, tok, c.sg.g, blk, c.sg.layer, policy);
+          for (int h = 0; h < D / 64; ++h) {
+            tma_load_5d(dst + h * (kTileTokens * 128), &tm_k, full, h * 64, tok, c.sg.g, blk, c.sg.layer, policy);
+            tma_load_5d(dst + TILE_BYTES + h * (kTileTokens * 128), &tm_v, full, h * 64, tok, c.sg.g, blk, c.sg.layer, policy);
+          }
         }
         if (!told && i == STAGES - 1) {                     // the ring is full: time for the hand-over of a cut item
-          publish_cut_item(p, *slice, cta, cta, prefix);
+          if (leader) publish_cut_item(p, *slice, cta, cta, prefix);
           told = true;
         }
         c.next_tile(prefix, p.batch, hkv);
       }
-      if (!told) publish_cut_item(p, *slice, cta, cta, prefix);
+      if (!told && leader) publish_cut_item(p, *slice, cta, cta, prefix);
       if (!ok) {
         // a wait expired: report, then stay until this CTA's copies in flight have landed
-        if (p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
+        if (p.d_status && leader) *p.d_status = SPECVLM_ERR_TIMEOUT;
         const uint64_t t0 = global_timer_ns();
         for (int k = i > STAGES ? i - STAGES : 0; k < i; ++k)
           while (!mbar_test_wait(bar_full + 8 * (k % STAGES), (k / STAGES) & 1) && global_timer_ns() - t0 < kWaitLimitNs) {

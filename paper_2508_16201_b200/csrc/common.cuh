@@ -141,7 +141,8 @@ __device__ __forceinline__ void fence_proxy_async() {
 // issue behind `lane == 0`, 133 behind this; with operands that change from tile to tile 760 in the first form.
 // Verification, sustained, at 80 layers of 6400 tokens: a tree of 208 rows 669 -> 648 us (4310 -> 3700 cycles a
 // tile), 48 rows 360 -> 353.5; 40 layers x 4 sequences, 72 rows 1974 -> 1954.  Not in the rating passes, whose
-// issuer is never late: 32 polling lanes there cost 0.6 to 1 % at the power cap; nor for the decode kernel's copies (even).
+// issuer is never late: 32 polling lanes there cost 0.6 to 1 % at the power cap; nor for the copies of the decode kernel with a CTA per item (even), but on slices
+// (9 layers of 16 sequences, d = 64, 56.0 -> 54.9 us; 13 layers of 43 856 tokens, 16 rows, 598 -> 594).
 __device__ __forceinline__ bool elect_one() {
   uint32_t e;
   asm volatile(
