@@ -92,23 +92,32 @@ inline int32_t launch_status() {
 }
 
 // Launches `kern` so that it may be scheduled while the kernel before it in the stream still runs
-// (programmatic stream serialization).  The kernel itself has to wait (griddepcontrol.wait) for that
-// kernel's completion, in every CTA and before its first access to global memory.
+// (programmatic stream serialization), in clusters of `cluster` CTAs along x.  The kernel itself has to wait
+// (griddepcontrol.wait) for that kernel's completion, in every CTA and before its first access to global memory.
 template <typename... KArgs, typename... Args>
-inline int32_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                            const Args&... args) {
+inline int32_t launch_clusters_after(void (*kern)(KArgs...), dim3 grid, int cluster, dim3 block, size_t smem, cudaStream_t st,
+                                     const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   if (cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...) != cudaSuccess) return SPECVLM_ERR_CUDA;
   return launch_status();
+}
+template <typename... KArgs, typename... Args>
+inline int32_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                            const Args&... args) {
+  return launch_clusters_after(kern, grid, 1, block, smem, st, args...);
 }
 
 inline int sm_count() {

@@ -37,6 +37,23 @@ def test_append_bit_exact_and_lengths(paged):
         assert n == cap[b] and np.array_equal(gk[b], rk) and np.array_equal(gv[b], rv)
 
 
+@pytest.mark.parametrize("L,B,n_new", [(1, 1, 8), (1, 1, 9), (1, 2, 8), (1, 2, 9), (3, 2, 5)])
+def test_append_one_cta_or_two_launches(L, B, n_new):
+    """8 KV heads x 16 chunks a row: 1024, 1152, 2048, 2304 and 3840 chunks, on both sides of what one CTA takes."""
+    H, D = 8, 128
+    lens = [70 - 9 * b for b in range(B)]
+    cap = [n + n_new for n in lens]
+    cache, k_host, v_host = make_cache(L, H, D, cap, paged=True, seed=54)
+    cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    new_k, new_v = (synth.randn_bf16((L, B, n_new, H, D), "cuda", 55, t) for t in ("nk", "nv"))
+    specvlm.append_kv(cache, new_k, new_v)
+    assert cache.seq_lens.cpu().tolist() == cap
+    gk, gv = host_view(cache.k, cache.block_table, cap), host_view(cache.v, cache.block_table, cap)
+    for b in range(B):
+        assert np.array_equal(gk[b], oracle.append_kv(k_host[b], bits(new_k[:, b]), lens[b])[0])
+        assert np.array_equal(gv[b], oracle.append_kv(v_host[b], bits(new_v[:, b]), lens[b])[0])
+
+
 def test_append_without_room_is_reported_and_changes_nothing():
     L, H, D = 1, 2, 64
     cache, k_host, _ = make_cache(L, H, D, [20, 20], paged=False, seed=52)

@@ -263,6 +263,28 @@ def test_accept_small_exact_loop_and_ties():
     assert int(g[0, 1]) == 13 and int(g[1, 0]) == 0 and int(g[1, 3]) == 255
 
 
+@pytest.mark.parametrize("rows,vocab", [(1, 1), (1, 4096), (1, 4097), (8, 4096), (8, 4095), (9, 4096), (6, 1024), (7, 31), (5, 33)])
+def test_accept_one_cluster_or_two_launches(rows, vocab):
+    """Up to eight rows of 4096 logits go in one launch: both sides of the line, rows that start off a 16-byte boundary, ties."""
+    B = 3
+    x = torch.randn((B, rows, vocab), generator=torch.Generator().manual_seed(rows * 131 + vocab))
+    x[0, 0, vocab - 1] = x[0, 0, 0] = 9.0                             # the lower index wins
+    am = x.numpy().argmax(2)
+    drafts = am[:, :-1].astype(np.int32).copy()
+    if rows > 1:
+        drafts[1, 0] += 1                                             # rejected at once
+        drafts[2, rows // 2 - 1] += 1                                 # and in the middle
+    n, nxt, g = specvlm.accept(x.cuda(), torch.from_numpy(drafts).cuda(), want_argmax=True)
+    assert np.array_equal(g.cpu().numpy(), am)
+    want = [rows - 1, 0, 0 if rows == 1 else rows // 2 - 1]
+    assert n.cpu().tolist() == want and nxt.cpu().tolist() == [int(am[b, want[b]]) for b in range(B)]
+    par = torch.tensor([[t - 1 for t in range(rows)]] * B, dtype=torch.int32, device="cuda")     # the chain as a tree
+    tok = torch.from_numpy(np.concatenate([np.zeros((B, 1), np.int32), drafts], 1)).cuda()
+    tn, tnxt, path, tg = specvlm.accept_tree(x.cuda(), tok, par, want_argmax=True)
+    assert torch.equal(tn, n) and torch.equal(tnxt, nxt) and torch.equal(tg, g)
+    assert path.cpu().tolist() == [list(range(1, k + 1)) + [-1] * (rows - 1 - k + 1) for k in want]
+
+
 # ------------------------------------------------------------------------------- select
 def _select_case(n_frames_list, T, perm, seed, ties=False):
     rng = np.random.default_rng(seed)
