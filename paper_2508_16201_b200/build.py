@@ -1,15 +1,18 @@
-"""Build libspecvlm.so (all CUDA kernels + the C ABI) for sm_100a with nvcc, in-tree."""
+"""Build libspecvlm.so (all CUDA kernels + the C ABI) for sm_100a with nvcc, and the CPython module that calls it with
+g++, in-tree."""
 from __future__ import annotations
 
 import concurrent.futures
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libspecvlm.so")
+BINDING = os.path.join(HERE, "_binding.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "--use_fast_math", "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
@@ -54,6 +57,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if (not os.path.exists(LIB)) or any(os.path.getmtime(o) > os.path.getmtime(LIB) for o in objs):
         subprocess.run([NVCC, "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a", "-ldl"],
                        check=True)
+    src = os.path.join(CSRC, "binding.cpp")
+    if not os.path.exists(BINDING) or os.path.getmtime(BINDING) < max(os.path.getmtime(p) for p in (src, LIB)):
+        subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+                        "-I" + sysconfig.get_paths()["include"], src, "-o", BINDING, "-L" + HERE, "-l:libspecvlm.so",
+                        "-Wl,-rpath,$ORIGIN"], check=True)
     return LIB
 
 

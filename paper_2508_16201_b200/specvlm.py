@@ -1,4 +1,5 @@
-"""Thin ctypes binding over libspecvlm.so: argument marshalling only.
+"""Thin binding over libspecvlm.so: argument marshalling only (the calls that run kernels through the CPython module
+``_binding``, size queries and test hooks through ctypes).
 
 Every function has the name and the meaning of the C entry point declared in
 ``include/specvlm.h``; tensors are torch CUDA tensors whose ``data_ptr()`` is passed straight
@@ -8,7 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
-from ctypes import POINTER, byref, c_float, c_int32, c_int64, c_size_t, c_void_p
+from ctypes import POINTER, addressof, byref, c_float, c_int32, c_int64, c_size_t, c_void_p
 
 import torch
 
@@ -144,6 +145,25 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The CPython module with the entry points that run kernels (csrc/binding.cpp).  Raises if it is missing."""
+    global _native
+    if _native is None:
+        lib()
+        torch.cuda.current_device()                     # initialises CUDA, or says why it cannot
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise RuntimeError("_binding.so is missing or does not load: build it with "
+                               "`python -m paper_2508_16201_b200.build` (there is no fallback path)") from e
+        _binding.init(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        _native = _binding
+    return _native
+
+
 def version() -> str:
     return lib().specvlm_version().decode()
 
@@ -247,9 +267,9 @@ def draft_decode_attn(kv: KvCache, q: torch.Tensor, sm_scale: float, out: torch.
         out = torch.empty_like(q)
     if ws is None:
         ws = _ws(attn_workspace_bytes(kv, B, Hq, 0), q.device)
-    rc = lib().specvlm_draft_decode_attn(byref(kv.struct), _ptr(q), B, Hq, float(sm_scale), _ptr(out),
-                                         _ptr(lse), _ptr(ws), ws.numel(), _ptr(d_status), _stream())
-    _check(rc, "specvlm_draft_decode_attn")
+    rc = native().draft_decode_attn(addressof(kv.struct), q, B, Hq, float(sm_scale), out, lse, ws, ws.numel(), d_status)
+    if rc:
+        _check(rc, "specvlm_draft_decode_attn")
     return out
 
 
@@ -263,9 +283,10 @@ def verify_attn(kv: KvCache, q: torch.Tensor, gamma: int, sm_scale: float,
         out = torch.empty_like(q)
     if ws is None:
         ws = _ws(attn_workspace_bytes(kv, B, Hq, gamma), q.device)
-    rc = lib().specvlm_verify_attn(byref(kv.struct), _ptr(q), B, Hq, gamma, float(sm_scale), _ptr(out),
-                                   _ptr(lse), _ptr(ws), ws.numel(), _ptr(d_status), _stream())
-    _check(rc, "specvlm_verify_attn")
+    rc = native().verify_attn(addressof(kv.struct), q, B, Hq, gamma, float(sm_scale), out, lse, ws, ws.numel(),
+                              d_status)
+    if rc:
+        _check(rc, "specvlm_verify_attn")
     return out
 
 
@@ -289,10 +310,10 @@ def stage1_row_lse(kv: KvCache, q_text: torch.Tensor, text_cu, text_start, sm_sc
     assert q_text.is_contiguous() and q_text.dtype == torch.bfloat16 and n_text_all == text_cu[-1]
     if row_lse is None:
         row_lse = torch.empty((L, n_text_all, Hq), dtype=torch.float32, device=q_text.device)
-    rc = lib().specvlm_stage1_row_lse(byref(kv.struct), _ptr(q_text), _i32(text_cu), _i32(text_start),
-                                      len(text_start), Hq, float(sm_scale), _ptr(row_lse), _ptr(d_status),
-                                      _stream())
-    _check(rc, "specvlm_stage1_row_lse")
+    rc = native().stage1_row_lse(addressof(kv.struct), q_text, text_cu, text_start, len(text_start), Hq,
+                                 float(sm_scale), row_lse, d_status)
+    if rc:
+        _check(rc, "specvlm_stage1_row_lse")
     return row_lse
 
 
@@ -308,11 +329,10 @@ def stage1_scores(kv: KvCache, q_text: torch.Tensor, text_cu, text_start, video_
         scores = torch.empty(int(video_cu[-1]), dtype=torch.float32, device=q_text.device)
     if ws is None:
         ws = _ws(stage1_scores_workspace_bytes(kv, text_cu, video_len, Hq), q_text.device)
-    rc = lib().specvlm_stage1_scores(byref(kv.struct), _ptr(q_text), _i32(text_cu), _i32(text_start),
-                                     _i32(video_start), _i32(video_len), _i32(video_cu), batch, Hq,
-                                     float(sm_scale), _ptr(row_lse), _ptr(scores), _ptr(ws), ws.numel(),
-                                     _ptr(d_status), _stream())
-    _check(rc, "specvlm_stage1_scores")
+    rc = native().stage1_scores(addressof(kv.struct), q_text, text_cu, text_start, video_start, video_len, video_cu,
+                                batch, Hq, float(sm_scale), row_lse, scores, ws, ws.numel(), d_status)
+    if rc:
+        _check(rc, "specvlm_stage1_scores")
     return scores
 
 
@@ -326,12 +346,11 @@ def stage1_scores_layers(kv: KvCache, q_text: torch.Tensor, text_cu, text_start,
     L, n_text_all, Hq, D = q_text.shape
     batch = len(video_len)
     assert q_text.is_contiguous() and q_text.dtype == torch.bfloat16 and n_text_all == text_cu[-1]
-    rc = lib().specvlm_stage1_scores_layers(byref(kv.struct), _ptr(q_text), _i32(text_cu), _i32(text_start),
-                                            _i32(video_start), _i32(video_len), _i32(video_cu), batch, Hq,
-                                            float(sm_scale), _ptr(row_lse), _ptr(scores), _ptr(ws), ws.numel(),
-                                            int(layer_begin), int(layer_end), 1 if finish else 0,
-                                            _ptr(d_status), _stream())
-    _check(rc, "specvlm_stage1_scores_layers")
+    rc = native().stage1_scores_layers(addressof(kv.struct), q_text, text_cu, text_start, video_start, video_len,
+                                       video_cu, batch, Hq, float(sm_scale), row_lse, scores, ws, ws.numel(),
+                                       int(layer_begin), int(layer_end), 1 if finish else 0, d_status)
+    if rc:
+        _check(rc, "specvlm_stage1_scores_layers")
     return scores
 
 
@@ -342,10 +361,10 @@ def select(scores: torch.Tensor, video_cu, n_frames, tokens_per_frame: int, k_st
     assert scores.dtype == torch.float32 and scores.is_contiguous()
     if kept_idx is None:
         kept_idx = torch.empty(max(int(kept_cu[-1]), 1), dtype=torch.int32, device=scores.device)
-    rc = lib().specvlm_select(_ptr(scores), _i32(video_cu), _i32(n_frames), int(tokens_per_frame),
-                              _i32(k_stage1), _i32(k_total), _i32(kept_cu), batch, _ptr(kept_idx),
-                              _ptr(d_status), _stream())
-    _check(rc, "specvlm_select")
+    rc = native().select(scores, video_cu, n_frames, int(tokens_per_frame), k_stage1, k_total, kept_cu, batch, kept_idx,
+                         d_status)
+    if rc:
+        _check(rc, "specvlm_select")
     return kept_idx
 
 
@@ -359,10 +378,10 @@ def select_top_p(scores: torch.Tensor, video_cu, n_frames, tokens_per_frame: int
         kept_idx = torch.empty(max(int(kept_cu[-1]), 1), dtype=torch.int32, device=scores.device)
     if k_stage1_out is None:
         k_stage1_out = torch.empty(batch, dtype=torch.int32, device=scores.device)
-    rc = lib().specvlm_select_top_p(_ptr(scores), _i32(video_cu), _i32(n_frames), int(tokens_per_frame),
-                                    _i32(lambda_permille), _i32(k_total), _i32(kept_cu), batch, _ptr(kept_idx),
-                                    _ptr(k_stage1_out), _ptr(d_status), _stream())
-    _check(rc, "specvlm_select_top_p")
+    rc = native().select_top_p(scores, video_cu, n_frames, int(tokens_per_frame), lambda_permille, k_total, kept_cu,
+                               batch, kept_idx, k_stage1_out, d_status)
+    if rc:
+        _check(rc, "specvlm_select_top_p")
     return kept_idx, k_stage1_out
 
 
@@ -388,10 +407,10 @@ def gather_kv(src: KvCache, kept_idx: torch.Tensor, kept_cu, video_start, video_
               dst: KvCache, d_status: torch.Tensor | None = None) -> None:
     batch = len(video_len)
     assert kept_idx.dtype == torch.int32
-    rc = lib().specvlm_gather_kv(byref(src.struct), _ptr(kept_idx), _i32(kept_cu), _i32(video_start),
-                                 _i32(video_len), _i32(src_len), batch, byref(dst.struct), _ptr(d_status),
-                                 _stream())
-    _check(rc, "specvlm_gather_kv")
+    rc = native().gather_kv(addressof(src.struct), kept_idx, kept_cu, video_start, video_len, src_len, batch,
+                            addressof(dst.struct), d_status)
+    if rc:
+        _check(rc, "specvlm_gather_kv")
 
 
 # ---------------------------------------------------------------------------------- cache maintenance
@@ -399,17 +418,17 @@ def append_kv(kv: KvCache, new_k: torch.Tensor, new_v: torch.Tensor, d_status: t
     """new_k / new_v: bf16 [n_layers][batch][n_new][n_kv_heads][head_dim]; kv.seq_lens is updated."""
     assert new_k.dtype == torch.bfloat16 and new_k.is_contiguous() and new_v.is_contiguous()
     assert new_k.shape == new_v.shape and new_k.dim() == 5
-    rc = lib().specvlm_append_kv(byref(kv.struct), _ptr(new_k), _ptr(new_v), new_k.shape[1], new_k.shape[2],
-                                 _ptr(kv.seq_lens), _ptr(d_status), _stream())
-    _check(rc, "specvlm_append_kv")
+    rc = native().append_kv(addressof(kv.struct), new_k, new_v, new_k.shape[1], new_k.shape[2], kv.seq_lens, d_status)
+    if rc:
+        _check(rc, "specvlm_append_kv")
 
 
 def rollback_kv(seq_lens: torch.Tensor, accept_len: torch.Tensor, gamma: int,
                 d_status: torch.Tensor | None = None) -> None:
     assert seq_lens.dtype == torch.int32 and accept_len.dtype == torch.int32
-    rc = lib().specvlm_rollback_kv(_ptr(seq_lens), _ptr(accept_len), seq_lens.numel(), int(gamma), _ptr(d_status),
-                                   _stream())
-    _check(rc, "specvlm_rollback_kv")
+    rc = native().rollback_kv(seq_lens, accept_len, seq_lens.numel(), int(gamma), d_status)
+    if rc:
+        _check(rc, "specvlm_rollback_kv")
 
 
 # ---------------------------------------------------------------------------------- tree drafting
@@ -424,9 +443,10 @@ def verify_tree_attn(kv: KvCache, q: torch.Tensor, parents: torch.Tensor, sm_sca
         out = torch.empty_like(q)
     if ws is None:
         ws = _ws(int(lib().specvlm_verify_tree_workspace_bytes(byref(kv.struct), B, Hq, N)), q.device)
-    rc = lib().specvlm_verify_tree_attn(byref(kv.struct), _ptr(q), _ptr(parents), B, Hq, N, float(sm_scale),
-                                        _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), _ptr(d_status), _stream())
-    _check(rc, "specvlm_verify_tree_attn")
+    rc = native().verify_tree_attn(addressof(kv.struct), q, parents, B, Hq, N, float(sm_scale), out, lse, ws,
+                                   ws.numel(), d_status)
+    if rc:
+        _check(rc, "specvlm_verify_tree_attn")
     return out
 
 
@@ -448,9 +468,9 @@ def accept_tree(target_logits: torch.Tensor, node_tokens: torch.Tensor, parents:
     assert node_tokens.dtype == torch.int32 and parents.dtype == torch.int32
     dev = target_logits.device
     n, nxt, path, g, ws = out if out is not None else accept_tree_buffers(B, N, V, dev, want_argmax)
-    rc = lib().specvlm_accept_tree(_ptr(target_logits), _ptr(node_tokens), _ptr(parents), B, N, V, _ptr(n), _ptr(nxt),
-                                   _ptr(path), _ptr(g), _ptr(ws), ws.numel(), _stream())
-    _check(rc, "specvlm_accept_tree")
+    rc = native().accept_tree(target_logits, node_tokens, parents, B, N, V, n, nxt, path, g, ws, ws.numel())
+    if rc:
+        _check(rc, "specvlm_accept_tree")
     return n, nxt, path, g
 
 
@@ -487,9 +507,9 @@ def compact_tree_kv(kv: KvCache, path: torch.Tensor, accept_len: torch.Tensor,
                     d_status: torch.Tensor | None = None) -> None:
     """Moves the accepted nodes' rows behind the root and shortens kv.seq_lens accordingly."""
     B, N = path.shape
-    rc = lib().specvlm_compact_tree_kv(byref(kv.struct), _ptr(path), _ptr(accept_len), B, N, _ptr(kv.seq_lens),
-                                       _ptr(d_status), _stream())
-    _check(rc, "specvlm_compact_tree_kv")
+    rc = native().compact_tree_kv(addressof(kv.struct), path, accept_len, B, N, kv.seq_lens, d_status)
+    if rc:
+        _check(rc, "specvlm_compact_tree_kv")
 
 
 # ---------------------------------------------------------------------------------- accept
@@ -514,9 +534,9 @@ def accept(target_logits: torch.Tensor, draft_tokens: torch.Tensor, want_argmax:
         accept_len, next_token, g = out
     if ws is None:
         ws = _ws(accept_workspace_bytes(B, gamma, V), dev)
-    rc = lib().specvlm_accept(_ptr(target_logits), _ptr(draft_tokens), B, gamma, V, _ptr(accept_len),
-                              _ptr(next_token), _ptr(g), _ptr(ws), ws.numel(), _stream())
-    _check(rc, "specvlm_accept")
+    rc = native().accept(target_logits, draft_tokens, B, gamma, V, accept_len, next_token, g, ws, ws.numel())
+    if rc:
+        _check(rc, "specvlm_accept")
     return accept_len, next_token, g
 
 

@@ -139,3 +139,33 @@ def test_kernels_with_tensor_memory_release_their_successor_after_the_allocation
                 # up to the kernel's end: the first line that is a closing brace alone
                 assert "pdl_launch_next()" not in kernel[:kernel.index("\n}\n")], (f, kernel[:80])
     assert seen == 4
+
+
+def test_binding_takes_what_ctypes_took():
+    """The CPython module: device pointers as tensors, addresses or None, host arrays as any sequence, integers modulo
+    2^32; a wrong number or type of arguments is refused.  Every call here is one that the library rejects on the host."""
+    import numpy as np
+    import torch
+    from paper_2508_16201_b200 import _binding
+    bad = specvlm.ERR_INVALID_ARG
+    _binding.init(lambda: 0, lambda device: 0)
+    try:
+        kv = specvlm.KvStruct()
+        assert _binding.draft_decode_attn(ctypes.addressof(kv), None, 1, 4, 0.1, None, None, None, 0, None) == bad
+        t = torch.zeros(16)
+        for one, cu in (([5], [0, 10]), ((5,), (0, 10)), (np.array([5]), torch.tensor([0, 10])), ([5.0], ["0", 10])):
+            # k_stage1 = 5 > k_total = 3
+            assert _binding.select(t, cu, [2], 5, one, [3], [0, 3], 1, t, None) == bad
+        many = list(range(1, 200))                             # longer than the array on the stack
+        assert _binding.select(t, [0] + many, many, 1, [5] * 199, [3] * 199, [0] + many, 199, t, None) == bad
+        assert _binding.rollback_kv(t, t, 1, -1, None) == bad   # gamma < 0
+        assert _binding.rollback_kv(t, t, 1, (1 << 32) - 1, None) == bad
+        for call, args in ((_binding.rollback_kv, (t, t, 1)), (_binding.rollback_kv, (t, t, 1.5, 0, None)),
+                           (_binding.select, (t, 7, [2], 5, [5], [3], [0, 3], 1, t, None)),
+                           (_binding.select, (t, None, [2], 5, [5], [3], [0, 3], 1, t, None))):
+            with pytest.raises(TypeError):
+                call(*args)
+        with pytest.raises(AttributeError):
+            _binding.rollback_kv("no tensor", t, 1, 0, None)
+    finally:
+        _binding.init(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
