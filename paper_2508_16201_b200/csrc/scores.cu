@@ -571,8 +571,19 @@ __global__ void scores_finish_kernel(const __grid_constant__ ScoreParams p, floa
   if (j >= p.sum_video) return;
   int b = 0;
   while (b + 1 < p.batch && p.seq[b + 1].score_off <= j) ++b;
+  // sixteen layers' loads in flight: with the compiler's four a thread of 80 layers waited twenty times for L2
+  constexpr int kFlight = 16;
   float acc = 0.f;
-  for (int l = 0; l < p.n_layers; ++l) acc += p.partial[(size_t)l * p.sum_video + j];
+  const float* const part = p.partial + j;
+  int l = 0;
+  for (; l + kFlight <= p.n_layers; l += kFlight) {
+    float x[kFlight];
+#pragma unroll
+    for (int u = 0; u < kFlight; ++u) x[u] = part[(size_t)(l + u) * p.sum_video];
+#pragma unroll
+    for (int u = 0; u < kFlight; ++u) acc += x[u];
+  }
+  for (; l < p.n_layers; ++l) acc += part[(size_t)l * p.sum_video];
   scores[j] = acc / ((float)p.n_layers * (float)p.n_q_heads * (float)p.seq[b].n_text);
 }
 
