@@ -207,13 +207,28 @@ __device__ __forceinline__ void store_bf16x4(__nv_bfloat16* dst, const float4& v
   *reinterpret_cast<uint2*>(dst) = packed;
 }
 
+constexpr int kMaxRows16Cluster = 8;       // the portable cluster size
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
 // ---------------------------------------------------------------------------------------------
 // One CTA per item.  4 consumer warps each own 16 of a tile's 64 tokens; they are merged once at the end.
 // The last warp is the TMA producer.
 // ---------------------------------------------------------------------------------------------
 // NG consumer groups of 4 warps take alternate tiles (NG = 2 where an SM holds a single CTA, so
 // that eight warps hide each other's latencies as two resident CTAs would).
-template <int D, int STAGES, int NG>
+// SPLIT: a cluster of gridDim.x CTAs per item, CTA r on tiles r, r + gridDim.x, ..; their results meet over distributed
+// shared memory, each CTA folding its share of the output positions.  For a few short items, whose tiles one CTA would
+// work through one after the other at 0.35 us each.
+template <int D, int STAGES, int NG, bool SPLIT>
 __global__ void __launch_bounds__(32 * (4 * NG + 1))
 attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                    const AttnParams p) {
@@ -237,6 +252,7 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = blockIdx.y, lb = blockIdx.z;
   const int layer = lb / p.batch, b = lb - layer * p.batch;
+  const int rank = SPLIT ? (int)blockIdx.x : 0, n_cta = SPLIT ? (int)gridDim.x : 1;
 
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -263,13 +279,14 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     mbar_arrive_expect_tx(bar_full, STAGE_BYTES);
 #pragma unroll
     for (int h = 0; h < D / 64; ++h) {
-      tma_load_5d(base + h * (kTileTokens * 128), &tm_k, bar_full, h * 64, 0, g, b, layer, policy);
-      tma_load_5d(base + TILE_BYTES + h * (kTileTokens * 128), &tm_v, bar_full, h * 64, 0, g, b, layer, policy);
+      tma_load_5d(base + h * (kTileTokens * 128), &tm_k, bar_full, h * 64, rank * kTileTokens, g, b, layer, policy);
+      tma_load_5d(base + TILE_BYTES + h * (kTileTokens * 128), &tm_v, bar_full, h * 64, rank * kTileTokens, g, b, layer, policy);
     }
   }
 
   const int kv_len = clamp_len(p.seq_lens[b], p.max_seq_len);
-  const int n_my = (kv_len + kTileTokens - 1) / kTileTokens;
+  const int n_all = (kv_len + kTileTokens - 1) / kTileTokens;
+  const int n_my = SPLIT ? (n_all + n_cta - 1 - rank) / n_cta : n_all;
 
   if (warp == 4 * NG) {
     // ------------------------------------------------------------------ producer
@@ -288,13 +305,14 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         const int s = i % STAGES;
         if (i >= STAGES) ok = mbar_wait(bar_empty + 8 * s, ((i / STAGES) - 1) & 1, abort_flag);
         if (!ok) break;
+        const int t = i * n_cta + rank;
         int blk, tok;
         if (p.block_table) {
-          blk = p.block_table[(size_t)b * p.max_blocks + i / tiles_per_block];
-          tok = (i % tiles_per_block) * kTileTokens;
+          blk = p.block_table[(size_t)b * p.max_blocks + t / tiles_per_block];
+          tok = (t % tiles_per_block) * kTileTokens;
         } else {
           blk = b;
-          tok = i * kTileTokens;
+          tok = t * kTileTokens;
         }
         const uint32_t full = bar_full + 8 * s;
         mbar_arrive_expect_tx(full, STAGE_BYTES);
@@ -323,7 +341,8 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   }
 
   // -------------------------------------------------------------------- consumers
-  if (n_my == 0) {
+  if (n_all == 0) {
+    if (rank != 0) return;
     // An empty sequence: its outputs are zero, its LSE -inf.  The ring stays untouched: the tile that the producer
     // asked for before it knew the length may still be landing there, with whatever the cache rows hold.
     for (int idx = tid; idx < p.rows * (D / 8); idx += 128 * NG) {
@@ -339,6 +358,8 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   Rows16<D> st;
   st.start(p, p.n_q, p.rows, lb, g, kv_len, lane);
   bool alive = true;
+  // a CTA without a tile of its own: the one asked for before the length was known lands where the merge buffer will be
+  if (SPLIT && n_my == 0 && spec && !mbar_wait(bar_full, 0, abort_flag)) alive = false;
   for (int i = grp; i < n_my; i += NG) {
     const int s = i % STAGES;
     if (!mbar_wait(bar_full + 8 * s, (i / STAGES) & 1, abort_flag)) {
@@ -346,7 +367,8 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       break;
     }
     const uint32_t k_base = base + s * STAGE_BYTES;
-    st.tile(k_base, k_base + TILE_BYTES, smem + s * STAGE_BYTES + TILE_BYTES, i * kTileTokens, kv_len, p.scale_log2, cw, lane);
+    st.tile(k_base, k_base + TILE_BYTES, smem + s * STAGE_BYTES + TILE_BYTES, (i * n_cta + rank) * kTileTokens, kv_len,
+            p.scale_log2, cw, lane);
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_empty + 8 * s);
   }
@@ -354,13 +376,66 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   // ------------------------------------------------------------ merge the consumer warps' partials
   // (named barrier over the consumer threads; the producer warp has no part in it)
   asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
-  if (!alive || *abort_flag) return;   // a wait expired somewhere in this CTA: leave outputs alone
+  const bool gave_up = !alive || *abort_flag;   // a wait expired somewhere in this CTA (the flag tells all of it)
+  if (!SPLIT && gave_up) return;       // leave outputs alone
   constexpr int NW = 4 * NG;                                           // consumer warps
   float* const o_sm = reinterpret_cast<float*>(smem);                  // [NW][16][OPITCH]
   float* const m_sm = o_sm + NW * 16 * OPITCH;                         // [NW][16]
   float* const l_sm = m_sm + NW * 16;                                  // [NW][16]
   st.publish(o_sm, m_sm, l_sm, p.rows, warp, lane);
   asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
+  if constexpr (SPLIT) {
+    // this CTA's result, normalised, and its log-sum-exps: behind the merge buffer, for the whole cluster to read
+    float* const part_o = l_sm + NW * 16;                              // [16][D]
+    float* const part_lse = part_o + 16 * D;                           // [16]
+    for (int idx = tid; idx < p.rows * (D / 4); idx += 128 * NG) {
+      const int r = idx / (D / 4), c = (idx - r * (D / 4)) * 4;
+      float4 acc;
+      const float lse2 = rows16_merge<D, NW>(o_sm, m_sm, l_sm, r, c, acc);
+      *reinterpret_cast<float4*>(part_o + r * D + c) = acc;
+      if (c == 0) part_lse[r] = gave_up ? __uint_as_float(kUnwritten) : lse2;
+    }
+    cluster_barrier();
+    for (int idx = rank * 128 * NG + tid; idx < p.rows * (D / 4); idx += n_cta * 128 * NG) {
+      const int r = idx / (D / 4), c = (idx - r * (D / 4)) * 4;
+      float lse[kMaxRows16Cluster];
+      float4 x[kMaxRows16Cluster];
+#pragma unroll
+      for (int k = 0; k < kMaxRows16Cluster; ++k) {
+        lse[k] = -INFINITY;
+        x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k < n_cta) {
+          lse[k] = ld_cluster_f32(cluster_map(smem_u32(part_lse + r), k));
+          x[k] = ld_cluster_f32x4(cluster_map(smem_u32(part_o + r * D + c), k));
+        }
+      }
+      float mm = -INFINITY, den = 0.f;
+      bool lost = false;
+#pragma unroll
+      for (int k = 0; k < kMaxRows16Cluster; ++k) {
+        lost |= unwritten(lse[k]);
+        mm = fmaxf(mm, lse[k]);
+      }
+      if (lost) continue;                                              // a part is missing: leave the row alone
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < kMaxRows16Cluster; ++k) {
+        const float w = lse[k] == -INFINITY ? 0.f : fast_exp2(lse[k] - mm);
+        acc.x += w * x[k].x;
+        acc.y += w * x[k].y;
+        acc.z += w * x[k].z;
+        acc.w += w * x[k].w;
+        den += w;
+      }
+      const float inv = den > 0.f ? 1.f / den : 0.f;
+      const int t = r / p.group, h = g * p.group + (r - t * p.group);
+      const size_t orow = ((size_t)lb * p.n_q + t) * p.n_q_heads + h;
+      store_bf16x4(p.out + orow * D + c, make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+      if (p.lse && c == 0) p.lse[orow] = den > 0.f ? (mm + log2f(den)) * kLn2 : -INFINITY;
+    }
+    cluster_barrier();                                                 // nobody reads this CTA's shared memory any more
+    return;
+  }
   for (int idx = tid; idx < p.rows * (D / 4); idx += 128 * NG) {
     const int r = idx / (D / 4), c = (idx - r * (D / 4)) * 4;
     float4 acc;
@@ -573,7 +648,31 @@ static std::atomic<int> g_forced_splits{0};
 
 constexpr int kRows16Max = 16;     // windows up to this many rows run on the 16-row kernels
 
-// CTAs of a launch on slices, or 0 for a CTA per item.
+// Time that one CTA takes for a tile, us.
+static double rows16_tile_us(const specvlm_kv_t* kv) {
+  return (kv->head_dim == 128 ? 0.35 : 0.25) * (kv->block_table ? 1.25 : 1.0);
+}
+
+// CTAs per item of a launch without slices: the number that is the fastest where every CTA has an SM of its own.  The
+// hand-over costs 1.3 us: one layer of 4 items of 200 tokens 3.7 us with a CTA each, 4.3 with two; of 755 / 1600 / 3200
+// tokens 6.5 / 9.1 / 16 with one (7.4 / 8.3 on slices from 1600) and 4.4 / 5.0 / 6.3 with eight.  Clusters do not use
+// every SM of a GPC: 16 of eight CTAs no longer run side by side (4 layers of 800 tokens 7.3 -> 8.4), 24 of four do (2 layers
+// x 3 sequences of 800 tokens 8.0 -> 5.4).
+static int rows16_cluster(const specvlm_kv_t* kv, int64_t items, int64_t tiles) {
+  if (g_forced_splits.load(std::memory_order_relaxed) == 1) return 1;
+  int best = 1;
+  double best_us = rows16_tile_us(kv) * tiles;
+  for (int n = 2; n <= kMaxRows16Cluster; n *= 2) {
+    const double us = 1.3 + rows16_tile_us(kv) * ((tiles + n - 1) / n);
+    if (items * n <= (n == 2 ? 144 : n == 4 ? 96 : 64) && us < best_us) {
+      best = n;
+      best_us = us;
+    }
+  }
+  return best;
+}
+
+// CTAs of a launch on slices, or 0 for a CTA (or a cluster) per item.
 static int rows16_slices(const specvlm_kv_t* kv, int32_t batch) {
   const int64_t items = (int64_t)kv->n_layers * batch * kv->n_kv_heads;
   const int64_t tiles = (kv->max_seq_len + kTileTokens - 1) / kTileTokens, sms = sm_count();
@@ -593,10 +692,19 @@ static int rows16_slices(const specvlm_kv_t* kv, int32_t batch) {
   // 755 / 6400 / 50 000 tokens 9.6 / 55.4 / 405 against 15.5 / 59.3 / 399; 28 layers x 4 ragged paged sequences of up to
   // 755 / 6400 / 25 600 tokens 22.4 / 152 / 600 against 31.0 / 142 / 531.
   const double hbm = (double)items * tiles * (256.0 * kv->head_dim) / 6.65e6;
-  const double tile_us = (kv->head_dim == 128 ? 0.35 : 0.25) * (kv->block_table ? 1.25 : 1.0);
+  const double tile_us = rows16_tile_us(kv);
   const double ragged = batch > 1 ? 0.85 : 1.0;
   double per_item;
-  if (items <= sms) {
+  const int n = rows16_cluster(kv, items, tiles);
+  bool on_slices;
+  if (n > 1) {
+    // A cluster per item against slices that mostly keep to item boundaries (their merge folds many parts of few items).
+    // 4 items of 6400 / 12 800 tokens 8.6 / 12.7 us against 10.1 / 12.8; 24 ragged paged ones of up to 3200 / 6400 / 12 800
+    // 10.0 / 16.0 / 31.0 against 10.6 / 14.0 / 23.5: with two thirds of the SMs busy the longest item's CTAs slow down.
+    const double longest = tile_us * ((tiles + n - 1) / n), even = (double)(items * tiles < sms ? items * tiles : sms);
+    per_item = 3.9 + (longest > hbm ? longest : hbm) * (items * n > 64 ? 1.2 : 1.0);
+    on_slices = 6.0 + ragged * hbm + 0.04 * even / items + 0.5 < per_item;
+  } else if (items <= sms) {
     const double longest = tile_us * tiles;
     per_item = 3.0 + (longest > hbm ? longest : hbm);
   } else {
@@ -604,8 +712,8 @@ static int rows16_slices(const specvlm_kv_t* kv, int32_t batch) {
     const double stream = (1.0 + 0.2 / rounds) * ragged * hbm, serial = rounds * tiles * 0.75 * kv->head_dim / 128;
     per_item = 3.0 + (stream > serial ? stream : serial);
   }
-  const double slices = 4.5 + ragged * hbm + 2.0 * (1.0 + (double)items / sms);
-  if (slices + 1.5 >= per_item) return 0;
+  if (n == 1) on_slices = 4.5 + ragged * hbm + 2.0 * (1.0 + (double)items / sms) + 1.5 < per_item;
+  if (!on_slices) return 0;
   const int even = sched_active_ctas(items * tiles, (int)sms);
   // slices that keep to item boundaries may use more CTAs: every item rounds its own up
   const int64_t aligned = items * sched_active_ctas(tiles, (int)sms);
@@ -624,14 +732,14 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
                        float sm_scale, void* out, float* lse, void* ws, size_t ws_bytes, int32_t* d_status,
                        cudaStream_t st, const int32_t* tree_parents);
 
-template <int D, int STAGES, int NG>
+template <int D, int STAGES, int NG, bool SPLIT>
 static int32_t launch_rows16_s(const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& p,
                                dim3 grid, cudaStream_t st) {
   constexpr int SMEM = STAGES * 2 * kTileTokens * D * 2 + 1024 + 16 * STAGES + 16;
-  auto kern = attn_rows16_kernel<D, STAGES, NG>;
+  auto kern = attn_rows16_kernel<D, STAGES, NG, SPLIT>;
   static std::atomic<uint64_t> attr_done{0};
   if (!smem_attr_once(attr_done, reinterpret_cast<const void*>(kern), SMEM)) return SPECVLM_ERR_CUDA;
-  return launch_after(kern, grid, dim3(32 * (4 * NG + 1)), (size_t)SMEM, st, tk, tv, p);
+  return launch_clusters_after(kern, grid, (int)grid.x, dim3(32 * (4 * NG + 1)), (size_t)SMEM, st, tk, tv, p);
 }
 
 // Ring depth: 3 stages let two CTAs share an SM; a launch with no more CTAs than SMs would leave
@@ -642,8 +750,9 @@ static int32_t launch_rows16(const CUtensorMap& tk, const CUtensorMap& tv, const
                              dim3 grid, cudaStream_t st) {
   const int64_t ctas = (int64_t)grid.x * grid.y * grid.z;
   constexpr int kDeep = D == 128 ? 6 : 12;
-  return ctas <= sm_count() ? launch_rows16_s<D, kDeep, 2>(tk, tv, p, grid, st)
-                            : launch_rows16_s<D, 3, 1>(tk, tv, p, grid, st);
+  if (grid.x > 1) return launch_rows16_s<D, kDeep, 2, true>(tk, tv, p, grid, st);
+  return ctas <= sm_count() ? launch_rows16_s<D, kDeep, 2, false>(tk, tv, p, grid, st)
+                            : launch_rows16_s<D, 3, 1, false>(tk, tv, p, grid, st);
 }
 
 template <int D>
@@ -712,7 +821,8 @@ static int32_t attn_common(const specvlm_kv_t* kv, const void* q, int32_t batch,
   p.max_seq_len = kv->max_seq_len;
   p.scale_log2 = sm_scale * kLog2e;
 
-  dim3 grid(1, (unsigned)kv->n_kv_heads, (unsigned)lb64);
+  const int n = rows16_cluster(kv, lb64 * kv->n_kv_heads, (kv->max_seq_len + kTileTokens - 1) / kTileTokens);
+  dim3 grid((unsigned)n, (unsigned)kv->n_kv_heads, (unsigned)lb64);
   return kv->head_dim == 128 ? launch_rows16<128>(tk, tv, p, grid, st) : launch_rows16<64>(tk, tv, p, grid, st);
 }
 

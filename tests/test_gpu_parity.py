@@ -105,6 +105,30 @@ def test_decode_ragged_batch_paged_poisoned():
 
 
 @pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("lens", [[513], [450, 400], [1500], [700, 64, 1, 200], [577] * 18])
+def test_decode_with_a_cluster_per_item(lens, paged, D):
+    """Clusters of two to eight CTAs per item: tiles that the CTAs share unevenly, CTAs without a tile (the contiguous
+    cache asks for one before the length is known), NaN past every end."""
+    _run_attn(1, 28, 4, D, lens, 0, paged=paged, seed=70 + len(lens), decode_api=True, poison=True)
+
+
+def test_decode_with_a_cluster_per_item_and_an_empty_sequence():
+    from gpu_util import make_cache
+    lens = [1000, 0, 70]
+    cache, k, v = make_cache(1, 4, 128, [max(n, 1) for n in lens], paged=False, seed=71)
+    cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    cache.k[:, 1], cache.v[:, 1] = float("nan"), float("nan")
+    q = synth.randn_bf16((1, 3, 28, 128), "cuda", 71, "Q")
+    lse = torch.zeros((1, 3, 28), dtype=torch.float32, device="cuda")
+    out = f64(specvlm.draft_decode_attn(cache, q, 0.1, lse=lse))
+    assert (out[0, 1] == 0).all() and torch.isneginf(lse[0, 1]).all()
+    for b in (0, 2):
+        ref, _ = oracle.attention(bits(q)[0, b][None], k[b][0], v[b][0], lens[b], 0.1)
+        assert row_rel_err(out[0, b], ref[0]) <= ATTN_TOL
+
+
+@pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("lens", [[1], [64, 0, 65], [0, 0], [3, 1000, 63, 130], [2111], [257] * 40])
 def test_decode_on_slices(lens, D):
     """The slice kernel at every kind of slice: one tile, empty sequences between others, all empty, items cut
