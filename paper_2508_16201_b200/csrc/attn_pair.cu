@@ -22,8 +22,9 @@
 // per KV head, 80 layers of 6400 tokens (each part used to stream K and V on a set of CTAs of its own): 642 ->
 // 554 us, 827 -> 677 us under sustained load at the power cap.  What it took, same case: the parts in step
 // (both softmaxes, then both waiting for the tensor pipe) 684 us; taking turns 610; the next S issued before
-// the bookkeeping commits, waits that test before they suspend, and P handed over in two halves 554.  A
-// share of the exponentials on the FMA pipe is slower (2 / 4 of 16 pairs: 571 / 604 us).
+// the bookkeeping commits, waits that test before they suspend, and P handed over in two halves 554; products issued by an
+// elected lane of a whole warp instead of by lane 0 (of 4310 cycles a tile the issuers took 2750) 3700 cycles, sustained
+// 669 -> 648 us.  A share of the exponentials on the FMA pipe is slower (2 / 4 of 16 pairs: 571 / 604 us).
 #include "attn_tc.cuh"
 
 namespace specvlm {
