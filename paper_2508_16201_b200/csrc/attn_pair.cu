@@ -381,6 +381,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       for (int item = cta; item < n_items; item += ctas) {
         const int lb = item / hkv, kvh = item - lb * hkv, b = lb % p.batch;
         if (prefix[b + 1] != prefix[b]) continue;
+        if constexpr (TREE) check_tree(p.parents + (size_t)b * p.n_win, p.n_win, lane, p.d_status);
         for (int idx = my_row; idx < rows * (D / 8); idx += 128) {
           const int r = idx / (D / 8), c8 = idx - r * (D / 8);
           const int t = r / p.group, h = kvh * p.group + (r - t * p.group);
@@ -421,7 +422,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       const int win0 = kv_len - p.n_win;
       uint64_t my_a;
       if constexpr (TREE) {
-        my_a = row_on ? __ldcg(p.anc + (size_t)sg.b * p.n_win + q0 + my_t) : 0ull;
+        const uint64_t a = tree_mask(p.parents + (size_t)sg.b * p.n_win, p.n_win, row_on ? q0 + my_t : 0, p.d_status);
+        my_a = row_on ? a : 0ull;
       } else {
         my_a = row_on ? (uint64_t)(win0 + q0 + my_t + 1) : 0ull;
       }
@@ -592,8 +594,8 @@ static int32_t launch_pair_t(const CUtensorMap& tk, const CUtensorMap& tv, const
 int32_t attn_pair_launch(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const AttnTcParams& p,
                          int head_dim, int grid, cudaStream_t st) {
   if (head_dim == 128)
-    return p.anc ? launch_pair_t<128, true>(tk, tv, tq, p, grid, st) : launch_pair_t<128, false>(tk, tv, tq, p, grid, st);
-  return p.anc ? launch_pair_t<64, true>(tk, tv, tq, p, grid, st) : launch_pair_t<64, false>(tk, tv, tq, p, grid, st);
+    return p.parents ? launch_pair_t<128, true>(tk, tv, tq, p, grid, st) : launch_pair_t<128, false>(tk, tv, tq, p, grid, st);
+  return p.parents ? launch_pair_t<64, true>(tk, tv, tq, p, grid, st) : launch_pair_t<64, false>(tk, tv, tq, p, grid, st);
 }
 
 }  // namespace specvlm

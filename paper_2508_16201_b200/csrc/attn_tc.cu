@@ -363,6 +363,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       for (int item = cta; item < n_items; item += (int)gridDim.x) {
         const int lb = item / hkv, g = item - lb * hkv, b = lb % p.batch;
         if (prefix[b + 1] != prefix[b]) continue;
+        if constexpr (TREE) check_tree(p.parents + (size_t)b * p.n_win, p.n_win, lane, p.d_status);
         for (int idx = st; idx < rows * (D / 8); idx += 256) {
           const int r = idx / (D / 8), c8 = idx - r * (D / 8);
           const int t = r / p.group, h = g * p.group + (r - t * p.group);
@@ -404,7 +405,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const bool warp_on = rows > 32 * quarter;         // warp-uniform: some row of this quadrant is in use
         uint64_t my_a;                                       // the row's window mask (tree) or key limit (chain)
         if constexpr (TREE) {
-          my_a = my_row < rows ? __ldcg(p.anc + (size_t)sg.b * p.n_win + my_row / p.group) : 0ull;
+          const uint64_t a = tree_mask(p.parents + (size_t)sg.b * p.n_win, p.n_win, my_row < rows ? my_row / p.group : 0, p.d_status);
+          my_a = my_row < rows ? a : 0ull;
         } else {
           my_a = my_row < rows ? (uint64_t)(win0 + my_row / p.group + 1) : 0ull;
         }
@@ -552,7 +554,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           const int r = row0(h) + lr + 8 * e;
           const int t = r / p.group;
           if constexpr (TREE) {
-            vis[h][e] = r < rows ? __ldcg(p.anc + (size_t)sg.b * p.n_win + t) : 0ull;
+            const uint64_t a = tree_mask(p.parents + (size_t)sg.b * p.n_win, p.n_win, r < rows ? t : 0, p.d_status);
+            vis[h][e] = r < rows ? a : 0ull;
           } else {
             lim[h][e] = r < rows ? win0 + t + 1 : 0;
           }
@@ -1007,36 +1010,6 @@ static int32_t launch_merge(const AttnTcParams& p, int ctas, cudaStream_t st) {
                       st, p, grid);
 }
 
-// Ancestor masks of a draft tree: bit w of anc[b][t] says that node t attends window position w
-// (itself and the nodes on its path to a root).  parents[b][t] < t, -1 for a root.
-__global__ void tree_ancestors_kernel(const int32_t* parents, int n, int n_nodes,
-                                      uint64_t* __restrict__ anc, int32_t* d_status) {
-  pdl_launch_next();
-  pdl_wait();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int t = i % n_nodes;
-  const int32_t* par = parents + (i - t);
-  uint64_t a = 1ull << t;
-  int cur = t;
-  for (int step = 0; step < n_nodes; ++step) {
-    const int pp = par[cur];
-    if (pp < 0) break;
-    if (pp >= cur) {                      // not a tree in topological order: the node sees itself only
-      if (d_status) *d_status = SPECVLM_ERR_INVALID_ARG;
-      a = 1ull << t;
-      break;
-    }
-    a |= 1ull << pp;
-    cur = pp;
-  }
-  anc[i] = a;
-}
-
-size_t attn_tc_tree_extra_bytes(int32_t batch, int32_t n_nodes) {
-  return round_up((size_t)batch * n_nodes * sizeof(uint64_t), 256);
-}
-
 int32_t attn_merge_launch(const AttnTcParams& p, int head_dim, int ctas, cudaStream_t st) {
   return head_dim == 128 ? launch_merge<128>(p, ctas, st) : launch_merge<64>(p, ctas, st);
 }
@@ -1045,7 +1018,7 @@ template <int D, int M>
 static int32_t launch_tc(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& tq, const AttnTcParams& p,
                          int grid, cudaStream_t st) {
   constexpr int kSmem = TcCfg<D, M>::TOTAL;
-  return p.anc ? launch_tc_kernel<attn_tc_kernel<D, M, true>>(kSmem, tk, tv, tq, p, grid, st)
+  return p.parents ? launch_tc_kernel<attn_tc_kernel<D, M, true>>(kSmem, tk, tv, tq, p, grid, st)
                : launch_tc_kernel<attn_tc_kernel<D, M, false>>(kSmem, tk, tv, tq, p, grid, st);
 }
 
@@ -1065,8 +1038,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   // A window of more than 128 rows is cut into parts of equal numbers of query tokens that share one launch.
   const SlicePlan pl = attn_tc_plan(kv, batch, group, n_q);
   const SliceScratch sc = tc_scratch(kv, pl, group);
-  if (ws_bytes < sc.bytes() + (tree_parents ? attn_tc_tree_extra_bytes(batch, n_q) : 0))
-    return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < sc.bytes()) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
   if (tree_parents && n_q > kMaxTreeNodes) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
   if (pl.q_per * group > 128) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
   const int ctas = pl.ctas, n_parts = pl.n_parts;
@@ -1078,14 +1050,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   if (rc != SPECVLM_OK) return rc;
 
   AttnTcParams p = slice_params(kv, q, batch, n_q_heads, n_q, sm_scale, out, lse, d_status, n_parts, pl.q_per, ws, sc);
-  if (tree_parents) {
-    uint64_t* anc = reinterpret_cast<uint64_t*>(static_cast<uint8_t*>(ws) + sc.bytes());
-    const int n = batch * n_q;
-    rc = launch_after(tree_ancestors_kernel, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, st, tree_parents, n, n_q, anc,
-                      d_status);
-    if (rc != SPECVLM_OK) return rc;
-    p.anc = anc;
-  }
+  p.parents = tree_parents;
 
   CUtensorMap tq;
   rc = encode_q_map(&tq, q, kv->head_dim, group, n_q, pl.q_per, kv->n_kv_heads, (int64_t)kv->n_layers * batch);

@@ -18,7 +18,7 @@ struct AttnTcParams {
   const int32_t* block_table; // [B][max_blocks] or null
   const int32_t* seq_lens;    // [B]
   int32_t* d_status;
-  const uint64_t* anc;        // [B][n_win] ancestor masks of a draft tree (<= 64 nodes), or null: the window is a chain
+  const int32_t* parents;     // [B][n_win] parents of a draft tree's nodes (<= 64), or null: the window is a chain
   int32_t batch, n_layers, n_q_heads, n_kv_heads, group;
   int32_t n_win;              // tokens of the whole window
   int32_t n_parts, q_per;     // the window is cut into n_parts parts of q_per tokens (the last may be shorter)
@@ -133,6 +133,39 @@ __device__ __noinline__ void mask_s_half(uint32_t saddr, int tile_tok0, int win0
     tmem_st_16x256b_x8(saddr + 64 * c, v);
   }
   tmem_st_wait();
+}
+
+// The window mask of a draft tree's node t (another one in each lane), by a whole warp: bit w says that it attends window
+// position w, itself and the nodes on its path to a root.  par[t] < t, -1 for a root; a node whose path breaks that rule
+// sees itself only, and that is reported.  The parents sit in two registers of the warp, a step up is two shuffles:
+// a launch of its own for the masks cost a tree call 2.2 us on the host and 1 us on the device.
+static __device__ __noinline__ uint64_t tree_mask(const int32_t* par, int n_nodes, int t, int32_t* d_status) {
+  const int lane = threadIdx.x & 31;
+  const int lo = lane < n_nodes ? __ldcg(par + lane) : -1, hi = lane + 32 < n_nodes ? __ldcg(par + lane + 32) : -1;
+  uint64_t a = 1ull << t;
+  int cur = t;
+  bool going = true;
+#pragma unroll 1
+  while (__any_sync(0xffffffffu, going)) {
+    const int p0 = __shfl_sync(0xffffffffu, lo, cur & 31), p1 = __shfl_sync(0xffffffffu, hi, cur & 31);
+    const int up = cur < 32 ? p0 : p1;
+    if (!going) continue;
+    if (up < 0) {
+      going = false;
+    } else if (up >= cur) {
+      if (d_status) *d_status = SPECVLM_ERR_INVALID_ARG;
+      a = 1ull << t;
+      going = false;
+    } else {
+      a |= 1ull << up;
+      cur = up;
+    }
+  }
+  return a;
+}
+// The nodes of a sequence that no tile brings up (it has no token), for the report alone.
+__device__ __forceinline__ void check_tree(const int32_t* par, int n_nodes, int lane, int32_t* d_status) {
+  for (int t0 = 0; t0 < n_nodes; t0 += 32) tree_mask(par, n_nodes, t0 + lane < n_nodes ? t0 + lane : n_nodes - 1, d_status);
 }
 
 // A row maximum grew past the lazy-rescale threshold: the rows' O accumulators (16-lane half,
@@ -308,7 +341,7 @@ inline AttnTcParams slice_params(const specvlm_kv_t* kv, const void* q, int32_t 
   p.block_table = kv->block_table;
   p.seq_lens = kv->seq_lens;
   p.d_status = d_status;
-  p.anc = nullptr;
+  p.parents = nullptr;
   p.batch = batch;
   p.n_layers = kv->n_layers;
   p.n_q_heads = n_q_heads;
