@@ -703,7 +703,7 @@ static int rows16_slices(const specvlm_kv_t* kv, int32_t batch) {
     // 10.0 / 16.0 / 31.0 against 10.6 / 14.0 / 23.5: with two thirds of the SMs busy the longest item's CTAs slow down.
     const double longest = tile_us * ((tiles + n - 1) / n), even = (double)(items * tiles < sms ? items * tiles : sms);
     per_item = 3.9 + (longest > hbm ? longest : hbm) * (items * n > 64 ? 1.2 : 1.0);
-    on_slices = 6.0 + ragged * hbm + 0.04 * even / items + 0.5 < per_item;
+    on_slices = 6.0 + ragged * hbm + 0.04 * even / items < per_item;
   } else if (items <= sms) {
     const double longest = tile_us * tiles;
     per_item = 3.0 + (longest > hbm ? longest : hbm);
