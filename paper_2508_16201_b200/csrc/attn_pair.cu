@@ -22,7 +22,8 @@
 // per KV head, 80 layers of 6400 tokens (each part used to stream K and V on a set of CTAs of its own): 642 ->
 // 554 us, 827 -> 677 us under sustained load at the power cap.  What it took, same case: the parts in step
 // (both softmaxes, then both waiting for the tensor pipe) 684 us; taking turns 610; the next S issued before
-// the bookkeeping commits, waits that test before they suspend, and P handed over in two halves 554; products issued by an
+// the bookkeeping commits, waits that test before they suspend, and P handed over in two halves 554 (in 96 and 32
+// tokens, sustained 651 -> 643 us); products issued by an
 // elected lane of a whole warp instead of by lane 0 (of 4310 cycles a tile the issuers took 2750) 3700 cycles, sustained
 // 669 -> 648 us.  A share of the exponentials on the FMA pipe is slower (2 / 4 of 16 pairs: 571 / 604 us).
 #include "attn_tc.cuh"
@@ -97,8 +98,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
   const uint32_t bar_v_full = bar_k_empty + 8 * NKP, bar_v_empty = bar_v_full + 8 * NVP;
   const uint32_t bar_q_full = bar_v_empty + 8 * NVP, bar_q_empty = bar_q_full + 8;
   const uint32_t bar_s_full = bar_q_empty + 8;         // [2]: one per part
-  const uint32_t bar_p_half = bar_s_full + 16;         // [2]: the first 64 tokens' probabilities are in place
-  const uint32_t bar_p_full = bar_p_half + 16;         // [2]: ... and the rest
+  const uint32_t bar_p_most = bar_s_full + 16;         // [2]: the first 96 tokens' probabilities are in place
+  const uint32_t bar_p_full = bar_p_most + 16;         // [2]: ... and the rest
   const uint32_t bar_o_full = bar_p_full + 16;         // [2]
   const uint32_t bar_o_empty = bar_o_full + 16;        // [2]
   const uint32_t bar_turn = bar_o_empty + 16;          // [2][4]: the turn of part g's warp of a TMEM lane quadrant
@@ -137,7 +138,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     mbar_init(bar_q_empty, n_here);
     for (int g = 0; g < 2; ++g) {
       mbar_init(bar_s_full + 8 * g, 1);
-      mbar_init(bar_p_half + 8 * g, 4);
+      mbar_init(bar_p_most + 8 * g, 4);
       mbar_init(bar_p_full + 8 * g, 4);
       mbar_init(bar_o_full + 8 * g, 1);
       mbar_init(bar_o_empty + 8 * g, 4);
@@ -325,16 +326,17 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         const uint64_t db = umma_desc_advance(dv0, vp * 2 * SUB_BYTES);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          if (ok) ok = warp_wait_soon((u ? bar_p_full : bar_p_half) + 8 * g, i & 1, abort_flag);
+          if (ok) ok = warp_wait_soon((u ? bar_p_full : bar_p_most) + 8 * g, i & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
-          const int n_kt = u >= n_sub ? 0 : (tail && u == n_sub - 1 ? (last_rows + 15) >> 4 : kTileTokens / 16);
+          // 16 tokens per step: 8 columns of bf16 pairs of P, 16 rows of 128 bytes down the V sub-tile; the tile's first
+          // 96 tokens, then the other 32
+          const int n_kt = 4 * (n_sub - 1) + (tail ? (last_rows + 15) >> 4 : kTileTokens / 16);
 #pragma unroll
-          for (int kt = 0; kt < kTileTokens / 16; ++kt)
-            // 16 tokens per step: 8 columns of bf16 pairs of P, 16 rows of 128 bytes down the V sub-tile
+          for (int kt = u ? 6 : 0; kt < (u ? 8 : 6); ++kt)
             if (leader && kt < n_kt)
-              umma_bf16_ts(o_tmem, s_tmem + u * 32 + kt * 8, umma_desc_advance(db, u * SUB_BYTES + kt * 2048), kIdescPV,
-                           u > 0 || kt > 0 || j > 0 ? 1u : 0u);
+              umma_bf16_ts(o_tmem, s_tmem + kt * 8, umma_desc_advance(db, (kt >> 2) * SUB_BYTES + (kt & 3) * 2048), kIdescPV,
+                           kt > 0 || j > 0 ? 1u : 0u);
         }
         if (!ok) break;
         // S of the next tile first: the softmax is waiting for it
@@ -442,7 +444,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
           tc_fence_before_sync();
           __syncwarp();
           if (lane == 0) {
-            mbar_arrive(bar_p_half + 8 * g);
+            mbar_arrive(bar_p_most + 8 * g);
             mbar_arrive(bar_p_full + 8 * g);
           }
           continue;
@@ -504,11 +506,11 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             w[u] = pack_bf16x2(e0, e1);
           }
           tmem_st_x16(saddr + 16 * cc, w);
-          if (cc == 1) {
+          if (cc == 2) {
             tmem_st_wait();
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_p_half + 8 * g);
+            if (lane == 0) mbar_arrive(bar_p_most + 8 * g);
           }
         }
         pass_turn();

@@ -63,6 +63,14 @@ def test_tree_attention(Hq, Hkv, n_nodes, D, paged):
     _tree_case(2, Hq, Hkv, D, [300 + n_nodes, 128 + 3, n_nodes, 64 + n_nodes // 2], n_nodes, paged=paged, seed=60)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+def test_wide_tree_ends_at_every_step_of_a_tile(D):
+    """160 rows, sequences whose last tile ends around the steps of 16 tokens, the end of its first 64 and of the 96 that
+    are handed over first."""
+    tails = [1, 15, 16, 17, 48, 63, 64, 65, 80, 95, 96, 97, 111, 112, 113, 127, 128]
+    _tree_case(1, 16, 2, D, [128 + t for t in tails], 20, paged=D == 64, seed=66)
+
+
 def test_tree_with_chain_parents_equals_verify_attn():
     out, cache, q = _tree_case(1, 16, 4, 128, [200, 77], 6, paged=True, seed=61, chain=True)
     ref = specvlm.verify_attn(cache, q, 5, 1.0 / math.sqrt(128))
