@@ -45,11 +45,8 @@ struct Ptr {
   }
   AnyPtr get() const { return {v}; }
 };
+// An integer, or what stands for one (__index__: numpy's integers, tensors of one integer); a float is none.
 bool to_int(PyObject* o, unsigned long long& v) {
-  if (!PyLong_Check(o)) {
-    PyErr_Format(PyExc_TypeError, "int expected instead of %.200s", Py_TYPE(o)->tp_name);
-    return false;
-  }
   v = PyLong_AsUnsignedLongLongMask(o);
   return !PyErr_Occurred();
 }

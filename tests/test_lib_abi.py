@@ -160,6 +160,8 @@ def test_binding_takes_what_ctypes_took():
         assert _binding.select(t, [0] + many, many, 1, [5] * 199, [3] * 199, [0] + many, 199, t, None) == bad
         assert _binding.rollback_kv(t, t, 1, -1, None) == bad   # gamma < 0
         assert _binding.rollback_kv(t, t, 1, (1 << 32) - 1, None) == bad
+        for minus_one in (np.int64(-1), np.int8(-1), torch.tensor(-1)):     # whatever has __index__
+            assert _binding.rollback_kv(t, t, 1, minus_one, None) == bad
         for call, args in ((_binding.rollback_kv, (t, t, 1)), (_binding.rollback_kv, (t, t, 1.5, 0, None)),
                            (_binding.select, (t, 7, [2], 5, [5], [3], [0, 3], 1, t, None)),
                            (_binding.select, (t, None, [2], 5, [5], [3], [0, 3], 1, t, None))):
