@@ -3,7 +3,7 @@
 // and 0.1 us on each tensor's address, of 5 to 8 us that a short call takes on the host.
 //
 // Every function takes the C arguments in order without the stream, which is the current one of the current device:
-//   KvStruct    its address (int)       device pointer   a tensor (its data_ptr()), an address, or None
+//   KvStruct    its address (int)       device pointer   a tensor (its data_ptr()) or None; a number is refused
 //   host array  any sequence of integers; integers are taken modulo 2^32, as ctypes takes them
 // and returns the status.  The interpreter lock is released during the call.
 #define PY_SSIZE_T_CLEAN
@@ -28,15 +28,20 @@ struct AnyPtr {
 };
 
 // One class per kind of argument: set() converts, get() is what the C function takes.
+struct Kv {
+  static constexpr int kArgs = 1;
+  const specvlm_kv_t* v = nullptr;
+  bool set(PyObject* o) {
+    v = static_cast<const specvlm_kv_t*>(PyLong_AsVoidPtr(o));
+    return !PyErr_Occurred();
+  }
+  const specvlm_kv_t* get() const { return v; }
+};
 struct Ptr {
   static constexpr int kArgs = 1;
   void* v = nullptr;
   bool set(PyObject* o) {
     if (o == Py_None) return true;
-    if (PyLong_Check(o)) {
-      v = PyLong_AsVoidPtr(o);
-      return !PyErr_Occurred();
-    }
     PyObject* const a = PyObject_CallMethodNoArgs(o, g_data_ptr);
     if (!a) return false;
     v = PyLong_AsVoidPtr(a);
@@ -175,21 +180,21 @@ using Size = Int<size_t>;
 
 PyMethodDef g_methods[] = {
     {"init", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&init)), METH_FASTCALL, nullptr},
-    SPECVLM_ENTRY(stage1_row_lse, Ptr, Ptr, Array, Array, I32, I32, Float, Ptr, Ptr),
-    SPECVLM_ENTRY(stage1_scores, Ptr, Ptr, Array, Array, Array, Array, Array, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
-    SPECVLM_ENTRY(stage1_scores_layers, Ptr, Ptr, Array, Array, Array, Array, Array, I32, I32, Float, Ptr, Ptr, Ptr, Size, I32, I32,
+    SPECVLM_ENTRY(stage1_row_lse, Kv, Ptr, Array, Array, I32, I32, Float, Ptr, Ptr),
+    SPECVLM_ENTRY(stage1_scores, Kv, Ptr, Array, Array, Array, Array, Array, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
+    SPECVLM_ENTRY(stage1_scores_layers, Kv, Ptr, Array, Array, Array, Array, Array, I32, I32, Float, Ptr, Ptr, Ptr, Size, I32, I32,
                   I32, Ptr),
     SPECVLM_ENTRY(select, Ptr, Array, Array, I32, Array, Array, Array, I32, Ptr, Ptr),
     SPECVLM_ENTRY(select_top_p, Ptr, Array, Array, I32, Array, Array, Array, I32, Ptr, Ptr, Ptr),
-    SPECVLM_ENTRY(gather_kv, Ptr, Ptr, Array, Array, Array, Array, I32, Ptr, Ptr),
-    SPECVLM_ENTRY(draft_decode_attn, Ptr, Ptr, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
-    SPECVLM_ENTRY(verify_attn, Ptr, Ptr, I32, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
-    SPECVLM_ENTRY(verify_tree_attn, Ptr, Ptr, Ptr, I32, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
+    SPECVLM_ENTRY(gather_kv, Kv, Ptr, Array, Array, Array, Array, I32, Kv, Ptr),
+    SPECVLM_ENTRY(draft_decode_attn, Kv, Ptr, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
+    SPECVLM_ENTRY(verify_attn, Kv, Ptr, I32, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
+    SPECVLM_ENTRY(verify_tree_attn, Kv, Ptr, Ptr, I32, I32, I32, Float, Ptr, Ptr, Ptr, Size, Ptr),
     SPECVLM_ENTRY(accept, Ptr, Ptr, I32, I32, I32, Ptr, Ptr, Ptr, Ptr, Size),
     SPECVLM_ENTRY(accept_tree, Ptr, Ptr, Ptr, I32, I32, I32, Ptr, Ptr, Ptr, Ptr, Ptr, Size),
-    SPECVLM_ENTRY(append_kv, Ptr, Ptr, Ptr, I32, I32, Ptr, Ptr),
+    SPECVLM_ENTRY(append_kv, Kv, Ptr, Ptr, I32, I32, Ptr, Ptr),
     SPECVLM_ENTRY(rollback_kv, Ptr, Ptr, I32, I32, Ptr),
-    SPECVLM_ENTRY(compact_tree_kv, Ptr, Ptr, Ptr, I32, I32, Ptr, Ptr),
+    SPECVLM_ENTRY(compact_tree_kv, Kv, Ptr, Ptr, I32, I32, Ptr, Ptr),
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};

@@ -142,7 +142,7 @@ def test_kernels_with_tensor_memory_release_their_successor_after_the_allocation
 
 
 def test_binding_takes_what_ctypes_took():
-    """The CPython module: device pointers as tensors, addresses or None, host arrays as any sequence, integers modulo
+    """The CPython module: device pointers as tensors or None, host arrays as any sequence, integers modulo
     2^32; a wrong number or type of arguments is refused.  Every call here is one that the library rejects on the host."""
     import numpy as np
     import torch
@@ -167,7 +167,12 @@ def test_binding_takes_what_ctypes_took():
                            (_binding.select, (t, None, [2], 5, [5], [3], [0, 3], 1, t, None))):
             with pytest.raises(TypeError):
                 call(*args)
-        with pytest.raises(AttributeError):
-            _binding.rollback_kv("no tensor", t, 1, 0, None)
+        for no_tensor in ("no tensor", 0x1000, True, 0):         # a number is not taken for an address either
+            with pytest.raises(AttributeError):
+                _binding.rollback_kv(no_tensor, t, 1, -1, None)
+            with pytest.raises(AttributeError):
+                _binding.rollback_kv(t, t, 1, -1, no_tensor)
+        with pytest.raises(TypeError):
+            _binding.draft_decode_attn(t, None, 1, 4, 0.1, None, None, None, 0, None)   # a cache is its descriptor's address
     finally:
         _binding.init(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
