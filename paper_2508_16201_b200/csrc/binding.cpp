@@ -98,12 +98,16 @@ struct Array {
       data = big.data();
     }
     for (Py_ssize_t i = 0; ok && i < n; ++i) {
-      PyObject* const item = PySequence_Fast_GET_ITEM(seq, i);      // borrowed
       unsigned long long x = 0;
-      if (PyLong_CheckExact(item)) {
+      // a list is read in place, and an element's conversion may run code (or let another thread run) that shortens it:
+      // what is gone reads as 0, and the element is held while it is converted
+      PyObject* const item = i < PySequence_Fast_GET_SIZE(seq) ? PySequence_Fast_GET_ITEM(seq, i) : nullptr;
+      if (item && PyLong_CheckExact(item)) {
         ok = to_int(item, x);
-      } else {
+      } else if (item) {
+        Py_INCREF(item);
         PyObject* const whole = PyNumber_Long(item);
+        Py_DECREF(item);
         ok = whole && to_int(whole, x);
         Py_XDECREF(whole);
       }

@@ -162,6 +162,14 @@ def test_binding_takes_what_ctypes_took():
         assert _binding.rollback_kv(t, t, 1, (1 << 32) - 1, None) == bad
         for minus_one in (np.int64(-1), np.int8(-1), torch.tensor(-1)):     # whatever has __index__
             assert _binding.rollback_kv(t, t, 1, minus_one, None) == bad
+        class Empties:
+            """An element whose conversion empties the list that it is in."""
+            def __int__(self):
+                outer.clear()
+                return 5
+        for n in (1, 60, 199):                                 # on the stack and beyond it
+            outer = [Empties()] + [3] * (n - 1)
+            assert _binding.select(t, [0, 10], [2], 5, outer, [3], [0, 3], 1, t, None) == bad and outer == []
         for call, args in ((_binding.rollback_kv, (t, t, 1)), (_binding.rollback_kv, (t, t, 1.5, 0, None)),
                            (_binding.select, (t, 7, [2], 5, [5], [3], [0, 3], 1, t, None)),
                            (_binding.select, (t, None, [2], 5, [5], [3], [0, 3], 1, t, None))):
