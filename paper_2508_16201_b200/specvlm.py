@@ -157,7 +157,7 @@ def native():
         try:
             from . import _binding
         except ImportError as e:
-            raise RuntimeError("_binding.so is missing or does not load: build it with "
+            raise RuntimeError("the module _binding is missing or does not load: build it with "
                                "`python -m paper_2508_16201_b200.build` (there is no fallback path)") from e
         _binding.init(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
         _native = _binding

@@ -28,12 +28,11 @@ def pytest_collection_modifyitems(config, items):
 
 @pytest.fixture(scope="session", autouse=True)
 def _library_is_built():
-    """The CUDA library is built in-tree and kept out of the history: a fresh checkout compiles it
-    (nvcc, sm_100a; works without a GPU) before the first test needs it.  There is no other path to
-    fall back to, so a failed build fails the session here."""
-    from paper_2508_16201_b200 import specvlm
-    if not os.path.exists(specvlm.LIB_PATH):
-        from paper_2508_16201_b200 import build
+    """The CUDA library and the module that calls it are built in-tree and kept out of the history: a fresh checkout
+    compiles them (nvcc, sm_100a, and g++; works without a GPU) before the first test needs them.  There is no other path
+    to fall back to, so a failed build fails the session here."""
+    from paper_2508_16201_b200 import build
+    if not build.is_built():
         build.build()
     yield
 

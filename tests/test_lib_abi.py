@@ -141,6 +141,19 @@ def test_kernels_with_tensor_memory_release_their_successor_after_the_allocation
     assert seen == 4
 
 
+def test_a_tree_without_the_module_counts_as_not_built(monkeypatch, tmp_path):
+    """The module carries the interpreter's suffix, so that another one does not load it; a tree that has the library
+    alone is built before the tests run."""
+    import sysconfig
+    from paper_2508_16201_b200 import _binding, build
+    assert build.BINDING == _binding.__file__ and build.BINDING.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert build.is_built()
+    for name in ("LIB", "BINDING"):
+        with monkeypatch.context() as m:
+            m.setattr(build, name, str(tmp_path / "not built"))
+            assert not build.is_built()
+
+
 def test_binding_takes_what_ctypes_took():
     """The CPython module: device pointers as tensors or None, host arrays as any sequence, integers modulo
     2^32; a wrong number or type of arguments is refused.  Every call here is one that the library rejects on the host."""
