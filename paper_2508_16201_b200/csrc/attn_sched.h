@@ -72,6 +72,15 @@ SPECVLM_HD Segment segment_at(int64_t f, int64_t slice_end, const int* prefix, i
   return s;
 }
 
+// CTAs that a caller's scratch has room for, of a launch of up to total_tiles tiles on at most `grid`.  Slices that keep to
+// item boundaries take up to items * ceil(t / 2) CTAs for items of t tiles, at most twice the even split's; whether they are
+// used depends on how the tiles fall on items.  The room depends on the number of tiles alone and never falls as it rises,
+// so that a workspace sized for the longest sequences and the largest batch serves every shorter and smaller call.
+SPECVLM_HD int sched_scratch_ctas(int64_t total_tiles, int grid) {
+  const int even = sched_active_ctas(total_tiles, grid);
+  return 2 * even < grid ? 2 * even : grid;
+}
+
 // Where the items are fewer than the CTAs, slices that keep to item boundaries: an item of t tiles gets ceil(t / q)
 // CTAs of its own, as equal as its tiles allow.  No CTA then works on two items, one after the other (with a few tiles a
 // CTA the second one's hand-over is as long as its tiles).  part_prefix[b] = CTAs of one KV head of the sequences < b.

@@ -944,15 +944,21 @@ static void tc_parts(int rows, int group, int& n_parts, int& q_per) {
   q_per = (n_q + n_parts - 1) / n_parts;               // the parts are made as equal as the tokens allow
 }
 
-// CTAs of a launch's set (as many as the SMs allow and the tile count is worth).  A window of one
-// part is one set; a wider one has a set per two parts (attn_pair.cu), the sets side by side in one launch
-// over the same slices, so that all but the first reader of a tile find it in the L2 cache.
+// The most CTAs of a launch's set.  A window of one part is one set; a wider one has a set per two parts (attn_pair.cu),
+// the sets side by side in one launch over the same slices, so that all but the first reader of a tile find it in the L2
+// cache.
+static int tc_ctas_max(int n_parts) {
+  const int per_set = sm_count() / ((n_parts + 1) / 2);
+  return per_set < 1 ? 1 : per_set;
+}
+static int64_t tc_tiles_max(const specvlm_kv_t* kv, int32_t batch) {
+  return (int64_t)kv->n_layers * batch * kv->n_kv_heads * ((kv->max_seq_len + kBigTokens - 1) / kBigTokens);
+}
+
+// CTAs of a launch's set (as many as the SMs allow and the tile count is worth).
 static int tc_set_ctas(const specvlm_kv_t* kv, int32_t batch, int n_parts) {
-  const int64_t tiles_max = (int64_t)kv->n_layers * batch * kv->n_kv_heads *
-                            ((kv->max_seq_len + kBigTokens - 1) / kBigTokens);
-  int per_set = sm_count() / ((n_parts + 1) / 2);
-  if (per_set < 1) per_set = 1;
-  const int even = sched_active_ctas(tiles_max, per_set);
+  const int per_set = tc_ctas_max(n_parts);
+  const int even = sched_active_ctas(tc_tiles_max(kv, batch), per_set);
   // slices that keep to item boundaries may use more CTAs: every item rounds its own up
   const int64_t items = (int64_t)kv->n_layers * batch * kv->n_kv_heads;
   const int64_t aligned = items * sched_active_ctas((kv->max_seq_len + kBigTokens - 1) / kBigTokens, per_set);
@@ -971,7 +977,10 @@ static SliceScratch tc_scratch(const specvlm_kv_t* kv, const SlicePlan& pl, int 
 }
 
 size_t attn_tc_ws_bytes(const specvlm_kv_t* kv, int32_t batch, int rows, int group) {
-  return tc_scratch(kv, attn_tc_plan(kv, batch, group, rows / group), group).bytes();
+  SlicePlan pl;
+  tc_parts(rows, group, pl.n_parts, pl.q_per);
+  pl.ctas = sched_scratch_ctas(tc_tiles_max(kv, batch), tc_ctas_max(pl.n_parts));
+  return tc_scratch(kv, pl, group).bytes();
 }
 
 // Queries as a 5-D tensor (channel, head in group, query token, KV head, layer * batch + sequence):
@@ -1038,7 +1047,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
   // A window of more than 128 rows is cut into parts of equal numbers of query tokens that share one launch.
   const SlicePlan pl = attn_tc_plan(kv, batch, group, n_q);
   const SliceScratch sc = tc_scratch(kv, pl, group);
-  if (ws_bytes < sc.bytes()) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < attn_tc_ws_bytes(kv, batch, rows, group)) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
   if (tree_parents && n_q > kMaxTreeNodes) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
   if (pl.q_per * group > 128) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
   const int ctas = pl.ctas, n_parts = pl.n_parts;

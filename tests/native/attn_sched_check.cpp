@@ -140,7 +140,28 @@ static int check_aligned(const std::vector<int>& tiles, int n_layers, int hkv, i
   return 0;
 }
 
+// The room of a caller's scratch: enough for both kinds of slices, never less for more tiles.
+static int check_scratch(int grid) {
+  int last = 0;
+  for (int64_t total = 1; total <= 5 * grid; ++total) {
+    const int room = sched_scratch_ctas(total, grid);
+    if (room < last || room > grid) return 50;
+    last = room;
+    if (room < sched_active_ctas(total, grid)) return 51;
+    for (int64_t t = 1; t <= total; ++t) {
+      if (total % t != 0 || total / t > grid) continue;      // items of t tiles
+      const int64_t aligned = total / t * sched_active_ctas(t, grid);
+      if (room < (aligned < grid ? aligned : grid)) return 52;
+    }
+  }
+  return 0;
+}
+
 int main() {
+  for (int grid : {1, 2, 7, 49, 74, 148, 592}) {
+    const int rc = check_scratch(grid);
+    if (rc) { std::printf("scratch of %d CTAs failed: property %d\n", grid, rc); return 1; }
+  }
   unsigned rng = 12345u;
   auto rnd = [&](int m) { rng = rng * 1664525u + 1013904223u; return (int)((rng >> 8) % (unsigned)m); };
   struct Fixed { std::vector<int> tiles; int L, H, grid; };

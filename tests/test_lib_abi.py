@@ -83,6 +83,29 @@ def test_host_validation_without_gpu():
     assert rc == specvlm.ERR_UNSUPPORTED_SHAPE
 
 
+def _cache_of(layers, kv_heads, head_dim, max_seq_len):
+    kv = specvlm.KvStruct()
+    kv.n_layers, kv.n_kv_heads, kv.head_dim, kv.max_seq_len, kv.block_tokens = layers, kv_heads, head_dim, max_seq_len, 64
+    return kv
+
+
+@pytest.mark.parametrize("layers,group,n_q", [(1, 8, 3), (1, 8, 6), (2, 8, 9), (1, 8, 16), (1, 8, 26), (3, 16, 60), (80, 8, 6)])
+def test_a_workspace_for_the_largest_verification_serves_every_smaller_one(layers, group, n_q):
+    """The size query never falls as the batch or the sequences grow (chain up to nine tokens, tree beyond)."""
+    def size(batch, tokens):
+        kv = ctypes.byref(_cache_of(layers, 8, 128, tokens))
+        if n_q <= 9:
+            return specvlm.lib().specvlm_attn_workspace_bytes(kv, batch, 8 * group, n_q - 1)
+        return specvlm.lib().specvlm_verify_tree_workspace_bytes(kv, batch, 8 * group, n_q)
+
+    lengths = [1, 64, 65, 128, 129, 256, 257, 384, 385, 640, 1000, 2048, 2049, 6400, 50000]
+    sizes = [[size(batch, tokens) for tokens in lengths] for batch in range(1, 41)]
+    for batch, row in enumerate(sizes):
+        assert row[0] > 0 and row == sorted(row), (batch, row)
+        if batch:
+            assert all(a <= b for a, b in zip(sizes[batch - 1], row)), (batch, sizes[batch - 1], row)
+
+
 def test_missing_library_raises_and_package_is_oracle_free(monkeypatch, tmp_path):
     """No fallback: with the library file absent every call through the binding raises; and the
     package's sources neither import nor include anything of the oracle."""
