@@ -255,8 +255,8 @@ int32_t specvlm_gather_kv(const specvlm_kv_t* src, const int32_t* kept_idx, cons
  * batch <= 127 when group * (gamma+1) > 16.  A window of more than 128 rows (group * (gamma+1))
  * is cut into parts of at most 128 rows that run side by side in one launch, so that the cache
  * still comes from HBM once (the later readers of a tile find it in the L2 cache).
- * A workspace of the size for the largest batch and the largest max_seq_len serves every smaller call of the same
- * cache shape and window: the size never falls as either grows.
+ * A workspace of the size for the largest max_seq_len (and, where group * (gamma+1) > 16, the largest batch) serves
+ * every smaller call of the same cache shape and window: the size never falls as either grows.
  */
 size_t specvlm_attn_workspace_bytes(const specvlm_kv_t* kv, int32_t batch, int32_t n_q_heads,
                                     int32_t gamma);

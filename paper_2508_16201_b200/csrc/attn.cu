@@ -672,57 +672,70 @@ static int rows16_cluster(const specvlm_kv_t* kv, int64_t items, int64_t tiles) 
   return best;
 }
 
-// CTAs of a launch on slices, or 0 for a CTA (or a cluster) per item.
-static int rows16_slices(const specvlm_kv_t* kv, int32_t batch) {
-  const int64_t items = (int64_t)kv->n_layers * batch * kv->n_kv_heads;
-  const int64_t tiles = (kv->max_seq_len + kTileTokens - 1) / kTileTokens, sms = sm_count();
-  const int forced = g_forced_splits.load(std::memory_order_relaxed);
-  if (batch > kSchedMaxBatch || forced == 1) return 0;
-  if (forced > 1) {
-    const int64_t n = items * (forced < tiles ? forced : tiles);
-    return (int)(n < 4 * sms ? n : 4 * sms);
-  }
-  // Estimated times in us, from the host's bound on the lengths.  A CTA per item: about 3 us around the
-  // tiles; while the items fit the SMs the longest one counts (one CTA takes 0.35 us a tile at d = 128, a
-  // quarter more with a block table) or HBM does; beyond, rounds of two CTAs per SM at 0.75 us a tile, or HBM with
-  // a last round that is partly empty.  Slices: 4.5 us with the merge kernel, the bytes, 2 us for every
+// Whether slices are worth a workspace: estimated times in us, from the host's bound on the lengths, against a CTA per item.
+static bool rows16_slices_beat_ctas(const specvlm_kv_t* kv, int32_t batch, int64_t items, int64_t tiles) {
+  // A CTA per item: about 3 us around the tiles; while the items fit the SMs the longest one counts (one CTA takes 0.35 us
+  // a tile at d = 128, a quarter more with a block table) or HBM does; beyond, rounds of two CTAs per SM at 0.75 us a tile,
+  // or HBM with a last round that is partly empty.  Slices: 4.5 us with the merge kernel, the bytes, 2 us for every
   // item boundary of a CTA.  A batch is taken as ragged (slices balance it; so do many rounds): 0.85 of the bytes.
   // Slices have to win by 1.5 us: they cost a second launch.  Measured, 4 KV heads of d = 128, CTA per item / slices:
-  // 1 layer of 755 / 1500 / 6400 / 50 000 tokens 6.6 / 10.8 / 37.9 / 281 against 6.8 / 7.1 / 8.6 / 21.4; 28 layers of
-  // 755 / 6400 / 50 000 tokens 9.6 / 55.4 / 405 against 15.5 / 59.3 / 399; 28 layers x 4 ragged paged sequences of up to
-  // 755 / 6400 / 25 600 tokens 22.4 / 152 / 600 against 31.0 / 142 / 531.
+  // 1 layer of 1600 / 3200 / 6400 / 12 800 tokens 11.3 / 20.1 / 38.0 / 73.7 against 7.4 / 8.5 / 10.3 / 11.2; 20 layers of
+  // 2560 / 5120 / 10 240 tokens 20.7 / 37.7 / 72.7 against 23.8 / 37.9 / 65.9; 28 layers of 640 / 1280 / 5120 tokens
+  // 6.3 / 11.9 / 46.4 against 12.9 / 16.2 / 50.0; 28 layers x 4 ragged paged sequences of up to 640 / 1280 tokens
+  // 18.1 / 34.0 against 28.1 / 41.4.
+  const int64_t sms = sm_count();
   const double hbm = (double)items * tiles * (256.0 * kv->head_dim) / 6.65e6;
-  const double tile_us = rows16_tile_us(kv);
   const double ragged = batch > 1 ? 0.85 : 1.0;
   double per_item;
-  const int n = rows16_cluster(kv, items, tiles);
-  bool on_slices;
-  if (n > 1) {
-    // A cluster per item against slices that mostly keep to item boundaries (their merge folds many parts of few items).
-    // 4 items of 6400 / 12 800 tokens 8.6 / 12.7 us against 10.1 / 12.8; 24 ragged paged ones of up to 3200 / 6400 / 12 800
-    // 10.0 / 16.0 / 31.0 against 10.6 / 14.0 / 23.5: with two thirds of the SMs busy the longest item's CTAs slow down.
-    const double longest = tile_us * ((tiles + n - 1) / n), even = (double)(items * tiles < sms ? items * tiles : sms);
-    per_item = 3.9 + (longest > hbm ? longest : hbm) * (items * n > 64 ? 1.2 : 1.0);
-    on_slices = 6.0 + ragged * hbm + 0.04 * even / items < per_item;
-  } else if (items <= sms) {
-    const double longest = tile_us * tiles;
+  if (items <= sms) {
+    const double longest = rows16_tile_us(kv) * tiles;
     per_item = 3.0 + (longest > hbm ? longest : hbm);
   } else {
     const double rounds = (double)((items + 2 * sms - 1) / (2 * sms));
     const double stream = (1.0 + 0.2 / rounds) * ragged * hbm, serial = rounds * tiles * 0.75 * kv->head_dim / 128;
     per_item = 3.0 + (stream > serial ? stream : serial);
   }
-  if (n == 1) on_slices = 4.5 + ragged * hbm + 2.0 * (1.0 + (double)items / sms) + 1.5 < per_item;
-  if (!on_slices) return 0;
+  return 4.5 + ragged * hbm + 2.0 * (1.0 + (double)items / sms) + 1.5 < per_item;
+}
+
+// CTAs of a launch on slices, or 0 for a CTA (or a cluster) per item.  *scratch_ctas: the CTAs that the workspace has to
+// have room for, 0 for none.  It does not depend on whether a cluster takes the slices' place: the choice between the two
+// turns back and forth with the length, and a workspace sized for the longest sequences has to serve the shorter ones.
+static int rows16_slices(const specvlm_kv_t* kv, int32_t batch, int* scratch_ctas) {
+  const int64_t items = (int64_t)kv->n_layers * batch * kv->n_kv_heads;
+  const int64_t tiles = (kv->max_seq_len + kTileTokens - 1) / kTileTokens, sms = sm_count();
+  const int forced = g_forced_splits.load(std::memory_order_relaxed);
+  *scratch_ctas = 0;
+  if (batch > kSchedMaxBatch || forced == 1) return 0;
+  if (forced > 1) {
+    const int64_t n = items * (forced < tiles ? forced : tiles);
+    return *scratch_ctas = (int)(n < 4 * sms ? n : 4 * sms);
+  }
+  if (!rows16_slices_beat_ctas(kv, batch, items, tiles)) return 0;
+  *scratch_ctas = sched_scratch_ctas(items * tiles, (int)sms);
+  const int n = rows16_cluster(kv, items, tiles);
+  if (n > 1) {
+    // A cluster per item against slices that mostly keep to item boundaries (their merge folds many parts of few items).
+    // 4 items of 6400 / 12 800 tokens 8.6 / 12.7 us against 10.1 / 12.8; 24 ragged paged ones of up to 3200 / 6400 / 12 800
+    // 10.0 / 16.0 / 31.0 against 10.6 / 14.0 / 23.5: with two thirds of the SMs busy the longest item's CTAs slow down.
+    const double hbm = (double)items * tiles * (256.0 * kv->head_dim) / 6.65e6, ragged = batch > 1 ? 0.85 : 1.0;
+    const double longest = rows16_tile_us(kv) * ((tiles + n - 1) / n), even = (double)(items * tiles < sms ? items * tiles : sms);
+    const double cluster = 3.9 + (longest > hbm ? longest : hbm) * (items * n > 64 ? 1.2 : 1.0);
+    if (6.0 + ragged * hbm + 0.04 * even / items >= cluster) return 0;
+  }
   const int even = sched_active_ctas(items * tiles, (int)sms);
   // slices that keep to item boundaries may use more CTAs: every item rounds its own up
   const int64_t aligned = items * sched_active_ctas(tiles, (int)sms);
   return aligned > even && items <= sms ? (int)(aligned < sms ? aligned : sms) : even;
 }
 
+static size_t rows16_scratch_bytes(const specvlm_kv_t* kv, int scratch_ctas, int rows) {
+  return scratch_ctas == 0 ? 256 : SliceScratch(scratch_ctas, rows, kv->head_dim).bytes();
+}
 static size_t rows16_ws_bytes(const specvlm_kv_t* kv, int32_t batch, int rows) {
-  const int ctas = rows16_slices(kv, batch);
-  return ctas == 0 ? 256 : SliceScratch(ctas, rows, kv->head_dim).bytes();
+  int scratch_ctas;
+  rows16_slices(kv, batch, &scratch_ctas);
+  return rows16_scratch_bytes(kv, scratch_ctas, rows);
 }
 
 // tcgen05 path (attn_tc.cu)
@@ -792,11 +805,14 @@ static int32_t attn_common(const specvlm_kv_t* kv, const void* q, int32_t batch,
   rc = encode_kv_map(&tv, kv, kv->v, kTileTokens);
   if (rc != SPECVLM_OK) return rc;
 
-  const int ctas = rows16_slices(kv, batch);
+  int scratch_ctas;
+  const int ctas = rows16_slices(kv, batch, &scratch_ctas);
+  if (scratch_ctas > 0) {
+    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SPECVLM_ERR_INVALID_ARG;
+    if (ws_bytes < rows16_scratch_bytes(kv, scratch_ctas, rows)) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
+  }
   if (ctas > 0) {
     const SliceScratch sc(ctas, rows, kv->head_dim);
-    if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SPECVLM_ERR_INVALID_ARG;
-    if (ws_bytes < sc.bytes()) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
     const AttnTcParams p = slice_params(kv, q, batch, n_q_heads, n_q, sm_scale, out, lse, d_status, 1, n_q, ws, sc);
     rc = kv->head_dim == 128 ? launch_slices<128>(tk, tv, p, ctas, st) : launch_slices<64>(tk, tv, p, ctas, st);
     return rc != SPECVLM_OK ? rc : attn_merge_launch(p, kv->head_dim, ctas, st);
@@ -841,7 +857,8 @@ extern "C" int32_t specvlm_debug_attn_merge(const specvlm_kv_t* kv, int32_t batc
   if (!out || !ws || !n_ctas || n_q_heads < 1 || n_q < 1 || n_q_heads % kv->n_kv_heads != 0) return SPECVLM_ERR_INVALID_ARG;
   const int group = n_q_heads / kv->n_kv_heads;
   if (group > 16 || n_q > 9 || batch > kSchedMaxBatch) return SPECVLM_ERR_UNSUPPORTED_SHAPE;
-  const SlicePlan pl = group * n_q > kRows16Max ? attn_tc_plan(kv, batch, group, n_q) : SlicePlan{rows16_slices(kv, batch), 1, n_q};
+  int room;
+  const SlicePlan pl = group * n_q > kRows16Max ? attn_tc_plan(kv, batch, group, n_q) : SlicePlan{rows16_slices(kv, batch, &room), 1, n_q};
   const int grid = pl.n_parts * pl.ctas;
   *n_ctas = grid;
   if (grid == 0) return SPECVLM_ERR_UNSUPPORTED_SHAPE;

@@ -106,6 +106,28 @@ def test_a_workspace_for_the_largest_verification_serves_every_smaller_one(layer
             assert all(a <= b for a, b in zip(sizes[batch - 1], row)), (batch, sizes[batch - 1], row)
 
 
+@pytest.mark.parametrize("layers,kv_heads,head_dim", [(1, 4, 128), (1, 1, 64), (2, 4, 64), (8, 4, 128), (16, 4, 128), (28, 4, 128)])
+@pytest.mark.parametrize("batch", [1, 3, 16])
+def test_a_decode_workspace_for_the_longest_sequences_serves_shorter_ones(layers, kv_heads, head_dim, batch):
+    """As the lengths grow a cluster of CTAs per item and slices take turns, and the slices' scratch comes and goes; the size
+    query never falls."""
+    table = (ctypes.c_int32 * 1)()
+    for paged in (False, True):
+        last = 256
+        for tokens in sorted({*range(64, 4096, 64), *range(4096, 60000, 256), *range(8704, 9344, 64)}):
+            kv = _cache_of(layers, kv_heads, head_dim, tokens)
+            kv.block_table = ctypes.addressof(table) if paged else None
+            size = specvlm.lib().specvlm_attn_workspace_bytes(ctypes.byref(kv), batch, 7 * kv_heads, 0)
+            assert size >= last, (paged, tokens, last, size)
+            last = size
+
+
+def test_decode_asks_for_scratch_only_where_slices_beat_a_cta_per_item():
+    """64 items of 2560 tokens (d = 128): no slices, and a call without a workspace is accepted."""
+    kv = _cache_of(16, 4, 128, 2560)
+    assert specvlm.lib().specvlm_attn_workspace_bytes(ctypes.byref(kv), 1, 28, 0) == 256
+
+
 def test_missing_library_raises_and_package_is_oracle_free(monkeypatch, tmp_path):
     """No fallback: with the library file absent every call through the binding raises; and the
     package's sources neither import nor include anything of the oracle."""
