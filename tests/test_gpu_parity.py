@@ -128,6 +128,31 @@ def test_decode_with_a_cluster_per_item_and_an_empty_sequence():
         assert row_rel_err(out[0, b], ref[0]) <= ATTN_TOL
 
 
+@pytest.mark.parametrize("L,tokens,paged,slices", [
+    (3, 2560, False, False), (3, 10240, False, True),        # 12 items: clusters of four 7.3 / 18.5 us, slices 8.3 / 16.4
+    (4, 2560, True, False), (4, 5120, True, True),           # 16 paged ones: 8.3 / 13.4, slices 9.0 / 10.8
+    (14, 2560, False, False), (16, 5120, False, False),      # clusters of two 14.0 / 28.4, slices 18.3 / 31.8
+    (18, 2560, False, False), (18, 10240, False, False)])    # 16.3 / 57.8, slices 20.4 / 61.0
+def test_decode_takes_the_faster_of_cluster_and_slices(L, tokens, paged, slices):
+    """Which of the two runs is seen from whether the call has a second kernel."""
+    if paged:
+        blocks = -(-tokens // 64)
+        k, v = (torch.zeros((L, blocks, 4, 64, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        table = torch.arange(blocks, dtype=torch.int32, device="cuda").view(1, -1)
+    else:
+        k, v = (torch.zeros((L, 1, 4, tokens, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        table = None
+    cache = specvlm.KvCache(k, v, torch.full((1,), tokens, dtype=torch.int32, device="cuda"), tokens, table)
+    q = torch.zeros((L, 1, 28, 128), dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(specvlm.attn_workspace_bytes(cache, 1, 28, 0), dtype=torch.uint8, device="cuda")
+    out = specvlm.draft_decode_attn(cache, q, 0.1, ws=ws).unsqueeze(2)
+    if slices:
+        assert specvlm.debug_attn_merge(cache, out, ws) > 0
+    else:
+        with pytest.raises(specvlm.SpecvlmError, match="shape"):
+            specvlm.debug_attn_merge(cache, out, ws)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("lens", [[1], [64, 0, 65], [0, 0], [3, 1000, 63, 130], [2111], [257] * 40])
 def test_decode_on_slices(lens, D):
