@@ -225,124 +225,23 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
 // ---------------------------------------------------------------------------------------------
 // NG consumer groups of 4 warps take alternate tiles (NG = 2 where an SM holds a single CTA, so
 // that eight warps hide each other's latencies as two resident CTAs would).
-// SPLIT: a cluster of gridDim.x CTAs per item, CTA r on tiles r, r + gridDim.x, ..; their results meet over distributed
+// SPLIT: a cluster of n_cta CTAs per item, CTA r on tiles r, r + n_cta, ..; their results meet over distributed
 // shared memory, each CTA folding its share of the output positions.  For a few short items, whose tiles one CTA would
 // work through one after the other at 0.35 us each.
+//
+// The consumer warps of an item, or of a cluster's CTA.
 template <int D, int STAGES, int NG, bool SPLIT>
-__global__ void __launch_bounds__(32 * (4 * NG + 1))
-attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                   const AttnParams p) {
-  constexpr int TILE_BYTES = kTileTokens * D * 2;
-  constexpr int STAGE_BYTES = 2 * TILE_BYTES;
+__device__ __forceinline__ void rows16_consume(const AttnParams& p, uint8_t* smem, uint32_t base, volatile int* abort_flag,
+                                               int kv_len, int n_my, int rank, int n_cta) {
+  constexpr int TILE_BYTES = kTileTokens * D * 2, STAGE_BYTES = 2 * TILE_BYTES;
   constexpr int OPITCH = Rows16<D>::OPITCH;
-  // A consumer group must see every phase of the ring slots it waits on: with the groups on
-  // alternate tiles that holds only when a slot always belongs to the same group.  (A wait on a
-  // phase two behind the barrier returns at once, the group then releases a slot it never read,
-  // and the surplus arrival on the barrier is undefined behaviour: it faulted the kernel.)
-  static_assert(STAGES % NG == 0, "ring depth must be a multiple of the number of consumer groups");
-
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw_addr = smem_u32(smem_raw);
-  const uint32_t base = (raw_addr + 1023u) & ~1023u;
-  uint8_t* const smem = smem_raw + (base - raw_addr);
-  const uint32_t bar_full = base + STAGES * STAGE_BYTES;
-  const uint32_t bar_empty = bar_full + 8 * STAGES;
-  volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem + STAGES * STAGE_BYTES + 16 * STAGES);
-
+  const uint32_t bar_full = base + STAGES * STAGE_BYTES, bar_empty = bar_full + 8 * STAGES;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = blockIdx.y, lb = blockIdx.z;
-  const int layer = lb / p.batch, b = lb - layer * p.batch;
-  const int rank = SPLIT ? (int)blockIdx.x : 0, n_cta = SPLIT ? (int)gridDim.x : 1;
-
-  if (tid == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(bar_full + 8 * s, 1);
-      mbar_init(bar_empty + 8 * s, 4);
-    }
-    *abort_flag = 0;
-    mbar_fence_init();
-  }
-  if (tid == 32 * 4 * NG) {              // the producer's lane: descriptors are kernel parameters
-    tma_prefetch_desc(&tm_k);
-    tma_prefetch_desc(&tm_v);
-  }
-  __syncthreads();                       // the barriers are initialised
-  pdl_launch_next();
-  pdl_wait();
-
-  // The first tile of a contiguous cache sits at a known place whatever the sequence's
-  // length (rows past the cache's end are zero-filled by the copy): the producer asks for it
-  // before the length has even been read, which takes a global-memory round trip off the start.
   const bool spec = p.block_table == nullptr;
-  if (spec && tid == 32 * 4 * NG) {
-    const uint64_t policy = l2_policy_evict_first();
-    mbar_arrive_expect_tx(bar_full, STAGE_BYTES);
-#pragma unroll
-    for (int h = 0; h < D / 64; ++h) {
-      tma_load_5d(base + h * (kTileTokens * 128), &tm_k, bar_full, h * 64, rank * kTileTokens, g, b, layer, policy);
-      tma_load_5d(base + TILE_BYTES + h * (kTileTokens * 128), &tm_v, bar_full, h * 64, rank * kTileTokens, g, b, layer, policy);
-    }
-  }
-
-  const int kv_len = clamp_len(p.seq_lens[b], p.max_seq_len);
   const int n_all = (kv_len + kTileTokens - 1) / kTileTokens;
-  const int n_my = SPLIT ? (n_all + n_cta - 1 - rank) / n_cta : n_all;
 
-  if (warp == 4 * NG) {
-    // ------------------------------------------------------------------ producer
-    if (lane == 0 && n_my == 0 && spec) {
-      // an empty sequence: nobody will consume the tile asked for above; stay until it has landed
-      const uint64_t t0 = global_timer_ns();
-      while (!mbar_try_wait(bar_full, 0) && global_timer_ns() - t0 < kWaitLimitNs) {
-      }
-    }
-    if (lane == 0 && n_my > 0) {
-      const uint64_t policy = l2_policy_evict_first();
-      const int tiles_per_block = p.block_tokens / kTileTokens;   // used only when paged
-      int issued = spec ? 1 : 0;
-      bool ok = true;
-      for (int i = issued; i < n_my && ok; ++i) {
-        const int s = i % STAGES;
-        if (i >= STAGES) ok = mbar_wait(bar_empty + 8 * s, ((i / STAGES) - 1) & 1, abort_flag);
-        if (!ok) break;
-        const int t = i * n_cta + rank;
-        int blk, tok;
-        if (p.block_table) {
-          blk = p.block_table[(size_t)b * p.max_blocks + t / tiles_per_block];
-          tok = (t % tiles_per_block) * kTileTokens;
-        } else {
-          blk = b;
-          tok = t * kTileTokens;
-        }
-        const uint32_t full = bar_full + 8 * s;
-        mbar_arrive_expect_tx(full, STAGE_BYTES);
-        const uint32_t dst = base + s * STAGE_BYTES;
-#pragma unroll
-        for (int h = 0; h < D / 64; ++h) {
-          tma_load_5d(dst + h * (kTileTokens * 128), &tm_k, full, h * 64, tok, g, blk, layer, policy);
-          tma_load_5d(dst + TILE_BYTES + h * (kTileTokens * 128), &tm_v, full, h * 64, tok, g, blk,
-                      layer, policy);
-        }
-        issued = i + 1;
-      }
-      if (!ok) {
-        // a wait expired: report, then stay until this CTA's copies in flight have landed
-        if (p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
-        const int first = issued > STAGES ? issued - STAGES : 0;
-        for (int i = first; i < issued; ++i) {
-          const uint64_t t0 = global_timer_ns();
-          while (!mbar_try_wait(bar_full + 8 * (i % STAGES), (i / STAGES) & 1) &&
-                 global_timer_ns() - t0 < kWaitLimitNs) {
-          }
-        }
-      }
-    }
-    return;
-  }
-
-  // -------------------------------------------------------------------- consumers
   if (n_all == 0) {
-    if (rank != 0) return;
     // An empty sequence: its outputs are zero, its LSE -inf.  The ring stays untouched: the tile that the producer
     // asked for before it knew the length may still be landing there, with whatever the cache rows hold.
     for (int idx = tid; idx < p.rows * (D / 8); idx += 128 * NG) {
@@ -445,6 +344,135 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     store_bf16x4(p.out + orow * D + c, acc);
     if (p.lse && c == 0) p.lse[orow] = lse2 * kLn2;
   }
+}
+
+// SPLIT: launched in clusters of gridDim.x CTAs per item, a number that the host's bound on the lengths gives.  A sequence of
+// a few tiles is left to the first of them, since the hand-over would take longer (one layer, 4 items of d = 128 in a cache of
+// 800 tokens, alone / by eight: 40 tokens 2.9 / 4.1 us, 200 3.9 / 4.1, 400 4.8 / 4.1; d = 64: 200 tokens 3.0 / 3.3, 400
+// 3.8 / 3.3; by two, 36 items of d = 128: 200 tokens 4.1 / 4.5, 320 4.5 / 4.9, 400 5.2 / 5.1).  The producer serves both
+// forms in one loop and the consumers have code of their own for each: the other ways round cost a cluster's full lengths
+// 1 to 5 %.
+constexpr int kSoloTiles = 4, kSoloTilesPair = 6;
+template <int D, int STAGES, int NG, bool SPLIT>
+__global__ void __launch_bounds__(32 * (4 * NG + 1))
+attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                   const AttnParams p) {
+  constexpr int TILE_BYTES = kTileTokens * D * 2;
+  constexpr int STAGE_BYTES = 2 * TILE_BYTES;
+  // A consumer group must see every phase of the ring slots it waits on: with the groups on
+  // alternate tiles that holds only when a slot always belongs to the same group.  (A wait on a
+  // phase two behind the barrier returns at once, the group then releases a slot it never read,
+  // and the surplus arrival on the barrier is undefined behaviour: it faulted the kernel.)
+  static_assert(STAGES % NG == 0, "ring depth must be a multiple of the number of consumer groups");
+
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw_addr = smem_u32(smem_raw);
+  const uint32_t base = (raw_addr + 1023u) & ~1023u;
+  uint8_t* const smem = smem_raw + (base - raw_addr);
+  const uint32_t bar_full = base + STAGES * STAGE_BYTES;
+  const uint32_t bar_empty = bar_full + 8 * STAGES;
+  volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem + STAGES * STAGE_BYTES + 16 * STAGES);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = blockIdx.y, lb = blockIdx.z;
+  const int layer = lb / p.batch, b = lb - layer * p.batch;
+  const int rank = SPLIT ? (int)blockIdx.x : 0, n_cta = SPLIT ? (int)gridDim.x : 1;
+
+  if (tid == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(bar_full + 8 * s, 1);
+      mbar_init(bar_empty + 8 * s, 4);
+    }
+    *abort_flag = 0;
+    mbar_fence_init();
+  }
+  if (tid == 32 * 4 * NG) {              // the producer's lane: descriptors are kernel parameters
+    tma_prefetch_desc(&tm_k);
+    tma_prefetch_desc(&tm_v);
+  }
+  __syncthreads();                       // the barriers are initialised
+  pdl_launch_next();
+  pdl_wait();
+
+  // The first tile of a contiguous cache sits at a known place whatever the sequence's
+  // length (rows past the cache's end are zero-filled by the copy): the producer asks for it
+  // before the length has even been read, which takes a global-memory round trip off the start.
+  const bool spec = p.block_table == nullptr;
+  if (spec && tid == 32 * 4 * NG) {
+    const uint64_t policy = l2_policy_evict_first();
+    mbar_arrive_expect_tx(bar_full, STAGE_BYTES);
+#pragma unroll
+    for (int h = 0; h < D / 64; ++h) {
+      tma_load_5d(base + h * (kTileTokens * 128), &tm_k, bar_full, h * 64, rank * kTileTokens, g, b, layer, policy);
+      tma_load_5d(base + TILE_BYTES + h * (kTileTokens * 128), &tm_v, bar_full, h * 64, rank * kTileTokens, g, b, layer, policy);
+    }
+  }
+
+  const int kv_len = clamp_len(p.seq_lens[b], p.max_seq_len);
+  const int n_all = (kv_len + kTileTokens - 1) / kTileTokens;
+  const bool solo = SPLIT && n_all <= (n_cta == 2 ? kSoloTilesPair : kSoloTiles);
+  const int n_split = SPLIT ? (n_all + n_cta - 1 - rank) / n_cta : n_all;
+  const int n_my = !solo ? n_split : rank == 0 ? n_all : 0;
+
+  if (warp == 4 * NG) {
+    // ------------------------------------------------------------------ producer
+    if (lane == 0 && n_my == 0 && spec) {
+      // an empty sequence, or a CTA without a part: nobody will consume the tile asked for above; stay until it has landed
+      const uint64_t t0 = global_timer_ns();
+      while (!mbar_try_wait(bar_full, 0) && global_timer_ns() - t0 < kWaitLimitNs) {
+      }
+    }
+    if (lane == 0 && n_my > 0) {
+      const uint64_t policy = l2_policy_evict_first();
+      const int tiles_per_block = p.block_tokens / kTileTokens;   // used only when paged
+      int issued = spec ? 1 : 0;
+      bool ok = true;
+      for (int i = issued; i < n_my && ok; ++i) {
+        const int s = i % STAGES;
+        if (i >= STAGES) ok = mbar_wait(bar_empty + 8 * s, ((i / STAGES) - 1) & 1, abort_flag);
+        if (!ok) break;
+        const int t = solo ? i : i * n_cta + rank;
+        int blk, tok;
+        if (p.block_table) {
+          blk = p.block_table[(size_t)b * p.max_blocks + t / tiles_per_block];
+          tok = (t % tiles_per_block) * kTileTokens;
+        } else {
+          blk = b;
+          tok = t * kTileTokens;
+        }
+        const uint32_t full = bar_full + 8 * s;
+        mbar_arrive_expect_tx(full, STAGE_BYTES);
+        const uint32_t dst = base + s * STAGE_BYTES;
+#pragma unroll
+        for (int h = 0; h < D / 64; ++h) {
+          tma_load_5d(dst + h * (kTileTokens * 128), &tm_k, full, h * 64, tok, g, blk, layer, policy);
+          tma_load_5d(dst + TILE_BYTES + h * (kTileTokens * 128), &tm_v, full, h * 64, tok, g, blk,
+                      layer, policy);
+        }
+        issued = i + 1;
+      }
+      if (!ok) {
+        // a wait expired: report, then stay until this CTA's copies in flight have landed
+        if (p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
+        const int first = issued > STAGES ? issued - STAGES : 0;
+        for (int i = first; i < issued; ++i) {
+          const uint64_t t0 = global_timer_ns();
+          while (!mbar_try_wait(bar_full + 8 * (i % STAGES), (i / STAGES) & 1) &&
+                 global_timer_ns() - t0 < kWaitLimitNs) {
+          }
+        }
+      }
+    }
+    return;
+  }
+
+  if constexpr (SPLIT) {
+    if (solo) {
+      if (rank == 0) rows16_consume<D, STAGES, NG, false>(p, smem, base, abort_flag, kv_len, n_my, 0, 1);
+      return;
+    }
+  }
+  rows16_consume<D, STAGES, NG, SPLIT>(p, smem, base, abort_flag, kv_len, n_my, rank, n_cta);
 }
 
 // bar.sync 1 over n threads (whole warps) that also answers whether the predicate holds for all of them

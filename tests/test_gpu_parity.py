@@ -113,6 +113,30 @@ def test_decode_with_a_cluster_per_item(lens, paged, D):
     _run_attn(1, 28, 4, D, lens, 0, paged=paged, seed=70 + len(lens), decode_api=True, poison=True)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("paged", [False, True])
+def test_short_sequences_of_a_cluster_launch_are_left_to_one_cta(paged, D):
+    """Sequences of up to four tiles in a cache whose room calls for a cluster: what a CTA per item gives, bit for bit."""
+    from gpu_util import make_cache
+    lens = [1500, 256, 1, 200, 255, 64]
+    q = synth.randn_bf16((1, len(lens), 28, D), "cuda", 73, "Q")
+    outs = []
+    for splits in (0, 1):
+        cache, _, _ = make_cache(1, 4, D, lens, paged=paged, seed=73, poison_tail=True)
+        specvlm.debug_set_attn_splits(splits)
+        try:
+            lse = torch.empty((1, len(lens), 28), dtype=torch.float32, device="cuda")
+            outs.append((specvlm.draft_decode_attn(cache, q, 0.1, lse=lse), lse))
+        finally:
+            specvlm.debug_set_attn_splits(0)
+    for one, other in zip(*outs):
+        assert torch.equal(one[:, 1:], other[:, 1:])
+    assert not torch.equal(outs[0][0][:, 0], outs[1][0][:, 0])          # the long one really went to a cluster
+    for batch in (4, 11):                                              # clusters of four and of two
+        _run_attn(1, 28, 4, D, ([1500, 257, 256, 320, 384, 385, 448, 449] * 2)[:batch], 0, paged=paged, seed=74,
+                  decode_api=True, poison=True)
+
+
 def test_decode_with_a_cluster_per_item_and_an_empty_sequence():
     from gpu_util import make_cache
     lens = [1000, 0, 70]
