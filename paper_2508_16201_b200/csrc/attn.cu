@@ -284,9 +284,10 @@ __device__ __forceinline__ void rows16_consume(const AttnParams& p, uint8_t* sme
   st.publish(o_sm, m_sm, l_sm, p.rows, warp, lane);
   asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
   if constexpr (SPLIT) {
-    // this CTA's result, normalised, and its log-sum-exps: behind the merge buffer, for the whole cluster to read
+    // This CTA's result, normalised, behind the merge buffer, and its log-sum-exps, for the whole cluster to read.  The
+    // latter say whether the CTA gave up, and lie behind the ring, where no copy that was asked for before lands on them.
     float* const part_o = l_sm + NW * 16;                              // [16][D]
-    float* const part_lse = part_o + 16 * D;                           // [16]
+    float* const part_lse = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES + 16 * STAGES + 16);   // [16]
     for (int idx = tid; idx < p.rows * (D / 4); idx += 128 * NG) {
       const int r = idx / (D / 4), c = (idx - r * (D / 4)) * 4;
       float4 acc;
@@ -778,7 +779,7 @@ int32_t attn_tc_launch(const specvlm_kv_t* kv, const void* q, int32_t batch, int
 template <int D, int STAGES, int NG, bool SPLIT>
 static int32_t launch_rows16_s(const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& p,
                                dim3 grid, cudaStream_t st) {
-  constexpr int SMEM = STAGES * 2 * kTileTokens * D * 2 + 1024 + 16 * STAGES + 16;
+  constexpr int SMEM = STAGES * 2 * kTileTokens * D * 2 + 1024 + 16 * STAGES + 16 + (SPLIT ? 16 * 4 : 0);
   auto kern = attn_rows16_kernel<D, STAGES, NG, SPLIT>;
   static std::atomic<uint64_t> attr_done{0};
   if (!smem_attr_once(attr_done, reinterpret_cast<const void*>(kern), SMEM)) return SPECVLM_ERR_CUDA;
