@@ -219,6 +219,20 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
   return v;
 }
 
+// By a consumer thread of a CTA that gives up (a wait expired): it stays, bounded, until the producer has gone and the last
+// copies that it asked for have landed, since the CTA must not end under copies to its shared memory.  flags[0] is the abort
+// flag, flags[1] the copies asked for once the producer has gone, -1 before.
+template <int STAGES>
+__device__ __forceinline__ void await_copies(uint32_t bar_full, volatile int* flags) {
+  const uint64_t t0 = global_timer_ns();
+  while (flags[1] < 0 && global_timer_ns() - t0 < kWaitLimitNs) {
+  }
+  const int issued = flags[1];
+  for (int i = issued > STAGES ? issued - STAGES : 0; i < issued; ++i)
+    while (!mbar_try_wait(bar_full + 8 * (i % STAGES), (i / STAGES) & 1) && global_timer_ns() - t0 < kWaitLimitNs) {
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // One CTA per item.  4 consumer warps each own 16 of a tile's 64 tokens; they are merged once at the end.
 // The last warp is the TMA producer.
@@ -276,7 +290,10 @@ __device__ __forceinline__ void rows16_consume(const AttnParams& p, uint8_t* sme
   // (named barrier over the consumer threads; the producer warp has no part in it)
   asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
   const bool gave_up = !alive || *abort_flag;   // a wait expired somewhere in this CTA (the flag tells all of it)
-  if (!SPLIT && gave_up) return;       // leave outputs alone
+  if (!SPLIT && gave_up) {             // leave outputs alone
+    if (tid == 0) await_copies<STAGES>(bar_full, abort_flag);
+    return;
+  }
   constexpr int NW = 4 * NG;                                           // consumer warps
   float* const o_sm = reinterpret_cast<float*>(smem);                  // [NW][16][OPITCH]
   float* const m_sm = o_sm + NW * 16 * OPITCH;                         // [NW][16]
@@ -334,6 +351,7 @@ __device__ __forceinline__ void rows16_consume(const AttnParams& p, uint8_t* sme
       if (p.lse && c == 0) p.lse[orow] = den > 0.f ? (mm + log2f(den)) * kLn2 : -INFINITY;
     }
     cluster_barrier();                                                 // nobody reads this CTA's shared memory any more
+    if (gave_up && tid == 0) await_copies<STAGES>(bar_full, abort_flag);
     return;
   }
   for (int idx = tid; idx < p.rows * (D / 4); idx += 128 * NG) {
@@ -386,7 +404,8 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       mbar_init(bar_full + 8 * s, 1);
       mbar_init(bar_empty + 8 * s, 4);
     }
-    *abort_flag = 0;
+    abort_flag[0] = 0;
+    abort_flag[1] = -1;                  // see await_copies
     mbar_fence_init();
   }
   if (tid == 32 * 4 * NG) {              // the producer's lane: descriptors are kernel parameters
@@ -419,11 +438,12 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 
   if (warp == 4 * NG) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0 && n_my == 0 && spec) {
+    if (lane == 0 && n_my == 0) {
       // an empty sequence, or a CTA without a part: nobody will consume the tile asked for above; stay until it has landed
       const uint64_t t0 = global_timer_ns();
-      while (!mbar_try_wait(bar_full, 0) && global_timer_ns() - t0 < kWaitLimitNs) {
+      while (spec && !mbar_try_wait(bar_full, 0) && global_timer_ns() - t0 < kWaitLimitNs) {
       }
+      abort_flag[1] = 0;
     }
     if (lane == 0 && n_my > 0) {
       const uint64_t policy = l2_policy_evict_first();
@@ -465,6 +485,7 @@ attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
           }
         }
       }
+      abort_flag[1] = issued;
     }
     return;
   }
@@ -536,7 +557,8 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
       mbar_init(bar_full + 8 * s, 1);
       mbar_init(bar_empty + 8 * s, 4);
     }
-    *abort_flag = 0;
+    abort_flag[0] = 0;
+    abort_flag[1] = -1;                  // see await_copies
     mbar_fence_init();
   }
   if (tid == 32 * NW) {
@@ -595,6 +617,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
           while (!mbar_test_wait(bar_full + 8 * (k % STAGES), (k / STAGES) & 1) && global_timer_ns() - t0 < kWaitLimitNs) {
           }
       }
+      if (leader) abort_flag[1] = i;
     }
     return;
   }
@@ -668,6 +691,7 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
     i0 += sg.n_tiles;
     c.next_segment(prefix, p.batch, hkv);
   }
+  if (!alive && lane == 0) await_copies<STAGES>(bar_full, abort_flag);
 }
 
 // ---------------------------------------------------------------------------------------------
