@@ -427,6 +427,16 @@ int32_t specvlm_debug_attn_merge(const specvlm_kv_t* kv, int32_t batch, int32_t 
                                  void* stream);
 
 /*
+ * Test hook; the paper has no counterpart.  specvlm_draft_decode_attn with CTA lost_cta (0 .. n_ctas - 1, of the kernel that
+ * reads the cache; -1: none) giving up as if a wait of its had expired, if it has work: d_status then reads
+ * SPECVLM_ERR_TIMEOUT, and the heads that the CTA has a part of stay as they are in out and lse.  n_ctas (host int32 out):
+ * the kernel's CTAs.  No wait is made to expire.
+ */
+int32_t specvlm_debug_attn_give_up(const specvlm_kv_t* kv, const void* q, int32_t batch, int32_t n_q_heads, float sm_scale,
+                                   void* out, float* lse_or_null, void* ws, size_t ws_bytes, int32_t lost_cta,
+                                   int32_t* n_ctas, int32_t* d_status, void* stream);
+
+/*
  * Test hook, host only; the paper has no counterpart.  Reports how a verification window of n_q
  * query tokens at `group` = n_q_heads / n_kv_heads heads per KV head is cut into the parts that run
  * side by side in one launch: n_parts parts of q_per tokens (the last may be shorter), each of at

@@ -286,10 +286,14 @@ __device__ __forceinline__ void rows16_consume(const AttnParams& p, uint8_t* sme
     if (lane == 0) mbar_arrive(bar_empty + 8 * s);
   }
 
+  // test hook: the CTA that gives up although it has seen its tiles
+  if (p.lost_cta == (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x)) *abort_flag = 1;
   // ------------------------------------------------------------ merge the consumer warps' partials
   // (named barrier over the consumer threads; the producer warp has no part in it)
   asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
   const bool gave_up = !alive || *abort_flag;   // a wait expired somewhere in this CTA (the flag tells all of it)
+  // (the producer reports only the waits of its own, and it has none where the tiles fit the ring)
+  if (gave_up && tid == 0 && p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
   if (!SPLIT && gave_up) {             // leave outputs alone
     if (tid == 0) await_copies<STAGES>(bar_full, abort_flag);
     return;
@@ -668,7 +672,8 @@ attn_rows16_slices_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid
     const bool complete = sg.tile0 == 0 && sg.n_tiles == sg.item_tiles;
     const int slot = partial_slot(cta, T0, sg.item_begin);
     // and whether every consumer has seen all its tiles: one answer for all threads, so that a row is stored whole or not at all
-    const bool whole = bar_and(alive, 128 * NG);
+    const bool whole = bar_and(alive && cta != p.lost_cta, 128 * NG);
+    if (!whole && tid == 0 && p.d_status) *p.d_status = SPECVLM_ERR_TIMEOUT;
     st.publish(o_sm, m_sm, l_sm, p.rows, warp, lane);
     asm volatile("bar.sync 1, %0;" ::"n"(128 * NG) : "memory");
     if (whole) {
@@ -840,7 +845,7 @@ __global__ void give_up_kernel(const __grid_constant__ AttnTcParams p, int gcta,
 
 static int32_t attn_common(const specvlm_kv_t* kv, const void* q, int32_t batch, int32_t n_q_heads,
                            int32_t n_q, float sm_scale, void* out, float* lse, void* ws,
-                           size_t ws_bytes, int32_t* d_status, void* stream) {
+                           size_t ws_bytes, int32_t* d_status, void* stream, int lost_cta = -1, int32_t* n_ctas = nullptr) {
   int32_t rc = validate_kv(kv, batch, true);
   if (rc != SPECVLM_OK) return rc;
   if (!q || !out || n_q_heads < 1 || n_q < 1 || !(sm_scale > 0.f)) return SPECVLM_ERR_INVALID_ARG;
@@ -869,7 +874,9 @@ static int32_t attn_common(const specvlm_kv_t* kv, const void* q, int32_t batch,
   }
   if (ctas > 0) {
     const SliceScratch sc(ctas, rows, kv->head_dim);
-    const AttnTcParams p = slice_params(kv, q, batch, n_q_heads, n_q, sm_scale, out, lse, d_status, 1, n_q, ws, sc);
+    AttnTcParams p = slice_params(kv, q, batch, n_q_heads, n_q, sm_scale, out, lse, d_status, 1, n_q, ws, sc);
+    p.lost_cta = lost_cta;
+    if (n_ctas) *n_ctas = ctas;
     rc = kv->head_dim == 128 ? launch_slices<128>(tk, tv, p, ctas, st) : launch_slices<64>(tk, tv, p, ctas, st);
     return rc != SPECVLM_OK ? rc : attn_merge_launch(p, kv->head_dim, ctas, st);
   }
@@ -891,9 +898,11 @@ static int32_t attn_common(const specvlm_kv_t* kv, const void* q, int32_t batch,
   p.block_tokens = kv->block_tokens;
   p.max_seq_len = kv->max_seq_len;
   p.scale_log2 = sm_scale * kLog2e;
+  p.lost_cta = lost_cta;
 
   const int n = rows16_cluster(kv, lb64 * kv->n_kv_heads, (kv->max_seq_len + kTileTokens - 1) / kTileTokens);
   dim3 grid((unsigned)n, (unsigned)kv->n_kv_heads, (unsigned)lb64);
+  if (n_ctas) *n_ctas = (int32_t)(grid.x * grid.y * grid.z);
   return kv->head_dim == 128 ? launch_rows16<128>(tk, tv, p, grid, st) : launch_rows16<64>(tk, tv, p, grid, st);
 }
 
@@ -928,6 +937,13 @@ extern "C" int32_t specvlm_debug_attn_merge(const specvlm_kv_t* kv, int32_t batc
     if (marked != SPECVLM_OK) return marked;
   }
   return attn_merge_launch(p, kv->head_dim, pl.ctas, st);
+}
+
+extern "C" int32_t specvlm_debug_attn_give_up(const specvlm_kv_t* kv, const void* q, int32_t batch, int32_t n_q_heads, float sm_scale,
+                                              void* out, float* lse_or_null, void* ws, size_t ws_bytes, int32_t lost_cta,
+                                              int32_t* n_ctas, int32_t* d_status, void* stream) {
+  if (!n_ctas) return SPECVLM_ERR_INVALID_ARG;
+  return attn_common(kv, q, batch, n_q_heads, 1, sm_scale, out, lse_or_null, ws, ws_bytes, d_status, stream, lost_cta, n_ctas);
 }
 
 extern "C" size_t specvlm_attn_workspace_bytes(const specvlm_kv_t* kv, int32_t batch,

@@ -14,6 +14,7 @@ struct AttnParams {
   int32_t batch, n_q, n_q_heads, n_kv_heads, group, rows;   // rows = group * n_q
   int32_t max_blocks, block_tokens, max_seq_len;
   float scale_log2;           // sm_scale * log2(e)
+  int32_t lost_cta;           // test hook: the CTA that gives up as if a wait had expired; -1 as a rule
 };
 
 }  // namespace specvlm

@@ -27,6 +27,7 @@ struct AttnTcParams {
   int32_t align;              // slices may keep to item boundaries (attn_sched.h): no more items than CTAs
   int32_t lse_block;          // floats from one 64-channel block's LSEs to the next one's
   float scale_log2;           // sm_scale * log2(e)
+  int32_t lost_cta;           // test hook (attn.cu): the CTA that gives up as if a wait had expired; -1 as a rule
 };
 
 constexpr float kRescaleThreshold = 8.f;   // log2 units
@@ -357,6 +358,7 @@ inline AttnTcParams slice_params(const specvlm_kv_t* kv, const void* q, int32_t 
   p.align = (int64_t)p.n_layers * batch * p.n_kv_heads <= sc.grid / n_parts && batch <= kSchedAlignedBatch;
   p.lse_block = 2 * sc.grid * p.rows;
   p.scale_log2 = sm_scale * kLog2e;
+  p.lost_cta = -1;
   return p;
 }
 

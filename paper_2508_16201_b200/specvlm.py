@@ -57,6 +57,7 @@ EXPORTS = [
     "specvlm_verify_tree_workspace_bytes", "specvlm_verify_tree_attn", "specvlm_accept_tree",
     "specvlm_compact_tree_kv", "specvlm_debug_poison_shared_memory", "specvlm_debug_wait_timeout",
     "specvlm_debug_set_attn_splits", "specvlm_debug_window_parts", "specvlm_debug_attn_merge",
+    "specvlm_debug_attn_give_up",
 ]
 
 
@@ -106,6 +107,9 @@ def lib():
         L.specvlm_debug_attn_merge.restype = c_int32
         L.specvlm_debug_attn_merge.argtypes = [kvp, c_int32, c_int32, c_int32, c_void_p, c_void_p, c_void_p, c_size_t,
                                                c_int32, i32p, c_void_p]
+        L.specvlm_debug_attn_give_up.restype = c_int32
+        L.specvlm_debug_attn_give_up.argtypes = [kvp, c_void_p, c_int32, c_int32, c_float, c_void_p, c_void_p, c_void_p, c_size_t,
+                                                 c_int32, i32p, c_void_p, c_void_p]
         L.specvlm_debug_set_attn_splits.restype = None
         L.specvlm_debug_set_attn_splits.argtypes = [c_int32]
         L.specvlm_verify_tree_workspace_bytes.restype = c_size_t
@@ -500,6 +504,17 @@ def debug_attn_merge(kv: KvCache, out: torch.Tensor, ws: torch.Tensor, lse: torc
     rc = lib().specvlm_debug_attn_merge(byref(kv.struct), B, Hq, NQ, _ptr(out), _ptr(lse), _ptr(ws), ws.numel(), int(lost_cta),
                                         byref(n), _stream())
     _check(rc, "specvlm_debug_attn_merge")
+    return n.value
+
+
+def debug_attn_give_up(kv: KvCache, q: torch.Tensor, sm_scale: float, out: torch.Tensor, lse: torch.Tensor, ws: torch.Tensor,
+                       d_status: torch.Tensor, lost_cta: int = -1) -> int:
+    """draft_decode_attn with one CTA giving up as if a wait of its had expired; returns the number of CTAs (test hook)."""
+    L, B, Hq, D = q.shape
+    n = c_int32()
+    rc = lib().specvlm_debug_attn_give_up(byref(kv.struct), _ptr(q), B, Hq, float(sm_scale), _ptr(out), _ptr(lse), _ptr(ws),
+                                          ws.numel(), int(lost_cta), byref(n), _ptr(d_status), _stream())
+    _check(rc, "specvlm_debug_attn_give_up")
     return n.value
 
 

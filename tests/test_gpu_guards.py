@@ -218,3 +218,48 @@ def test_items_with_a_part_that_was_given_up_are_left_alone(Hq, Hkv, gamma, D, l
         assert torch.equal(left, cut) and parts >= 2 * int(cut.sum())   # a cut item has parts in two CTAs at least
     finally:
         specvlm.debug_set_attn_splits(0)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("splits,lens", [(0, [1500, 700, 0, 100]),       # a cluster per item; two of them left to one CTA
+                                         (1, [1500, 40, 0, 300]),        # a CTA per item
+                                         (5, [1500, 40, 0, 900])])       # slices
+def test_decode_reports_a_cta_that_gives_up(splits, lens, paged, D):
+    """Every CTA in turn gives up as if a wait of its had expired: the call reports it if the CTA had work, stores nothing for
+    the items it has a part of (one item, or those of its slice), and everything else bit for bit.  No wait is made to
+    expire."""
+    L, Hkv, Hq, B = 1, 2, 8, len(lens)
+    cache, _, _ = make_cache(L, Hkv, D, [max(n, 1) for n in lens], paged=paged, seed=82)
+    cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    q = synth.randn_bf16((L, B, Hq, D), "cuda", 83, "Q")
+    specvlm.debug_set_attn_splits(splits)
+    try:
+        ws = torch.full((specvlm.attn_workspace_bytes(cache, B, Hq, 0),), 255, dtype=torch.uint8, device="cuda")
+
+        def run(cta):
+            out, lse, st = torch.full_like(q, 7.0), torch.full((L, B, Hq), 7.0, device="cuda"), _status()
+            n = specvlm.debug_attn_give_up(cache, q, 0.1, out, lse, ws, st, cta)
+            torch.cuda.synchronize()
+            return n, out, lse, int(st.item())
+
+        n, whole, whole_lse, st = run(-1)
+        assert st == 0 and torch.equal(whole, specvlm.draft_decode_attn(cache, q, 0.1, ws=ws)) and (whole_lse != 7.0).all()
+        lost = torch.zeros((B, Hkv), dtype=torch.int32)
+        for cta in range(n):
+            _, out, lse, st = run(cta)
+            stored = (out != 7.0).any(-1)
+            assert torch.equal(stored, lse != 7.0)
+            assert torch.equal(out[stored], whole[stored]) and torch.equal(lse[stored], whole_lse[stored])
+            items = stored.view(B, Hkv, Hq // Hkv)
+            assert torch.equal(items.any(-1), items.all(-1))
+            left = ~items.all(-1)
+            assert st == (specvlm.ERR_TIMEOUT if left.any() else 0)
+            assert left.any() or splits != 1 or lens[cta // Hkv] == 0           # a CTA per item: all but the empty sequence's
+            lost += left.cpu()
+        for b, length in enumerate(lens):
+            tiles = -(-length // 64)
+            parts = min(tiles, 1 if splits == 1 or (splits == 0 and tiles <= 4) else 2)
+            assert (lost[b] >= parts).all() and (parts > 1 or (lost[b] == parts).all()), (b, lost[b])
+    finally:
+        specvlm.debug_set_attn_splits(0)
