@@ -61,11 +61,12 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ 
   append_chunks(p);
 }
 
-// The same for what one CTA moves about as fast as the chip would, and the lengths behind its barrier instead of a second
-// launch, which costs the host 2.2 us and the stream 0.9: 6 tokens of one layer, 8 KV heads of d = 128 (768 chunks) 7.3 ->
-// 3.6 us of host time, 2.6 -> 2.9 on the device.  A cluster of eight CTAs was slower on the device beyond that
-// (3072 chunks 2.5 -> 3.4, 15 360 chunks 2.7 -> 5.3).
-constexpr int kAppendSmallThreads = 1024, kAppendSmallChunks = 2 * kAppendSmallThreads;
+// The same for what one CTA moves with a chunk a thread, and the lengths behind its barrier instead of a second launch,
+// which costs the host 3.4 us.  Device time of an append and a rollback, two launches / one: 128 chunks 3.30 / 2.86 us, 768
+// (6 tokens of one layer, 8 KV heads of d = 128) 3.39 / 3.28, 896 3.38 / 3.39, 1024 3.39 / 3.51, 1536 3.49 / 4.39, 2048
+// 3.43 / 4.62: beyond the line one SM's copies take longer than the launch.  A cluster of eight CTAs was slower on the
+// device too (3072 chunks 2.5 -> 3.4, 15 360 chunks 2.7 -> 5.3).
+constexpr int kAppendSmallThreads = 768, kAppendSmallChunks = kAppendSmallThreads;
 __global__ void __launch_bounds__(kAppendSmallThreads) append_small_kernel(const __grid_constant__ AppendParams p, int32_t* seq_lens) {
   pdl_launch_next();
   pdl_wait();

@@ -71,3 +71,16 @@ def host_view(t, table, seq_lens):
             seq = tc[:, blocks].permute(0, 2, 1, 3, 4).reshape(L, H, nb * BT, D)[:, :, :n, :]
         out.append(bits(seq.contiguous()))
     return out
+
+
+def launches(call):
+    """Number of kernels that `call` launches on the current stream, from a captured graph (which is not run)."""
+    from cuda.bindings import driver
+    call()                                                   # what is set up on a first call is not captured
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    err, _, n = driver.cuGraphGetNodes(driver.CUgraph(graph.raw_cuda_graph()))
+    assert int(err) == 0
+    return n

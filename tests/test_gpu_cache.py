@@ -8,7 +8,7 @@ import pytest
 import torch
 
 import oracle
-from gpu_util import host_view, make_cache
+from gpu_util import host_view, launches, make_cache
 from helpers import bits, f64, row_rel_err
 from paper_2508_16201_b200 import specvlm, synth
 
@@ -37,9 +37,10 @@ def test_append_bit_exact_and_lengths(paged):
         assert n == cap[b] and np.array_equal(gk[b], rk) and np.array_equal(gv[b], rv)
 
 
-@pytest.mark.parametrize("L,B,n_new", [(1, 1, 8), (1, 1, 9), (1, 2, 8), (1, 2, 9), (3, 2, 5)])
+@pytest.mark.parametrize("L,B,n_new", [(1, 1, 1), (1, 1, 6), (1, 1, 7), (1, 1, 8), (1, 1, 9), (1, 2, 3), (1, 2, 8), (1, 2, 9),
+                                       (3, 2, 5)])
 def test_append_one_cta_or_two_launches(L, B, n_new):
-    """8 KV heads x 16 chunks a row: 1024, 1152, 2048, 2304 and 3840 chunks, on both sides of what one CTA takes."""
+    """8 KV heads x 16 chunks a row: 128 to 3840 chunks, on both sides of the 768 that one CTA takes with a chunk a thread."""
     H, D = 8, 128
     lens = [70 - 9 * b for b in range(B)]
     cap = [n + n_new for n in lens]
@@ -52,6 +53,7 @@ def test_append_one_cta_or_two_launches(L, B, n_new):
     for b in range(B):
         assert np.array_equal(gk[b], oracle.append_kv(k_host[b], bits(new_k[:, b]), lens[b])[0])
         assert np.array_equal(gv[b], oracle.append_kv(v_host[b], bits(new_v[:, b]), lens[b])[0])
+    assert launches(lambda: specvlm.append_kv(cache, new_k, new_v)) == (1 if L * B * n_new * 128 <= 768 else 2)
 
 
 def test_append_without_room_is_reported_and_changes_nothing():
