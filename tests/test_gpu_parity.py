@@ -336,10 +336,12 @@ def test_accept_small_exact_loop_and_ties():
     assert int(g[0, 1]) == 13 and int(g[1, 0]) == 0 and int(g[1, 3]) == 255
 
 
-@pytest.mark.parametrize("rows,vocab", [(1, 1), (1, 4096), (1, 4097), (8, 4096), (8, 4095), (9, 4096), (6, 1024), (7, 31), (5, 33)])
-def test_accept_one_cluster_or_two_launches(rows, vocab):
-    """Up to eight rows of 4096 logits go in one launch: both sides of the line, rows that start off a 16-byte boundary, ties."""
-    B = 3
+@pytest.mark.parametrize("rows,vocab,B", [(1, 1, 3), (1, 4096, 3), (1, 4097, 3), (8, 4096, 3), (8, 4095, 3), (9, 4096, 3), (6, 1024, 3),
+                                          (7, 31, 3), (5, 33, 3), (6, 1024, 24), (6, 1024, 25), (1, 100, 24), (1, 100, 25)])
+def test_accept_one_cluster_or_two_launches(rows, vocab, B):
+    """Up to eight rows of 4096 logits of up to 24 sequences go in one launch: both sides of the lines, rows that start off a
+    16-byte boundary, ties."""
+    from gpu_util import launches
     x = torch.randn((B, rows, vocab), generator=torch.Generator().manual_seed(rows * 131 + vocab))
     x[0, 0, vocab - 1] = x[0, 0, 0] = 9.0                             # the lower index wins
     am = x.numpy().argmax(2)
@@ -349,13 +351,18 @@ def test_accept_one_cluster_or_two_launches(rows, vocab):
         drafts[2, rows // 2 - 1] += 1                                 # and in the middle
     n, nxt, g = specvlm.accept(x.cuda(), torch.from_numpy(drafts).cuda(), want_argmax=True)
     assert np.array_equal(g.cpu().numpy(), am)
-    want = [rows - 1, 0, 0 if rows == 1 else rows // 2 - 1]
+    want = [rows - 1, 0, 0 if rows == 1 else rows // 2 - 1] + [rows - 1] * (B - 3)
     assert n.cpu().tolist() == want and nxt.cpu().tolist() == [int(am[b, want[b]]) for b in range(B)]
     par = torch.tensor([[t - 1 for t in range(rows)]] * B, dtype=torch.int32, device="cuda")     # the chain as a tree
     tok = torch.from_numpy(np.concatenate([np.zeros((B, 1), np.int32), drafts], 1)).cuda()
     tn, tnxt, path, tg = specvlm.accept_tree(x.cuda(), tok, par, want_argmax=True)
     assert torch.equal(tn, n) and torch.equal(tnxt, nxt) and torch.equal(tg, g)
     assert path.cpu().tolist() == [list(range(1, k + 1)) + [-1] * (rows - 1 - k + 1) for k in want]
+    x, d = x.cuda(), torch.from_numpy(drafts).cuda()
+    one = rows <= 8 and vocab <= 4096 and B <= 24
+    bufs = specvlm.accept_tree_buffers(B, rows, vocab, "cuda")
+    assert launches(lambda: specvlm.accept(x, d, ws=bufs[4])) == (1 if one else 2)
+    assert launches(lambda: specvlm.accept_tree(x, tok, par, out=bufs)) == (1 if one else 2)
 
 
 # ------------------------------------------------------------------------------- select
