@@ -88,6 +88,65 @@ def test_tree_bad_parents_are_reported():
     assert int(status.item()) == specvlm.ERR_INVALID_ARG
 
 
+BAD_TREES = [(4, 2, 4, 1),          # 8 rows
+             (8, 8, 41, 37),        # 41 rows, the fault among the nodes 32..: the second half of the parents
+             (64, 8, 16, 9),        # 128 rows
+             (64, 8, 26, 5), (64, 8, 26, 20),       # 208 rows, the fault in the first and in the second part
+             (28, 4, 64, 50)]       # four parts
+
+
+def _bad_tree(rng, n_nodes, bad, late):
+    """A tree in which node `bad` names itself or a later node as its parent, and the parents that amount to the same: a node
+    whose path meets the fault sees itself only."""
+    par = _random_tree(rng, n_nodes)
+    par[bad] = min(bad + 1, n_nodes - 1) if late else bad
+    par[n_nodes - 1] = bad                                            # a child below the fault
+    seen = list(par)
+    for t in range(n_nodes):
+        at = t
+        while at >= 0 and par[at] < at:
+            at = par[at]
+        if at >= 0:
+            seen[t] = -1
+    return par, seen
+
+
+@pytest.mark.parametrize("late", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,n_nodes,bad", BAD_TREES)
+def test_a_node_below_a_bad_parent_sees_itself_only(Hq, Hkv, n_nodes, bad, late):
+    D, lens = 64, [40 + n_nodes, 130 + n_nodes]
+    rng = np.random.default_rng(67)
+    cache, k_host, v_host = make_cache(1, Hkv, D, lens, paged=True, seed=67, poison_tail=True)
+    good = _random_tree(rng, n_nodes)
+    par, seen = _bad_tree(rng, n_nodes, bad, late)
+    assert seen.count(-1) > 2
+    q = synth.randn_bf16((1, 2, n_nodes, Hq, D), "cuda", 67, "Qt")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = specvlm.verify_tree_attn(cache, q, torch.tensor([good, par], dtype=torch.int32, device="cuda"), 0.125, d_status=status)
+    assert int(status.item()) == specvlm.ERR_INVALID_ARG
+    for b, parents in enumerate((good, seen)):
+        ref, _ = oracle.attention_tree(bits(q)[0, b], k_host[b][0], v_host[b][0], lens[b], parents, 0.125)
+        assert row_rel_err(f64(out[0, b]), ref) <= 1e-2
+
+
+@pytest.mark.parametrize("Hq,Hkv,n_nodes,bad", BAD_TREES)
+def test_bad_parents_of_an_empty_sequence_are_reported(Hq, Hkv, n_nodes, bad):
+    """Its nodes are in no tile: the tree is looked at for the report alone."""
+    rng = np.random.default_rng(68)
+    cache, _, _ = make_cache(1, Hkv, 64, [100 + n_nodes, 1], paged=False, seed=68)
+    cache.seq_lens[1] = 0
+    good = _random_tree(rng, n_nodes)
+    q = synth.randn_bf16((1, 2, n_nodes, Hq, 64), "cuda", 68, "Qt")
+    outs = []
+    for par, expect in ((good, 0), (_bad_tree(rng, n_nodes, bad, True)[0], specvlm.ERR_INVALID_ARG)):
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        outs.append(specvlm.verify_tree_attn(cache, q, torch.tensor([good, par], dtype=torch.int32, device="cuda"), 0.125,
+                                             d_status=status))
+        assert int(status.item()) == expect
+        assert (outs[-1][0, 1] == 0).all()
+    assert torch.equal(*outs)
+
+
 @pytest.mark.parametrize("batch,n_nodes,vocab", [(1, 26, 152064), (5, 9, 4099), (16, 32, 1000), (3, 64, 4099), (2, 47, 152064)])
 def test_tree_accept_bit_exact(batch, n_nodes, vocab):
     rng = np.random.default_rng(63)
