@@ -714,8 +714,8 @@ static double rows16_tile_us(const specvlm_kv_t* kv) {
 }
 
 // CTAs per item of a launch without slices: the number that is the fastest where every CTA has an SM of its own.  The
-// hand-over costs 1.3 us: one layer of 4 items of 200 tokens 3.7 us with a CTA each, 4.3 with two; of 755 / 1600 / 3200
-// tokens 6.5 / 9.1 / 16 with one (7.4 / 8.3 on slices from 1600) and 4.4 / 5.0 / 6.3 with eight.  Clusters do not use
+// hand-over costs 1.3 us: one layer of 4 items of 200 tokens 3.7 us with a CTA each, 4.3 with two; of 800 / 1600 / 3200
+// tokens 7.0 / 11.3 / 20.1 with one (7.4 / 8.5 on slices from 1600) and 4.4 / 5.0 / 6.3 with eight.  Clusters do not use
 // every SM of a GPC: 16 of eight CTAs no longer run side by side (4 layers of 800 tokens 7.3 -> 8.4), 24 of four do (2 layers
 // x 3 sequences of 800 tokens 8.0 -> 5.4).
 static int rows16_cluster(const specvlm_kv_t* kv, int64_t items, int64_t tiles) {

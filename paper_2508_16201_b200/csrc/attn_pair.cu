@@ -18,14 +18,18 @@
 // What bounds it: per tile and SM two parts cost 32 UMMAs of 64 cycles and 2 x 128 exponentials per
 // thread, 2048 cycles each of the tensor pipe and of a scheduler's special-function unit, against about
 // 2500 cycles in which HBM delivers the tile; a part's chain Q K^T -> softmax -> P V is serial (one S
-// buffer per part fits the tensor memory), 4000 cycles of which the two parts overlap.  26 nodes at 8 heads
-// per KV head, 80 layers of 6400 tokens (each part used to stream K and V on a set of CTAs of its own): 642 ->
-// 554 us, 827 -> 677 us under sustained load at the power cap.  What it took, same case: the parts in step
-// (both softmaxes, then both waiting for the tensor pipe) 684 us; taking turns 610; the next S issued before
-// the bookkeeping commits, waits that test before they suspend, and P handed over in two halves 554 (in 96 and 32
-// tokens, sustained 651 -> 643 us); products issued by an
-// elected lane of a whole warp instead of by lane 0 (of 4310 cycles a tile the issuers took 2750) 3700 cycles, sustained
-// 669 -> 648 us.  A share of the exponentials on the FMA pipe is slower (2 / 4 of 16 pairs: 571 / 604 us).
+// buffer per part fits the tensor memory), some 3700 cycles of which the two parts overlap.
+//
+// 26 nodes at 8 heads per KV head, 80 layers of 6400 tokens, cool / under sustained load at the power cap, in us:
+//   a set of CTAs per part, each streaming K and V                                        642 / 827
+//   two parts a CTA, in step (both softmaxes, then both waiting for the tensor pipe)      684
+//   taking turns                                                                          610
+//   the next S issued before the bookkeeping commits, waits that test before they
+//   suspend, P handed over in two halves                                                  554 / 677
+//   products issued by an elected lane of a whole warp instead of by lane 0 (of 4310
+//   cycles a tile the issuers took 2750; then 3700)                                       548 / 648 (669 before, same box)
+//   P handed over as 96 and 32 tokens                                                           643 (651)
+// A share of the exponentials on the FMA pipe is slower (2 / 4 of 16 pairs: 571 / 604 against 554).
 #include "attn_tc.cuh"
 
 namespace specvlm {

@@ -7,6 +7,8 @@
 // number of tiles (+-1) and an item is cut only where a slice boundary falls inside it.  A CTA's
 // slice is a sequence of "segments" (maximal runs inside one item); only its first and its last
 // segment can be partial, which bounds the scratch memory to two partial results per CTA.
+// Where the items are fewer than the CTAs the slices keep to item boundaries instead (aligned_slice): one
+// segment a CTA, the tiles as even as the items allow.
 #pragma once
 #include <stdint.h>
 

@@ -286,8 +286,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
   } else if (warp == 2) {
     // ================================================================ O += P V issuer
-    // The whole warp walks the slice; one lane issues.  The others lend a hand where a sequence ends inside a sub-tile, the V rows past its end hold
-    // whatever the page held, and are cleared so that a zero probability times a stale non-finite
+    // The whole warp walks the slice; one lane issues.  The others lend a hand where a sequence ends inside a sub-tile: the V
+    // rows past its end hold whatever the page held, and are cleared so that a zero probability times a stale non-finite
     // value cannot reach O.
     setmaxnreg_dec<kRegsLight>();
     if (active) {

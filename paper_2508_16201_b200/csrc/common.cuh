@@ -150,14 +150,14 @@ __device__ __forceinline__ void fence_proxy_async() {
 }
 
 // True in one lane of the (whole, converged) warp, the same one every time.  What a warp issues for itself -- tensor
-// instructions, their commits, TMA copies -- goes behind this in code that all of its lanes run: in a branch of
-// `lane == 0` the compiler takes the operands for different in each lane and moves them to the uniform registers that
-// these instructions read one instruction at a time.  Eight tcgen05.mma of fixed operands: 402 cycles to
-// issue behind `lane == 0`, 133 behind this; with operands that change from tile to tile 760 in the first form.
-// Verification, sustained, at 80 layers of 6400 tokens: a tree of 208 rows 669 -> 648 us (4310 -> 3700 cycles a
-// tile), 48 rows 360 -> 353.5; 40 layers x 4 sequences, 72 rows 1974 -> 1954.  Not in the rating passes, whose
-// issuer is never late: 32 polling lanes there cost 0.6 to 1 % at the power cap; nor for the copies of the decode kernel with a CTA per item (even), but on slices
-// (9 layers of 16 sequences, d = 64, 56.0 -> 54.9 us; 13 layers of 43 856 tokens, 16 rows, 598 -> 594).
+// instructions, their commits, TMA copies -- goes behind this in code that all of its lanes run, and not into a branch of
+// `lane == 0`: eight tcgen05.mma of fixed operands take 402 cycles to issue there and 133 behind this; with operands that
+// change from tile to tile 760 in the first form.  (Why was not looked into: the operands are in uniform registers, and
+// presumably the compiler can keep them there only where no lane stands out.)  Verification, sustained, at 80 layers of 6400
+// tokens: a tree of 208 rows 669 -> 648 us (4310 -> 3700 cycles a tile), 48 rows 360 -> 353.5.  Not in the rating passes,
+// whose issuer is never late: 32 polling lanes there cost 0.6 to 1 % at the power cap; nor for the copies of the decode kernel
+// with a CTA per item (even), but on slices (9 layers of 16 sequences, d = 64, 56.0 -> 54.9 us; 13 layers of 43 856 tokens,
+// 16 rows, 598 -> 594).
 __device__ __forceinline__ bool elect_one() {
   uint32_t e;
   asm volatile(

@@ -571,7 +571,9 @@ __global__ void scores_finish_kernel(const __grid_constant__ ScoreParams p, floa
   if (j >= p.sum_video) return;
   int b = 0;
   while (b + 1 < p.batch && p.seq[b + 1].score_off <= j) ++b;
-  // sixteen layers' loads in flight: with the compiler's four a thread of 80 layers waited twenty times for L2
+  // sixteen layers' loads in flight (this kernel alone in a replayed graph: 80 layers of 6272 scores 2.87 -> 2.57 us, 64 of
+  // 23 040 2.57 -> 2.36, one layer even; nothing that shows beside the passes): with the compiler's four a thread of 80
+  // layers waited twenty times for L2
   constexpr int kFlight = 16;
   float acc = 0.f;
   const float* const part = p.partial + j;
