@@ -379,7 +379,7 @@ constexpr int kSoloTiles = 4, kSoloTilesPair = 6;
 // (CTAs per SM are as many as the ring allows; without that the compiler held d = 64 to 96 registers and spilled: 6 layers of
 // 800 tokens, 24 items, 4.4 -> 4.2 us, 112 items of d = 128 and 755 tokens 9.83 -> 9.65)
 template <int D, int STAGES, int NG, bool SPLIT>
-__global__ void __launch_bounds__(32 * (4 * NG + 1), NG == 2 ? 1 : 2)
+__global__ void __launch_bounds__(32 * (4 * NG + 1), NG == 2 ? 1 : D == 64 ? 4 : 2)
 attn_rows16_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                    const AttnParams p) {
   constexpr int TILE_BYTES = kTileTokens * D * 2;
