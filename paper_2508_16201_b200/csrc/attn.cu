@@ -775,14 +775,16 @@ static int rows16_slices(const specvlm_kv_t* kv, int32_t batch, int* scratch_cta
   *scratch_ctas = sched_scratch_ctas(items * tiles, (int)sms);
   const int n = rows16_cluster(kv, items, tiles);
   if (n > 1) {
-    // A cluster per item, 3.9 us around its CTAs' tiles or the bytes, against slices, 6.5 us around the bytes.  Measured,
-    // cluster / slices: 12 items of 640 / 2560 / 10 240 tokens 4.9 / 7.3 / 18.5 against 7.0 / 8.3 / 16.4; 16 paged ones of
-    // 2560 / 5120 / 10 240 8.3 / 13.4 / 23.9 against 9.0 / 10.8 / 15.7; 64 of 1280 / 2560 / 5120 / 10 240 7.5 / 15.3 / 28.4 /
-    // 52.6 against 11.0 / 20.5 / 31.8 / 55.0; 72 ragged ones of up to 1280 / 2560 / 10 240 7.5 / 11.3 / 47.2 against 12.9 /
-    // 16.1 / 48.3.
+    // A cluster per item, 3.9 us around its CTAs' tiles or the bytes, which half the SMs do not stream as well, against
+    // slices, 6.5 us around the bytes (in pages 6) and more for many parts an item.  Measured, cluster / slices: 1 item
+    // (d = 64) of 10 240 tokens 8.5 / 11.6; 12 items of 640 / 2560 / 10 240 4.9 / 7.3 / 18.5 against 7.0 / 8.3 / 16.4; 16 paged ones of 2560 / 5120 /
+    // 10 240 8.3 / 13.4 / 23.9 against 9.0 / 10.8 / 15.7; 40 of 2560 / 10 240 / 20 480 11.3 / 38.8 / 75.5 against 14.2 / 37.3 /
+    // 64.7; 64 of 1280 / 2560 / 5120 / 10 240 7.5 / 15.3 / 28.4 / 52.6 against 11.0 / 20.5 / 31.8 / 55.0; 72 ragged ones of up to
+    // 1280 / 2560 / 10 240 7.5 / 11.3 / 47.2 against 12.9 / 16.1 / 48.3.
     const double hbm = (double)items * tiles * (256.0 * kv->head_dim) / 6.65e6, ragged = batch > 1 ? 0.85 : 1.0;
     const double longest = 1.08 * rows16_tile_us(kv) * ((tiles + n - 1) / n);
-    if (6.5 + ragged * hbm >= 3.9 + (longest > hbm ? longest : hbm)) return 0;
+    const double parts = (double)(items * tiles < sms ? items * tiles : sms) / items;
+    if ((kv->block_table ? 6.0 : 6.5) + ragged * hbm + 0.04 * parts >= 3.9 + (longest > 1.05 * hbm ? longest : 1.05 * hbm)) return 0;
   }
   const int even = sched_active_ctas(items * tiles, (int)sms);
   // slices that keep to item boundaries may use more CTAs: every item rounds its own up

@@ -156,7 +156,7 @@ def test_decode_with_a_cluster_per_item_and_an_empty_sequence():
     (3, 2560, False, False), (3, 10240, False, True),        # 12 items: clusters of four 7.3 / 18.5 us, slices 8.3 / 16.4
     (4, 2560, True, False), (4, 5120, True, True),           # 16 paged ones: 8.3 / 13.4, slices 9.0 / 10.8
     (14, 2560, False, False), (16, 5120, False, False),      # clusters of two 14.0 / 28.4, slices 18.3 / 31.8
-    (18, 2560, False, False), (18, 10240, False, False)])    # 16.3 / 57.8, slices 20.4 / 61.0
+    (18, 2560, False, False), (10, 20480, False, True)])     # 16.3, slices 20.4; 75.5, slices 64.7
 def test_decode_takes_the_faster_of_cluster_and_slices(L, tokens, paged, slices):
     """Which of the two runs is seen from whether the call has a second kernel."""
     if paged:
