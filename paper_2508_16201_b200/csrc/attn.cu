@@ -784,7 +784,7 @@ static int rows16_slices(const specvlm_kv_t* kv, int32_t batch, int* scratch_cta
     const double hbm = (double)items * tiles * (256.0 * kv->head_dim) / 6.65e6, ragged = batch > 1 ? 0.85 : 1.0;
     const double longest = 1.08 * rows16_tile_us(kv) * ((tiles + n - 1) / n);
     const double parts = (double)(items * tiles < sms ? items * tiles : sms) / items;
-    if ((kv->block_table ? 6.0 : 6.5) + ragged * hbm + 0.04 * parts >= 3.9 + (longest > 1.05 * hbm ? longest : 1.05 * hbm)) return 0;
+    if ((kv->block_table ? 6.0 : 6.5) + ragged * hbm + 0.04 * parts >= 3.9 + (longest > 1.09 * hbm ? longest : 1.09 * hbm)) return 0;
   }
   const int even = sched_active_ctas(items * tiles, (int)sms);
   // slices that keep to item boundaries may use more CTAs: every item rounds its own up
