@@ -61,17 +61,23 @@ __global__ void __launch_bounds__(256) append_kv_kernel(const __grid_constant__ 
   append_chunks(p);
 }
 
-// The same for what one CTA moves with a chunk a thread, and the lengths behind its barrier instead of a second launch,
-// which costs the host 3.4 us.  Device time of an append and a rollback, two launches / one: 128 chunks 3.30 / 2.86 us, 768
-// (6 tokens of one layer, 8 KV heads of d = 128) 3.39 / 3.28, 896 3.38 / 3.39, 1024 3.39 / 3.51, 1536 3.49 / 4.39, 2048
-// 3.43 / 4.62: beyond the line one SM's copies take longer than the launch.  A cluster of eight CTAs was slower on the
-// device too (3072 chunks 2.5 -> 3.4, 15 360 chunks 2.7 -> 5.3).
-constexpr int kAppendSmallThreads = 768, kAppendSmallChunks = kAppendSmallThreads;
+// The same for what one CTA, or a cluster of up to three, moves with a chunk a thread, and the lengths behind its barrier
+// instead of a second launch, which costs the host 3.4 us.  Device time of an append and a rollback, two launches / one:
+// 128 chunks 3.30 / 2.77 us, 768 (6 tokens of one layer, 8 KV heads of d = 128) 3.38 / 3.18; with more than a CTA 1152 3.39 /
+// 3.78, 1536 3.59 / 3.89, 2048 3.40 / 3.90 (in one CTA, two chunks a thread, 3.99 / 4.39 / 4.62): there it pays where the host
+// is the one that is waited for, and not in a graph.  A cluster of eight was slower yet (3072 chunks 2.5 -> 3.4).
+constexpr int kAppendSmallThreads = 768, kAppendSmallCtas = 3;
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kAppendSmallThreads) append_small_kernel(const __grid_constant__ AppendParams p, int32_t* seq_lens) {
   pdl_launch_next();
   pdl_wait();
   append_chunks(p);
-  __syncthreads();                         // every thread has read the lengths
+  if constexpr (CLUSTER) {                 // every thread has read the lengths
+    cluster_barrier();
+    if (blockIdx.x != 0) return;
+  } else {
+    __syncthreads();
+  }
   for (int b = threadIdx.x; b < p.batch; b += kAppendSmallThreads) {
     const int n = seq_lens[b];
     if (n >= 0 && n + p.n_new <= p.max_seq_len) seq_lens[b] = n + p.n_new;
@@ -214,13 +220,16 @@ extern "C" int32_t specvlm_append_kv(const specvlm_kv_t* kv, const void* new_k, 
   p.n_layers = c.n_layers; p.batch = batch; p.n_new = n_new; p.n_kv_heads = c.n_kv_heads;
   p.chunks_per_row = c.head_dim / 8;
   const int64_t total = (int64_t)p.n_layers * batch * n_new * p.n_kv_heads * p.chunks_per_row;
-  if (total <= kAppendSmallChunks)
-    return launch_after(append_small_kernel, dim3(1), dim3(kAppendSmallThreads), 0, static_cast<cudaStream_t>(stream), p,
-                        seq_lens_inout);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const int64_t small = (total + kAppendSmallThreads - 1) / kAppendSmallThreads;
+  if (small == 1)
+    return launch_after(append_small_kernel<false>, dim3(1), dim3(kAppendSmallThreads), 0, st, p, seq_lens_inout);
+  if (small <= kAppendSmallCtas && !being_captured(st))
+    return launch_clusters_after(append_small_kernel<true>, dim3((unsigned)small), (int)small, dim3(kAppendSmallThreads), 0, st, p,
+                                 seq_lens_inout);
   int64_t blocks = (total + 255) / 256;
   const int64_t cap = (int64_t)sm_count() * 8;
   if (blocks > cap) blocks = cap;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   rc = launch_after(append_kv_kernel, dim3((unsigned)blocks), dim3(256), 0, st, p);
   if (rc != SPECVLM_OK) return rc;
   // the lengths change only after every row has been placed by the kernel above

@@ -91,6 +91,16 @@ inline int32_t launch_status() {
   return cudaGetLastError() == cudaSuccess ? SPECVLM_OK : SPECVLM_ERR_CUDA;
 }
 
+// Whether launches on the stream go into a graph, whose replays cost no launch of the host's.
+inline bool being_captured(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();                    // the default stream beside a capture: not ours to report
+    return false;
+  }
+  return status != cudaStreamCaptureStatusNone;
+}
+
 // Launches `kern` so that it may be scheduled while the kernel before it in the stream still runs
 // (programmatic stream serialization), in clusters of `cluster` CTAs along x.  The kernel itself has to wait
 // (griddepcontrol.wait) for that kernel's completion, in every CTA and before its first access to global memory.

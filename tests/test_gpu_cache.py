@@ -40,7 +40,8 @@ def test_append_bit_exact_and_lengths(paged):
 @pytest.mark.parametrize("L,B,n_new", [(1, 1, 1), (1, 1, 6), (1, 1, 7), (1, 1, 8), (1, 1, 9), (1, 2, 3), (1, 2, 8), (1, 2, 9),
                                        (3, 2, 5)])
 def test_append_one_cta_or_two_launches(L, B, n_new):
-    """8 KV heads x 16 chunks a row: 128 to 3840 chunks, on both sides of the 768 that one CTA takes with a chunk a thread."""
+    """8 KV heads x 16 chunks a row: 128 to 3840 chunks, on both sides of the 768 that one CTA takes with a chunk a thread
+    and of the 2304 that a cluster of three does, which a graph does not take."""
     H, D = 8, 128
     lens = [70 - 9 * b for b in range(B)]
     cap = [n + n_new for n in lens]
