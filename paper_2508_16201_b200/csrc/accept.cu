@@ -138,9 +138,11 @@ __device__ __forceinline__ void walk_tree(const int* g_sm, const int32_t* node_t
 // 2.87 / 2.26 us for one sequence, 2.98 / 2.58 for 16; 8 rows of 4096 3.18 / 2.95 for 24, 3.17 / 3.21 for 32, 3.59 / 3.94
 // for 48; 1 row, seven of whose eight CTAs have none, 2.77 / 2.53 for 24, 2.77 / 3.84 for 64, 4.3 / 10.7 for 512.  With 8000
 // logits a row, a whole chunk for a CTA, the device would take 4.1 us instead of 2.6.
-constexpr int kAcceptSmallRows = 8, kAcceptSmallVocab = kAcceptChunk / 2, kAcceptSmallBatch = 24;
-static bool accept_small(int batch, int rows, int vocab) {
-  return rows <= kAcceptSmallRows && vocab <= kAcceptSmallVocab && batch <= kAcceptSmallBatch;
+// Up to 64 sequences the host's launch is longer than what the device loses, but in a graph.
+constexpr int kAcceptSmallRows = 8, kAcceptSmallVocab = kAcceptChunk / 2, kAcceptSmallBatch = 24, kAcceptSmallBatchEager = 64;
+static bool accept_small(int batch, int rows, int vocab, cudaStream_t st) {
+  return rows <= kAcceptSmallRows && vocab <= kAcceptSmallVocab &&
+         (batch <= kAcceptSmallBatch || (batch <= kAcceptSmallBatchEager && !being_captured(st)));
 }
 __global__ void __launch_bounds__(kAcceptThreads)
 accept_small_kernel(const float* logits, int vocab, int rows, const int32_t* tokens, const int32_t* parents,
@@ -241,7 +243,7 @@ extern "C" int32_t specvlm_accept(const float* target_logits, const int32_t* dra
   if (ws_bytes < specvlm_accept_workspace_bytes(batch, gamma, vocab)) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
   const int n_chunks = (vocab + kAcceptChunk - 1) / kAcceptChunk;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (accept_small(batch, gamma + 1, vocab))
+  if (accept_small(batch, gamma + 1, vocab, st))
     return launch_accept_small(target_logits, vocab, batch, gamma + 1, draft_tokens, nullptr, accept_len, next_token,
                                nullptr, target_argmax_or_null, st);
   Cand* part = static_cast<Cand*>(ws);
@@ -308,7 +310,7 @@ extern "C" int32_t specvlm_accept_tree(const float* target_logits, const int32_t
   if (ws_bytes < specvlm_accept_workspace_bytes(batch, n_nodes - 1, vocab)) return SPECVLM_ERR_WORKSPACE_TOO_SMALL;
   const int n_chunks = (vocab + kAcceptChunk - 1) / kAcceptChunk;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (accept_small(batch, n_nodes, vocab))
+  if (accept_small(batch, n_nodes, vocab, st))
     return launch_accept_small(target_logits, vocab, batch, n_nodes, node_tokens, parents, accept_len, next_token, path,
                                target_argmax_or_null, st);
   Cand* part = static_cast<Cand*>(ws);

@@ -337,10 +337,10 @@ def test_accept_small_exact_loop_and_ties():
 
 
 @pytest.mark.parametrize("rows,vocab,B", [(1, 1, 3), (1, 4096, 3), (1, 4097, 3), (8, 4096, 3), (8, 4095, 3), (9, 4096, 3), (6, 1024, 3),
-                                          (7, 31, 3), (5, 33, 3), (6, 1024, 24), (6, 1024, 25), (1, 100, 24), (1, 100, 25)])
+                                          (7, 31, 3), (5, 33, 3), (6, 1024, 24), (6, 1024, 25), (1, 100, 24), (1, 100, 25), (8, 1024, 64), (8, 1024, 65)])
 def test_accept_one_cluster_or_two_launches(rows, vocab, B):
-    """Up to eight rows of 4096 logits of up to 24 sequences go in one launch: both sides of the lines, rows that start off a
-    16-byte boundary, ties."""
+    """Up to eight rows of 4096 logits of up to 24 sequences go in one launch, of up to 64 outside a graph: both sides of the
+    lines, rows that start off a 16-byte boundary, ties."""
     from gpu_util import launches
     x = torch.randn((B, rows, vocab), generator=torch.Generator().manual_seed(rows * 131 + vocab))
     x[0, 0, vocab - 1] = x[0, 0, 0] = 9.0                             # the lower index wins
